@@ -84,6 +84,10 @@ struct ising_ctx {
   unsigned long long* rec = nullptr;  // [kRecCap][2]: anti-bond count, up-spin count
   int64_t rec_count = 0;
   unsigned long long* meas = nullptr;  // [2]
+  // resident strips (the automatic choice where they are the fastest; G = 0: not used)
+  StripShape strip{0, 0, 0.0};
+  unsigned long long* strip_x = nullptr;  // boundary exchange buffer (G > 1)
+  int* strip_status = nullptr;            // pinned host word a strip sets when a wait gave up
   int kernel = ISING_KERNEL_HALF, k = 1, tile_rows = 1, tile_words = 4, grid = 0, block = 0;
   __nv_bfloat16* nn_w = nullptr;    // BF16 weights of the block proposal
   __nv_bfloat16* nn_w2t = nullptr;
@@ -137,6 +141,10 @@ void free_all(ising_ctx* c) {
   cudaFree(c->spins);
   cudaFree(c->rec);
   cudaFree(c->meas);
+  cudaFree(c->strip_x);
+  cudaFreeHost(c->strip_status);
+  c->strip_x = nullptr;
+  c->strip_status = nullptr;
   cudaFree(c->nn_w);
   cudaFree(c->nn_w2t);
   cudaFree(c->blk_stats);
@@ -165,6 +173,16 @@ bool beta_ok(double beta) { return std::isfinite(beta) && beta > 0.0; }
 int check_ctx(ising_ctx* c) {
   if (!c) return fail(ISING_EINVAL, "null context");
   return ISING_OK;
+}
+
+// Where the resident strips are the automatic choice: everywhere they fit in
+// shared memory, except lattices from 6144 up that tile into 32-word tiles
+// (flips/ns, strips against the best tiled shape: L = 2048 1220 / 709, 4096
+// 2057 / 1627, 6144 2384 / 2192, 8192 2569 / 2706).  The other automatic paths
+// there, one launch per half sweep or per sweep, gave 115 at L = 1000 and 200 at
+// L = 2048; one CTA with int8 spins 0.25 at L = 64 (strips: 7).
+bool strip_applies(int layout, int L) {
+  return layout == ISING_LAYOUT_I8 || L <= 6144 || words_per_row(L) % 32 != 0 || L % 64 != 0;
 }
 
 // Kernel configuration validity for this lattice.
@@ -199,7 +217,24 @@ int validate_kernel(const ising_ctx* c, int kernel, int k, int tile_rows, int ti
   return fail(ISING_EINVAL, "kernel %d does not apply to the int8 layout", kernel);
 }
 
+// Buffers of the strips' boundary exchange, once per context.
+int ensure_strip(ising_ctx* c) {
+  if (c->strip.G <= 1 || c->strip_x) return ISING_OK;
+  void* p = nullptr;
+  int st = dev_alloc(&p, strip_xbuf_words(c->L, c->strip.G, c->strip.K) * sizeof(unsigned long long));
+  if (st) return st;
+  c->strip_x = (unsigned long long*)p;
+  cudaError_t e = cudaHostAlloc((void**)&c->strip_status, sizeof(int), cudaHostAllocDefault);
+  if (e != cudaSuccess) {
+    c->strip_status = nullptr;
+    return fail(ISING_ENOMEM, "pinned status word: %s", cudaGetErrorString(e));
+  }
+  *c->strip_status = 0;
+  return ISING_OK;
+}
+
 void resolve_auto(ising_ctx* c) {
+  c->strip = strip_applies(c->layout, c->L) ? choose_strip(c->L, c->sms) : StripShape{0, 0, 0.0};
   if (c->layout == ISING_LAYOUT_BITS) {
     if (c->Wc % 4 == 0 && c->L % 64 == 0 && c->L >= 256) {
       c->kernel = ISING_KERNEL_TILED;
@@ -297,7 +332,27 @@ int sweep_chunk(ising_ctx* c, int64_t t0, int n, int m) {
   const RngParams rng = c->rng();
   if (fault("launch")) return fail(ISING_ECUDA, "sweep launch failed (injected)");
 
-  if (c->layout == ISING_LAYOUT_BITS && c->kernel == ISING_KERNEL_HALF) {
+  if (c->strip.G > 0) {
+    Timed tm(c);
+    StripArgs a{};
+    a.planes = c->layout == ISING_LAYOUT_BITS ? c->bits[c->cur] : nullptr;
+    a.spins = c->layout == ISING_LAYOUT_BITS ? nullptr : c->spins;
+    a.L = c->L;
+    a.Wc = c->Wc;
+    a.G = c->strip.G;
+    a.K = c->strip.K;
+    a.t0 = (uint32_t)t0;
+    a.n = n;
+    a.m = m;
+    a.to_rec = first_t < 0 ? 0 : (int)(first_t - t0 + 1);
+    a.rec0 = rec0 % kRecCap;
+    a.rec_cap = kRecCap;
+    a.rec = c->rec;
+    a.xbuf = c->strip_x;
+    a.status = c->strip_status;
+    a.limit = kClusterSpinLimit;
+    if (int st = launch_result(c, launch_strip_sweep(a, rng, c->stream), "strip sweep")) return st;
+  } else if (c->layout == ISING_LAYOUT_BITS && c->kernel == ISING_KERNEL_HALF) {
     for (int64_t t = t0; t < t0 + n; ++t) {
       const int64_t sl = slot_of(t);
       for (int col = 0; col < 2; ++col) {
@@ -352,6 +407,8 @@ int to_host_sync(ising_ctx* c, void* dst, const void* src, size_t bytes) {
   if (fault("copy")) return fail(ISING_ECUDA, "device-to-host copy failed (injected)");
   CUDA_TRY(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(cudaStreamSynchronize(c->stream));
+  if (c->strip_status && *(volatile int*)c->strip_status)
+    return fail(ISING_ETIMEOUT, "a strip's wait for its neighbour timed out");
   if (c->cluster_gctl) {
     // a grid barrier of the persistent cluster kernel that gave up stays recorded until the next seed
     int status = 0;
@@ -431,7 +488,8 @@ int ising_create(ising_ctx** out, int L, double beta, int layout, void* stream) 
   }
   if (!st) {
     resolve_auto(c);
-    if (c->kernel == ISING_KERNEL_TILED) st = ensure_second_buffer(c);
+    st = ensure_strip(c);
+    if (!st && c->kernel == ISING_KERNEL_TILED && c->strip.G == 0) st = ensure_second_buffer(c);
   }
   if (!st) {
     // all -1 start: zero bits / int8 0xff
@@ -467,6 +525,7 @@ int ising_seed(ising_ctx* c, uint64_t seed) {
   c->rec_count = 0;
   c->sw_steps = 0;
   c->wolff_steps = 0;
+  if (c->strip_status) *c->strip_status = 0;
   cudaError_t e;
   if (c->wolff) {
     e = cudaMemsetAsync(c->wolff, 0, sizeof(WolffCtl), c->stream);
@@ -735,7 +794,8 @@ int ising_set_kernel(ising_ctx* c, int kernel, int k, int tile_rows, int tile_wo
     return fail(ISING_EINVAL, "grid must be >= 0 and block a multiple of 32 in [32, 1024]");
   if (kernel == ISING_KERNEL_AUTO) {
     resolve_auto(c);
-    if (c->kernel == ISING_KERNEL_TILED)
+    if (int st = ensure_strip(c)) return st;
+    if (c->kernel == ISING_KERNEL_TILED && c->strip.G == 0)
       if (int st = ensure_second_buffer(c)) return st;
     return ok();
   }
@@ -744,6 +804,7 @@ int ising_set_kernel(ising_ctx* c, int kernel, int k, int tile_rows, int tile_wo
   if (int st = validate_kernel(c, kernel, k, tile_rows, tile_words)) return st;
   if (kernel == ISING_KERNEL_TILED)
     if (int st = ensure_second_buffer(c)) return st;
+  c->strip = StripShape{0, 0, 0.0};
   c->kernel = kernel;
   c->k = kernel == ISING_KERNEL_TILED ? k : 1;
   c->tile_rows = tile_rows;

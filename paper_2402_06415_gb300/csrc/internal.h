@@ -130,6 +130,36 @@ cudaError_t launch_tiled32_sweep_bits(const BitsLattice& in, uint32_t* out, cons
                                       unsigned long long* rec_base, int n_tile_rows,
                                       int tile_words, int grid, cudaStream_t s);
 size_t tiled32_smem_bytes(int L, int k, int n_tile_rows, int tile_words);
+// Resident strips (k_strip.cu): n sweeps in one launch, in place, on packed
+// planes or int8 spins (the other pointer null).  G row strips, one CTA each
+// (cooperative launch; needs L >= 2 K G), K sweeps between exchanges.
+constexpr int kStripThreads = 512, kSplitThreads = 768;
+constexpr int kStripBlocks = 3;  // Philox blocks drawn for every word before the lazy ones
+struct StripArgs {
+  uint32_t* planes;
+  int8_t* spins;
+  int L, Wc, G, K;
+  uint32_t t0;
+  int n;
+  int m, to_rec;       // record every m sweeps; sweeps until the first record (0: none)
+  long long rec0, rec_cap;  // ring slot of the first record
+  unsigned long long* rec;
+  unsigned long long* xbuf;  // strip_xbuf_words(L, G, K) words (G > 1), zeroed by the launcher
+  int* status;         // host-visible word, set to 1 when a wait gave up
+  long long limit;     // clock64 cycles a wait may take
+  FastDiv fwc;         // set by the launcher
+};
+// Strips and sweeps per exchange for an L x L lattice, and the modelled time per
+// sweep (G = 0: the strips do not fit in shared memory).
+struct StripShape {
+  int G, K;
+  double us;
+};
+constexpr int kStripMaxK = 8;
+StripShape choose_strip(int L, int sms);
+size_t strip_smem_bytes(int L, int G, int K);
+size_t strip_xbuf_words(int L, int G, int K);
+cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, cudaStream_t s);
 cudaError_t launch_measure_bits(const BitsLattice& lat, unsigned long long* out2,
                                 cudaStream_t s);
 cudaError_t launch_unpack_bits(const BitsLattice& lat, int8_t* spins, cudaStream_t s);

@@ -158,6 +158,113 @@ __device__ __forceinline__ uint32_t flip_mask_rk(const Classes& k, uint32_t vali
   return (k.ge2 & valid) | acc;
 }
 
+// Planes of Philox blocks b = B0 .. B1-1 for the undecided lanes D of one
+// word; cls marks the lanes that test against t4 (the others test against t8).
+// Accepted lanes are added to acc.  Stops early once no lane of the warp is
+// undecided (warp vote), so every lane of the warp must call it.
+template <int B0, int B1>
+__device__ __forceinline__ void lazy_planes(uint32_t g, uint32_t t, uint32_t rep, uint32_t colour,
+                                            const RngParams& rng, uint32_t& D, uint32_t cls,
+                                            uint32_t& acc) {
+#pragma unroll
+  for (int b = B0; b < B1; ++b) {
+    if (!__any_sync(0xffffffffu, D != 0u)) break;
+    const uint4 r = philox10_rk(make_uint4(g, t, rep, ctr_w(kTagMet, colour, b)), rng.rk0, rng.rk1);
+    const uint32_t p[4] = {r.x, r.y, r.z, r.w};
+    // the block's 4 planes as one 4-bit comparison (borrow of u - T from the
+    // block's last plane up, equality chain), then merged into (acc, D)
+    uint32_t bor = 0u, eq = D;
+#pragma unroll
+    for (int q = 3; q >= 0; --q) {
+      const int k = 4 * b + q;
+      const uint32_t m4 = rng.tm4[k], m8 = rng.tm8[k];
+      const uint32_t tm = (cls & m4) | (~cls & m8);  // lane's threshold bit
+      bor = (~p[q] & tm) | (~p[q] & bor) | (tm & bor);
+      eq &= ~(tm ^ p[q]);
+    }
+    acc |= D & bor;
+    D = eq;
+  }
+}
+
+// lazy_planes for two independent words at once (one warp vote for both; two
+// Philox chains in flight per thread).
+template <int B0, int B1>
+__device__ __forceinline__ void lazy_planes2(uint32_t ga, uint32_t gb, uint32_t t, uint32_t rep,
+                                             uint32_t colour, const RngParams& rng, uint32_t& Da,
+                                             uint32_t clsa, uint32_t& acca, uint32_t& Db,
+                                             uint32_t clsb, uint32_t& accb) {
+#pragma unroll
+  for (int b = B0; b < B1; ++b) {
+    if (!__any_sync(0xffffffffu, (Da | Db) != 0u)) break;
+    const uint32_t cw = ctr_w(kTagMet, colour, b);
+    const uint4 ra = philox10_rk(make_uint4(ga, t, rep, cw), rng.rk0, rng.rk1);
+    const uint4 rb = philox10_rk(make_uint4(gb, t, rep, cw), rng.rk0, rng.rk1);
+    const uint32_t pa[4] = {ra.x, ra.y, ra.z, ra.w};
+    const uint32_t pb[4] = {rb.x, rb.y, rb.z, rb.w};
+    uint32_t bora = 0u, borb = 0u, eqa = Da, eqb = Db;
+#pragma unroll
+    for (int q = 3; q >= 0; --q) {
+      const int k = 4 * b + q;
+      const uint32_t m4 = rng.tm4[k], m8 = rng.tm8[k];
+      const uint32_t ta = (clsa & m4) | (~clsa & m8);
+      const uint32_t tb = (clsb & m4) | (~clsb & m8);
+      bora = (~pa[q] & ta) | (~pa[q] & bora) | (ta & bora);
+      borb = (~pb[q] & tb) | (~pb[q] & borb) | (tb & borb);
+      eqa &= ~(ta ^ pa[q]);
+      eqb &= ~(tb ^ pb[q]);
+    }
+    acca |= Da & bora;
+    accb |= Db & borb;
+    Da = eqa;
+    Db = eqb;
+  }
+}
+
+// Planes 0..7 (Philox blocks 0 and 1) of one or two words, all evaluated, as
+// one strict comparison of the top 8 bits: u_8 < T_8 is the borrow out of the
+// bit-sliced subtraction u_8 - T_8, carried from plane 7 (the least
+// significant of the eight) up to plane 0 with one majority function per
+// plane, borrow' = maj(~u_k, T_k, borrow); lanes whose 8 bits equal the
+// threshold's stay undecided.  Gives the same (acc, D) as the MSB-first test
+// over the same planes with one logic operation less per plane.  Block 1 is
+// drawn first, so only one block's planes are live at a time.
+template <int NW>
+__device__ __forceinline__ void planes8(const uint32_t (&g)[NW], uint32_t t, uint32_t rep,
+                                        uint32_t colour, const RngParams& rng, uint32_t (&D)[NW],
+                                        const uint32_t (&cls)[NW], uint32_t (&acc)[NW]) {
+  uint32_t bor[NW], eq[NW];
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    bor[w] = 0u;
+    eq[w] = D[w];
+  }
+#pragma unroll
+  for (int b = 1; b >= 0; --b) {
+    const uint32_t cw = ctr_w(kTagMet, colour, b);
+    uint4 r[NW];
+#pragma unroll
+    for (int w = 0; w < NW; ++w) r[w] = philox10_rk(make_uint4(g[w], t, rep, cw), rng.rk0, rng.rk1);
+#pragma unroll
+    for (int q = 3; q >= 0; --q) {
+      const int k = 4 * b + q;
+      const uint32_t m4 = rng.tm4[k], m8 = rng.tm8[k];
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        const uint32_t p = q == 0 ? r[w].x : q == 1 ? r[w].y : q == 2 ? r[w].z : r[w].w;
+        const uint32_t tm = (cls[w] & m4) | (~cls[w] & m8);  // lane's threshold bit
+        bor[w] = (~p & tm) | (~p & bor[w]) | (tm & bor[w]);
+        eq[w] &= ~(tm ^ p);
+      }
+    }
+  }
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    acc[w] |= D[w] & bor[w];
+    D[w] = eq[w];
+  }
+}
+
 // Valid-lane mask of word w when the colour row has n sites (n = L/2).
 __device__ __forceinline__ uint32_t valid_mask(int w, int Wc, int n) {
   if (w < Wc - 1) return 0xffffffffu;

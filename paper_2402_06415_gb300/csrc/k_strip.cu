@@ -1,0 +1,415 @@
+// Resident strips: many checkerboard Metropolis sweeps of one lattice per
+// launch (arXiv 2402.06415, Results A: the two sublattices updated in turn),
+// for lattices whose sweep is too short for a launch of its own.
+//
+// G CTAs (one per SM, all co-resident) own G row strips of full width and keep
+// them as two bit planes in shared memory, with a halo of H = 2K rows above
+// and below.  A group of K sweeps runs with CTA barriers only: every half
+// sweep invalidates one more halo row on each side, and halo sites are updated
+// with their owners' (sweep, site) random numbers, so after K sweeps exactly
+// the own rows are correct.  Then each CTA hands its H outer rows to its two
+// neighbours through global memory and waits for theirs (a flag per CTA; there
+// is no grid barrier).  G = 1 keeps the whole lattice in one CTA without halo.
+// Rows are whole, so any even L works: the x wrap and a ragged last word are a
+// select per word.
+//
+// What bounds it: up to L ~ 500 the dependent chain of a half sweep (shared
+// loads, neighbour classes, one Philox block, the plane test, a CTA barrier) and
+// the exchange (0.9 us).  There four threads share a word, one Philox block
+// each (SPLIT), and draw the next half sweep's block while this one's loads and
+// shuffles are in flight: a half sweep of 32 words takes 0.19 us against 0.62
+// with one thread per word.  Above, three blocks per word on the multiply pipe
+// (4 cycles per 32 x 32 -> 64 product and sub-partition).  Time per sweep, before
+// (launches per sweep or half sweep; int8: one CTA) and with strips: L = 64 int8
+// 16.4 -> 0.55 us, L = 256 8.3 -> 1.14, L = 1000 8.2 -> 1.9, L = 2048 21 -> 3.4.
+#include "internal.h"
+#include "ising_device.cuh"
+
+namespace ising {
+namespace {
+
+// kBlocks Philox blocks (4 kBlocks planes) of a word as one strict comparison
+// (planes8 with a variable number of blocks).
+template <int NB>
+__device__ __forceinline__ void planes_first(uint32_t g, uint32_t t, uint32_t rep, uint32_t colour,
+                                             const RngParams& rng, uint32_t& D, uint32_t cls, uint32_t& acc) {
+  uint32_t bor = 0u, eq = D;
+#pragma unroll
+  for (int b = NB - 1; b >= 0; --b) {
+    const uint4 r = philox10_rk(make_uint4(g, t, rep, ctr_w(kTagMet, colour, b)), rng.rk0, rng.rk1);
+    const uint32_t p[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int q = 3; q >= 0; --q) {
+      const int k = 4 * b + q;
+      const uint32_t tm = (cls & rng.tm4[k]) | (~cls & rng.tm8[k]);  // lane's threshold bit
+      bor = (~p[q] & tm) | (~p[q] & bor) | (tm & bor);
+      eq &= ~(tm ^ p[q]);
+    }
+  }
+  acc |= D & bor;
+  D = eq;
+}
+
+// Boundary words travel as 8-byte (tag, word) pairs, written and polled with
+// single 8-byte accesses: the reader sees the word as soon as it sees the tag,
+// so an exchange is one store and one load through L2, without a fence, a flag
+// or a second load.
+__device__ __forceinline__ void send_word(unsigned long long* slot, uint32_t tag, uint32_t word) {
+  const unsigned long long v = ((unsigned long long)tag << 32) | word;
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(slot), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long poll_word(const unsigned long long* slot) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(slot) : "memory");
+  return v;
+}
+// Waits for the pair with this tag; false (and *status = 1) after `limit` cycles.
+__device__ __forceinline__ bool recv_word(const unsigned long long* slot, uint32_t tag, long long limit, int* status,
+                                          uint32_t& word) {
+  unsigned long long v = poll_word(slot);
+  if ((uint32_t)(v >> 32) != tag) {
+    const long long start = clock64();
+    do {
+      if (clock64() - start > limit) {
+        *reinterpret_cast<volatile int*>(status) = 1;
+        return false;
+      }
+      v = poll_word(slot);
+    } while ((uint32_t)(v >> 32) != tag);
+  }
+  word = (uint32_t)v;
+  return true;
+}
+
+template <bool WHOLE, bool I8, bool SPLIT>
+__global__ void __launch_bounds__(SPLIT ? kSplitThreads : kStripThreads) k_strip(StripArgs a, RngParams rng) {
+  extern __shared__ uint32_t strip_smem[];
+  const int L = a.L, Wc = a.Wc, n_half = L / 2;
+  const int nb = n_half - 32 * (Wc - 1);                       // valid bits of a row's last word
+  const uint32_t last_mask = nb >= 32 ? 0xffffffffu : ((1u << nb) - 1u);
+  const int G = WHOLE ? 1 : a.G, H = WHOLE ? 0 : 2 * a.K;
+  const int b = blockIdx.x, tid = threadIdx.x, nth = blockDim.x, lane = tid & 31;
+  const int y0 = (int)((long long)b * L / G), y1 = (int)((long long)(b + 1) * L / G);
+  const int R = y1 - y0, rows = R + 2 * H;
+  const int plane = ((L + G - 1) / G + 2 * H) * Wc;
+  auto P = [plane](int c) { return strip_smem + c * plane; };
+  const int LW = L * Wc, n_words = rows * Wc;
+  // word i of the strip is group g = i + goff of the lattice, modulo L * Wc
+  const int goff = (y0 - H) * Wc;
+  auto group_of = [&](int i) {
+    int g = i + goff;
+    if (!WHOLE) {
+      g += g < 0 ? LW : 0;
+      g -= g >= LW ? LW : 0;
+    }
+    return g;
+  };
+  if (I8) {
+    // one warp per word: lane j reads the site's byte
+    for (int i = tid >> 5; i < 2 * n_words; i += nth >> 5) {
+      const int c = i >= n_words, g = group_of(i - c * n_words);
+      const int y = (int)fdiv((uint32_t)g, a.fwc), w = g - y * Wc;
+      const int j = 32 * w + lane;
+      const bool up = j < n_half && a.spins[(size_t)y * L + 2 * j + ((y + c) & 1)] > 0;
+      const uint32_t v = __ballot_sync(0xffffffffu, up);
+      if (lane == 0) P(c)[i - c * n_words] = v;
+    }
+  } else {
+    for (int i = tid; i < 2 * n_words; i += nth) {
+      const int c = i >= n_words, k = i - c * n_words;
+      P(c)[k] = __ldcg(&a.planes[(size_t)c * LW + group_of(k)]);
+    }
+  }
+  __syncthreads();
+  // slots of this strip: 2 x 4 hw boundary pairs (two buffers used in turn), then
+  // one "lattice read" token
+  const int hw = H * Wc;
+  const size_t per_cta = 8 * (size_t)hw + 1;
+  unsigned long long* const mine = WHOLE ? nullptr : a.xbuf + b * per_cta;
+  const unsigned long long* const up_slots = WHOLE ? nullptr : a.xbuf + (b == 0 ? G - 1 : b - 1) * per_cta;
+  const unsigned long long* const dn_slots = WHOLE ? nullptr : a.xbuf + (b == G - 1 ? 0 : b + 1) * per_cta;
+  if (!WHOLE && tid == 0) send_word(mine + 8 * hw, 1u, 0u);
+  uint32_t exchanges = 0;
+  int to_rec = a.to_rec;  // sweeps until the next record (counting this one), 0 = never
+  long long slot = a.rec0;
+  // SPLIT: four threads per word, one Philox block each (planes 4q .. 4q + 3),
+  // always the same word, whose two spin words stay in registers
+  const int q = tid & 3;
+  const int wi = (WHOLE ? 0 : Wc) + (tid >> 2);
+  const bool mine_w = SPLIT && wi < n_words - (WHOLE ? 0 : Wc);
+  const int i1 = mine_w ? wi : (WHOLE ? 0 : Wc);
+  const int r1 = (int)fdiv((uint32_t)i1, a.fwc), w1 = i1 - r1 * Wc;
+  const uint32_t g1 = (uint32_t)group_of(i1);
+  const bool first1 = w1 == 0, last1 = w1 == Wc - 1;
+  const int o1 = (y0 + r1) & 1;  // x offset of colour 0
+  int iu1 = i1 - Wc, id1 = i1 + Wc;
+  if (WHOLE) {
+    iu1 += iu1 < 0 ? n_words : 0;
+    id1 -= id1 >= n_words ? n_words : 0;
+  }
+  const int il1 = first1 ? i1 + Wc - 1 : i1 - 1, ir1 = last1 ? i1 - Wc + 1 : i1 + 1;
+  const int shl1 = first1 ? nb - 1 : 31, shr1 = last1 ? nb - 1 : 31;
+  const uint32_t valid1 = mine_w ? (last1 ? last_mask : 0xffffffffu) : 0u;
+  const bool inner1 = mine_w && q == 0 && r1 >= H && r1 < H + R;
+  uint32_t m4[4], m8[4], own[2] = {0u, 0u};
+  uint4 pl = make_uint4(0u, 0u, 0u, 0u);
+  if (SPLIT) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      m4[k] = rng.tm4[4 * q + k];
+      m8[k] = rng.tm8[4 * q + k];
+    }
+    own[0] = P(0)[i1];
+    own[1] = P(1)[i1];
+    pl = philox10_rk(make_uint4(g1, a.t0, rng.replica, ctr_w(kTagMet, 0u, (uint32_t)q)), rng.rk0, rng.rk1);
+  }
+  for (int done = 0; done < a.n;) {
+    const int kk = min(a.K, a.n - done);
+    if (SPLIT) {
+      for (int s2 = 0; s2 < kk; ++s2) {
+        const uint32_t t = a.t0 + (uint32_t)(done + s2);
+        unsigned int anti = 0, ones = 0;
+        const bool meas = to_rec == 1;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          uint32_t* const So = P(c);
+          const uint32_t* const Sn = P(1 - c);
+          const bool left = ((o1 ^ c) & 1) == 0;
+          const uint32_t s = own[c], mid = own[1 - c];
+          const uint32_t up = Sn[iu1], dn = Sn[id1], x = Sn[left ? il1 : ir1];
+          // the next half sweep's planes do not depend on spins: drawn while
+          // this one's loads and shuffles are in flight
+          const uint4 nx = philox10_rk(make_uint4(g1, t + (uint32_t)c, rng.replica,
+                                                  ctr_w(kTagMet, (uint32_t)(1 - c), (uint32_t)q)),
+                                       rng.rk0, rng.rk1);
+          const uint32_t side = left ? (mid << 1) | ((x >> shl1) & 1u) : (mid >> 1) | ((x & 1u) << shr1);
+          const HalfClasses k = classify_hs(s, up ^ dn, up, dn, mid, side);
+          const uint32_t p[4] = {pl.x, pl.y, pl.z, pl.w};
+          uint32_t bor = 0u, eq = 0xffffffffu;
+#pragma unroll
+          for (int j = 3; j >= 0; --j) {
+            const uint32_t tm = (k.cls & m4[j]) | (~k.cls & m8[j]);
+            bor = (~p[j] & tm) | (~p[j] & bor) | (tm & bor);
+            eq &= ~(tm ^ p[j]);
+          }
+          // merge the four blocks' verdicts: the more significant block decides
+          // unless it is tied (eq)
+#pragma unroll
+          for (int st = 1; st <= 2; st <<= 1) {
+            const uint32_t ob = __shfl_xor_sync(0xffffffffu, bor, st), oe = __shfl_xor_sync(0xffffffffu, eq, st);
+            const bool hi = (q & st) == 0;
+            const uint32_t hb = hi ? bor : ob, he = hi ? eq : oe, lb = hi ? ob : bor;
+            bor = hb | (he & lb);
+            eq &= oe;
+          }
+          uint32_t D = ~k.ge2 & valid1;
+          uint32_t acc = D & bor;
+          D &= eq;
+          if (__any_sync(0xffffffffu, D != 0u))  // a tie over 16 planes: the other blocks
+            lazy_planes<4, 8>(g1, t, rng.replica, (uint32_t)c, rng, D, k.cls, acc);
+          const uint32_t ns = s ^ ((k.ge2 & valid1) | acc);
+          own[c] = ns;
+          if (mine_w && q == 0) So[i1] = ns;
+          if (c == 1 && meas && inner1) {
+            anti = __popc((ns ^ up) & valid1) + __popc((ns ^ dn) & valid1) + __popc((ns ^ mid) & valid1) +
+                   __popc((ns ^ side) & valid1);
+            ones = __popc(ns & valid1) + __popc(mid & valid1);
+          }
+          pl = nx;
+          __syncthreads();
+        }
+        if (meas) {
+          anti = __reduce_add_sync(0xffffffffu, anti);
+          ones = __reduce_add_sync(0xffffffffu, ones);
+          if (lane == 0 && (anti | ones)) {
+            atomicAdd(&a.rec[2 * slot], (unsigned long long)anti);
+            atomicAdd(&a.rec[2 * slot + 1], (unsigned long long)ones);
+          }
+        }
+        if (to_rec > 0 && --to_rec == 0) {
+          to_rec = a.m;
+          slot = slot + 1 == a.rec_cap ? 0 : slot + 1;
+        }
+      }
+    } else {
+      for (int h = 0; h < 2 * kk; ++h) {
+        const int c = h & 1;
+        const uint32_t t = a.t0 + (uint32_t)(done + (h >> 1));
+        const bool meas = c == 1 && to_rec == 1;
+        uint32_t* const So = P(c);
+        const uint32_t* const Sn = P(1 - c);
+        // rows still correct after this half sweep (a short last group starts further in)
+        const int margin = WHOLE ? 0 : h + 1 + 2 * (a.K - kk);
+        const int lo = margin * Wc, count = n_words - 2 * lo;
+        unsigned int anti = 0, ones = 0;
+        for (int base = tid & ~31; base < count; base += nth) {
+          const bool active = base + lane < count;
+          const int i = lo + (active ? base + lane : 0);
+          const int r = (int)fdiv((uint32_t)i, a.fwc), w = i - r * Wc;
+          int iu = i - Wc, id = i + Wc;
+          if (WHOLE) {
+            iu += iu < 0 ? n_words : 0;
+            id -= id >= n_words ? n_words : 0;
+          }
+          const bool first = w == 0, last = w == Wc - 1;
+          const int o = (y0 + r + c) & 1;  // H is even
+          const int ix = o == 0 ? (first ? i + Wc - 1 : i - 1) : (last ? i - Wc + 1 : i + 1);
+          const uint32_t s = So[i], up = Sn[iu], dn = Sn[id], mid = Sn[i], x = Sn[ix];
+          const uint32_t side = o == 0 ? (mid << 1) | ((x >> (first ? nb - 1 : 31)) & 1u)
+                                       : (mid >> 1) | ((x & 1u) << (last ? nb - 1 : 31));
+          const uint32_t valid = active ? (last ? last_mask : 0xffffffffu) : 0u;
+          const HalfClasses k = classify_hs(s, up ^ dn, up, dn, mid, side);
+          uint32_t D = ~k.ge2 & valid, acc = 0;
+          const uint32_t g = (uint32_t)group_of(i);
+          planes_first<kStripBlocks>(g, t, rng.replica, (uint32_t)c, rng, D, k.cls, acc);
+          lazy_planes<kStripBlocks, 8>(g, t, rng.replica, (uint32_t)c, rng, D, k.cls, acc);
+          const uint32_t ns = s ^ ((k.ge2 & valid) | acc);
+          if (active) So[i] = ns;
+          if (meas && r >= H && r < H + R) {
+            anti += __popc((ns ^ up) & valid) + __popc((ns ^ dn) & valid) + __popc((ns ^ mid) & valid) +
+                    __popc((ns ^ side) & valid);
+            ones += __popc(ns & valid) + __popc(mid & valid);
+          }
+        }
+        if (meas) {
+          anti = __reduce_add_sync(0xffffffffu, anti);
+          ones = __reduce_add_sync(0xffffffffu, ones);
+          if (lane == 0 && (anti | ones)) {
+            atomicAdd(&a.rec[2 * slot], (unsigned long long)anti);
+            atomicAdd(&a.rec[2 * slot + 1], (unsigned long long)ones);
+          }
+        }
+        if (c == 1 && to_rec > 0 && --to_rec == 0) {
+          to_rec = a.m;
+          slot = slot + 1 == a.rec_cap ? 0 : slot + 1;
+        }
+        __syncthreads();
+      }
+    }
+    done += kk;
+    if (WHOLE || done >= a.n) continue;
+    // exchange: own rows [H, 2H) go up, [R, R + H) go down; buffers alternate
+    const uint32_t tag = ++exchanges;
+    const size_t buf = (size_t)(tag & 1) * 4 * hw;
+    for (int i = tid; i < 4 * hw; i += nth) {
+      const int lower = i >= 2 * hw, rem = i - lower * 2 * hw;
+      const int c = rem >= hw, k = rem - c * hw;
+      send_word(mine + buf + i, tag, P(c)[(lower ? R * Wc : H * Wc) + k]);
+    }
+    bool ok = true;
+    for (int i = tid; i < 4 * hw; i += nth) {
+      const int lower = i >= 2 * hw, rem = i - lower * 2 * hw;
+      const int c = rem >= hw, k = rem - c * hw;
+      // the upper neighbour's lower rows, the lower neighbour's upper rows
+      uint32_t word = 0;
+      ok = ok && recv_word((lower ? dn_slots : up_slots + 2 * hw) + buf + rem, tag, a.limit, a.status, word);
+      P(c)[(lower ? (H + R) * Wc : 0) + k] = word;
+    }
+    if (!__syncthreads_and(ok)) return;
+    if (SPLIT) {
+      own[0] = P(0)[i1];
+      own[1] = P(1)[i1];
+    }
+  }
+  // the lattice is updated in place: both neighbours must have read their halos
+  if (!WHOLE && exchanges == 0) {
+    uint32_t word;
+    bool ok = true;
+    if (tid < 2) ok = recv_word((tid ? dn_slots : up_slots) + 8 * hw, 1u, a.limit, a.status, word);
+    if (!__syncthreads_and(ok)) return;
+  }
+  if (I8) {
+    const int n = R * Wc;
+    for (int i = tid >> 5; i < 2 * n; i += nth >> 5) {
+      const int c = i >= n, k = i - c * n;
+      const int r = (int)fdiv((uint32_t)k, a.fwc), w = k - r * Wc, y = y0 + r;
+      const uint32_t v = P(c)[H * Wc + k];
+      const int j = 32 * w + lane;
+      if (j < n_half) a.spins[(size_t)y * L + 2 * j + ((y + c) & 1)] = (v >> lane) & 1u ? 1 : -1;
+    }
+  } else {
+    const int n = R * Wc;
+    for (int i = tid; i < 2 * n; i += nth) {
+      const int c = i >= n, k = i - c * n;
+      a.planes[(size_t)c * LW + (size_t)y0 * Wc + k] = P(c)[H * Wc + k];
+    }
+  }
+}
+
+}  // namespace
+
+size_t strip_smem_bytes(int L, int G, int K) {
+  const int Wc = (L / 2 + 31) / 32;
+  const int H = G == 1 ? 0 : 2 * K;
+  return 2ull * (size_t)((L + G - 1) / G + 2 * H) * (size_t)Wc * sizeof(uint32_t);
+}
+
+size_t strip_xbuf_words(int L, int G, int K) {
+  const int Wc = (L / 2 + 31) / 32;
+  return G == 1 ? 0 : (size_t)G * (16 * (size_t)K * Wc + 1);
+}
+
+// Time model of one sweep in microseconds, fitted to sweeps of (G, K) on GB300
+// for L = 32 ... 8192 (within 15 %): per half sweep 0.10 + 0.085 us per resident
+// warp of an SM sub-partition with four threads per word (SPLIT), 0.45 + 0.25 us
+// with one, and 0.9 us per exchange.
+static double strip_model_us(int L, int Wc, int G, int K) {
+  const int R = (L + G - 1) / G;
+  const bool whole = G == 1;
+  const int most = (R + (whole ? 0 : 4 * K - 2)) * Wc;
+  double t = whole ? 0.0 : 0.9;
+  if (4 * most <= kSplitThreads) {
+    const int wps = ((most + 7) / 8 + 3) / 4;
+    t += 2 * K * (0.10 + 0.085 * wps);
+  } else {
+    for (int h = 0; h < 2 * K; ++h) {
+      const int words = (R + (whole ? 0 : 2 * (2 * K - 1 - h))) * Wc;
+      t += 0.45 + 0.25 * (((words + 31) / 32 + 3) / 4);
+    }
+  }
+  return t / K;
+}
+
+StripShape choose_strip(int L, int sms) {
+  const int Wc = (L / 2 + 31) / 32;
+  StripShape best{0, 0, 1e30};
+  for (int G = 1; G <= sms && G <= L / 2; ++G)
+    for (int K = 1; K <= (G == 1 ? 1 : kStripMaxK); ++K) {
+      if (G > 1 && L / G < 2 * K) break;  // the halo comes from the next strip only
+      if (strip_smem_bytes(L, G, K) > 200 * 1024) break;
+      const double t = strip_model_us(L, Wc, G, K);
+      if (t < best.us) best = {G, G == 1 ? 1 << 30 : K, t};
+    }
+  return best;
+}
+
+cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, cudaStream_t s) {
+  const bool whole = a.G == 1, i8 = a.spins != nullptr;
+  if (a.K > a.n) a.K = a.n;
+  const size_t smem = strip_smem_bytes(a.L, a.G, a.K);
+  const int words = (int)(((a.L + a.G - 1) / a.G + (whole ? 0 : 4 * a.K - 2)) * (long long)a.Wc);
+  const bool split = 4 * words <= kSplitThreads;
+  const void* fns[8] = {(const void*)k_strip<false, false, false>, (const void*)k_strip<true, false, false>,
+                        (const void*)k_strip<false, true, false>,  (const void*)k_strip<true, true, false>,
+                        (const void*)k_strip<false, false, true>,  (const void*)k_strip<true, false, true>,
+                        (const void*)k_strip<false, true, true>,   (const void*)k_strip<true, true, true>};
+  const int which = (whole ? 1 : 0) + (i8 ? 2 : 0) + (split ? 4 : 0);
+  static DeviceCache configured[8];
+  if ((long long)smem > configured[which].get()) {
+    cudaError_t e = cudaFuncSetAttribute(fns[which], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured[which].set((long long)smem);
+  }
+  int threads = (((split ? 4 : 1) * words + 31) / 32) * 32;
+  if (threads < 64) threads = 64;
+  if (!split && threads > kStripThreads) threads = kStripThreads;
+  a.fwc = make_fastdiv((uint32_t)a.Wc);
+  RngParams r = rng;
+  void* args[] = {&a, &r};
+  if (whole) return cudaLaunchKernel(fns[which], dim3(1), dim3(threads), args, smem, s);
+  cudaError_t e = cudaMemsetAsync(a.xbuf, 0, strip_xbuf_words(a.L, a.G, a.K) * 8, s);
+  if (e != cudaSuccess) return e;
+  return cudaLaunchCooperativeKernel(fns[which], dim3(a.G), dim3(threads), args, smem, s);
+}
+
+}  // namespace ising
