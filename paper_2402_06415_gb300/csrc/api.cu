@@ -233,19 +233,48 @@ int ensure_strip(ising_ctx* c) {
   return ISING_OK;
 }
 
+// 32-word tiles, four sweeps per launch, and the number of row strips that gives
+// whole waves of resident CTAs (2 or 3 per SM) with the fewest row updates per
+// SM, halo rows included (2K - 1 on average over the half sweeps).  L = 16384:
+// 76 strips, two waves of two CTAs, 3113 flips/ns (one sweep per launch and 152
+// strips, the choice before: 2310); 12288: 76, 3047; 8192: 76, 2706.
+void auto_tiles32(ising_ctx* c) {
+  constexpr int K = 4;
+  const int n_tx = c->Wc / 32;
+  c->k = K;
+  c->tile_words = 32;
+  int64_t best = INT64_MAX;
+  for (int per_sm = 2; per_sm <= 3; ++per_sm)
+    for (int waves = 1; waves <= 64; ++waves) {
+      const int n_ty = std::min(c->sms * per_sm * waves / n_tx, c->L / 8);
+      if (n_ty < 1) continue;
+      const int rows = (c->L + n_ty - 1) / n_ty;
+      // shared memory of an SM: 228 KB less 1 KB per CTA and the queue's 18 KB
+      const size_t smem = tiled32_smem_bytes(c->L, K, n_ty, 32) + 20 * 1024;
+      if (smem * per_sm > 227 * 1024) continue;
+      const int64_t cost = (int64_t)waves * per_sm * (rows + 2 * K - 1);
+      if (cost < best) {
+        best = cost;
+        c->tile_rows = n_ty;
+      }
+    }
+}
+
 void resolve_auto(ising_ctx* c) {
   c->strip = strip_applies(c->layout, c->L) ? choose_strip(c->L, c->sms) : StripShape{0, 0, 0.0};
   if (c->layout == ISING_LAYOUT_BITS) {
     if (c->Wc % 4 == 0 && c->L % 64 == 0 && c->L >= 256) {
       c->kernel = ISING_KERNEL_TILED;
-      c->k = 1;
-      int tw = 32;
-      while (tw > 4 && c->Wc % tw != 0) tw /= 2;
-      c->tile_words = tw;
-      // about 108-row strips: for L = 16384 that is 152 strips x 8 tiles,
-      // two tiles per resident CTA at 4 CTAs per SM
-      c->tile_rows = c->L >= 1024 ? (int)((int64_t)c->L * 152 / 16384) : c->L / 64;
-      if (c->tile_rows < 1) c->tile_rows = 1;
+      if (c->Wc % 32 == 0 && c->L >= 2048) {
+        auto_tiles32(c);
+      } else {
+        c->k = 1;
+        int tw = 32;
+        while (tw > 4 && c->Wc % tw != 0) tw /= 2;
+        c->tile_words = tw;
+        c->tile_rows = c->L >= 1024 ? (int)((int64_t)c->L * 152 / 16384) : c->L / 64;
+        if (c->tile_rows < 1) c->tile_rows = 1;
+      }
     } else {
       c->kernel = ISING_KERNEL_HALF;
     }
