@@ -7,13 +7,34 @@
 //   input gradient g1[q][c]  = sum_{t,o} gz2[q - d_t][o] W2[o][c][t]
 //   weight gradient dW2[o][c][t] += sum_p gz2[p][o] h1[p + d_t][c]
 // (p, q frame positions, d_t the offset of tap t, zero outside the frame).
-// Layers 1 and 3 (2 -> 32 and 32 -> 1 channels, a few per cent of the work) run
-// in FP32 on the CUDA cores.  Activations and dL/dz2 are rounded to BF16 for the
-// MMA operands (the master weights stay FP32, the operands see them in BF16),
-// so gradients agree with the FP32 kernel to BF16 rounding, not bit for bit.
-// Each CTA keeps its weight-gradient sums (dW2 in the accumulator registers of
-// its warps, the rest in shared memory) over all its samples and adds them to
-// the global gradient once.
+// Activations and dL/dz2 are rounded to BF16 for the MMA operands (the master
+// weights stay FP32, the operands see them in BF16), so gradients agree with the
+// FP32 kernel to BF16 rounding, not bit for bit.  Layers 1 and 3 (2 -> 32 and
+// 32 -> 1 channels) are FP32: layer 3 on the CUDA cores; layer 1 and its weight
+// gradient on mma.sync as well, with the FP32 operand (W1, dL/dz1) split into
+// three BF16 terms that hold it exactly; the other operand, the spins and the
+// known mask, is exact in BF16, so products are exact and sums FP32.
+//
+// A stage's loss terms sit at a few sites, so only the positions next to them
+// carry a gradient: h2 matters at the sites' 3 x 3 neighbourhoods (list l2 of the
+// plan), h1 at their 5 x 5 neighbourhoods (list l1); everywhere else the
+// gradients are exactly zero.  Over the 8 network stages of a 16 x 16 block that
+// is 666 and 1196 positions instead of 8 x 324 each.  A CTA takes up to kMaxW
+// windows of one stage at a time and keeps their activations packed in list
+// order, so the matrix rows are dense; tables per stage give, for every list
+// entry and tap, the row to gather (a zero row where there is none).  512 layer-1
+// rows at a time give each of the 16 warps one unit of 32 rows x 32 channels.
+// The windows of all stages are dealt to the CTAs in contiguous ranges of equal
+// estimated work, so a CTA builds the tables of one or two stages.
+//
+// What bounds it: the two gathered contractions, whose ldmatrix traffic (the
+// weights are read again by every warp) and mma.sync rate (8 cycles per
+// m16n8k16 and sub-partition) are about equal, and the barriers between phases.
+// 512 windows x 8 stages: kernel 1520 -> 192 us, loss and gradients through the
+// API 1560 -> 236 us (before: full frames, one sample at a time, and one thread
+// listing the loss sites).
+// Each CTA keeps its weight-gradient sums in registers over all its windows and
+// adds them to the global gradient once.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -25,32 +46,42 @@ namespace ising {
 namespace nnc {
 namespace {
 
-constexpr int kG = kMaxB + 4;     // padded grid side: frame plus a zero border
-constexpr int kGrid = kG * kG;    // 400 grid positions
-constexpr int kZeroPos = 0;       // a grid corner: always zero (padding rows)
+constexpr int kTcWarps = 16, kTcThreads = 32 * kTcWarps;
+constexpr int kCap1 = 512, kCap2 = 336, kCap3 = kMaxB * kMaxB;  // packed rows of layers 1, 2, 3
+constexpr int kMaxW = 12;                                        // windows of a stage at a time
+// layer-1 inputs of a row: columns 0 .. 15 (spin, known) of taps 0 .. 7; then, three
+// times (once per BF16 term of the weights), (spin, known) of tap 8, a one for the
+// bias and a zero; zeros up to 32
+constexpr int kXP = 40, kW1K = 64;  // row stride, K of the layer-1 product
+constexpr uint16_t kNone = 0xffff;
+static_assert(kCap1 >= kMaxFrame && kCap2 >= kMaxFrame, "one full-frame window must fit");
+static_assert(kCap1 == 32 * kTcWarps, "one unit of 32 layer-1 rows per warp");
 
 struct TrainTcSmem {
-  __nv_bfloat16 w2f[kC * kK2P];  // forward B operand: [o][t * 32 + c]
-  __nv_bfloat16 w2r[kC * kK2P];  // input-gradient B operand: [c][t * 32 + o]
-  __nv_bfloat16 h1[kGrid * kCP];   // layer-1 output, zero outside the frame
-  __nv_bfloat16 h2[kGrid * kCP];   // layer-2 output, zero outside the frame
-  __nv_bfloat16 gz2[kGrid * kCP];  // dL/dz2, zero outside the frame
-  float gz1[kMaxFrame * kC];       // dL/dz1 (FP32, frame positions)
-  float w1t[18 * kC];              // W1 as [ci * 9 + t][c] (lanes = channels)
-  float b1[kC], b2[kC], w3[kC * 9 + 1];
-  float xg[2][kGrid];              // input channels on the padded grid (zero border)
-  float g3g[kGrid];                // dL/dz3 on the padded grid (zero outside the sites)
-  float red[8][kC * 18 + kC];      // per-warp layer-1 gradient sums, reduced at the end
-  float tgt[kMaxB * kMaxB];
-  uint8_t tmask[kMaxB * kMaxB];
-  int16_t sites[kMaxB * kMaxB];    // frame positions of this sample's loss terms
-  int n_sites;
-  // this CTA's gradient sums (dW2 lives in registers)
-  float gw1[kC * 18], gb1[kC], gb2[kC], gw3[kC * 9], gb3;
+  __nv_bfloat16 w2f[kC * kK2P];          // W2 as [o][t * 32 + c]
+  __nv_bfloat16 h1[(kCap1 + 1) * kCP];   // layer-1 output rows (the last row is zero)
+  __nv_bfloat16 h2[(kCap2 + 1) * kCP];   // layer-2 output rows
+  __nv_bfloat16 gz2[(kCap2 + 1) * kCP];  // dL/dz2 rows (the last row is zero)
+  __nv_bfloat16 x[kCap1 * kXP];          // layer-1 input rows
+  // W1 and b1 in three BF16 terms, [c][K]: terms of taps 0 .. 7 at 0, 16, 32, of x columns 16 .. 27 at 48
+  __nv_bfloat16 w1s[kC * (kW1K + 8)];
+  uint32_t mask[kCap1];                  // layer-1 row: bit c set iff h1[c] > 0
+  alignas(16) float w3t[9 * kC];         // W3 as [t][c]
+  float b2[kC], b3;
+  float g3[kCap3];                       // dL/dz3 at the sites
+  // tables of the current stage
+  uint32_t p1[kMaxFrame];       // l1 entry: frame position, known taps << 16
+  uint16_t nb1[kMaxFrame * 9];  // l2 entry, tap -> l1 entry at p + d_t
+  uint16_t nb2[kMaxFrame * 9];  // l1 entry, tap -> l2 entry at q - d_t
+  uint16_t nb3[kMaxFrame * 9];  // l2 entry, tap -> site at p - d_t
+  uint16_t nb4[kCap3 * 9];      // site, tap -> l2 entry at p + d_t
+  uint16_t m3[kMaxFrame];       // l2 entry: taps of nb3 that exist
+  uint2 l3s[kMaxFrame];         // l2 entry: its first four sites, 16 bits each: tap | site << 4 (kNone: no more)
+  uint16_t at1[kMaxFrame], at2[kMaxFrame], at3[kMaxFrame];  // frame position -> list entry
+  int8_t win[kMaxW * kMaxFrame];
 };
-
-__device__ __forceinline__ int grid_of_frame(int p, int F) { return (p / F + 1) * kG + p % F + 1; }
-__device__ __forceinline__ int tap_off(int t) { return (t / 3 - 1) * kG + (t % 3 - 1); }
+constexpr int kRed = 30;  // per-warp sums added up at the end, rows of 32: 18 W1, b1, b2, 9 W3 (and one spare)
+static_assert(kTcWarps * kRed * kC * 4 <= (kCap1 + kCap2) * kCP * 2, "the sums fit the h1 and h2 buffers");
 
 __device__ __forceinline__ void ldm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
@@ -62,16 +93,6 @@ __device__ __forceinline__ void ldm_x4_t(uint32_t addr, uint32_t& r0, uint32_t& 
                : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
                : "r"(addr));
 }
-__device__ __forceinline__ void ldm_x2(uint32_t addr, uint32_t& r0, uint32_t& r1) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n"
-               : "=r"(r0), "=r"(r1)
-               : "r"(addr));
-}
-__device__ __forceinline__ void ldm_x2_t(uint32_t addr, uint32_t& r0, uint32_t& r1) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n"
-               : "=r"(r0), "=r"(r1)
-               : "r"(addr));
-}
 __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                          uint32_t b0, uint32_t b1) {
   asm volatile(
@@ -81,310 +102,496 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Implicit GEMM over the frame positions (rows) with N = 32 channels and
-// K = 9 taps x 32 channels: acc[p][n] = sum_{t,k} act[g(p) + sign * d_t][k] B[n][t * 32 + k].
-// sign = +1: forward (B = w2f); sign = -1: input gradient (B = w2r).  The
-// epilogue gets (frame position, channel, value) for every valid output.
-template <typename Epi>
-__device__ __forceinline__ void conv_gemm(const __nv_bfloat16* act, const __nv_bfloat16* Bm, int F, int sign,
-                                          Epi epi) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const int FF = F * F;
-  const int n_mt = (FF + 15) / 16;
-  for (int mt = warp; mt < n_mt; mt += nwarps) {
-    float acc[4][4];
+__device__ __forceinline__ void ldm_x2_t(uint32_t addr, uint32_t& r0, uint32_t& r1) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(addr));
+}
+// v0, v1 as a sum of three packed BF16 pairs, exactly (8 + 8 + 8 significand bits)
+__device__ __forceinline__ void split3(float v0, float v1, uint32_t (&o)[3]) {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-    const int row = mt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-    const int gpos = row < FF ? grid_of_frame(row, F) : -1;
-    const int acol = (lane >> 4) * 8;
-#pragma unroll 2
-    for (int kc = 0; kc < 18; ++kc) {
-      const int tap = kc >> 1, k0 = (kc & 1) * 16;
-      // padding rows read the zero corner (results dropped)
-      const int ga = gpos >= 0 ? gpos + sign * tap_off(tap) : kZeroPos;
-      uint32_t a0, a1, a2, a3;
-      ldm_x4(smem_addr(act + ga * kCP + k0 + acol), a0, a1, a2, a3);
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
-        uint32_t b0, b1;
-        ldm_x2(smem_addr(Bm + (nt * 8 + (lane & 7)) * kK2P + kc * 16 + ((lane >> 3) & 1) * 8), b0, b1);
-        mma_bf16(acc[nt], a0, a1, a2, a3, b0, b1);
-      }
-    }
-    const int g = lane >> 2, t2 = (lane & 3) * 2;
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      const int p = mt * 16 + g + half * 8;
-      if (p >= FF) continue;
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
-        epi(p, nt * 8 + t2, acc[nt][half * 2 + 0]);
-        epi(p, nt * 8 + t2 + 1, acc[nt][half * 2 + 1]);
-      }
-    }
+  for (int i = 0; i < 3; ++i) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
+    o[i] = *reinterpret_cast<const uint32_t*>(&h);
+    v0 -= __uint_as_float(o[i] << 16);
+    v1 -= __uint_as_float(o[i] & 0xffff0000u);
   }
 }
 
-__global__ void __launch_bounds__(kThreads, 1) k_nn_train_tc(const int8_t* __restrict__ windows, int n,
-                                                             const StagedPlan* __restrict__ plan,
-                                                             const float* __restrict__ params,
-                                                             float* __restrict__ grads,
-                                                             float* __restrict__ loss) {
+__device__ __forceinline__ void ldm_x4_row(const __nv_bfloat16* p, uint32_t (&r)[4]) {
+  ldm_x4(smem_addr(p), r[0], r[1], r[2], r[3]);
+}
+
+// Work of one window of a stage in units of about one layer-1 row, for the
+// division of the windows among the CTAs.
+__device__ __forceinline__ long long window_cost(const StagedPlan* plan, int k) {
+  return (plan->off1[k + 1] - plan->off1[k]) + (plan->off2[k + 1] - plan->off2[k]) +
+         4 * (plan->off3[k + 1] - plan->off3[k]) + 16;
+}
+
+__global__ void __launch_bounds__(kTcThreads, 1) k_nn_train_tc(const int8_t* __restrict__ windows, int n,
+                                                               const StagedPlan* __restrict__ plan,
+                                                               const float* __restrict__ params,
+                                                               float* __restrict__ grads, float* __restrict__ loss) {
   extern __shared__ uint4 smem_raw[];
   TrainTcSmem& S = *reinterpret_cast<TrainTcSmem*>(smem_raw);
   const int B = plan->B, F = frame_of(B), FF = F * F;
   const float invn = 1.f / (float)n;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // weights: FP32 for layers 1 and 3, BF16 operand layouts of W2
-  for (int i = threadIdx.x; i < kC * kC * 9; i += blockDim.x) {
-    const int o = i / (kC * 9), c = (i / 9) % kC, t = i % 9;  // W2[o][c][t]
-    const __nv_bfloat16 v = __float2bfloat16_rn(params[kOffW2 + i]);
-    S.w2f[o * kK2P + t * kC + c] = v;
-    S.w2r[c * kK2P + t * kC + o] = v;
-  }
-  for (int i = threadIdx.x; i < kC * 18; i += blockDim.x) {
-    const int c = i / 18, j = i % 18;  // W1[c][ci][t], j = ci * 9 + t
-    S.w1t[j * kC + c] = params[kOffW1 + i];
-    S.gw1[i] = 0.f;
-  }
-  for (int i = threadIdx.x; i < kC * 9 + 1; i += blockDim.x) S.w3[i] = params[kOffW3 + i];
-  for (int i = threadIdx.x; i < kC * 9; i += blockDim.x) S.gw3[i] = 0.f;
-  for (int i = threadIdx.x; i < kC; i += blockDim.x) {
-    S.b1[i] = params[kOffB1 + i];
-    S.b2[i] = params[kOffB2 + i];
-    S.gb1[i] = 0.f;
-    S.gb2[i] = 0.f;
-  }
-  if (threadIdx.x == 0) S.gb3 = 0.f;
-  // grids start (and outside the frame stay) zero
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const __nv_bfloat16 z = __float2bfloat16_rn(0.f);
-  for (int i = threadIdx.x; i < kGrid * kCP; i += blockDim.x) S.h1[i] = S.h2[i] = S.gz2[i] = z;
-  for (int i = threadIdx.x; i < kGrid; i += blockDim.x) S.xg[0][i] = S.xg[1][i] = S.g3g[i] = 0.f;
+  for (int i = tid; i < kC * kC * 9; i += kTcThreads) {
+    const int o = i / (kC * 9), c = (i / 9) % kC, t = i % 9;  // W2[o][c][t]
+    S.w2f[o * kK2P + t * kC + c] = __float2bfloat16_rn(params[kOffW2 + i]);
+  }
+  for (int i = tid; i < kC * (kW1K + 8); i += kTcThreads) S.w1s[i] = z;
   __syncthreads();
+  for (int i = tid; i < kC * 19; i += kTcThreads) {
+    const int c = i / 19, j = i % 19;  // column j = 2 t + ci; 18: the bias
+    float v = j < 18 ? params[kOffW1 + c * 18 + (j & 1) * 9 + (j >> 1)] : params[kOffB1 + c];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const __nv_bfloat16 h = __float2bfloat16_rn(v);
+      S.w1s[c * (kW1K + 8) + (j < 16 ? 16 * q + j : 48 + 4 * q + j - 16)] = h;
+      v -= bf(h);
+    }
+  }
+  for (int i = tid; i < kC * 9; i += kTcThreads) S.w3t[(i % 9) * kC + i / 9] = params[kOffW3 + i];
+  for (int i = tid; i < kCap1 * kXP; i += kTcThreads) {
+    const int j = i % kXP;
+    S.x[i] = j == 18 || j == 22 || j == 26 ? __float2bfloat16_rn(1.f) : z;
+  }
+  if (tid < kC) S.b2[tid] = params[kOffB2 + tid];
+  if (tid == 0) S.b3 = params[kOffB3];
+  if (tid < kCP) {
+    S.h1[kCap1 * kCP + tid] = z;
+    S.h2[kCap2 * kCP + tid] = z;
+    S.gz2[kCap2 * kCP + tid] = z;
+  }
 
-  // dW2 accumulators: warp w owns tap w (both 16-row o tiles x four 8-column c
-  // tiles) and one tile of tap 8 (o tile w >> 2, c tile w & 3)
-  float dw[9][4];
-#pragma unroll
-  for (int a = 0; a < 9; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) dw[a][b] = 0.f;
-  // layer-1 gradient sums of this thread: channel o = lane, positions of
-  // warp `warp`'s slice, all samples (j = ci * 9 + t; gw1s[18] = bias)
-  float gw1s[19];
-#pragma unroll
-  for (int j = 0; j < 19; ++j) gw1s[j] = 0.f;
-  float my_loss = 0.f;
+  // gradient sums of this thread over all its CTA's windows.  dW2: tap warp & 7
+  // (both halves of the output channels x four tiles of input channels) and one
+  // tile of tap 8, over every second 16 rows; dW1 and db1: 32 channels x 24
+  // columns (as x) over this warp's rows; W3[lane][tap] over this warp's sites.
+  const int my_tap = warp & 7, my_half = warp >> 3, t8m = my_tap >> 2, t8n = my_tap & 3;
+  float dw[9][4] = {}, dw1[2][3][4] = {}, gw3s[9] = {};
+  float gb3s = 0.f, my_loss = 0.f;
+  float4 gb2s = make_float4(0.f, 0.f, 0.f, 0.f);  // channels 4 (lane & 7) ..
+
   const int n_net = plan->n_net;
-  const int total = n * n_net;
-  for (int smp = blockIdx.x; smp < total; smp += gridDim.x) {
-    const int k = smp / n_net;
-    const int stage = plan->net_ids[smp - k * n_net];
-    const int8_t* win = windows + (size_t)k * FF;
-    for (int i = threadIdx.x; i < FF; i += blockDim.x) {
-      const int fy = i / F, fx = i - (i / F) * F;
-      const bool e = known_at(*plan, fy, fx, stage);
-      const int gi = grid_of_frame(i, F);
-      S.xg[0][gi] = e ? (float)win[i] : 0.f;
-      S.xg[1][gi] = e ? 1.f : 0.f;
-      S.g3g[gi] = 0.f;
-      if (fy >= 1 && fy <= B && fx >= 1 && fx <= B) {
-        const int ii = (fy - 1) * B + fx - 1;
-        S.tgt[ii] = win[i] > 0 ? 1.f : 0.f;
-        S.tmask[ii] = plan->stage_of[ii] == stage ? 1 : 0;
+  long long total = 0;
+  for (int s = 0; s < n_net; ++s) total += (long long)n * window_cost(plan, plan->net_ids[s]);
+  long long before = 0;
+  for (int s = 0; s < n_net; ++s) {
+    const int stage = plan->net_ids[s];
+    const long long cost = window_cost(plan, stage);
+    // this CTA's windows: those whose start before + i cost lies in [b, b + 1) total / grid
+    auto first_of = [&](long long b) {
+      const long long x = b * total - before * (long long)gridDim.x, d = cost * (long long)gridDim.x;
+      const long long i = x <= 0 ? 0 : (x + d - 1) / d;
+      return (int)(i < n ? i : n);
+    };
+    const int k_lo = first_of(blockIdx.x), k_hi = first_of((long long)blockIdx.x + 1);
+    before += (long long)n * cost;
+    if (k_lo >= k_hi) continue;
+    const int16_t* l1 = plan->l1 + plan->off1[stage];
+    const int16_t* l2 = plan->l2 + plan->off2[stage];
+    const int16_t* l3 = plan->l3 + plan->off3[stage];
+    const uint16_t* m1 = plan->m1 + plan->off1[stage];
+    const int n1 = plan->off1[stage + 1] - plan->off1[stage], n2 = plan->off2[stage + 1] - plan->off2[stage];
+    const int n3 = plan->off3[stage + 1] - plan->off3[stage];
+    const int W = min(min(kMaxW, kCap1 / n1), min(kCap2 / n2, kCap3 / n3));
+    const FastDiv f1 = make_fastdiv((uint32_t)n1), f2 = make_fastdiv((uint32_t)n2), f3 = make_fastdiv((uint32_t)n3);
+
+    // ---- tables of the stage ----
+    __syncthreads();
+    for (int i = tid; i < FF; i += kTcThreads) S.at1[i] = S.at2[i] = S.at3[i] = kNone;
+    __syncthreads();
+    for (int e = tid; e < n1; e += kTcThreads) {
+      S.at1[l1[e]] = (uint16_t)e;
+      S.p1[e] = (uint32_t)l1[e] | ((uint32_t)m1[e] << 16);
+    }
+    for (int e = tid; e < n2; e += kTcThreads) S.at2[l2[e]] = (uint16_t)e;
+    for (int e = tid; e < n3; e += kTcThreads) S.at3[(l3[e] / B + 1) * F + l3[e] % B + 1] = (uint16_t)e;
+    __syncthreads();
+    auto look = [&](const uint16_t* at, int p, int t, int sign) {
+      const int y = p / F + sign * (t / 3 - 1), x = p % F + sign * (t % 3 - 1);
+      return y >= 0 && y < F && x >= 0 && x < F ? at[y * F + x] : kNone;
+    };
+    for (int i = tid; i < n2 * 9; i += kTcThreads) {
+      S.nb1[i] = look(S.at1, l2[i / 9], i % 9, +1);
+      S.nb3[i] = look(S.at3, l2[i / 9], i % 9, -1);
+    }
+    for (int i = tid; i < n1 * 9; i += kTcThreads) S.nb2[i] = look(S.at2, l1[i / 9], i % 9, -1);
+    for (int i = tid; i < n3 * 9; i += kTcThreads)
+      S.nb4[i] = look(S.at2, (l3[i / 9] / B + 1) * F + l3[i / 9] % B + 1, i % 9, +1);
+    __syncthreads();
+    for (int e = tid; e < n2; e += kTcThreads) {
+      uint32_t m = 0;
+      uint32_t l[4] = {kNone, kNone, kNone, kNone};
+      int q = 0;
+      for (int t = 0; t < 9; ++t) {
+        const uint32_t site = S.nb3[e * 9 + t];
+        if (site == kNone) continue;
+        m |= 1u << t;
+        const uint32_t x = (uint32_t)t | (site << 4);
+        if (q == 0) l[0] = x;
+        else if (q == 1) l[1] = x;
+        else if (q == 2) l[2] = x;
+        else if (q == 3) l[3] = x;
+        ++q;
       }
+      S.m3[e] = (uint16_t)m;
+      S.l3s[e] = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
     }
-    if (threadIdx.x == 0) {
-      int m = 0;
-      for (int ii = 0; ii < B * B; ++ii)
-        if (plan->stage_of[ii] == stage) S.sites[m++] = (int16_t)((ii / B + 1) * F + ii % B + 1);
-      S.n_sites = m;
-    }
-    __syncthreads();
-    // layer 1 (FP32): h1 = relu(W1 * x + b1), stored in BF16; lanes = channels
-    for (int i = threadIdx.x; i < FF * kC; i += blockDim.x) {
-      const int c = i % kC, p = i / kC, gp = grid_of_frame(p, F);
-      float zz = S.b1[c];
-#pragma unroll
-      for (int t = 0; t < 9; ++t)
-        zz += S.w1t[t * kC + c] * S.xg[0][gp + tap_off(t)] + S.w1t[(9 + t) * kC + c] * S.xg[1][gp + tap_off(t)];
-      S.h1[gp * kCP + c] = __float2bfloat16_rn(fmaxf(zz, 0.f));
-    }
-    __syncthreads();
-    // layer 2 forward on the tensor cores
-    conv_gemm(S.h1, S.w2f, F, +1, [&](int p, int o, float v) {
-      S.h2[grid_of_frame(p, F) * kCP + o] = __float2bfloat16_rn(fmaxf(v + S.b2[o], 0.f));
-    });
-    __syncthreads();
-    // layer 3 and the loss at this sample's sites: eight lanes per site
-    for (int base = warp * 4; base < S.n_sites; base += (int)(blockDim.x >> 3)) {
-      const int si = base + (lane >> 3);
-      const int sub = lane & 7, c0 = 4 * sub;
-      float zz = 0.f;
-      int p = 0;
-      if (si < S.n_sites) {
-        p = S.sites[si];
-        const int gp = grid_of_frame(p, F);
+
+    for (int k0 = k_lo; k0 < k_hi; k0 += W) {
+      const int nw = min(W, k_hi - k0), R1 = nw * n1, R2 = nw * n2, R3 = nw * n3;
+      for (int i = tid; i < nw * FF; i += kTcThreads) S.win[i] = windows[(size_t)k0 * FF + i];
+      __syncthreads();
+      // ---- layer-1 input rows ----
+      if (tid < R1) {  // one row per thread (R1 <= kCap1)
+        const int w = (int)fdiv((uint32_t)tid, f1);
+        const uint32_t pm = S.p1[tid - w * n1];
+        const int8_t* at = S.win + w * FF + (int)(pm & 0xffffu);
+        uint32_t v[9];  // (spin, known)
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
-          const __nv_bfloat16* h = &S.h2[(gp + tap_off(t)) * kCP + c0];
-          zz += S.w3[(c0 + 0) * 9 + t] * bf(h[0]) + S.w3[(c0 + 1) * 9 + t] * bf(h[1]) +
-                S.w3[(c0 + 2) * 9 + t] * bf(h[2]) + S.w3[(c0 + 3) * 9 + t] * bf(h[3]);
+          v[t] = 0u;
+          if (pm & (0x10000u << t))  // an int8 is exact in BF16
+            v[t] = (__float_as_uint((float)at[(t / 3 - 1) * F + t % 3 - 1]) >> 16) | 0x3f800000u;
         }
+        uint4* row = reinterpret_cast<uint4*>(S.x + tid * kXP);
+        row[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        row[1] = make_uint4(v[4], v[5], v[6], v[7]);
+        uint32_t* tail = reinterpret_cast<uint32_t*>(row + 2);
+        tail[0] = tail[2] = tail[4] = v[8];
       }
-      zz += __shfl_xor_sync(0xffffffffu, zz, 4);
-      zz += __shfl_xor_sync(0xffffffffu, zz, 2);
-      zz += __shfl_xor_sync(0xffffffffu, zz, 1);
-      if (si < S.n_sites && sub == 0) {
-        zz += S.w3[kC * 9];
-        const int fy = p / F, fx = p - (p / F) * F;
-        const float y = S.tgt[(fy - 1) * B + fx - 1];
-        my_loss += (fmaxf(zz, 0.f) - zz * y + log1pf(expf(-fabsf(zz)))) * invn;
-        S.g3g[grid_of_frame(p, F)] = (1.f / (1.f + expf(-zz)) - y) * invn;
-      }
-    }
-    __syncthreads();
-    // layer 3 gradients (FP32) and dL/dz2 = (W3^T g3) . (h2 > 0), stored in BF16
-    for (int i = threadIdx.x; i < kC * 9 + 1; i += blockDim.x) {
-      float s = 0.f;
-      for (int j = 0; j < S.n_sites; ++j) {
-        const int gp = grid_of_frame(S.sites[j], F);
-        if (i == kC * 9) {
-          s += S.g3g[gp];
-        } else {
-          const int c = i / 9, t = i % 9;
-          s += S.g3g[gp] * bf(S.h2[(gp + tap_off(t)) * kCP + c]);
-        }
-      }
-      if (i == kC * 9)
-        S.gb3 += s;
-      else
-        S.gw3[i] += s;
-    }
-    for (int i = threadIdx.x; i < FF * kC; i += blockDim.x) {
-      const int c = i % kC, q = i / kC, gqp = grid_of_frame(q, F);
-      float s = 0.f;
+      __syncthreads();
+      const int u0 = warp * 32;  // this warp's unit of 32 layer-1 rows
+      // ---- layer 1: h1 = relu(W1 * x + b1), W1 in three BF16 terms (exact products, FP32 sums) ----
+      if (u0 < R1) {
+        float acc[2][4][4] = {};
+        uint32_t ax[2][2][4];  // columns 0 .. 15 and 16 .. 31 of two times 16 rows
 #pragma unroll
-      for (int t = 0; t < 9; ++t) s += S.w3[c * 9 + t] * S.g3g[gqp - tap_off(t)];
-      const int gq = gqp * kCP + c;
-      const float v = bf(S.h2[gq]) > 0.f ? s : 0.f;
-      S.gz2[gq] = __float2bfloat16_rn(v);
-      S.gz1[q * kC + c] = v;  // FP32 dL/dz2 for the bias sum below (overwritten by g1)
-    }
-    __syncthreads();
-    // bias of layer 2 from the FP32 dL/dz2 (one thread per channel)
-    if (threadIdx.x < kC) {
-      float s = 0.f;
-      for (int q = 0; q < FF; ++q) s += S.gz1[q * kC + threadIdx.x];
-      S.gb2[threadIdx.x] += s;
-    }
-    // weight gradient of layer 2 on the tensor cores: K = frame positions
-    {
-      const int n_kt = (FF + 15) / 16;
-      for (int kt = 0; kt < n_kt; ++kt) {
-        // this lane's frame position in the A (gz2^T) and B (h1) tiles
-        const int pa = kt * 16 + (lane & 7) + ((lane >> 4) << 3);          // A: mat = lane >> 3, rows p
-        const int pb = kt * 16 + (lane & 7) + (((lane >> 3) & 1) << 3);    // B: rows p
-        const int ga = pa < FF ? grid_of_frame(pa, F) : -1;
-        const int gb = pb < FF ? grid_of_frame(pb, F) : -1;
-        const int oa = ((lane >> 3) & 1) * 8;   // A column (o) offset within the 16-row tile
-        const int cb = (lane >> 4) * 8;         // B column (c) offset: second n tile
-        // A tiles: gz2^T for o tiles 0 and 1
-        uint32_t a[2][4];
+        for (int m = 0; m < 2; ++m)
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-          ldm_x4_t(smem_addr(S.gz2 + (ga >= 0 ? ga : kZeroPos) * kCP + mt * 16 + oa), a[mt][0], a[mt][1],
-                   a[mt][2], a[mt][3]);
-        // tap `warp`: both o tiles, four c tiles
-        {
-          const int t = warp;
-          const int gbt = gb >= 0 ? gb + tap_off(t) : kZeroPos;
+          for (int k = 0; k < 2; ++k)
+            ldm_x4_row(S.x + (u0 + m * 16 + (lane & 15)) * kXP + k * 16 + (lane >> 4) * 8, ax[m][k]);
+        const __nv_bfloat16* wr =
+            S.w1s + ((lane & 7) + ((lane >> 4) << 3)) * (kW1K + 8) + ((lane >> 3) & 1) * 8;
 #pragma unroll
-          for (int np = 0; np < 2; ++np) {
-            uint32_t b0, b1, b2, b3;
-            ldm_x4_t(smem_addr(S.h1 + gbt * kCP + np * 16 + cb), b0, b1, b2, b3);
+        for (int q = 3; q >= 0; --q) {  // taps 0 .. 7 last, their smallest term first
+          uint32_t bw[8];
+          ldm_x4(smem_addr(wr + q * 16), bw[0], bw[1], bw[2], bw[3]);
+          ldm_x4(smem_addr(wr + q * 16 + 16 * (kW1K + 8)), bw[4], bw[5], bw[6], bw[7]);
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-              mma_bf16(dw[mt * 4 + np * 2 + 0], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
-              mma_bf16(dw[mt * 4 + np * 2 + 1], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b2, b3);
+          for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) {
+              const uint32_t(&a)[4] = ax[m][q == 3 ? 1 : 0];
+              mma_bf16(acc[m][nt], a[0], a[1], a[2], a[3], bw[2 * nt], bw[2 * nt + 1]);
             }
+        }
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            const int row = u0 + m * 16 + (lane >> 2) + half * 8;
+            uint32_t pos = 0u;
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) {
+              const int c = nt * 8 + (lane & 3) * 2;
+              const __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(acc[m][nt][2 * half], 0.f),
+                                                             fmaxf(acc[m][nt][2 * half + 1], 0.f));
+              *reinterpret_cast<__nv_bfloat162*>(&S.h1[row * kCP + c]) = h;
+              pos |= (bf(h.x) > 0.f ? 1u << c : 0u) | (bf(h.y) > 0.f ? 2u << c : 0u);
+            }
+            pos |= __shfl_xor_sync(0xffffffffu, pos, 1);
+            pos |= __shfl_xor_sync(0xffffffffu, pos, 2);
+            if ((lane & 3) == 0) S.mask[row] = row < R1 ? pos : 0u;
+          }
+      }
+      __syncthreads();
+      // ---- layer 2 forward on the tensor cores: units of 32 rows x 32 channels ----
+      for (int r0 = warp * 32; r0 < R2; r0 += kTcWarps * 32) {
+        float acc[2][4][4] = {};
+        int e9[2], base[2];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+          const int row = r0 + m * 16 + (lane & 15), w = (int)fdiv((uint32_t)row, f2);
+          e9[m] = row < R2 ? (row - w * n2) * 9 : -1;
+          base[m] = w * n1;
+        }
+        const __nv_bfloat16* b_base = S.w2f + ((lane & 7) + ((lane >> 4) << 3)) * kK2P + ((lane >> 3) & 1) * 8;
+        int nx[2];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) nx[m] = e9[m] < 0 ? kNone : S.nb1[e9[m]];
+#pragma unroll 1
+        for (int t = 0; t < 9; ++t) {
+          const __nv_bfloat16* ar[2];
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            const int i = nx[m];
+            if (t < 8 && e9[m] >= 0) nx[m] = S.nb1[e9[m] + t + 1];
+            ar[m] = S.h1 + (i == kNone ? kCap1 : base[m] + i) * kCP + (lane >> 4) * 8;
+          }
+#pragma unroll
+          for (int k = 0; k < kC; k += 16) {
+            uint32_t av[2][4], bv[8];
+            ldm_x4_row(ar[0] + k, av[0]);
+            ldm_x4_row(ar[1] + k, av[1]);
+            ldm_x4(smem_addr(b_base + t * kC + k), bv[0], bv[1], bv[2], bv[3]);
+            ldm_x4(smem_addr(b_base + 16 * kK2P + t * kC + k), bv[4], bv[5], bv[6], bv[7]);
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+              for (int nt = 0; nt < 4; ++nt)
+                mma_bf16(acc[m][nt], av[m][0], av[m][1], av[m][2], av[m][3], bv[2 * nt], bv[2 * nt + 1]);
           }
         }
-        // tap 8: o tile warp >> 2, c tile warp & 3
-        {
-          const int mt = warp >> 2, nt = warp & 3;
-          const int gbt = gb >= 0 ? gb + tap_off(8) : kZeroPos;
-          uint32_t b0, b1;
-          ldm_x2_t(smem_addr(S.h1 + gbt * kCP + nt * 8), b0, b1);
-          mma_bf16(dw[8], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            const int row = r0 + m * 16 + (lane >> 2) + half * 8;
+            if (row >= R2) continue;
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) {
+              const int o = nt * 8 + (lane & 3) * 2;
+              *reinterpret_cast<__nv_bfloat162*>(&S.h2[row * kCP + o]) =
+                  __floats2bfloat162_rn(fmaxf(acc[m][nt][2 * half] + S.b2[o], 0.f),
+                                        fmaxf(acc[m][nt][2 * half + 1] + S.b2[o + 1], 0.f));
+            }
+          }
+      }
+      __syncthreads();
+      // ---- layer 3 and the loss: eight lanes per site ----
+      for (int base = warp * 4; base < R3; base += kTcWarps * 4) {
+        const int si = base + (lane >> 3);
+        const int sub = lane & 7, c0 = 4 * sub;
+        float zz = 0.f;
+        int w = 0, j = 0;
+        if (si < R3) {
+          w = (int)fdiv((uint32_t)si, f3);
+          j = si - w * n3;
+#pragma unroll
+          for (int t = 0; t < 9; ++t) {
+            const __nv_bfloat16* h = &S.h2[(w * n2 + S.nb4[j * 9 + t]) * kCP + c0];
+            const float* w3 = &S.w3t[t * kC + c0];
+            zz += w3[0] * bf(h[0]) + w3[1] * bf(h[1]) + w3[2] * bf(h[2]) + w3[3] * bf(h[3]);
+          }
+        }
+        zz += __shfl_xor_sync(0xffffffffu, zz, 4);
+        zz += __shfl_xor_sync(0xffffffffu, zz, 2);
+        zz += __shfl_xor_sync(0xffffffffu, zz, 1);
+        if (si < R3 && sub == 0) {
+          zz += S.b3;
+          const float y = S.win[w * FF + (l3[j] / B + 1) * F + l3[j] % B + 1] > 0 ? 1.f : 0.f;
+          my_loss += (fmaxf(zz, 0.f) - zz * y + log1pf(expf(-fabsf(zz)))) * invn;
+          const float g = (1.f / (1.f + expf(-zz)) - y) * invn;
+          S.g3[si] = g;
+          gb3s += g;
         }
       }
-    }
-    __syncthreads();
-    // input gradient of layer 2 on the tensor cores: dL/dz1 = (W2^T * gz2) . (h1 > 0)
-    conv_gemm(S.gz2, S.w2r, F, -1, [&](int q, int c, float v) {
-      S.gz1[q * kC + c] = bf(S.h1[grid_of_frame(q, F) * kCP + c]) > 0.f ? v : 0.f;
-    });
-    __syncthreads();
-    // layer 1 gradients (FP32): lane = output channel, warp = a slice of the
-    // positions, sums kept in registers over all samples
-    for (int p = warp; p < FF; p += (int)(blockDim.x >> 5)) {
-      const float g = S.gz1[p * kC + lane];
-      const int gp = grid_of_frame(p, F);
-      gw1s[18] += g;
+      __syncthreads();
+      // ---- layer 3 gradients (FP32): lane = channel, one site per warp ----
+      for (int si = warp; si < R3; si += kTcWarps) {
+        const int w = (int)fdiv((uint32_t)si, f3), j = si - w * n3;
+        const float g = S.g3[si];
 #pragma unroll
-      for (int t = 0; t < 9; ++t) {
-        gw1s[t] += g * S.xg[0][gp + tap_off(t)];
-        gw1s[9 + t] += g * S.xg[1][gp + tap_off(t)];
+        for (int t = 0; t < 9; ++t) gw3s[t] += g * bf(S.h2[(w * n2 + S.nb4[j * 9 + t]) * kCP + lane]);
       }
+      // dL/dz2 = (W3^T g3) . (h2 > 0) in BF16, and its FP32 sum for the bias: eight lanes per row, four
+      // channels each; a row next to at most four sites (every staged one) reads them from one list entry
+      for (int r = warp * 4 + (lane >> 3); r < R2; r += kTcWarps * 4) {
+        const int w = (int)fdiv((uint32_t)r, f2), e = r - w * n2, c0 = (lane & 7) * 4;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        auto add = [&](int t, int site) {
+          const float4 w3 = *reinterpret_cast<const float4*>(&S.w3t[t * kC + c0]);
+          const float g = S.g3[w * n3 + site];
+          v.x += w3.x * g;
+          v.y += w3.y * g;
+          v.z += w3.z * g;
+          v.w += w3.w * g;
+        };
+        const uint32_t m = S.m3[e];
+        if (__popc(m) <= 4) {
+          const uint2 l = S.l3s[e];
+          const uint32_t x[4] = {l.x & 0xffffu, l.x >> 16, l.y & 0xffffu, l.y >> 16};
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (x[q] != kNone) add((int)(x[q] & 15u), (int)(x[q] >> 4));
+        } else {
+          for (uint32_t mm = m; mm; mm &= mm - 1) {
+            const int t = __ffs(mm) - 1;
+            add(t, S.nb3[e * 9 + t]);
+          }
+        }
+        const uint2 h = *reinterpret_cast<const uint2*>(&S.h2[r * kCP + c0]);
+        v.x = __uint_as_float(h.x << 16) > 0.f ? v.x : 0.f;
+        v.y = __uint_as_float(h.x & 0xffff0000u) > 0.f ? v.y : 0.f;
+        v.z = __uint_as_float(h.y << 16) > 0.f ? v.z : 0.f;
+        v.w = __uint_as_float(h.y & 0xffff0000u) > 0.f ? v.w : 0.f;
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+        *reinterpret_cast<uint2*>(&S.gz2[r * kCP + c0]) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+        gb2s.x += v.x;
+        gb2s.y += v.y;
+        gb2s.z += v.z;
+        gb2s.w += v.w;
+      }
+      __syncthreads();
+      // ---- weight gradient of layer 2 on the tensor cores: K = rows ----
+      for (int p0 = my_half * 16; p0 < R2; p0 += 32) {
+        // this lane's rows in the A (gz2^T) and B (h1) tiles; past the end: zero rows
+        const int pa = p0 + (lane & 7) + ((lane >> 4) << 3), pb = p0 + (lane & 15);
+        const int w = (int)fdiv((uint32_t)pb, f2);
+        const uint16_t* nb = &S.nb1[(pb - w * n2) * 9];
+        const int i = pb < R2 ? nb[my_tap] : kNone, i8 = pb < R2 ? nb[8] : kNone;
+        uint32_t av[2][4], bv[8], b8[2];
+        const __nv_bfloat16* ga = S.gz2 + (pa < R2 ? pa : kCap2) * kCP + ((lane >> 3) & 1) * 8;
+        ldm_x4_t(smem_addr(ga), av[0][0], av[0][1], av[0][2], av[0][3]);
+        ldm_x4_t(smem_addr(ga + 16), av[1][0], av[1][1], av[1][2], av[1][3]);
+        const __nv_bfloat16* hb = S.h1 + (i == kNone ? kCap1 : w * n1 + i) * kCP + (lane >> 4) * 8;
+        ldm_x4_t(smem_addr(hb), bv[0], bv[1], bv[2], bv[3]);
+        ldm_x4_t(smem_addr(hb + 16), bv[4], bv[5], bv[6], bv[7]);
+        ldm_x2_t(smem_addr(S.h1 + (i8 == kNone ? kCap1 : w * n1 + i8) * kCP + t8n * 8), b8[0], b8[1]);
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt)
+            mma_bf16(dw[m * 4 + nt], av[m][0], av[m][1], av[m][2], av[m][3], bv[2 * nt], bv[2 * nt + 1]);
+        const uint32_t* a8 = av[0];
+        mma_bf16(dw[8], t8m ? av[1][0] : a8[0], t8m ? av[1][1] : a8[1], t8m ? av[1][2] : a8[2], t8m ? av[1][3] : a8[3],
+                 b8[0], b8[1]);
+      }
+      // ---- input gradient of layer 2, transposed: D[c][q] = sum_{t,o} W2[o][c][t] gz2[q - d_t][o], one
+      // unit of 32 rows q per warp; masked with h1 > 0 it is dL/dz1^T, whose accumulator layout is the A
+      // operand of the layer-1 weight gradient dW1[c][j] += sum_q dL/dz1[q][c] x[q][j] ----
+      if (u0 < R1) {
+        float acc[2][4][4] = {};
+        int e9[2], base[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int q = u0 + h * 16 + (lane & 7) + ((lane >> 4) << 3), w = (int)fdiv((uint32_t)q, f1);
+          e9[h] = q < R1 ? (q - w * n1) * 9 : -1;
+          base[h] = w * n2;
+        }
+        const __nv_bfloat16* a_base = S.w2f + ((lane & 7) + ((lane >> 4) << 3)) * kK2P + ((lane >> 3) & 1) * 8;
+        int nx[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) nx[h] = e9[h] < 0 ? kNone : S.nb2[e9[h]];
+#pragma unroll 1
+        for (int t = 0; t < 9; ++t) {
+          const __nv_bfloat16* br[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int i = nx[h];
+            if (t < 8 && e9[h] >= 0) nx[h] = S.nb2[e9[h] + t + 1];
+            br[h] = S.gz2 + (i == kNone ? kCap2 : base[h] + i) * kCP + ((lane >> 3) & 1) * 8;
+          }
+#pragma unroll
+          for (int k = 0; k < kC; k += 16) {
+            uint32_t av[2][4], bv[8];
+            ldm_x4_t(smem_addr(a_base + k * kK2P + t * kC), av[0][0], av[0][1], av[0][2], av[0][3]);
+            ldm_x4_t(smem_addr(a_base + k * kK2P + t * kC + 16), av[1][0], av[1][1], av[1][2], av[1][3]);
+            ldm_x4(smem_addr(br[0] + k), bv[0], bv[1], bv[2], bv[3]);
+            ldm_x4(smem_addr(br[1] + k), bv[4], bv[5], bv[6], bv[7]);
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+              for (int nt = 0; nt < 4; ++nt)
+                mma_bf16(acc[m][nt], av[m][0], av[m][1], av[m][2], av[m][3], bv[2 * nt], bv[2 * nt + 1]);
+          }
+        }
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) {  // 16 rows at a time
+          uint32_t xb[6];
+          const __nv_bfloat16* xr = S.x + (u0 + kk * 16 + (lane & 15)) * kXP;
+          ldm_x4_t(smem_addr(xr + (lane >> 4) * 8), xb[0], xb[1], xb[2], xb[3]);
+          ldm_x2_t(smem_addr(xr + 16), xb[4], xb[5]);
+          uint2 mk[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            mk[h] = *reinterpret_cast<const uint2*>(&S.mask[u0 + kk * 16 + h * 8 + (lane & 3) * 2]);
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            uint32_t a[4][3];  // A registers (rows g, g + 8; columns of tile 2 kk, 2 kk + 1), three terms each
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              const float* d = acc[m][2 * kk + (r >> 1)] + 2 * (r & 1);
+              const uint32_t bit = 1u << (m * 16 + (lane >> 2) + (r & 1) * 8);
+              split3(mk[r >> 1].x & bit ? d[0] : 0.f, mk[r >> 1].y & bit ? d[1] : 0.f, a[r]);
+            }
+#pragma unroll
+            for (int q = 2; q >= 0; --q)
+#pragma unroll
+              for (int nt = 0; nt < 3; ++nt)
+                mma_bf16(dw1[m][nt], a[0][q], a[1][q], a[2][q], a[3][q], xb[2 * nt], xb[2 * nt + 1]);
+          }
+        }
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
-  // flush this CTA's sums
-  {
-    const int g = lane >> 2, t2 = (lane & 3) * 2;
-    auto put = [&](const float (&d)[4], int t, int mt, int nt) {
+  // add this CTA's sums to the global gradient: the warps' sums meet in shared
+  // memory (the h1 and h2 buffers)
+  const int g = lane >> 2, t2 = (lane & 3) * 2;
+  float* red = reinterpret_cast<float*>(S.h1);
+  if (my_half == 1) {
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) red[((my_tap * 9 + q) * 4 + e) * 32 + lane] = dw[q][e];
+  }
+  __syncthreads();
+  if (my_half == 0) {
+#pragma unroll
+    for (int q = 0; q < 9; ++q)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const int o = mt * 16 + g + (e >> 1) * 8, c = nt * 8 + t2 + (e & 1);
-        if (d[e] != 0.f) atomicAdd(&grads[kOffW2 + (o * kC + c) * 9 + t], d[e]);
+        const float v = dw[q][e] + red[((my_tap * 9 + q) * 4 + e) * 32 + lane];
+        const int m = q < 8 ? q >> 2 : t8m, nt = q < 8 ? q & 3 : t8n, t = q < 8 ? my_tap : 8;
+        const int o = m * 16 + g + (e >> 1) * 8, c = nt * 8 + t2 + (e & 1);
+        if (v != 0.f) atomicAdd(&grads[kOffW2 + (o * kC + c) * 9 + t], v);
       }
-    };
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt) put(dw[mt * 4 + nt], warp, mt, nt);
-    put(dw[8], 8, warp >> 2, warp & 3);
-  }
-  // layer-1 sums: reduce the warps' partial sums in shared memory
-#pragma unroll
-  for (int j = 0; j < 18; ++j) S.red[warp][lane * 18 + j] = gw1s[j];
-  S.red[warp][kC * 18 + lane] = gw1s[18];
-  __syncthreads();
-  for (int i = threadIdx.x; i < kC * 18 + kC; i += blockDim.x) {
-    float s = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += S.red[w][i];
-    if (i < kC * 18)
-      S.gw1[i] += s;  // [o][ci * 9 + t] = W1[o][ci][t]
-    else
-      S.gb1[i - kC * 18] += s;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < kC * 18; i += blockDim.x)
-    if (S.gw1[i] != 0.f) atomicAdd(&grads[kOffW1 + i], S.gw1[i]);
-  for (int i = threadIdx.x; i < kC * 9; i += blockDim.x)
-    if (S.gw3[i] != 0.f) atomicAdd(&grads[kOffW3 + i], S.gw3[i]);
-  for (int i = threadIdx.x; i < kC; i += blockDim.x) {
-    if (S.gb1[i] != 0.f) atomicAdd(&grads[kOffB1 + i], S.gb1[i]);
-    if (S.gb2[i] != 0.f) atomicAdd(&grads[kOffB2 + i], S.gb2[i]);
-  }
-  if (threadIdx.x == 0 && S.gb3 != 0.f) atomicAdd(&grads[kOffB3], S.gb3);
+  float* mine = red + warp * kRed * kC;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) my_loss += __shfl_xor_sync(0xffffffffu, my_loss, o);
-  if (lane == 0) atomicAdd(loss, my_loss);
+  for (int m = 0; m < 2; ++m)
+#pragma unroll
+    for (int nt = 0; nt < 3; ++nt)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int c = m * 16 + g + (e >> 1) * 8, j = nt * 8 + t2 + (e & 1);  // column j = 2 t + ci
+        if (j < 19) mine[(j == 18 ? 18 : (j & 1) * 9 + (j >> 1)) * kC + c] = dw1[m][nt][e];
+      }
+#pragma unroll
+  for (int o = 8; o <= 16; o <<= 1) {
+    gb2s.x += __shfl_xor_sync(0xffffffffu, gb2s.x, o);
+    gb2s.y += __shfl_xor_sync(0xffffffffu, gb2s.y, o);
+    gb2s.z += __shfl_xor_sync(0xffffffffu, gb2s.z, o);
+    gb2s.w += __shfl_xor_sync(0xffffffffu, gb2s.w, o);
+  }
+  if (lane < 8) *reinterpret_cast<float4*>(&mine[19 * kC + 4 * lane]) = gb2s;
+#pragma unroll
+  for (int t = 0; t < 9; ++t) mine[(20 + t) * kC + lane] = gw3s[t];
+  __syncthreads();
+  for (int i = tid; i < 29 * kC; i += kTcThreads) {
+    float v = 0.f;
+    for (int w = 0; w < kTcWarps; ++w) v += red[w * kRed * kC + i];
+    const int j = i / kC, c = i % kC;
+    const int at = j < 18 ? kOffW1 + c * 18 + j : j == 18 ? kOffB1 + c : j == 19 ? kOffB2 + c : kOffW3 + c * 9 + j - 20;
+    if (v != 0.f) atomicAdd(&grads[at], v);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    my_loss += __shfl_xor_sync(0xffffffffu, my_loss, o);
+    gb3s += __shfl_xor_sync(0xffffffffu, gb3s, o);
+  }
+  if (lane == 0) {
+    atomicAdd(loss, my_loss);
+    if (gb3s != 0.f) atomicAdd(&grads[kOffB3], gb3s);
+  }
 }
 
 }  // namespace
@@ -401,7 +608,7 @@ cudaError_t nn_train_tc(const int8_t* windows, int count, const StagedPlan* d_pl
     attr.set(1);
   }
   const int g = std::max(1, std::min(count * n_net, grid));
-  k_nn_train_tc<<<g, kThreads, sizeof(TrainTcSmem), s>>>(windows, count, d_plan, params, grads, loss);
+  k_nn_train_tc<<<g, kTcThreads, sizeof(TrainTcSmem), s>>>(windows, count, d_plan, params, grads, loss);
   return cudaGetLastError();
 }
 
