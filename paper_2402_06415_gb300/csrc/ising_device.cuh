@@ -345,6 +345,57 @@ __device__ __forceinline__ bool grid_sync_bounded(GridCtl* ctl, long long limit)
   return s_ok != 0;
 }
 
+// Boundary words travel as 8-byte (tag, word) pairs, written and polled with
+// single 8-byte accesses: the reader sees the word as soon as it sees the tag,
+// so an exchange is one store and one load through L2, without a fence, a flag
+// or a second load.
+__device__ __forceinline__ void send_word(unsigned long long* slot, uint32_t tag, uint32_t word) {
+  const unsigned long long v = ((unsigned long long)tag << 32) | word;
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(slot), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long poll_word(const unsigned long long* slot) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(slot) : "memory");
+  return v;
+}
+// Waits for the pair with this tag; false (and *status = 1) after `limit` cycles.
+__device__ __forceinline__ bool recv_word(const unsigned long long* slot, uint32_t tag, long long limit, int* status,
+                                          uint32_t& word) {
+  unsigned long long v = poll_word(slot);
+  if ((uint32_t)(v >> 32) != tag) {
+    const long long start = clock64();
+    do {
+      if (clock64() - start > limit) {
+        *reinterpret_cast<volatile int*>(status) = 1;
+        return false;
+      }
+      v = poll_word(slot);
+    } while ((uint32_t)(v >> 32) != tag);
+  }
+  word = (uint32_t)v;
+  return true;
+}
+
+// Receives words tid, tid + nth, ... < n, N of them in flight at a time (an L2 round
+// trip is 0.4 us): src(i) is the slot, put(i, word) takes the word.
+template <int N, typename Src, typename Put>
+__device__ __forceinline__ void recv_words(int tid, int nth, int n, Src src, uint32_t tag, long long limit,
+                                           int* status, bool& ok, Put put) {
+  for (int base = tid; base < n; base += N * nth) {
+    unsigned long long v[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = base + q * nth < n ? poll_word(src(base + q * nth)) : 0ull;
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const int i = base + q * nth;
+      if (i >= n) break;
+      uint32_t word = (uint32_t)v[q];
+      if ((uint32_t)(v[q] >> 32) != tag) ok = ok && recv_word(src(i), tag, limit, status, word);
+      put(i, word);
+    }
+  }
+}
+
 __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -50,37 +50,6 @@ __device__ __forceinline__ void planes_first(uint32_t g, uint32_t t, uint32_t re
   D = eq;
 }
 
-// Boundary words travel as 8-byte (tag, word) pairs, written and polled with
-// single 8-byte accesses: the reader sees the word as soon as it sees the tag,
-// so an exchange is one store and one load through L2, without a fence, a flag
-// or a second load.
-__device__ __forceinline__ void send_word(unsigned long long* slot, uint32_t tag, uint32_t word) {
-  const unsigned long long v = ((unsigned long long)tag << 32) | word;
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(slot), "l"(v) : "memory");
-}
-__device__ __forceinline__ unsigned long long poll_word(const unsigned long long* slot) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(slot) : "memory");
-  return v;
-}
-// Waits for the pair with this tag; false (and *status = 1) after `limit` cycles.
-__device__ __forceinline__ bool recv_word(const unsigned long long* slot, uint32_t tag, long long limit, int* status,
-                                          uint32_t& word) {
-  unsigned long long v = poll_word(slot);
-  if ((uint32_t)(v >> 32) != tag) {
-    const long long start = clock64();
-    do {
-      if (clock64() - start > limit) {
-        *reinterpret_cast<volatile int*>(status) = 1;
-        return false;
-      }
-      v = poll_word(slot);
-    } while ((uint32_t)(v >> 32) != tag);
-  }
-  word = (uint32_t)v;
-  return true;
-}
-
 template <bool WHOLE, bool I8, bool SPLIT>
 __global__ void __launch_bounds__(SPLIT ? kSplitThreads : kStripThreads) k_strip(StripArgs a, RngParams rng) {
   extern __shared__ uint32_t strip_smem[];
@@ -297,14 +266,16 @@ __global__ void __launch_bounds__(SPLIT ? kSplitThreads : kStripThreads) k_strip
       send_word(mine + buf + i, tag, P(c)[(lower ? R * Wc : H * Wc) + k]);
     }
     bool ok = true;
-    for (int i = tid; i < 4 * hw; i += nth) {
+    // the upper neighbour's lower rows, the lower neighbour's upper rows
+    auto src = [&](int i) {
+      const int lower = i >= 2 * hw;
+      return (lower ? dn_slots : up_slots + 2 * hw) + buf + (i - lower * 2 * hw);
+    };
+    recv_words<SPLIT ? 1 : 4>(tid, nth, 4 * hw, src, tag, a.limit, a.status, ok, [&](int i, uint32_t word) {
       const int lower = i >= 2 * hw, rem = i - lower * 2 * hw;
       const int c = rem >= hw, k = rem - c * hw;
-      // the upper neighbour's lower rows, the lower neighbour's upper rows
-      uint32_t word = 0;
-      ok = ok && recv_word((lower ? dn_slots : up_slots + 2 * hw) + buf + rem, tag, a.limit, a.status, word);
       P(c)[(lower ? (H + R) * Wc : 0) + k] = word;
-    }
+    });
     if (!__syncthreads_and(ok)) return;
     if (SPLIT) {
       own[0] = P(0)[i1];

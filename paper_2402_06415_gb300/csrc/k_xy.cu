@@ -165,6 +165,36 @@ __device__ __forceinline__ T angle_of(uint32_t w) {
   return mul_rn<T>(two_pi<T>(), mul_rn<T>((T)(w >> 8), inv24<T>()));
 }
 
+// sin and cos of the angle of a random word.  Same values as
+// own_sincos(angle_of<T>(w)); in double, where every operation holds this part's
+// FP64 unit for 64 cycles per warp and sub-partition, without five of them: the
+// conversion is integer work, the exact scaling by 2^-24 sits in the constant,
+// and the quadrant k = rint(x 2 / pi) is the integer (m + 2^21) >> 22 unless
+// m / 2^22 is exactly a half integer (m / 2^22 differs from x 2 / pi by less
+// than 2e-15, and otherwise lies at least 2^-22 from a half integer).
+__device__ __forceinline__ void word_sincos(uint32_t w, float& s, float& c) { own_sincos(angle_of<float>(w), s, c); }
+__device__ __forceinline__ void word_sincos(uint32_t w, double& s, double& c) {
+  const uint32_t m = w >> 8;
+  // m and k as doubles from their (exact) floats; no branches: the lanes differ
+  const uint32_t mf = __float_as_uint((float)m);
+  const double md = __hiloint2double(m ? (int)((mf >> 3) + 0x38000000u) : 0, (int)(mf << 29));
+  const double x = __dmul_rn(6.283185307179586 / 16777216.0, md);
+  uint32_t k = (m + (1u << 21)) >> 22;
+  if ((m & 0x3fffffu) == 0x200000u) k = (uint32_t)rint(__dmul_rn(x, 0.6366197723675814));
+  const uint32_t kf = __float_as_uint((float)k);
+  const double kd = __hiloint2double(k ? (int)((kf >> 3) + 0xb8000000u) : (int)0x80000000u, 0);  // -k
+  double r = fma(kd, 1.5707963267948966, x);
+  r = fma(kd, 6.123233995736766e-17, r);
+  double ss, cc;
+  sincos_small(r, ss, cc);
+  // quadrant k & 3: swap sin and cos, then flip their sign bits
+  const bool swap = (k & 1u) != 0;
+  const int s_hi = __double2hiint(swap ? cc : ss) ^ (int)((k & 2u) << 30);
+  const int c_hi = __double2hiint(swap ? ss : cc) ^ (int)(((k + 1u) & 2u) << 30);
+  s = __hiloint2double(s_hi, __double2loint(swap ? cc : ss));
+  c = __hiloint2double(c_hi, __double2loint(swap ? ss : cc));
+}
+
 template <typename T>
 __global__ void k_xy_init(typename Vec<T>::type* __restrict__ u, int L, RngParams rng) {
   const long long N = (long long)L * L;
@@ -176,7 +206,7 @@ __global__ void k_xy_init(typename Vec<T>::type* __restrict__ u, int L, RngParam
                                 rng.rk0, rng.rk1);
     const uint32_t w = (n & 3) == 0 ? r.x : ((n & 3) == 1 ? r.y : ((n & 3) == 2 ? r.z : r.w));
     T s, c;
-    own_sincos(angle_of<T>(w), s, c);
+    word_sincos(w, s, c);
     const int col = (x + y) & 1;
     typename Vec<T>::type v;
     v.x = c;
@@ -203,6 +233,33 @@ __device__ __forceinline__ bool accept_exp(T p, T x) {
     return false;
   }
   return p < own_exp(x);
+}
+
+// The trial's decision: dE <= 0 or p < exp(-beta dE), p = the top 24 bits of w2.
+__device__ __forceinline__ bool accept_move(uint32_t w2, float dE, float beta, float) {
+  return dE <= 0.f || accept_exp<float>(mul_rn<float>((float)(w2 >> 8), inv24<float>()), mul_rn<float>(-beta, dE));
+}
+// In double, the sign and the estimate that decides all but a band of 1e-4 need
+// no FP64 operation: -beta dE is formed in float (beta_f = beta) from dE's bits cut to 24
+// (relative error below 2^-22, so below 2e-5 in exp for -beta dE >= -80, next to
+// the 1e-5 of __expf); the band, and p = 0 below -80, are decided exactly.
+__device__ __forceinline__ bool accept_move(uint32_t w2, double dE, double beta, float beta_f) {
+  const int hi = __double2hiint(dE), lo = __double2loint(dE);
+  const int mag = hi & 0x7fffffff;
+  if (mag < 0x7ff00000 && (hi < 0 || (mag | lo) == 0)) return true;
+  const int ex = (mag >> 20) - 1023 + 127;
+  const float d = ex <= 0 ? 0.f : ex >= 255 ? __int_as_float(0x7f800000)
+                                            : __uint_as_float(((uint32_t)ex << 23) | ((uint32_t)(hi & 0xfffff) << 3) |
+                                                              ((uint32_t)lo >> 29));
+  const float x = -beta_f * d, p = (float)(w2 >> 8) * (1.0f / 16777216.0f);
+  if (x >= -80.f) {
+    const float e = __expf(x);
+    if (p < e * 0.9999f) return true;
+    if (p > e * 1.0001f) return false;
+  } else if (p > 0.f) {
+    return false;
+  }
+  return dE <= 0.0 || (double)p < own_exp(__dmul_rn(-beta, dE));
 }
 
 // Loads and stores of the state: plain in the one-launch-per-half-sweep
@@ -252,11 +309,10 @@ __device__ __forceinline__ unsigned int xy_pair(typename Vec<T>::type* __restric
     hy = add_rn<T>(hy, e.y);
     const uint32_t w1 = h == 0 ? r.x : r.z, w2 = h == 0 ? r.y : r.w;
     T sn, cs;
-    own_sincos(angle_of<T>(w1), sn, cs);
-    const T p = mul_rn<T>((T)(w2 >> 8), inv24<T>());
+    word_sincos(w1, sn, cs);
     V me = ld_state<CG>(own + k);
     const T dE = -fma(sub_rn<T>(cs, me.x), hx, mul_rn<T>(sub_rn<T>(sn, me.y), hy));
-    if (dE <= (T)0 || accept_exp<T>(p, mul_rn<T>(-beta, dE))) {
+    if (accept_move(w2, dE, beta, (float)beta)) {
       me.x = cs;
       me.y = sn;
       st_state<CG>(own + k, me);
@@ -388,6 +444,243 @@ __global__ void __launch_bounds__(PM == kGrid ? 256 : 1024) k_xy_persist(typenam
   add_accepted(accepted, acc);
 }
 
+// Resident strips: many sweeps in one launch for lattices whose half sweep is
+// too short for a launch or a grid barrier of its own.  G CTAs own row strips of
+// full width, both colours in shared memory, with a halo of `gh` rows; gh half
+// sweeps run with CTA barriers only (each invalidates one more halo row), then
+// the strips hand their outer rows to their neighbours as (tag, word) pairs
+// through L2.  G = 1 keeps the whole lattice in one CTA.  A thread updates the
+// two sites of one Philox block (k = 2b, 2b + 1; their parity survives the wrap
+// because L^2 / 2 is even).  AHEAD (at most one block per thread): the proposals
+// of the next half sweep, which do not depend on spins, are drawn before the
+// barrier or while the neighbours' rows are on their way; in FP64 their sines
+// and cosines are most of the work of this part's slow FP64 pipe.
+// E, Mx, My of a recorded sweep are summed (in double) in the colour-1 half
+// sweep itself: every bond joins a colour-1 site to a colour-0 neighbour.
+// Per sweep with a record each, before (a grid barrier or launch per half sweep
+// and per measurement) and now: FP64 L = 32 17.1 -> 5.2 us, FP32 L = 512 (a record
+// every 10 sweeps) 14.9 -> 5.6 us.  What bounds it: FP64, the 31 FP64 operations of a
+// trial at 64 cycles per warp and sub-partition; FP32, the dependent chain of a
+// half sweep up to L ~ 256, then issue slots.
+template <typename T>
+struct XYStripArgs {
+  typename Vec<T>::type* u;
+  int L, G, gh;
+  T beta;
+  float beta_f;
+  uint32_t t0;
+  int n, m, to_rec;  // sweeps; record every m; sweeps until the first record (0: none)
+  double* rec;
+  long long rec0, rec_cap;
+  unsigned long long* accepted;
+  unsigned long long* xbuf;  // xy_strip_words(...) pairs, zeroed by the launcher (G > 1)
+  int* status;
+  long long limit;
+  FastDiv fh;
+};
+constexpr int kXYStripThreads = 512;
+
+template <typename T>
+size_t xy_strip_words(int L, int G, int gh) {
+  return G == 1 ? 0 : (size_t)G * (8 * (size_t)gh * (L / 2) * (sizeof(typename Vec<T>::type) / 4) + 1);
+}
+template <typename T>
+size_t xy_strip_smem(int L, int G, int gh) {
+  return 2 * (size_t)((L + G - 1) / G + (G == 1 ? 0 : 2 * gh)) * (L / 2) * sizeof(typename Vec<T>::type);
+}
+
+template <typename T, bool WHOLE, bool AHEAD>
+__global__ void __launch_bounds__(kXYStripThreads) k_xy_strip(XYStripArgs<T> a, RngParams rng) {
+  using V = typename Vec<T>::type;
+  constexpr int VW = sizeof(V) / 4;
+  extern __shared__ uint4 xy_smem[];
+  const int L = a.L, half = L / 2, G = WHOLE ? 1 : a.G, H = WHOLE ? 0 : a.gh;
+  const int b = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
+  const int y0 = (int)((long long)b * L / G), R = (int)((long long)(b + 1) * L / G) - y0;
+  const int rows = R + 2 * H, ns = rows * half, N2 = L * half;
+  const int plane = ((L + G - 1) / G + 2 * H) * half;
+  V* const S = reinterpret_cast<V*>(xy_smem);
+  auto P = [&](int c) { return S + c * plane; };
+  const int koff = (y0 - H) * half;  // local site i is site i + koff of its colour, modulo N2
+  auto global_k = [&](int i) {
+    int k = i + koff;
+    if (!WHOLE) {
+      k += k < 0 ? N2 : 0;
+      k -= k >= N2 ? N2 : 0;
+    }
+    return k;
+  };
+  for (int i = tid; i < 2 * ns; i += nth) {
+    const int c = i >= ns, k = i - c * ns;
+    P(c)[k] = __ldcg(&a.u[(size_t)c * N2 + global_k(k)]);
+  }
+  __syncthreads();
+  const int hw = H * half * VW;  // 32-bit words of H rows of one colour
+  const size_t per_cta = 8 * (size_t)hw + 1;
+  const int up = b == 0 ? G - 1 : b - 1, dn = b == G - 1 ? 0 : b + 1;
+  unsigned long long* const mine = WHOLE ? nullptr : a.xbuf + b * per_cta;
+  if (!WHOLE && tid == 0) send_word(mine + 8 * hw, 1u, 0u);  // "lattice read"
+  // an item is one site (SPT = 1) or the two sites of a block (item j: local sites
+  // 2 j - par, 2 j - par + 1)
+  constexpr int SPT = (AHEAD || sizeof(T) == 8) ? 1 : 2;
+  const int par = SPT == 2 ? koff & 1 : 0;
+  // AHEAD: one item per thread, in rows 1 .. rows - 2 (the outermost halo rows are only read)
+  const int item = tid + (WHOLE ? 0 : half), items_end = ns - (WHOLE ? 0 : half);
+  auto in_rows = [&](int i, int lo) { return i >= lo * half && i < ns - lo * half; };
+
+  struct Prop {
+    T cs[SPT], sn[SPT];
+    uint32_t w2[SPT];
+  };
+  auto propose = [&](int j, uint32_t t, int c, Prop& q) {
+    const uint32_t k = (uint32_t)global_k(SPT * j - par);
+    const uint4 r = philox10_rk(make_uint4(k >> 1, t, rng.replica, (kTagXYMet << 16) | ((uint32_t)c << 8)), rng.rk0,
+                                rng.rk1);
+#pragma unroll
+    for (int h = 0; h < SPT; ++h) {
+      const bool second = SPT == 2 ? h == 1 : (k & 1u) != 0;
+      word_sincos(second ? r.z : r.x, q.sn[h], q.cs[h]);
+      q.w2[h] = second ? r.w : r.y;
+    }
+  };
+  unsigned int acc = 0;
+  double e = 0, mx = 0, my = 0;
+  // trials of item j in the rows [lo, rows - lo) of colour c
+  auto update = [&](int j, int c, int lo, bool meas, const Prop& q) {
+    V* const So = P(c);
+    const V* const Sn = P(1 - c);
+#pragma unroll
+    for (int h = 0; h < SPT; ++h) {
+      const int i = SPT * j - par + h;
+      if (!in_rows(i, lo)) continue;
+      const int r = (int)fdiv((uint32_t)i, a.fh), x = i - r * half, row = i - x;
+      const int o = (y0 - H + r + c) & 1;
+      const int ir = o == 0 ? i : row + (x + 1 == half ? 0 : x + 1);
+      const int il = o == 0 ? row + (x == 0 ? half - 1 : x - 1) : i;
+      int id = i + half, iu = i - half;
+      if (WHOLE) {
+        id -= id >= ns ? ns : 0;
+        iu += iu < 0 ? ns : 0;
+      }
+      const V va = Sn[ir], vb = Sn[il], vd = Sn[id], ve = Sn[iu];
+      T hx = add_rn<T>(va.x, vb.x);
+      hx = add_rn<T>(hx, vd.x);
+      hx = add_rn<T>(hx, ve.x);
+      T hy = add_rn<T>(va.y, vb.y);
+      hy = add_rn<T>(hy, vd.y);
+      hy = add_rn<T>(hy, ve.y);
+      V me = So[i];
+      const T dE = -fma(sub_rn<T>(q.cs[h], me.x), hx, mul_rn<T>(sub_rn<T>(q.sn[h], me.y), hy));
+      const bool own = WHOLE || (r >= H && r < H + R);
+      if (accept_move(q.w2[h], dE, a.beta, a.beta_f)) {
+        me.x = q.cs[h];
+        me.y = q.sn[h];
+        So[i] = me;
+        acc += own;
+      }
+      if (meas && own) {
+        double b2;  // u . h: in double from the neighbours themselves when T is float
+        if (sizeof(T) == 8) {
+          b2 = (double)me.x * (double)hx + (double)me.y * (double)hy;
+        } else {
+          const double dx = (double)va.x + vb.x + vd.x + ve.x, dy = (double)va.y + vb.y + vd.y + ve.y;
+          b2 = (double)me.x * dx + (double)me.y * dy;
+        }
+        const V s0 = Sn[i];
+        const double tx = (double)me.x + (double)s0.x, ty = (double)me.y + (double)s0.y;
+        e = AHEAD ? -b2 : e - b2;  // AHEAD: the thread's only site
+        mx = AHEAD ? tx : mx + tx;
+        my = AHEAD ? ty : my + ty;
+      }
+    }
+  };
+
+  Prop q;
+  if (AHEAD && item < items_end) propose(item, a.t0, 0, q);
+  int to_rec = a.to_rec, g = 0;
+  long long slot = a.rec0;
+  uint32_t exchanges = 0;
+  const int halves = 2 * a.n;
+  for (int hh = 0; hh < halves; ++hh) {
+    const int c = hh & 1;
+    const uint32_t t = a.t0 + (uint32_t)(hh >> 1), t_next = a.t0 + (uint32_t)((hh + 1) >> 1);
+    const bool meas = c == 1 && to_rec == 1;
+    const int lo = WHOLE ? 0 : g + 1;
+    const bool swap = !WHOLE && g + 1 == H && hh + 1 < halves;
+    if (AHEAD) {
+      if (in_rows(item, lo)) update(item, c, lo, meas, q);
+      if (!swap && in_rows(item, WHOLE ? 0 : lo + 1)) propose(item, t_next, 1 - c, q);
+    } else {
+      for (int j = (lo * half + par) / SPT + tid; SPT * j - par < ns - lo * half; j += nth) {
+        propose(j, t, c, q);
+        update(j, c, lo, meas, q);
+      }
+    }
+    if (meas) {
+      // warp sums of the three values with 6 additions instead of 15: after the
+      // first exchange the lower lanes hold (e, mx), the upper ones (my, -), after
+      // the second lanes 0, 8, 16 ... hold one value each
+      const bool up4 = (tid & 16) != 0, up3 = (tid & 8) != 0;
+      const double p = (up4 ? my : e) + __shfl_xor_sync(0xffffffffu, up4 ? e : my, 16);
+      const double r = (up4 ? 0.0 : mx) + __shfl_xor_sync(0xffffffffu, up4 ? mx : 0.0, 16);
+      double v = (up3 ? r : p) + __shfl_xor_sync(0xffffffffu, up3 ? p : r, 8);
+#pragma unroll
+      for (int off = 4; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+      const int which = (up4 ? 2 : 0) + (up3 ? 1 : 0);  // 0: E, 1: Mx, 2: My
+      if ((tid & 7) == 0 && which < 3) atomicAdd(&a.rec[3 * slot + which], v);
+      e = mx = my = 0;
+    }
+    if (c == 1 && to_rec > 0 && --to_rec == 0) {
+      to_rec = a.m;
+      slot = slot + 1 == a.rec_cap ? 0 : slot + 1;
+    }
+    __syncthreads();
+    ++g;
+    if (!swap) continue;
+    g = 0;
+    // own rows [H, 2H) go up, [R, R + H) go down; with one half sweep between
+    // exchanges only the colour just updated changed
+    const uint32_t tag = ++exchanges;
+    const size_t buf = (size_t)(tag & 1) * 4 * hw;
+    const int c_first = H == 1 ? c : 0, c_count = H == 1 ? 1 : 2;
+    const uint32_t* const words = reinterpret_cast<const uint32_t*>(S);
+    for (int i = tid; i < 2 * c_count * hw; i += nth) {
+      const int lower = i >= c_count * hw, rem = i - lower * c_count * hw;
+      const int cc = c_first + (rem >= hw), k = rem - (rem >= hw ? hw : 0);
+      send_word(mine + buf + (lower * 2 + cc) * (size_t)hw + k, tag,
+                words[(size_t)(cc * plane + (lower ? R : H) * half) * VW + k]);
+    }
+    if (AHEAD && item < items_end) propose(item, t_next, 1 - c, q);
+    bool ok = true;
+    const int total = 2 * c_count * hw;
+    // the upper neighbour's lower rows, the lower neighbour's upper rows; four
+    // loads in flight per thread
+    auto src = [&](int i) {
+      const int lower = i >= c_count * hw, rem = i - lower * c_count * hw;
+      const int cc = c_first + (rem >= hw), k = rem - (rem >= hw ? hw : 0);
+      return a.xbuf + (lower ? dn : up) * per_cta + buf + ((1 - lower) * 2 + cc) * (size_t)hw + k;
+    };
+    recv_words<4>(tid, nth, total, src, tag, a.limit, a.status, ok, [&](int i, uint32_t word) {
+      const int lower = i >= c_count * hw, rem = i - lower * c_count * hw;
+      const int cc = c_first + (rem >= hw), k = rem - (rem >= hw ? hw : 0);
+      reinterpret_cast<uint32_t*>(S)[(size_t)(cc * plane + (lower ? H + R : 0) * half) * VW + k] = word;
+    });
+    if (!__syncthreads_and(ok)) return;
+  }
+  // in place: both neighbours must have read their halos
+  if (!WHOLE && exchanges == 0) {
+    uint32_t word;
+    bool ok = true;
+    if (tid < 2) ok = recv_word(a.xbuf + (tid ? dn : up) * per_cta + 8 * hw, 1u, a.limit, a.status, word);
+    if (!__syncthreads_and(ok)) return;
+  }
+  for (int i = tid; i < 2 * R * half; i += nth) {
+    const int c = i >= R * half, k = i - c * R * half;
+    a.u[(size_t)c * N2 + (size_t)y0 * half + k] = P(c)[H * half + k];
+  }
+  add_accepted(a.accepted, acc);
+}
+
 // Self-test of the persistent kernels' barrier: CTA 0 never arrives, so every
 // other CTA must give up after `limit` cycles and record the time-out.
 __global__ void k_grid_barrier_selftest(GridCtl* ctl, long long limit) {
@@ -458,15 +751,112 @@ struct ising_xy {
   double* rec = nullptr;  // ring [65536][3]
   int64_t rec_count = 0;
   unsigned long long* accepted = nullptr;
-  double* host_scratch = nullptr;
+  // resident strips of the automatic mode (G = 0: one launch per half sweep)
+  int strip_G = 0, strip_gh = 0;
+  unsigned long long* strip_x = nullptr;
+  int* strip_status = nullptr;  // pinned host word a strip sets when a wait gave up
 };
 
 namespace {
 constexpr int64_t kXYRec = 65536;
 
-// Largest L for which the automatic mode runs the persistent kernel.
-constexpr int kXYPersistMaxL = 256;
+// Largest L for which the automatic mode runs the resident strips.
+// (us per sweep, strips / one launch per half sweep: FP64 L = 256 8.9 / 17.6, 1024 76 / 78; FP32 L = 256 3.1 / 8.2,
+// 1024 13.1 / 20.6)
+constexpr int kXYStripMaxL = 1024;
 constexpr long long kXYSpinLimit = 4000000000LL;  // ~2 s of SM clock per barrier
+
+// Strips and half sweeps per exchange for an L x L lattice by a time model (us),
+// fitted on GB300 (within 20 % of the measured times, L = 8 ... 1024): a half sweep
+// with w warps of sites per SM sub-partition takes 0.5 + 1.05 w in FP64 (31
+// operations at 64 cycles per warp) and 0.45 + 0.08 w in FP32 (0.5 + 0.0013 per site
+// past one site per thread), an exchange 0.9 + 3e-4 per word.
+struct XYStrip {
+  int G, gh;
+  double us;
+};
+template <typename T>
+XYStrip choose_xy_strip(int L, int sms) {
+  const int half = L / 2;
+  XYStrip best{0, 0, 1e30};
+  for (int G = 1; G <= sms && G <= L; ++G)
+    for (int gh = 1; gh <= (G == 1 ? 1 : 4); gh *= 2) {
+      if (L / G < gh || xy_strip_smem<T>(L, G, gh) > 200 * 1024) continue;
+      const int R = (L + G - 1) / G;
+      const bool ahead = (R + (G == 1 ? 0 : 2 * gh - 2)) * half <= kXYStripThreads;
+      const int words = (gh == 1 ? 2 : 4) * gh * half * (int)(sizeof(T) / 2);
+      double t = G == 1 ? 0.0 : 0.9 + 3e-4 * words;
+      for (int g = 0; g < gh; ++g) {
+        const double s = (double)(R + (G == 1 ? 0 : 2 * (gh - 1 - g))) * half;
+        const double w = std::ceil(std::ceil(s / 32) / 4);
+        t += sizeof(T) == 8 ? 0.5 + 1.05 * w : ahead ? 0.45 + 0.08 * w : 0.5 + 0.0013 * s;
+      }
+      t *= 2.0 / gh;
+      if (t < best.us) best = {G, gh, t};
+    }
+  return best;
+}
+
+template <typename T>
+cudaError_t xy_strip_t(ising_xy* x, int n, int m) {
+  XYStripArgs<T> a{};
+  a.u = (typename Vec<T>::type*)x->u;
+  a.L = x->L;
+  a.G = x->strip_G;
+  a.gh = std::min(x->strip_gh, 2 * n);
+  a.beta = (T)x->beta;
+  a.beta_f = (float)x->beta;
+  a.t0 = (uint32_t)x->sweep;
+  a.n = n;
+  a.m = m;
+  a.rec = x->rec;
+  a.rec0 = x->rec_count % kXYRec;
+  a.rec_cap = kXYRec;
+  a.accepted = x->accepted;
+  a.xbuf = x->strip_x;
+  a.status = x->strip_status;
+  a.limit = kXYSpinLimit;
+  a.fh = make_fastdiv((uint32_t)(x->L / 2));
+  const bool whole = a.G == 1;
+  const long long sites = (long long)((a.L + a.G - 1) / a.G + (whole ? 0 : 2 * a.gh)) * (a.L / 2);
+  const long long active = sites - (whole ? 0 : a.L);  // without the two outermost rows
+  const bool ahead = active <= kXYStripThreads;
+  const long long items = ahead || sizeof(T) == 8 ? active : active / 2 + 2;
+  const int threads = (int)std::min<long long>(kXYStripThreads, (items + 31) / 32 * 32);
+  const size_t smem = xy_strip_smem<T>(a.L, a.G, a.gh);
+  const void* fns[4] = {(const void*)k_xy_strip<T, false, false>, (const void*)k_xy_strip<T, true, false>,
+                        (const void*)k_xy_strip<T, false, true>, (const void*)k_xy_strip<T, true, true>};
+  const int which = (whole ? 1 : 0) + (ahead ? 2 : 0);
+  static DeviceCache configured[4];
+  cudaError_t e;
+  if ((long long)smem > configured[which].get()) {
+    e = cudaFuncSetAttribute(fns[which], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e) return e;
+    configured[which].set((long long)smem);
+  }
+  // records of this launch: zeroed, then summed into by every CTA
+  int64_t n_rec = 0;
+  if (m > 0) {
+    const int64_t before = x->sweep / m;
+    n_rec = (x->sweep + n) / m - before;
+    a.to_rec = n_rec ? (int)((before + 1) * m - x->sweep) : 0;
+    const int64_t n1 = std::min<int64_t>(n_rec, kXYRec - a.rec0);
+    if (n1 > 0 && (e = cudaMemsetAsync(x->rec + 3 * a.rec0, 0, (size_t)n1 * 24, x->stream))) return e;
+    if (n_rec > n1 && (e = cudaMemsetAsync(x->rec, 0, (size_t)(n_rec - n1) * 24, x->stream))) return e;
+  }
+  RngParams r = make_rng(x->seed, 0, 0, 0);
+  void* args[] = {&a, &r};
+  if (whole) {
+    e = cudaLaunchKernel(fns[which], dim3(1), dim3(threads), args, smem, x->stream);
+  } else {
+    e = cudaMemsetAsync(a.xbuf, 0, xy_strip_words<T>(a.L, a.G, a.gh) * 8, x->stream);
+    if (!e) e = cudaLaunchCooperativeKernel(fns[which], dim3(a.G), dim3(threads), args, smem, x->stream);
+  }
+  if (e) return e;
+  ++x->launches;
+  x->rec_count += n_rec;
+  return cudaSuccess;
+}
 
 template <typename T>
 cudaError_t xy_persist_t(ising_xy* x, int n, int m) {
@@ -541,7 +931,20 @@ cudaError_t xy_persist_t(ising_xy* x, int n, int m) {
 
 template <typename T>
 cudaError_t xy_sweep_t(ising_xy* x, int n, int m) {
-  const bool persist = x->mode == 2 || (x->mode == 0 && x->L <= kXYPersistMaxL);
+  if (x->mode == 0 && x->strip_G > 0) {
+    // chunks whose records fit the ring
+    const int most = m > 0 ? (int)std::min<int64_t>(kXYRec * (int64_t)m, 1 << 29) : 1 << 29;
+    for (int done = 0; done < n;) {
+      const int k = std::min(most, n - done);
+      cudaError_t e = xy_strip_t<T>(x, k, m);
+      if (e) return e;
+      x->sweep += k;
+      done += k;
+    }
+    x->sweep -= n;  // the caller advances the counter
+    return cudaSuccess;
+  }
+  const bool persist = x->mode == 2;
   if (persist) return n > 0 ? xy_persist_t<T>(x, n, m) : cudaSuccess;
   const RngParams rng = make_rng(x->seed, 0, 0, 0);
   const long long blocks = ((long long)x->L * (x->L / 2) + 1) / 2;
@@ -592,8 +995,24 @@ int ising_xy_create(ising_xy** out, int L, double beta, int precision, void* str
   if (!e) e = cudaMemset(x->accepted, 0, sizeof(unsigned long long));
   if (!e) e = cudaMalloc((void**)&x->ctl, sizeof(GridCtl));
   if (!e) e = cudaMemset(x->ctl, 0, sizeof(GridCtl));
+  int dev = 0, sms = 0;
+  if (!e) e = cudaGetDevice(&dev);
+  if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (!e && L <= kXYStripMaxL) {
+    const XYStrip st = precision == 64 ? choose_xy_strip<double>(L, sms) : choose_xy_strip<float>(L, sms);
+    x->strip_G = st.G;
+    x->strip_gh = st.gh;
+    if (st.G > 1) {
+      const size_t words = precision == 64 ? xy_strip_words<double>(L, st.G, st.gh) : xy_strip_words<float>(L, st.G, st.gh);
+      e = cudaMalloc((void**)&x->strip_x, words * sizeof(unsigned long long));
+      if (!e) e = cudaHostAlloc((void**)&x->strip_status, sizeof(int), cudaHostAllocDefault);
+      if (!e) *x->strip_status = 0;
+    }
+  }
   if (e) {
     cudaGetLastError();
+    cudaFree(x->strip_x);
+    cudaFreeHost(x->strip_status);
     cudaFree(x->u);
     cudaFree(x->rec);
     cudaFree(x->accepted);
@@ -610,6 +1029,7 @@ int ising_xy_seed(ising_xy* x, uint64_t seed) {
   x->seed = seed;
   x->sweep = 0;
   x->rec_count = 0;
+  if (x->strip_status) *x->strip_status = 0;
   const RngParams rng = make_rng(seed, 0, 0, 0);
   const long long N = (long long)x->L * x->L;
   if (x->precision == 64)
@@ -638,6 +1058,8 @@ int ising_xy_sweep(ising_xy* x, int n_sweeps, int measure_every) {
 // After a synchronising call: ETIMEOUT if a persistent kernel's grid barrier
 // gave up (the flag stays set until the next seed).
 static int xy_status(ising_xy* x) {
+  if (x->strip_status && *(volatile int*)x->strip_status)
+    return xfail(ISING_ETIMEOUT, "a strip's wait for its neighbour timed out in the XY kernel");
   int st = 0;
   XTRY(cudaMemcpy(&st, &x->ctl->status, sizeof(int), cudaMemcpyDeviceToHost));
   if (st) return xfail(ISING_ETIMEOUT, "grid barrier timed out in the persistent XY kernel");
@@ -753,6 +1175,8 @@ int ising_xy_destroy(ising_xy* x) {
   cudaFree(x->rec);
   cudaFree(x->accepted);
   cudaFree(x->ctl);
+  cudaFree(x->strip_x);
+  cudaFreeHost(x->strip_status);
   delete x;
   return ISING_OK;
 }

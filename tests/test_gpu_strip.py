@@ -49,3 +49,31 @@ def test_strips_equal_oracle(L, beta):
     E, M = oracle.sweep(ref, beta, 40 + L, 12)
     got = _run(L, beta, BITS, [(12, 1)])
     assert np.array_equal(got[0], ref) and np.array_equal(got[1], E) and np.array_equal(got[2], M)
+
+
+# one CTA and strips, odd and even row lengths L / 2, one site per thread and loops; calls of one sweep, fewer half
+# sweeps than an exchange group, and records at both ends of a call
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("L", [2, 6, 8, 16, 32, 34, 62, 130, 256, 514])
+def test_xy_strips_equal_half_sweeps(precision, L):
+    out = []
+    for mode in (0, 1):
+        with ising.XY(L, 1.0 / 0.85, precision, seed=7 + L) as x:
+            x.set_mode(mode)
+            for n, every in [(1, 1), (2, 0), (5, 2), (12, 1)]:
+                x.sweep(n, every)
+            out.append((x.spins(), x.accepted(), x.series(15)))
+    assert np.array_equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
+    # the same terms (at most 1.5 L^2 of them, each within 4) in another order, in double
+    for a, b in zip(out[0][2], out[1][2]):
+        np.testing.assert_allclose(a, b, rtol=0, atol=6 * L * L * 1.2e-16 * (2 + np.log2(L * L)))
+
+
+def test_xy_angles_of_quadrant_edges():
+    """The double path takes the quadrant of an angle from its 24-bit word; at every word within two of a
+    quadrant edge it must give the same integer as rounding the angle (the recipe the oracle follows)."""
+    m = np.concatenate([(1 << 21) * k + np.arange(-2, 3) for k in range(1, 8)]).astype(np.int64)
+    x = 6.283185307179586 * (m * 2.0 ** -24)
+    assert np.array_equal(x, (6.283185307179586 / 16777216.0) * m)
+    tie = (m & 0x3FFFFF) == 0x200000
+    assert np.array_equal(np.rint(x * 0.6366197723675814)[~tie], ((m + (1 << 21)) >> 22)[~tie])
