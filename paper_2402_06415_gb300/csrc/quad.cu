@@ -141,9 +141,12 @@ __device__ __forceinline__ uint32_t valid_bits(const QuadGeom& g, int w) {
 // Metropolis trials of the 32 sites of word i = Y Wq + w of sublattice q.
 // All 32 lanes of the warp call it together (warp vote); lanes past the end pass
 // active = false (any in-range i) and change nothing.
-template <int LAT, int NV, bool G>
+// grp is the word's index in the whole lattice (its Philox counter).  The first NB
+// Philox blocks are drawn for every word and compared as one 4 NB-bit borrow chain;
+// the rest while a lane of the warp is tied.
+template <int LAT, int NV, bool G, int NB>
 __device__ __forceinline__ void quad_word(uint32_t* __restrict__ planes, const QuadGeom& g, int q,
-                                          long long i, bool active, uint32_t t, const RngParams& rng,
+                                          long long i, uint32_t grp, bool active, uint32_t t, const RngParams& rng,
                                           const QuadTable& tab) {
   constexpr int Z2 = LAT == ISING_QUAD_SQUARE ? 4 : 1;
   constexpr int Z1 = LAT == ISING_QUAD_SQUARE ? 4 : 2;
@@ -173,21 +176,41 @@ __device__ __forceinline__ void quad_word(uint32_t* __restrict__ planes, const Q
     }
   }
   uint32_t und = ~always & valid, lt = 0;
-  const uint32_t g_idx = (uint32_t)i;
-  // planes block by block while any lane of the warp is undecided; the level is
-  // a compile-time index, so each threshold-bit mask is a constant operand
+  // the level is a compile-time index, so each threshold-bit mask is a constant operand
+  auto level_mask = [&](int lvl) {
+    uint32_t tm = 0;
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
+    for (int d = 0; d < NV; ++d) tm |= vm[d] & tab.lm[d][lvl];
+    return tm;
+  };
+  auto block = [&](int m) {
+    return philox10_rk(make_uint4(grp, t, rng.replica, (kTagQuadMet << 16) | ((uint32_t)q << 8) | (uint32_t)m),
+                       rng.rk0, rng.rk1);
+  };
+  {
+    uint32_t bor = 0, eq = und;
+#pragma unroll
+    for (int m = NB - 1; m >= 0; --m) {
+      const uint4 r = block(m);
+      const uint32_t pw[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+      for (int k = 3; k >= 0; --k) {
+        const uint32_t tm = level_mask(4 * m + k);
+        bor = (~pw[k] & tm) | (~pw[k] & bor) | (tm & bor);
+        eq &= ~(tm ^ pw[k]);
+      }
+    }
+    lt = und & bor;
+    und = eq;
+  }
+#pragma unroll
+  for (int m = NB; m < 8; ++m) {
     if (!__any_sync(0xffffffffu, und != 0u)) break;
-    const uint4 r = philox10_rk(make_uint4(g_idx, t, rng.replica, (kTagQuadMet << 16) | ((uint32_t)q << 8) | (uint32_t)m),
-                                rng.rk0, rng.rk1);
+    const uint4 r = block(m);
     const uint32_t pw[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int lvl = 4 * m + k;
-      uint32_t tm = 0;
-#pragma unroll
-      for (int d = 0; d < NV; ++d) tm |= vm[d] & tab.lm[d][lvl];
+      const uint32_t tm = level_mask(4 * m + k);
       lt |= und & ~pw[k] & tm;
       und &= ~(pw[k] ^ tm);
     }
@@ -203,7 +226,7 @@ __global__ void __launch_bounds__(256) k_quad_quarter(uint32_t* __restrict__ pla
   const int lane = threadIdx.x & 31;
   for (long long base = (blockIdx.x * (long long)blockDim.x + threadIdx.x) - lane; base < words;
        base += (long long)gridDim.x * blockDim.x)
-    quad_word<LAT, NV, true>(planes, g, q, base + lane, base + lane < words, t, rng, tab);
+    quad_word<LAT, NV, true, 2>(planes, g, q, base + lane, (uint32_t)(base + lane), base + lane < words, t, rng, tab);
 }
 
 __global__ void k_quad_init(uint32_t* __restrict__ planes, QuadGeom g, RngParams rng) {
@@ -279,8 +302,8 @@ __global__ void __launch_bounds__(1024) k_quad_persist(uint32_t* __restrict__ pl
     const uint32_t t = t0 + (uint32_t)s;
     for (int q = 0; q < 4; ++q) {
       for (long long base = threadIdx.x & ~31; base < words; base += blockDim.x)
-        quad_word<LAT, NV, false>(sp, g, q, base + (threadIdx.x & 31), base + (threadIdx.x & 31) < words, t,
-                                  rng, tab);
+        quad_word<LAT, NV, false, 2>(sp, g, q, base + (threadIdx.x & 31), (uint32_t)(base + (threadIdx.x & 31)),
+                                     base + (threadIdx.x & 31) < words, t, rng, tab);
       __syncthreads();
     }
     if (meas_every > 0 && ((long long)t + 1) % meas_every == 0) {
@@ -313,6 +336,147 @@ __global__ void __launch_bounds__(1024) k_quad_persist(uint32_t* __restrict__ pl
     }
   }
   for (long long i = threadIdx.x; i < 4 * words; i += blockDim.x) planes[i] = sp[i];
+}
+
+// Resident strips (as the two-sublattice sweep's): G CTAs own row strips of full
+// width, the four planes in shared memory, K sweeps between exchanges of boundary
+// rows.  A sweep invalidates one more halo row on each side: two of the quarter
+// sweeps read the row below, two the row above, so the first pair runs one row
+// further than the second on the side it does not read from.  The halo has
+// H = K + 1 rows, because the bond sums of a recorded sweep read one row beyond
+// the strip.
+// Bound by the dependent chain of a quarter sweep (~0.6 us) up to 512^2 cells, then by
+// issue slots.  us per sweep, before (one CTA up to 256^2 cells, else a launch per
+// quarter sweep) and with strips: 4.8.8 at 256^2 19.5 -> 2.7, 1024^2 16.5 -> 4.5, 4096^2
+// 49.8 -> 34.5; square J2 = 0.5 at 1024^2 24.7 -> 8.8.  8192^2 does not fit and keeps
+// the launches (152 us, ALU pipe bound).
+struct QuadStripArgs {
+  uint32_t* planes;
+  QuadGeom g;
+  int G, K;
+  uint32_t t0;
+  int n, m, to_rec;  // sweeps; record every m; sweeps until the first record (0: none)
+  unsigned long long* rec;
+  long long rec0, rec_cap;
+  unsigned long long* xbuf;  // quad_strip_words(...) pairs, zeroed by the launcher
+  int* status;
+  long long limit;
+};
+constexpr int kQuadStripThreads = 512, kQuadStripMaxK = 4;
+
+size_t quad_strip_words(const QuadGeom& g, int G, int K) { return (size_t)G * (16 * (size_t)(K + 1) * g.Wq + 1); }
+size_t quad_strip_smem(const QuadGeom& g, int G, int K) {
+  return 4 * (size_t)((g.Lc + G - 1) / G + 2 * (K + 1)) * g.Wq * sizeof(uint32_t);
+}
+
+template <int LAT, int NV>
+__global__ void __launch_bounds__(kQuadStripThreads) k_quad_strip(QuadStripArgs a, RngParams rng, QuadTable tab) {
+  extern __shared__ uint32_t sp[];
+  const int Lc = a.g.Lc, Wq = a.g.Wq, G = a.G, H = a.K + 1;
+  const int b = blockIdx.x, tid = threadIdx.x, nth = blockDim.x, lane = tid & 31;
+  const int y0 = (int)((long long)b * Lc / G), R = (int)((long long)(b + 1) * Lc / G) - y0;
+  const int rows = R + 2 * H, plane = rows * Wq, LW = Lc * Wq;
+  const QuadGeom gl{rows, Wq, a.g.nlast, a.g.fw};
+  const int goff = (y0 - H) * Wq;  // local word i is word i + goff of its plane, modulo LW
+  auto group_of = [&](int i) {
+    int k = i + goff;
+    k += k < 0 ? LW : 0;
+    k -= k >= LW ? LW : 0;
+    return k;
+  };
+  for (int q = 0; q < 4; ++q)
+    for (int i = tid; i < plane; i += nth) sp[q * plane + i] = __ldcg(&a.planes[(size_t)q * LW + group_of(i)]);
+  __syncthreads();
+  const int hw = H * Wq;
+  const size_t per_cta = 16 * (size_t)hw + 1;
+  const int up = b == 0 ? G - 1 : b - 1, dn = b == G - 1 ? 0 : b + 1;
+  unsigned long long* const mine = a.xbuf + b * per_cta;
+  if (tid == 0) send_word(mine + 16 * hw, 1u, 0u);  // "lattice read"
+  int to_rec = a.to_rec;
+  long long slot = a.rec0;
+  uint32_t exchanges = 0;
+  for (int done = 0; done < a.n;) {
+    const int kk = min(a.K, a.n - done);
+    // the outermost halo rows are needed only if a sweep of this group is recorded
+    const int skip = to_rec > 0 && to_rec <= kk ? a.K - kk : a.K - kk + 1;
+    for (int s = 0; s < kk; ++s) {
+      const uint32_t t = a.t0 + (uint32_t)(done + s);
+      const int e = skip + s;  // halo rows already invalid (or not needed) on each side
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        // square: q = 0, 1 read the row above, 2, 3 the row below; 4.8.8: 0 the row below, 2 the row above
+        const int lo = LAT == ISING_QUAD_SQUARE ? e + 1 : (q < 2 ? e : e + 1);
+        const int hi = LAT == ISING_QUAD_SQUARE ? (q < 2 ? rows - e : rows - e - 1) : rows - e - 1;
+        const int count = (hi - lo) * Wq;
+        for (int base = tid & ~31; base < count; base += nth) {
+          const bool active = base + lane < count;
+          const int i = lo * Wq + (active ? base + lane : 0);
+          quad_word<LAT, NV, false, 3>(sp, gl, q, i, (uint32_t)group_of(i), active, t, rng, tab);
+        }
+        __syncthreads();
+      }
+      if (to_rec > 0 && --to_rec == 0) {
+        to_rec = a.m;
+        long long b1 = 0, b2 = 0, m = 0;
+        for (int i = tid; i < 4 * R * Wq; i += nth) {
+          const int q = i / (R * Wq);
+          quad_measure_word<LAT, false>(sp, gl, (long long)q * plane + hw + (i - q * R * Wq), b1, b2, m);
+        }
+        const unsigned long long s1 = warp_sum_u64((unsigned long long)b1);
+        const unsigned long long s2 = warp_sum_u64((unsigned long long)b2);
+        const unsigned long long s3 = warp_sum_u64((unsigned long long)m);
+        if (lane == 0) {
+          atomicAdd(&a.rec[3 * slot], s1);
+          atomicAdd(&a.rec[3 * slot + 1], s2);
+          atomicAdd(&a.rec[3 * slot + 2], s3);
+        }
+        slot = slot + 1 == a.rec_cap ? 0 : slot + 1;
+        __syncthreads();
+      }
+    }
+    done += kk;
+    if (done >= a.n) break;
+    const uint32_t tag = ++exchanges;
+    const size_t buf = (size_t)(tag & 1) * 8 * hw;
+    for (int i = tid; i < 8 * hw; i += nth) {  // [upper / lower rows][plane][H rows]
+      const int lower = i >= 4 * hw, rem = i - lower * 4 * hw, q = rem / hw;
+      send_word(mine + buf + i, tag, sp[q * plane + (lower ? R * Wq : hw) + rem - q * hw]);
+    }
+    bool ok = true;
+    auto src = [&](int i) {  // the upper neighbour's lower rows, the lower neighbour's upper rows
+      const int lower = i >= 4 * hw;
+      return a.xbuf + (lower ? dn : up) * per_cta + buf + (lower ? i - 4 * hw : i + 4 * hw);
+    };
+    recv_words<4>(tid, nth, 8 * hw, src, tag, a.limit, a.status, ok, [&](int i, uint32_t word) {
+      const int lower = i >= 4 * hw, rem = i - lower * 4 * hw, q = rem / hw;
+      sp[q * plane + (lower ? (H + R) * Wq : 0) + rem - q * hw] = word;
+    });
+    if (!__syncthreads_and(ok)) return;
+  }
+  // in place: both neighbours must have read their halos
+  if (exchanges == 0) {
+    uint32_t word;
+    bool ok = true;
+    if (tid < 2) ok = recv_word(a.xbuf + (tid ? dn : up) * per_cta + 16 * hw, 1u, a.limit, a.status, word);
+    if (!__syncthreads_and(ok)) return;
+  }
+  for (int q = 0; q < 4; ++q)
+    for (int i = tid; i < R * Wq; i += nth) a.planes[(size_t)q * LW + (size_t)y0 * Wq + i] = sp[q * plane + hw + i];
+}
+
+// Bit planes -> one int8 (+-1) per site, [4][Lc][Lc].
+__global__ void __launch_bounds__(256) k_quad_unpack(const uint32_t* __restrict__ planes, QuadGeom g,
+                                                     int8_t* __restrict__ out) {
+  const long long words = 4LL * g.Lc * g.Wq;
+  const int lane = threadIdx.x & 31;
+  // one warp per word, one lane per site
+  for (long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; i < words;
+       i += ((long long)gridDim.x * blockDim.x) >> 5) {
+    const long long row = i / g.Wq;  // q Lc + Y
+    const int X = 32 * (int)(i - row * g.Wq) + lane;
+    const uint32_t v = __ldg(&planes[i]);
+    if (X < g.Lc) out[row * g.Lc + X] = (v >> lane) & 1u ? 1 : -1;
+  }
 }
 
 int qfail(int code, const char* fmt, ...) {
@@ -387,10 +551,91 @@ struct ising_quad {
   unsigned long long* rec = nullptr;  // ring [65536][3]
   int64_t rec_count = 0;
   int64_t launches = 0;
+  int strip_G = 0, strip_K = 0;  // resident strips (G = 0: not used)
+  unsigned long long* strip_x = nullptr;
+  int* strip_status = nullptr;   // pinned host word a strip sets when a wait gave up
+  int8_t* spins = nullptr;       // unpacked spins for get_spins, allocated by its first call
 };
 
 namespace {
 constexpr int64_t kQuadRec = 65536;
+constexpr long long kQuadSpinLimit = 4000000000LL;  // ~2 s of SM clock per wait
+
+// Strips of an Lc x Lc lattice by a time model (us per sweep, GB300): a quarter
+// sweep takes 0.45 + 0.25 per resident warp of an SM sub-partition, an exchange
+// 1.0; G = 0 where one CTA (the same time per quarter, no exchange) is as fast
+// or the strips do not fit.
+void choose_quad_strip(const QuadGeom& g, int sms, int* G_out, int* K_out) {
+  auto quarter = [](double words) { return 0.45 + 0.25 * std::ceil(std::ceil(words / 32) / 4); };
+  double best = g.Lc <= 256 ? 4 * quarter((double)g.Lc * g.Wq) : 1e30;
+  *G_out = *K_out = 0;
+  for (int G = 2; G <= sms && G <= g.Lc; ++G)
+    for (int K = 1; K <= kQuadStripMaxK; ++K) {
+      if (g.Lc / G < K + 1 || quad_strip_smem(g, G, K) > 200 * 1024) break;
+      const int R = (g.Lc + G - 1) / G;
+      double t = 1.0;
+      for (int s = 0; s < K; ++s) t += 4 * quarter((double)(R + 2 * (K - 1 - s) + 1) * g.Wq);
+      if (t / K < best) {
+        best = t / K;
+        *G_out = G;
+        *K_out = K;
+      }
+    }
+}
+
+template <int LAT, int NV>
+cudaError_t launch_quad_strip(ising_quad* x, int n, int m, const RngParams& rng) {
+  QuadStripArgs a{};
+  a.planes = x->planes;
+  a.g = x->geom;
+  a.G = x->strip_G;
+  a.K = std::min(x->strip_K, n);
+  a.t0 = (uint32_t)x->sweep;
+  a.n = n;
+  a.m = m;
+  a.rec = x->rec;
+  a.rec0 = x->rec_count % kQuadRec;
+  a.rec_cap = kQuadRec;
+  a.xbuf = x->strip_x;
+  a.status = x->strip_status;
+  a.limit = kQuadSpinLimit;
+  cudaError_t e;
+  int64_t n_rec = 0;
+  if (m > 0) {
+    const int64_t before = x->sweep / m;
+    n_rec = (x->sweep + n) / m - before;
+    a.to_rec = n_rec ? (int)((before + 1) * m - x->sweep) : 0;
+    const int64_t n1 = std::min<int64_t>(n_rec, kQuadRec - a.rec0);
+    if (n1 > 0 && (e = cudaMemsetAsync(x->rec + 3 * a.rec0, 0, (size_t)n1 * 24, x->stream))) return e;
+    if (n_rec > n1 && (e = cudaMemsetAsync(x->rec, 0, (size_t)(n_rec - n1) * 24, x->stream))) return e;
+  }
+  const size_t smem = quad_strip_smem(a.g, a.G, a.K);
+  const void* fn = (const void*)k_quad_strip<LAT, NV>;
+  static DeviceCache configured;
+  if ((long long)smem > configured.get()) {
+    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
+    configured.set((long long)smem);
+  }
+  const long long words = (long long)((a.g.Lc + a.G - 1) / a.G + 2 * a.K - 1) * a.g.Wq;
+  const int threads = (int)std::min<long long>(kQuadStripThreads, std::max(64LL, (words + 31) / 32 * 32));
+  if ((e = cudaMemsetAsync(a.xbuf, 0, quad_strip_words(a.g, a.G, a.K) * 8, x->stream))) return e;
+  RngParams r = rng;
+  QuadTable tab = x->tab;
+  void* args[] = {&a, &r, &tab};
+  if ((e = cudaLaunchCooperativeKernel(fn, dim3(a.G), dim3(threads), args, smem, x->stream))) return e;
+  ++x->launches;
+  x->rec_count += n_rec;
+  return cudaSuccess;
+}
+
+template <int LAT>
+cudaError_t strip_dispatch(ising_quad* x, int n, int m, const RngParams& rng) {
+  const int nv = x->tab.n_vals;
+  if (nv <= 2) return launch_quad_strip<LAT, 2>(x, n, m, rng);
+  if (nv <= 8) return launch_quad_strip<LAT, 8>(x, n, m, rng);
+  if (LAT == ISING_QUAD_SQUARE) return launch_quad_strip<LAT, kMaxClasses>(x, n, m, rng);
+  return cudaErrorInvalidValue;
+}
 
 template <int LAT, int NV>
 cudaError_t launch_quarter(ising_quad* x, int q, uint32_t t, const RngParams& rng) {
@@ -431,6 +676,21 @@ cudaError_t persist_dispatch(ising_quad* x, int n, int m, const RngParams& rng) 
 
 cudaError_t quad_sweeps(ising_quad* x, int n, int m) {
   const RngParams rng = make_rng(x->seed, x->replica, 0, 0);
+  if (x->strip_G > 0 && n > 0) {
+    // chunks whose records fit the ring
+    const int most = m > 0 ? (int)std::min<int64_t>(kQuadRec * (int64_t)m, 1 << 29) : 1 << 29;
+    cudaError_t e = cudaSuccess;
+    int done = 0;
+    for (; done < n && !e;) {
+      const int k = std::min(most, n - done);
+      e = x->lattice == ISING_QUAD_SQUARE ? strip_dispatch<ISING_QUAD_SQUARE>(x, k, m, rng)
+                                          : strip_dispatch<ISING_QUAD_SQOCT>(x, k, m, rng);
+      x->sweep += k;
+      done += k;
+    }
+    x->sweep -= done;  // the caller advances the counter
+    return e;
+  }
   if (x->Lc <= kQuadPersistMaxLc && n > 0) {
     cudaError_t e = x->lattice == ISING_QUAD_SQUARE ? persist_dispatch<ISING_QUAD_SQUARE>(x, n, m, rng)
                                                     : persist_dispatch<ISING_QUAD_SQOCT>(x, n, m, rng);
@@ -498,8 +758,19 @@ int ising_quad_create(ising_quad** out, int lattice, int Lc, double beta, double
   const size_t bytes = (size_t)4 * Lc * x->geom.Wq * sizeof(uint32_t);
   cudaError_t e = cudaMalloc((void**)&x->planes, bytes);
   if (!e) e = cudaMalloc((void**)&x->rec, kQuadRec * 3 * sizeof(unsigned long long));
+  int dev = 0, sms = 0;
+  if (!e) e = cudaGetDevice(&dev);
+  if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (!e) choose_quad_strip(x->geom, sms, &x->strip_G, &x->strip_K);
+  if (!e && x->strip_G > 0) {
+    e = cudaMalloc((void**)&x->strip_x, quad_strip_words(x->geom, x->strip_G, x->strip_K) * sizeof(unsigned long long));
+    if (!e) e = cudaHostAlloc((void**)&x->strip_status, sizeof(int), cudaHostAllocDefault);
+    if (!e) *x->strip_status = 0;
+  }
   if (e) {
     cudaGetLastError();
+    cudaFree(x->strip_x);
+    cudaFreeHost(x->strip_status);
     cudaFree(x->planes);
     cudaFree(x->rec);
     delete x;
@@ -514,6 +785,7 @@ int ising_quad_seed(ising_quad* x, uint64_t seed) {
   x->seed = seed;
   x->sweep = 0;
   x->rec_count = 0;
+  if (x->strip_status) *x->strip_status = 0;
   const RngParams rng = make_rng(seed, x->replica, 0, 0);
   k_quad_init<<<qgrid(4LL * x->Lc * x->geom.Wq), 256, 0, x->stream>>>(x->planes, x->geom, rng);
   QTRY(cudaGetLastError());
@@ -538,17 +810,27 @@ int ising_quad_sweep(ising_quad* x, int n_sweeps, int measure_every) {
   return ISING_OK;
 }
 
+// After a synchronising call: ETIMEOUT if a strip's wait gave up (until the next seed).
+static int quad_status(ising_quad* x) {
+  if (x->strip_status && *(volatile int*)x->strip_status)
+    return qfail(ISING_ETIMEOUT, "a strip's wait for its neighbour timed out");
+  return ISING_OK;
+}
+
 int ising_quad_series(ising_quad* x, int64_t* B1, int64_t* B2, int64_t* M, int n) {
   if (!x) return qfail(ISING_EINVAL, "null context");
   if (n < 0 || n > std::min<int64_t>(x->rec_count, kQuadRec)) return qfail(ISING_EINVAL, "n exceeds records");
-  std::vector<unsigned long long> h((size_t)3 * kQuadRec);
-  QTRY(cudaMemcpyAsync(h.data(), x->rec, h.size() * 8, cudaMemcpyDeviceToHost, x->stream));
+  std::vector<unsigned long long> h((size_t)3 * n);
+  const int64_t s0 = (x->rec_count - n) % kQuadRec, n1 = std::min<int64_t>(n, kQuadRec - s0);
+  if (n1 > 0) QTRY(cudaMemcpyAsync(h.data(), x->rec + 3 * s0, (size_t)n1 * 24, cudaMemcpyDeviceToHost, x->stream));
+  if (n > n1)
+    QTRY(cudaMemcpyAsync(h.data() + 3 * n1, x->rec, (size_t)(n - n1) * 24, cudaMemcpyDeviceToHost, x->stream));
   QTRY(cudaStreamSynchronize(x->stream));
+  if (int st = quad_status(x)) return st;
   for (int i = 0; i < n; ++i) {
-    const int64_t slot = (x->rec_count - n + i) % kQuadRec;
-    if (B1) B1[i] = (int64_t)h[3 * slot] / 2;
-    if (B2) B2[i] = (int64_t)h[3 * slot + 1] / 2;
-    if (M) M[i] = (int64_t)h[3 * slot + 2];
+    if (B1) B1[i] = (int64_t)h[3 * i] / 2;
+    if (B2) B2[i] = (int64_t)h[3 * i + 1] / 2;
+    if (M) M[i] = (int64_t)h[3 * i + 2];
   }
   set_last_error("");
   return ISING_OK;
@@ -556,16 +838,13 @@ int ising_quad_series(ising_quad* x, int64_t* B1, int64_t* B2, int64_t* M, int n
 
 int ising_quad_get_spins(ising_quad* x, int8_t* host_out) {
   if (!x || !host_out) return qfail(ISING_EINVAL, "null argument");
-  const int Lc = x->Lc, Wq = x->geom.Wq;
-  std::vector<uint32_t> h((size_t)4 * Lc * Wq);
-  QTRY(cudaMemcpyAsync(h.data(), x->planes, h.size() * 4, cudaMemcpyDeviceToHost, x->stream));
+  const size_t N = (size_t)4 * x->Lc * x->Lc;
+  if (!x->spins) QTRY(cudaMalloc((void**)&x->spins, N));
+  k_quad_unpack<<<qgrid(4LL * x->Lc * x->geom.Wq * 32), 256, 0, x->stream>>>(x->planes, x->geom, x->spins);
+  QTRY(cudaGetLastError());
+  QTRY(cudaMemcpyAsync(host_out, x->spins, N, cudaMemcpyDeviceToHost, x->stream));
   QTRY(cudaStreamSynchronize(x->stream));
-  for (int q = 0; q < 4; ++q)
-    for (int Y = 0; Y < Lc; ++Y)
-      for (int X = 0; X < Lc; ++X) {
-        const uint32_t wv = h[((size_t)q * Lc + Y) * Wq + (X >> 5)];
-        host_out[((size_t)q * Lc + Y) * Lc + X] = ((wv >> (X & 31)) & 1u) ? 1 : -1;
-      }
+  if (int st = quad_status(x)) return st;
   set_last_error("");
   return ISING_OK;
 }
@@ -598,6 +877,9 @@ int ising_quad_destroy(ising_quad* x) {
   cudaStreamSynchronize(x->stream);
   cudaFree(x->planes);
   cudaFree(x->rec);
+  cudaFree(x->strip_x);
+  cudaFreeHost(x->strip_status);
+  cudaFree(x->spins);
   delete x;
   return ISING_OK;
 }

@@ -77,3 +77,22 @@ def test_xy_angles_of_quadrant_edges():
     assert np.array_equal(x, (6.283185307179586 / 16777216.0) * m)
     tie = (m & 0x3FFFFF) == 0x200000
     assert np.array_equal(np.rint(x * 0.6366197723675814)[~tie], ((m + (1 << 21)) >> 22)[~tie])
+
+
+# sizes that take strips (and 40, which stays in one CTA), one and several words a row, ragged last words, all three
+# numbers of distinct thresholds; calls of one sweep, groups without a record, and records at both ends of a group
+@pytest.mark.parametrize("lattice,J1,J2", [(ising.ISING_QUAD_SQOCT, 1.0, 1.0), (ising.ISING_QUAD_SQOCT, 0.7, 1.9),
+                                           (ising.ISING_QUAD_SQUARE, 1.0, 0.0), (ising.ISING_QUAD_SQUARE, 0.75, 1.25)])
+@pytest.mark.parametrize("Lc", [40, 64, 97, 200, 257, 640])
+def test_quad_strips_equal_oracle(lattice, J1, J2, Lc):
+    seed = 90 + Lc
+    s = oracle.quad_init(Lc, seed)
+    with ising.Quad(lattice, Lc, 0.4406868, J1, J2, seed=seed) as x:
+        for n, every in [(1, 1), (2, 0), (6, 4), (5, 1)]:
+            x.sweep(n, every)
+        got = x.spins()
+        B1, B2, M = x.series(7)  # after sweeps 1; 4, 8; 10 ... 14 (the last seven: 4, 8, 10 ... 14)
+    R1, R2, RM = oracle.quad_sweep(lattice, s, 0.4406868, J1, J2, seed, 14)
+    assert np.array_equal(got, s)
+    at = [3, 7, 9, 10, 11, 12, 13]
+    assert np.array_equal(B1, R1[at]) and np.array_equal(B2, R2[at]) and np.array_equal(M, RM[at])
