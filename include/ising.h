@@ -369,13 +369,14 @@ int ising_sw_step(ising_ctx* ctx, int n_steps, int measure_every);
 
 /* How cluster steps (ising_sw_step, ising_wolff_step) run: AUTO = one
  * persistent launch per call for L < 768 (up to 64 x 64 sites one CTA with the
- * lattice in shared memory, else a cooperative grid with three bounded
- * grid-barrier phases per step: runs, unions, flips; a barrier wait gives up
+ * lattice in shared memory, else row strips resident in shared memory with
+ * bounded grid barriers around the unions across strips; a barrier wait gives up
  * after about 2 s and later synchronising calls then fail with ISING_ETIMEOUT;
  * work queued after the timed-out step, sweeps included, ran on a lattice the
  * step left half-updated, so the lattice and its records are undefined until
  * ising_seed, ising_set_spins or ising_set_bits),
- * a few kernels per step from L = 768 (from L = 2048 with tiled labelling in
+ * a few kernels per step from L = 768 (Wolff) or where the strips do not fit or
+ * the tiled labelling applies (Swendsen-Wang; L >= 2048 with tiled labelling in
  * shared memory; Wolff first tries growth from the seed, and its step is one
  * CUDA graph launch (eight steps per launch when nothing is recorded): the
  * growth kernel sets the condition of an IF node that holds the labelling

@@ -106,7 +106,8 @@ struct ising_ctx {
   WolffGraph wolff_graph;           // one Wolff step as a CUDA graph (growth + IF labelling)
   bool wolff_graph_broken = false;  // building it failed once: separate launches from then on
   int cluster_mode = ISING_CLUSTER_AUTO;
-  GridCtl* cluster_gctl = nullptr;  // barrier of the persistent cluster kernel
+  GridCtl* cluster_gctl = nullptr;  // barrier of the persistent cluster kernels
+  void* cluster_strip = nullptr;    // scratch of the strip form (cluster_strip_bytes)
   bool timing = false;
   std::vector<cudaEvent_t> ev;
   size_t ev_used = 0;
@@ -156,6 +157,8 @@ void free_all(ising_ctx* c) {
   wolff_graph_free(&c->wolff_graph);
   cudaFree(c->wolff);
   cudaFree(c->cluster_gctl);
+  cudaFree(c->cluster_strip);
+  c->cluster_strip = nullptr;
   c->wolff = nullptr;
   c->cluster_gctl = nullptr;
   c->sw_parent = nullptr;
@@ -217,13 +220,8 @@ int validate_kernel(const ising_ctx* c, int kernel, int k, int tile_rows, int ti
   return fail(ISING_EINVAL, "kernel %d does not apply to the int8 layout", kernel);
 }
 
-// Buffers of the strips' boundary exchange, once per context.
-int ensure_strip(ising_ctx* c) {
-  if (c->strip.G <= 1 || c->strip_x) return ISING_OK;
-  void* p = nullptr;
-  int st = dev_alloc(&p, strip_xbuf_words(c->L, c->strip.G, c->strip.K) * sizeof(unsigned long long));
-  if (st) return st;
-  c->strip_x = (unsigned long long*)p;
+int ensure_strip_status(ising_ctx* c) {
+  if (c->strip_status) return ISING_OK;
   cudaError_t e = cudaHostAlloc((void**)&c->strip_status, sizeof(int), cudaHostAllocDefault);
   if (e != cudaSuccess) {
     c->strip_status = nullptr;
@@ -231,6 +229,16 @@ int ensure_strip(ising_ctx* c) {
   }
   *c->strip_status = 0;
   return ISING_OK;
+}
+
+// Buffers of the strips' boundary exchange, once per context.
+int ensure_strip(ising_ctx* c) {
+  if (c->strip.G <= 1 || c->strip_x) return ISING_OK;
+  void* p = nullptr;
+  int st = dev_alloc(&p, strip_xbuf_words(c->L, c->strip.G, c->strip.K) * sizeof(unsigned long long));
+  if (st) return st;
+  c->strip_x = (unsigned long long*)p;
+  return ensure_strip_status(c);
 }
 
 // 32-word tiles, four sweeps per launch, and the number of row strips that gives
@@ -983,19 +991,49 @@ int cluster_checks(ising_ctx* c, int64_t counter, int n_steps, int measure_every
 }
 
 constexpr int kClusterPersistMaxL = 768;
+constexpr int kClusterSmemMaxL = 64;  // up to here one CTA holds the lattice (cluster_persist.cu)
 
 // Whether cluster steps on this context run as one persistent kernel per call.
-bool cluster_persistent(const ising_ctx* c) {
+bool cluster_persistent(const ising_ctx* c, bool wolff) {
   if (c->cluster_mode == ISING_CLUSTER_PERSISTENT) return true;
   if (c->cluster_mode == ISING_CLUSTER_KERNELS || c->cluster_mode == ISING_CLUSTER_GRAPH) return false;
-  // measured on GB300 at beta_c: one launch wins up to L = 512 (70 vs 76 us per
-  // step), the kernel-per-phase path at L = 1024 (137 vs 189 us)
-  return c->L < kClusterPersistMaxL;
+  // Swendsen-Wang: wherever the strips fit, except on lattices that the tiled
+  // labelling takes (us per step at beta_c, strips / kernels: L = 1024 56 / 134, 1536
+  // 112 / 221; tiled: 2048 170 / 111).  Wolff: below 768, where a step that grows from
+  // the seed is not yet worth a launch.
+  if (c->L <= kClusterSmemMaxL) return true;
+  if (wolff) return c->L < kClusterPersistMaxL;
+  return !sw_tiled(c->L) && cluster_strip_grid(c->L, c->sms) > 0;
 }
 
 // n persistent-kernel cluster steps from step0, records included.
 int cluster_persist_run(ising_ctx* c, bool wolff, int64_t step0, int n, int measure_every) {
   if (n <= 0) return ISING_OK;
+  const int G = c->L > kClusterSmemMaxL ? cluster_strip_grid(c->L, c->sms) : 0;
+  if (G > 0) {
+    if (!c->cluster_strip) {
+      if (int st = dev_alloc(&c->cluster_strip, cluster_strip_bytes(c->L, G))) return st;
+    }
+    if (int st = ensure_strip_status(c)) return st;
+    const int64_t m = measure_every;
+    // chunks whose records fit the ring
+    const int64_t most = m > 0 ? std::min<int64_t>(kRecCap * m, 1 << 29) : 1 << 29;
+    for (int64_t done = 0; done < n;) {
+      const int k = (int)std::min<int64_t>(most, n - done);
+      const int64_t t = step0 + done, before = m > 0 ? t / m : 0, n_rec = m > 0 ? (t + k) / m - before : 0;
+      if (int st = zero_records(c, c->rec_count, n_rec)) return st;
+      Timed tm(c);
+      cudaError_t e = launch_cluster_strip(c->lat(c->cur), wolff, (uint32_t)t, k, measure_every,
+                                           n_rec ? (int)((before + 1) * m - t) : 0, bond_threshold(c->beta), c->rng(),
+                                           G, c->cluster_strip, c->rec, c->rec_count % kRecCap, kRecCap, c->wolff,
+                                           c->strip_status, c->stream);
+      if (int st = launch_result(c, e, "cluster strips")) return st;
+      c->rec_count += n_rec;
+      done += k;
+    }
+    return ISING_OK;
+  }
+  if (int st = cluster_scratch(c)) return st;
   if (!c->cluster_gctl) {
     void* p = nullptr;
     if (int st = dev_alloc(&p, sizeof(GridCtl))) return st;
@@ -1055,7 +1093,7 @@ int ising_wolff_step(ising_ctx* c, int n_steps, int measure_every) {
     cudaError_t e = cudaMemsetAsync(c->wolff, 0, sizeof(WolffCtl), c->stream);
     if (e) return fail(ISING_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
   }
-  if (cluster_persistent(c)) {
+  if (cluster_persistent(c, true)) {
     if (int st = cluster_persist_run(c, true, c->wolff_steps, n_steps, measure_every)) return st;
     c->wolff_steps += n_steps;
     return ok();
@@ -1131,12 +1169,12 @@ int ising_sw_step(ising_ctx* c, int n_steps, int measure_every) {
   if (int st = check_ctx(c)) return st;
   if (int st = cluster_checks(c, c->sw_steps, n_steps, measure_every)) return st;
   NvtxRange nvtx("ising_sw_step");
-  if (int st = cluster_scratch(c)) return st;
-  if (cluster_persistent(c)) {
+  if (cluster_persistent(c, false)) {
     if (int st = cluster_persist_run(c, false, c->sw_steps, n_steps, measure_every)) return st;
     c->sw_steps += n_steps;
     return ok();
   }
+  if (int st = cluster_scratch(c)) return st;
   const uint32_t thr = bond_threshold(c->beta);
   const RngParams rng = c->rng();
   for (int k = 0; k < n_steps; ++k) {

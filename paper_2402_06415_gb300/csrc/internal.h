@@ -276,6 +276,18 @@ cudaError_t launch_cluster_persist(const BitsLattice& lat, bool wolff, uint32_t 
                                    GridCtl* gctl,
                                    WolffCtl* wctl, int sms, cudaStream_t s);
 
+// The same on resident row strips (cluster_strip.cu).  cluster_strip_grid: strips of
+// an L x L lattice (0: they do not fit in shared memory); scratch: device memory
+// of cluster_strip_bytes(L, G) bytes; the record slots are zero on entry; to_rec:
+// steps until the first record (0: none); *status: host-visible word set to 1
+// when a wait gave up.
+int cluster_strip_grid(int L, int sms);
+size_t cluster_strip_bytes(int L, int G);
+cudaError_t launch_cluster_strip(const BitsLattice& lat, bool wolff, uint32_t step0, int n_steps, int measure_every,
+                                 int to_rec, uint32_t thr, const RngParams& rng, int G, void* scratch,
+                                 unsigned long long* rec, long long rec0, long long rec_cap, WolffCtl* wctl,
+                                 int* status, cudaStream_t s);
+
 // Sets the message returned by ising_last_error() on the calling thread.
 void set_last_error(const char* msg);
 

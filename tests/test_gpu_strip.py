@@ -96,3 +96,23 @@ def test_quad_strips_equal_oracle(lattice, J1, J2, Lc):
     assert np.array_equal(got, s)
     at = [3, 7, 9, 10, 11, 12, 13]
     assert np.array_equal(B1, R1[at]) and np.array_equal(B2, R2[at]) and np.array_equal(M, RM[at])
+
+
+# a shared forest per CTA (L <= 160) and the global one, uneven strips of 2 to 10 rows, rows that are no multiple of a
+# 64-site block; one step, records, and a hot, critical and cold lattice
+@pytest.mark.parametrize("wolff", [False, True])
+@pytest.mark.parametrize("L", [66, 158, 160, 162, 330, 446, 450, 766, 1030])
+@pytest.mark.parametrize("beta", [0.2, 0.4406868, 1.5])
+def test_cluster_strips_equal_kernels(wolff, L, beta):
+    out = []
+    for mode in (ising.ISING_CLUSTER_PERSISTENT, ising.ISING_CLUSTER_KERNELS):
+        with ising.Lattice(L, beta, BITS, seed=3 + L) as lat:
+            lat.cluster_set_mode(mode)
+            step = lat.wolff_step if wolff else lat.sw_step
+            for n, every in [(1, 1), (2, 0), (6, 2)]:
+                step(n, every)
+            lat.sweep(1)
+            step(3, 1)
+            out.append((lat.spins(), *lat.series(), lat.wolff_stats()["flipped"] if wolff else 0))
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
