@@ -181,7 +181,7 @@ int check_ctx(ising_ctx* c) {
 // Where the resident strips are the automatic choice: everywhere they fit in
 // shared memory, except lattices from 6144 up that tile into 32-word tiles
 // (flips/ns, strips against the best tiled shape: L = 2048 1220 / 709, 4096
-// 2057 / 1627, 6144 2384 / 2192, 8192 2569 / 2706).  The other automatic paths
+// 2066 / 1627, 6144 2416 / 2192, 8192 2611 / 3094).  The other automatic paths
 // there, one launch per half sweep or per sweep, gave 115 at L = 1000 and 200 at
 // L = 2048; one CTA with int8 spins 0.25 at L = 64 (strips: 7).
 bool strip_applies(int layout, int L) {
@@ -244,8 +244,8 @@ int ensure_strip(ising_ctx* c) {
 // 32-word tiles, four sweeps per launch, and the number of row strips that gives
 // whole waves of resident CTAs (2 or 3 per SM) with the fewest row updates per
 // SM, halo rows included (2K - 1 on average over the half sweeps).  L = 16384:
-// 76 strips, two waves of two CTAs, 3113 flips/ns (one sweep per launch and 152
-// strips, the choice before: 2310); 12288: 76, 3047; 8192: 76, 2706.
+// 76 strips, two waves of two CTAs, 3530 flips/ns (one sweep per launch and 152
+// strips, the choice before, was 25 % slower); 12288: 50, 3456; 8192: 76, 3094.
 void auto_tiles32(ising_ctx* c) {
   constexpr int K = 4;
   const int n_tx = c->Wc / 32;
@@ -257,8 +257,8 @@ void auto_tiles32(ising_ctx* c) {
       const int n_ty = std::min(c->sms * per_sm * waves / n_tx, c->L / 8);
       if (n_ty < 1) continue;
       const int rows = (c->L + n_ty - 1) / n_ty;
-      // shared memory of an SM: 228 KB less 1 KB per CTA and the queue's 18 KB
-      const size_t smem = tiled32_smem_bytes(c->L, K, n_ty, 32) + 20 * 1024;
+      // shared memory of an SM: 228 KB less 1 KB per CTA and the queue's 24 KB
+      const size_t smem = tiled32_smem_bytes(c->L, K, n_ty, 32) + 26 * 1024;
       if (smem * per_sm > 227 * 1024) continue;
       const int64_t cost = (int64_t)waves * per_sm * (rows + 2 * K - 1);
       if (cost < best) {

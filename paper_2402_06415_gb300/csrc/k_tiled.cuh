@@ -146,6 +146,24 @@ __global__ void __launch_bounds__(256) k_tiled_bits(const uint32_t* __restrict__
     if (slots.slot[s] >= 0) block_add2(acc_anti[s], acc_ones[s], rec + 2 * (size_t)slots.slot[s]);
 }
 
+// Planes of blocks 2 .. 7 of one word by its lane alone (a full queue; not expected
+// at the automatic tile sizes): returns the accepted lanes.
+__device__ __noinline__ uint32_t finish_word(uint32_t g, uint32_t t, uint32_t rep, uint32_t colour,
+                                             const RngParams& rng, uint32_t D, uint32_t cls) {
+  uint32_t acc = 0;
+  for (int b = 2; b < 8 && D != 0u; ++b) {
+    const uint4 r = philox10_rk(make_uint4(g, t, rep, ctr_w(kTagMet, colour, b)), rng.rk0, rng.rk1);
+    const uint32_t p[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t tm = (cls & rng.tm4[4 * b + q]) | (~cls & rng.tm8[4 * b + q]);
+      acc |= D & tm & ~p[q];
+      D &= ~(tm ^ p[q]);
+    }
+  }
+  return acc;
+}
+
 // Tiled sweep with one warp per 32-word tile row segment.  Same tiling, halo
 // and results as k_tiled_bits; differences are for speed only:
 //  * the inner 32*TWW words of a row are updated by TWW warps (lane = word), the
@@ -153,10 +171,20 @@ __global__ void __launch_bounds__(256) k_tiled_bits(const uint32_t* __restrict__
 //    or modulo runs per word;
 //  * phase 1 evaluates the first two Philox blocks (8 planes) of every word as
 //    one 8-bit comparison (planes8); words with lanes still undecided (about 1
-//    in 10) go to a shared-memory
-//    queue, and phase 2 finishes them with all lanes of a warp busy on queued
-//    words, instead of every warp waiting for its slowest word;
+//    in 10) go to a shared-memory queue, one claim per pair of words and one
+//    16-byte entry per word, and phase 2 finishes them with all lanes of a warp
+//    busy on queued words, instead of every warp waiting for its slowest word.  A
+//    lane that finds the queue full finishes its words alone, so the hot loop has
+//    no warp vote;
 //  * per-sweep observables are summed in shared memory, not registers.
+//
+// What bounds it: the logic pipe.  A logic operation or shift holds it 2 cycles
+// per warp and sub-partition, and so does a 32 x 32 -> 64 product (4 cycles on its own
+// pipe); additions are nearly free beside them.  L = 16384, beta_c, (K, strips, words) =
+// (4, 76, 32): 3120 flips/ns with three 4-byte queue arrays, a claim per word and a vote
+// per pair; 3260 with one claim and one 16-byte entry; 3320 with the warp index known
+// to be uniform; 3540 with the position and group in the entry and no vote.  Philox
+// with its first rounds' word-independent parts formed by hand measured 8 % slower.
 //
 // MINB is the number of CTAs per SM the register budget is sized for: 3 (80
 // registers) for tiles that fit three CTAs' shared memory on an SM, 2 (up to
@@ -173,10 +201,10 @@ __global__ void __launch_bounds__(256, MINB) k_tiled32_bits(const uint32_t* __re
   // queue capacity: about 1 word in 10 is still undecided after 8 planes (11 %
   // in an ordered lattice), ~500 words per half sweep of a 72 x 64-word tile
   // and ~800 of a 216 x 32-word tile; a full queue sends the rest to the slow
-  // in-place path.  18 KB, so tiles of up to 200 KiB still fit an SM.
+  // lane alone.  24 KB, so tiles of up to 200 KiB still fit an SM.
   constexpr int QCAP = 1536;
   extern __shared__ uint4 smem4[];
-  __shared__ uint32_t q_pos[QCAP], q_d[QCAP], q_cls[QCAP];
+  __shared__ uint4 q_ent[QCAP];  // shared-memory index, undecided lanes, class lanes, group
   __shared__ int q_n[2];
   __shared__ unsigned long long s_anti[K], s_ones[K];
   uint32_t* S = reinterpret_cast<uint32_t*>(smem4);
@@ -186,7 +214,10 @@ __global__ void __launch_bounds__(256, MINB) k_tiled32_bits(const uint32_t* __re
   uint32_t* S1 = S + SR * SP;
   const int n_tx = Wc / TW;
   const int n_tiles = n_ty * n_tx;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  // the warp index through a shuffle: what depends on it (rows, parities, group
+  // bases) is then known to be uniform and leaves the logic pipe
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  constexpr int nwarps = 8;
   if (tid < K) {
     s_anti[tid] = 0ull;
     s_ones[tid] = 0ull;
@@ -260,36 +291,16 @@ __global__ void __launch_bounds__(256, MINB) k_tiled32_bits(const uint32_t* __re
         const uint32_t gv[1] = {g}, clsv[1] = {cls};
         planes8<1>(gv, t, rng.replica, c, rng, Dv, clsv, accv);
         const uint32_t D = Dv[0], acc = accv[0];
-        bool ovf = false;
         if (active) {
           So[r * SP + col] = s ^ ((k.ge2 & valid) | acc);
           if (D != 0u) {
             const int slot = atomicAdd(qn, 1);
-            if (slot < QCAP) {
-              q_pos[slot] = ((uint32_t)r << 8) | (uint32_t)col;
-              q_d[slot] = D;
-              q_cls[slot] = cls;
-            } else {
-              ovf = true;
-            }
+            if (slot < QCAP)
+              q_ent[slot] = make_uint4((uint32_t)(r * SP + col), D, cls, g);
+            else
+              So[r * SP + col] ^= finish_word(g, t, rng.replica, c, rng, D, cls);
           }
         }
-        // queue full (not expected at these tile sizes): finish in place
-        if (__any_sync(0xffffffffu, ovf)) {
-          uint32_t e = ovf ? D : 0u, acc2 = 0;
-          lazy_planes<2, 8>(g, t, rng.replica, c, rng, e, cls, acc2);
-          if (ovf) So[r * SP + col] ^= acc2;
-        }
-      };
-      // queue a word whose lanes are still undecided after phase 1 (returns
-      // false if the queue is full; the caller then finishes it in place)
-      auto enqueue = [&](int r, int col, uint32_t D, uint32_t cls) {
-        const int slot = atomicAdd(qn, 1);
-        if (slot >= QCAP) return false;
-        q_pos[slot] = ((uint32_t)r << 8) | (uint32_t)col;
-        q_d[slot] = D;
-        q_cls[slot] = cls;
-        return true;
       };
       // inner words of two adjacent rows (r, r+1) per thread: the two words
       // share the other colour's rows r and r+1 as neighbours
@@ -324,13 +335,20 @@ __global__ void __launch_bounds__(256, MINB) k_tiled32_bits(const uint32_t* __re
         const uint32_t Da = Dv[0], Db = Dv[1], acca = accv[0], accb = accv[1];
         So[r * SP + col] = sa ^ (ka.ge2 | acca);
         So[(r + 1) * SP + col] = sb ^ (kb.ge2 | accb);
-        const bool ovfa = Da != 0u && !enqueue(r, col, Da, ka.cls);
-        const bool ovfb = Db != 0u && !enqueue(r + 1, col, Db, kb.cls);
-        if (__any_sync(0xffffffffu, ovfa || ovfb)) {  // queue full: finish in place
-          uint32_t ea = ovfa ? Da : 0u, eb = ovfb ? Db : 0u, xa = 0, xb = 0;
-          lazy_planes2<2, 8>(ga, gb, t, rng.replica, c, rng, ea, ka.cls, xa, eb, kb.cls, xb);
-          if (ovfa) So[r * SP + col] ^= xa;
-          if (ovfb) So[(r + 1) * SP + col] ^= xb;
+        // queue the words whose lanes are still undecided, one claim for both
+        if ((Da | Db) != 0u) {
+          const int na = Da != 0u;
+          const int slot = atomicAdd(qn, na + (Db != 0u));
+          const uint32_t pos = (uint32_t)(r * SP + col);
+          if (slot + 2 <= QCAP) {
+            if (na) q_ent[slot] = make_uint4(pos, Da, ka.cls, ga);
+            if (Db != 0u) q_ent[slot + na] = make_uint4(pos + SP, Db, kb.cls, gb);
+          } else {
+            So[pos] ^= finish_word(ga, t, rng.replica, c, rng, Da, ka.cls);
+            So[pos + SP] ^= finish_word(gb, t, rng.replica, c, rng, Db, kb.cls);
+            // claimed entries below the capacity must not hold an old word
+            for (int e = slot; e < QCAP && e < slot + na + (Db != 0u); ++e) q_ent[e] = make_uint4(0u, 0u, 0u, 0u);
+          }
         }
       };
       // three kinds of work item (row pairs, the odd last row, the halo
@@ -365,13 +383,10 @@ __global__ void __launch_bounds__(256, MINB) k_tiled32_bits(const uint32_t* __re
       for (int base = warp * 32; base < n; base += blockDim.x) {
         const int e = base + lane;
         const bool act = e < n;
-        const uint32_t pos = act ? q_pos[e] : (3u | ((uint32_t)r_lo << 8));
-        uint32_t D = act ? q_d[e] : 0u, acc = 0;
-        const uint32_t cls = act ? q_cls[e] : 0u;
-        const int r = (int)(pos >> 8), col = (int)(pos & 255u);
-        const uint32_t g = (uint32_t)grow(r) * (uint32_t)Wc + (uint32_t)gcol(col);
-        lazy_planes<2, 8>(g, t, rng.replica, c, rng, D, cls, acc);
-        if (act && acc) So[r * SP + col] ^= acc;
+        const uint4 ent = act ? q_ent[e] : make_uint4(0u, 0u, 0u, 0u);
+        uint32_t D = ent.y, acc = 0;
+        lazy_planes<2, 8>(ent.w, t, rng.replica, c, rng, D, ent.z, acc);
+        if (act && acc) So[ent.x] ^= acc;
       }
       if (c == 1 && slots.slot[sw] >= 0) {
         __syncthreads();
