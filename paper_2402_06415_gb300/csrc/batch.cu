@@ -183,10 +183,32 @@ __device__ __forceinline__ void planes8_tab2(uint32_t ga, uint32_t gb, uint32_t 
   Db = eqb;
 }
 
+// Planes of blocks 2 .. 7 of one word by its lane alone (a full queue): returns the
+// accepted lanes.
+__device__ __noinline__ uint32_t finish_word_tab(uint32_t g, uint32_t t, uint32_t rep, uint32_t colour,
+                                                 const uint32_t (&rk0)[10], const uint32_t (&rk1)[10],
+                                                 const uint2* tm, uint32_t D, uint32_t cls) {
+  uint32_t acc = 0;
+  for (int b = 2; b < 8 && D != 0u; ++b) {
+    const uint4 r = philox10_rk(make_uint4(g, t, rep, ctr_w(kTagMet, colour, b)), rk0, rk1);
+    const uint32_t p[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint2 m = tm[4 * b + q];
+      const uint32_t tk = (cls & m.x) | (~cls & m.y);
+      acc |= D & tk & ~p[q];
+      D &= ~(tk ^ p[q]);
+    }
+  }
+  return acc;
+}
+
 // One round (ns sweeps from global sweep t0) of one item, in shared memory.
 struct ItemSmem {
   uint2 tm[kMaxRepPerItem][32];  // per replica and plane: threshold masks (t4, t8)
-  uint32_t q_idx[kQueueCap], q_d[kQueueCap], q_cls[kQueueCap];
+  // undecided words: shared-memory index | replica of the item << 16, undecided
+  // lanes, class lanes, group
+  uint4 q_ent[kQueueCap];
   int q_n[2];
 };
 
@@ -216,6 +238,10 @@ __device__ void run_item(const BatchDev& d, int item, uint32_t t0, int ns, bool 
     X.tm[qq][k] = make_uint2(0u - ((s_t4[qq] >> (31 - k)) & 1u), 0u - ((s_t8[qq] >> (31 - k)) & 1u));
   }
   __syncthreads();
+  // Bound by the logic pipe and the CTA barriers.  4096 replicas, flips/ns: 1591 with a
+  // claim and three stores per queued word and a vote per pair, 1719 with one claim per
+  // pair, 16-byte entries that carry address and group, and no vote; 1840 with
+  // 128-thread CTAs (finer barriers).
   // Half sweeps in two phases, as in the single-lattice tiled kernel: phase 1
   // draws the first two Philox blocks (8 planes) of every word and queues the
   // words with lanes still undecided (~7 %); phase 2 finishes the queued words
@@ -223,32 +249,22 @@ __device__ void run_item(const BatchDev& d, int item, uint32_t t0, int ns, bool 
   // its slowest word.  (Warp-owned replicas with only __syncwarp() between half
   // sweeps measured slower: too few resident warps per SM for this many
   // replicas.)
-  const int lane = threadIdx.x & 31;
+  // the warp's first thread through a shuffle: known to be uniform
+  const int lane = threadIdx.x & 31, warp0 = __shfl_sync(0xffffffffu, (int)(threadIdx.x & ~31u), 0);
   const int words = nr * plane;
   const int half = plane / 2, pairs = nr * half;  // word pairs (rows 2 yy, 2 yy + 1)
-  const FastDiv fplane = make_fastdiv((uint32_t)plane), fwc = make_fastdiv((uint32_t)Wc);
+  const FastDiv fwc = make_fastdiv((uint32_t)Wc);
   const FastDiv fhalf = make_fastdiv((uint32_t)half);
   for (int s = 0; s < ns; ++s) {
     const uint32_t t = t0 + (uint32_t)s;
     for (int c = 0; c < 2; ++c) {
       const int cur = c;  // queue counter of this half sweep (the other is reset meanwhile)
-      auto enq = [&](int idx, uint32_t D, uint32_t cls) {  // returns true if the queue was full
-        if (D == 0u) return false;
-        const int slot = atomicAdd(&X.q_n[cur], 1);
-        if (slot < kQueueCap) {
-          X.q_idx[slot] = (uint32_t)idx;
-          X.q_d[slot] = D;
-          X.q_cls[slot] = cls;
-          return false;
-        }
-        return true;
-      };
       // two vertically adjacent words of one replica per lane (rows 2 yy and
       // 2 yy + 1; L is even): they share the other colour's rows 2 yy, 2 yy + 1
       // as neighbours (and the half sum of that pair), the replica and the
       // index division, and their two Philox chains interleave; 80 registers
       // keep three CTAs of 256 threads per SM
-      for (int p0 = threadIdx.x & ~31; p0 < pairs; p0 += blockDim.x) {
+      for (int p0 = warp0; p0 < pairs; p0 += blockDim.x) {
         const int p = p0 + lane;
         const bool act = p < pairs;
         const int qq = act ? (int)fdiv((uint32_t)p, fhalf) : 0;
@@ -279,31 +295,34 @@ __device__ void run_item(const BatchDev& d, int item, uint32_t t0, int ns, bool 
           So[pa] = sa ^ ((ka.ge2 & valid) | acca);
           So[pb] = sb ^ ((kb.ge2 & valid) | accb);
         }
-        const bool ovfa = enq(qq * plane + pa, Da, ka.cls);
-        const bool ovfb = enq(qq * plane + pb, Db, kb.cls);
-        if (__any_sync(0xffffffffu, ovfa || ovfb)) {  // queue full: finish in place
-          uint32_t ea = ovfa ? Da : 0u, eb = ovfb ? Db : 0u, xa = 0, xb = 0;
-          planes_tab<2, 8, true>((uint32_t)pa, t, rep, (uint32_t)c, d.rk0, d.rk1, X.tm[qq], ea, ka.cls, xa);
-          planes_tab<2, 8, true>((uint32_t)pb, t, rep, (uint32_t)c, d.rk0, d.rk1, X.tm[qq], eb, kb.cls, xb);
-          if (ovfa) So[pa] ^= xa;
-          if (ovfb) So[pb] ^= xb;
+        // queue the words whose lanes are still undecided, one claim for both; a lane
+        // that finds the queue full finishes its words alone (no warp vote here)
+        if ((Da | Db) != 0u) {
+          const int na = Da != 0u, n = na + (Db != 0u);
+          const int slot = atomicAdd(&X.q_n[cur], n);
+          const uint32_t at = (uint32_t)(qq * per_rep + c * plane + pa), tag = (uint32_t)qq << 16;
+          if (slot + 2 <= kQueueCap) {
+            if (na) X.q_ent[slot] = make_uint4(at | tag, Da, ka.cls, (uint32_t)pa);
+            if (Db != 0u) X.q_ent[slot + na] = make_uint4((at + Wc) | tag, Db, kb.cls, (uint32_t)pb);
+          } else {
+            So[pa] ^= finish_word_tab((uint32_t)pa, t, rep, (uint32_t)c, d.rk0, d.rk1, X.tm[qq], Da, ka.cls);
+            So[pb] ^= finish_word_tab((uint32_t)pb, t, rep, (uint32_t)c, d.rk0, d.rk1, X.tm[qq], Db, kb.cls);
+            // claimed entries below the capacity must not hold an old word
+            for (int e = slot; e < kQueueCap && e < slot + n; ++e) X.q_ent[e] = make_uint4(0u, 0u, 0u, 0u);
+          }
         }
       }
       __syncthreads();
       const int nq = min(X.q_n[cur], kQueueCap);
       if (threadIdx.x == 0) X.q_n[cur ^ 1] = 0;
-      for (int b0 = threadIdx.x & ~31; b0 < nq; b0 += blockDim.x) {
+      for (int b0 = warp0; b0 < nq; b0 += blockDim.x) {
         const int e = b0 + lane;
         const bool act = e < nq;
-        const int idx = act ? (int)X.q_idx[e] : 0;
-        uint32_t D = act ? X.q_d[e] : 0u, acc = 0;
-        const uint32_t cls = act ? X.q_cls[e] : 0u;
-        const int qq = (int)fdiv((uint32_t)idx, fplane);
-        const int rem = idx - qq * plane;
-        const int y = (int)fdiv((uint32_t)rem, fwc), w = rem - y * Wc;
-        planes_tab<2, 8, true>((uint32_t)(y * Wc + w), t, (uint32_t)(r0 + qq), (uint32_t)c, d.rk0, d.rk1,
-                               X.tm[qq], D, cls, acc);
-        if (act && acc) sm[qq * per_rep + c * plane + y * Wc + w] ^= acc;
+        const uint4 ent = act ? X.q_ent[e] : make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t qq = ent.x >> 16;
+        uint32_t D = ent.y, acc = 0;
+        planes_tab<2, 8, true>(ent.w, t, (uint32_t)r0 + qq, (uint32_t)c, d.rk0, d.rk1, X.tm[qq], D, ent.z, acc);
+        if (act && acc) sm[ent.x & 0xffffu] ^= acc;
       }
       __syncthreads();
     }
@@ -735,6 +754,19 @@ int ising_batch_create(ising_batch** out, int n_ladders, const int* L, int n_bet
     if (!e) e = cudaMemcpy(b->d_q, q.data(), q.size() * 8, cudaMemcpyHostToDevice);
     if (!e) e = cudaMemset(b->d_ctr, 0, sizeof(BatchCounters));
     if (e) st = bfail(ISING_ECUDA, "batch setup copy: %s", cudaGetErrorString(e));
+  }
+  if (!st) {
+    // Default decomposition: 128 threads a CTA (six per SM) and the smaller of 256 and
+    // 512 words per item that leaves at most one item per resident CTA.  flips/ns for
+    // (256, 128) / (512, 128) / (512, 256) words and threads: 12.7 k words per colour
+    // plane in all 228 / 161 / 194, 83 k 1033 / 836 / 871, 166 k 1569 / 1349 / 1378, 331 k
+    // 1616 / 1922 / 1587.
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e) st = bfail(ISING_ECUDA, "device query: %s", cudaGetErrorString(e));
+    b->threads = 128;
+    b->words_per_item = o / 2 <= 256LL * 6 * sms ? 256 : 512;
   }
   if (!st) st = plan_items(b);
   if (st) {
