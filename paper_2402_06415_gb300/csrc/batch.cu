@@ -550,7 +550,7 @@ void bfree(ising_batch* b) {
   if (b->graph_exec) cudaGraphExecDestroy(b->graph_exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   void* ptrs[] = {b->spins, b->d_off, b->d_L, b->d_t4, b->d_t8, b->d_q, b->d_perm, b->d_slot,
-                  b->d_E, b->d_M, b->d_acc, b->d_att, b->d_serE, b->d_serM, b->d_serS,
+                  b->d_acc, b->d_serE, b->d_serM, b->d_serS,
                   b->d_item_l, b->d_item_i0, b->d_item_nr, b->d_cta_first, b->d_cta_items,
                   b->d_ctr, b->nn_w, b->nn_w2t, b->d_beta_slot, b->d_unit0, b->d_blk_stats, b->plan};
   for (void* p : ptrs) cudaFree(p);
@@ -738,12 +738,15 @@ int ising_batch_create(ising_batch** out, int n_ladders, const int* L, int n_bet
   A(&b->d_t4, (size_t)n_beta);
   A(&b->d_t8, (size_t)n_beta);
   A(&b->d_q, q.size());
-  A(&b->d_perm, (size_t)b->n_rep);
+  // what one call reads back lies together: perm, E, M; accepted, attempted
+  A(&b->d_perm, (size_t)3 * b->n_rep);
   A(&b->d_slot, (size_t)b->n_rep);
-  A(&b->d_E, (size_t)b->n_rep);
-  A(&b->d_M, (size_t)b->n_rep);
-  A(&b->d_acc, (size_t)b->n_rep);
-  A(&b->d_att, (size_t)b->n_rep);
+  A(&b->d_acc, (size_t)2 * b->n_rep);
+  if (!st) {
+    b->d_E = b->d_perm + b->n_rep;
+    b->d_M = b->d_E + b->n_rep;
+    b->d_att = b->d_acc + b->n_rep;
+  }
   A(&b->d_ctr, 1);
   if (!st) {
     cudaError_t e = cudaSuccess;
@@ -917,26 +920,25 @@ int ising_batch_status(ising_batch* b, int* status, int64_t* sweep) {
 
 int ising_batch_state(ising_batch* b, int32_t* perm, int64_t* E, int64_t* M) {
   if (int st = ising_batch_status(b, nullptr, nullptr)) return st;
-  std::vector<int> hp(b->n_rep), he(b->n_rep), hm(b->n_rep);
-  BTRY(cudaMemcpy(hp.data(), b->d_perm, hp.size() * 4, cudaMemcpyDeviceToHost));
-  BTRY(cudaMemcpy(he.data(), b->d_E, he.size() * 4, cudaMemcpyDeviceToHost));
-  BTRY(cudaMemcpy(hm.data(), b->d_M, hm.size() * 4, cudaMemcpyDeviceToHost));
-  for (int r = 0; r < b->n_rep; ++r) {
-    if (perm) perm[r] = hp[r];
-    if (E) E[r] = he[r];
-    if (M) M[r] = hm[r];
+  const size_t n = (size_t)b->n_rep;
+  std::vector<int> h(3 * n);
+  BTRY(cudaMemcpy(h.data(), b->d_perm, h.size() * 4, cudaMemcpyDeviceToHost));
+  for (size_t r = 0; r < n; ++r) {
+    if (perm) perm[r] = h[r];
+    if (E) E[r] = h[n + r];
+    if (M) M[r] = h[2 * n + r];
   }
   return ISING_OK;
 }
 
 int ising_batch_swap_counts(ising_batch* b, int64_t* accepts, int64_t* attempts) {
   if (int st = ising_batch_status(b, nullptr, nullptr)) return st;
-  std::vector<unsigned long long> ha(b->n_rep), ht(b->n_rep);
-  BTRY(cudaMemcpy(ha.data(), b->d_acc, ha.size() * 8, cudaMemcpyDeviceToHost));
-  BTRY(cudaMemcpy(ht.data(), b->d_att, ht.size() * 8, cudaMemcpyDeviceToHost));
-  for (int r = 0; r < b->n_rep; ++r) {
-    if (accepts) accepts[r] = (int64_t)ha[r];
-    if (attempts) attempts[r] = (int64_t)ht[r];
+  const size_t n = (size_t)b->n_rep;
+  std::vector<unsigned long long> h(2 * n);
+  BTRY(cudaMemcpy(h.data(), b->d_acc, h.size() * 8, cudaMemcpyDeviceToHost));
+  for (size_t r = 0; r < n; ++r) {
+    if (accepts) accepts[r] = (int64_t)h[r];
+    if (attempts) attempts[r] = (int64_t)h[n + r];
   }
   return ISING_OK;
 }

@@ -61,17 +61,6 @@ __device__ __forceinline__ void sincos_small(double r, double& s, double& c) {
   s = __dmul_rn(ps, r);
 }
 
-__device__ __forceinline__ void own_sincos(double x, double& s, double& c) {
-  const double k = rint(__dmul_rn(x, 0.6366197723675814));
-  double r = fma(-k, 1.5707963267948966, x);
-  r = fma(-k, 6.123233995736766e-17, r);
-  double ss, cc;
-  sincos_small(r, ss, cc);
-  const int q = ((int)k) & 3;
-  s = q == 0 ? ss : (q == 1 ? cc : (q == 2 ? -ss : -cc));
-  c = q == 0 ? cc : (q == 1 ? -ss : (q == 2 ? -cc : ss));
-}
-
 __device__ __forceinline__ double own_exp(double x) {
   if (x < -700.0) return 0.0;
   const double k = rint(__dmul_rn(x, 1.4426950408889634));
@@ -143,13 +132,6 @@ __device__ __forceinline__ float own_exp(float x) {
   return p * __int_as_float(((int)k + 127) << 23);
 }
 
-template <typename T> __device__ __forceinline__ T two_pi();
-template <> __device__ __forceinline__ double two_pi<double>() { return 6.283185307179586; }
-template <> __device__ __forceinline__ float two_pi<float>() { return 6.28318548f; }
-template <typename T> __device__ __forceinline__ T inv24();
-template <> __device__ __forceinline__ double inv24<double>() { return 1.0 / 16777216.0; }
-template <> __device__ __forceinline__ float inv24<float>() { return 1.0f / 16777216.0f; }
-
 template <typename T> __device__ __forceinline__ T mul_rn(T a, T b);
 template <> __device__ __forceinline__ double mul_rn<double>(double a, double b) { return __dmul_rn(a, b); }
 template <> __device__ __forceinline__ float mul_rn<float>(float a, float b) { return __fmul_rn(a, b); }
@@ -160,19 +142,18 @@ template <typename T> __device__ __forceinline__ T sub_rn(T a, T b);
 template <> __device__ __forceinline__ double sub_rn<double>(double a, double b) { return __dsub_rn(a, b); }
 template <> __device__ __forceinline__ float sub_rn<float>(float a, float b) { return __fsub_rn(a, b); }
 
-template <typename T>
-__device__ __forceinline__ T angle_of(uint32_t w) {
-  return mul_rn<T>(two_pi<T>(), mul_rn<T>((T)(w >> 8), inv24<T>()));
+// sin and cos of the angle of a random word, theta = 2 pi (m 2^-24) with m its top 24
+// bits: theta rounded, k = rint(theta 2 / pi), r = theta - k pi / 2 (two-part
+// constant), the polynomials at r, and the quadrant k & 3.  In double every
+// operation holds this part's FP64 unit for 64 cycles per warp and sub-partition,
+// so five of those steps are done otherwise with the same values: the conversion
+// is integer work, the exact scaling by 2^-24 sits in the constant, and k is the
+// integer (m + 2^21) >> 22 unless m / 2^22 is exactly a half integer (m / 2^22
+// differs from theta 2 / pi by less than 2e-15, and otherwise lies at least 2^-22
+// from a half integer).
+__device__ __forceinline__ void word_sincos(uint32_t w, float& s, float& c) {
+  own_sincos(__fmul_rn(6.28318548f, __fmul_rn((float)(w >> 8), 1.0f / 16777216.0f)), s, c);
 }
-
-// sin and cos of the angle of a random word.  Same values as
-// own_sincos(angle_of<T>(w)); in double, where every operation holds this part's
-// FP64 unit for 64 cycles per warp and sub-partition, without five of them: the
-// conversion is integer work, the exact scaling by 2^-24 sits in the constant,
-// and the quadrant k = rint(x 2 / pi) is the integer (m + 2^21) >> 22 unless
-// m / 2^22 is exactly a half integer (m / 2^22 differs from x 2 / pi by less
-// than 2e-15, and otherwise lies at least 2^-22 from a half integer).
-__device__ __forceinline__ void word_sincos(uint32_t w, float& s, float& c) { own_sincos(angle_of<float>(w), s, c); }
 __device__ __forceinline__ void word_sincos(uint32_t w, double& s, double& c) {
   const uint32_t m = w >> 8;
   // m and k as doubles from their (exact) floats; no branches: the lanes differ
@@ -222,14 +203,12 @@ __global__ void k_xy_init(typename Vec<T>::type* __restrict__ u, int L, RngParam
 // e (1 -+ 1e-4) the exact own_exp gives the same answer and is skipped; inside
 // that band (rare), or for x < -80 with p = 0, own_exp decides.  For x < -80,
 // exp(x) < 2^-115 < p whenever p > 0 (p is a multiple of 2^-24).
-template <typename T>
-__device__ __forceinline__ bool accept_exp(T p, T x) {
-  if (x >= (T)-80) {
-    const float e = __expf((float)x);
-    const float pf = (float)p;  // exact: p = k 2^-24, k < 2^24
-    if (pf < e * 0.9999f) return true;
-    if (pf > e * 1.0001f) return false;
-  } else if (p > (T)0) {
+__device__ __forceinline__ bool accept_exp(float p, float x) {
+  if (x >= -80.f) {
+    const float e = __expf(x);
+    if (p < e * 0.9999f) return true;
+    if (p > e * 1.0001f) return false;
+  } else if (p > 0.f) {
     return false;
   }
   return p < own_exp(x);
@@ -237,7 +216,12 @@ __device__ __forceinline__ bool accept_exp(T p, T x) {
 
 // The trial's decision: dE <= 0 or p < exp(-beta dE), p = the top 24 bits of w2.
 __device__ __forceinline__ bool accept_move(uint32_t w2, float dE, float beta, float) {
-  return dE <= 0.f || accept_exp<float>(mul_rn<float>((float)(w2 >> 8), inv24<float>()), mul_rn<float>(-beta, dE));
+  return dE <= 0.f || accept_exp((float)(w2 >> 8) * (1.0f / 16777216.0f), mul_rn<float>(-beta, dE));
+}
+// beta for the estimate below; NaN (every trial decided exactly) where dE's cut to
+// float range or beta's overflow would spoil it.
+__host__ __device__ __forceinline__ float beta_estimate(double beta) {
+  return beta <= 1e30 ? (float)beta : (float)(0.0 * INFINITY);
 }
 // In double, the sign and the estimate that decides all but a band of 1e-4 need
 // no FP64 operation: -beta dE is formed in float (beta_f = beta) from dE's bits cut to 24
@@ -246,7 +230,7 @@ __device__ __forceinline__ bool accept_move(uint32_t w2, float dE, float beta, f
 __device__ __forceinline__ bool accept_move(uint32_t w2, double dE, double beta, float beta_f) {
   const int hi = __double2hiint(dE), lo = __double2loint(dE);
   const int mag = hi & 0x7fffffff;
-  if (mag < 0x7ff00000 && (hi < 0 || (mag | lo) == 0)) return true;
+  if (mag <= 0x7ff00000 && (hi < 0 || (mag | lo) == 0)) return true;
   const int ex = (mag >> 20) - 1023 + 127;
   const float d = ex <= 0 ? 0.f : ex >= 255 ? __int_as_float(0x7f800000)
                                             : __uint_as_float(((uint32_t)ex << 23) | ((uint32_t)(hi & 0xfffff) << 3) |
@@ -256,7 +240,7 @@ __device__ __forceinline__ bool accept_move(uint32_t w2, double dE, double beta,
     const float e = __expf(x);
     if (p < e * 0.9999f) return true;
     if (p > e * 1.0001f) return false;
-  } else if (p > 0.f) {
+  } else if (x < -80.f && p > 0.f) {
     return false;
   }
   return dE <= 0.0 || (double)p < own_exp(__dmul_rn(-beta, dE));
@@ -312,7 +296,7 @@ __device__ __forceinline__ unsigned int xy_pair(typename Vec<T>::type* __restric
     word_sincos(w1, sn, cs);
     V me = ld_state<CG>(own + k);
     const T dE = -fma(sub_rn<T>(cs, me.x), hx, mul_rn<T>(sub_rn<T>(sn, me.y), hy));
-    if (accept_move(w2, dE, beta, (float)beta)) {
+    if (accept_move(w2, dE, beta, beta_estimate((double)beta))) {
       me.x = cs;
       me.y = sn;
       st_state<CG>(own + k, me);
@@ -751,6 +735,8 @@ struct ising_xy {
   double* rec = nullptr;  // ring [65536][3]
   int64_t rec_count = 0;
   unsigned long long* accepted = nullptr;
+  bool grid_used = false;            // a grid barrier ran since the last seed: its status is worth reading
+  double* host_layout = nullptr;     // spins in the host's layout, allocated by the first call that needs it
   // resident strips of the automatic mode (G = 0: one launch per half sweep)
   int strip_G = 0, strip_gh = 0;
   unsigned long long* strip_x = nullptr;
@@ -805,7 +791,7 @@ cudaError_t xy_strip_t(ising_xy* x, int n, int m) {
   a.G = x->strip_G;
   a.gh = std::min(x->strip_gh, 2 * n);
   a.beta = (T)x->beta;
-  a.beta_f = (float)x->beta;
+  a.beta_f = beta_estimate(x->beta);
   a.t0 = (uint32_t)x->sweep;
   a.n = n;
   a.m = m;
@@ -888,6 +874,7 @@ cudaError_t xy_persist_t(ising_xy* x, int n, int m) {
     threads = fp64 ? 32 : 64;
     grid = std::max(1LL, std::min((pairs + threads - 1) / threads, (long long)sms));
     fn = (const void*)k_xy_persist<T, kGrid>;
+    x->grid_used = true;
     e = cudaMemsetAsync(&x->ctl->count, 0, sizeof(unsigned int), x->stream);
     if (e) return e;
   }
@@ -1029,6 +1016,7 @@ int ising_xy_seed(ising_xy* x, uint64_t seed) {
   x->seed = seed;
   x->sweep = 0;
   x->rec_count = 0;
+  x->grid_used = false;
   if (x->strip_status) *x->strip_status = 0;
   const RngParams rng = make_rng(seed, 0, 0, 0);
   const long long N = (long long)x->L * x->L;
@@ -1060,6 +1048,7 @@ int ising_xy_sweep(ising_xy* x, int n_sweeps, int measure_every) {
 static int xy_status(ising_xy* x) {
   if (x->strip_status && *(volatile int*)x->strip_status)
     return xfail(ISING_ETIMEOUT, "a strip's wait for its neighbour timed out in the XY kernel");
+  if (!x->grid_used) return ISING_OK;
   int st = 0;
   XTRY(cudaMemcpy(&st, &x->ctl->status, sizeof(int), cudaMemcpyDeviceToHost));
   if (st) return xfail(ISING_ETIMEOUT, "grid barrier timed out in the persistent XY kernel");
@@ -1104,15 +1093,17 @@ int ising_xy_launch_count(ising_xy* x, int64_t* count) {
 int ising_xy_series(ising_xy* x, double* E, double* Mx, double* My, int n) {
   if (!x) return xfail(ISING_EINVAL, "null context");
   if (n < 0 || n > std::min<int64_t>(x->rec_count, kXYRec)) return xfail(ISING_EINVAL, "n exceeds records");
-  std::vector<double> h((size_t)3 * kXYRec);
-  XTRY(cudaMemcpyAsync(h.data(), x->rec, h.size() * 8, cudaMemcpyDeviceToHost, x->stream));
+  std::vector<double> h((size_t)3 * n);
+  const int64_t s0 = (x->rec_count - n) % kXYRec, n1 = std::min<int64_t>(n, kXYRec - s0);
+  if (n1 > 0) XTRY(cudaMemcpyAsync(h.data(), x->rec + 3 * s0, (size_t)n1 * 24, cudaMemcpyDeviceToHost, x->stream));
+  if (n > n1)
+    XTRY(cudaMemcpyAsync(h.data() + 3 * n1, x->rec, (size_t)(n - n1) * 24, cudaMemcpyDeviceToHost, x->stream));
   XTRY(cudaStreamSynchronize(x->stream));
   if (int st = xy_status(x)) return st;
   for (int i = 0; i < n; ++i) {
-    const int64_t slot = (x->rec_count - n + i) % kXYRec;
-    if (E) E[i] = h[3 * slot];
-    if (Mx) Mx[i] = h[3 * slot + 1];
-    if (My) My[i] = h[3 * slot + 2];
+    if (E) E[i] = h[3 * i];
+    if (Mx) Mx[i] = h[3 * i + 1];
+    if (My) My[i] = h[3 * i + 2];
   }
   set_last_error("");
   return ISING_OK;
@@ -1121,8 +1112,8 @@ int ising_xy_series(ising_xy* x, double* E, double* Mx, double* My, int n) {
 int ising_xy_get_spins(ising_xy* x, double* host_uv) {
   if (!x || !host_uv) return xfail(ISING_EINVAL, "null argument");
   const long long N = (long long)x->L * x->L;
-  double* d = nullptr;
-  XTRY(cudaMalloc((void**)&d, N * 2 * sizeof(double)));
+  if (!x->host_layout) XTRY(cudaMalloc((void**)&x->host_layout, N * 2 * sizeof(double)));
+  double* d = x->host_layout;
   if (x->precision == 64)
     k_xy_to_host_layout<double><<<grid_of(N), 256, 0, x->stream>>>((const double2*)x->u, x->L, d, 0);
   else
@@ -1130,7 +1121,6 @@ int ising_xy_get_spins(ising_xy* x, double* host_uv) {
   cudaError_t e = cudaGetLastError();
   if (!e) e = cudaMemcpyAsync(host_uv, d, N * 2 * sizeof(double), cudaMemcpyDeviceToHost, x->stream);
   if (!e) e = cudaStreamSynchronize(x->stream);
-  cudaFree(d);
   if (e) return xfail(ISING_ECUDA, "get spins: %s", cudaGetErrorString(e));
   if (int st = xy_status(x)) return st;
   set_last_error("");
@@ -1140,8 +1130,8 @@ int ising_xy_get_spins(ising_xy* x, double* host_uv) {
 int ising_xy_set_spins(ising_xy* x, const double* host_uv) {
   if (!x || !host_uv) return xfail(ISING_EINVAL, "null argument");
   const long long N = (long long)x->L * x->L;
-  double* d = nullptr;
-  XTRY(cudaMalloc((void**)&d, N * 2 * sizeof(double)));
+  if (!x->host_layout) XTRY(cudaMalloc((void**)&x->host_layout, N * 2 * sizeof(double)));
+  double* d = x->host_layout;
   cudaError_t e = cudaMemcpyAsync(d, host_uv, N * 2 * sizeof(double), cudaMemcpyHostToDevice, x->stream);
   if (!e) {
     if (x->precision == 64)
@@ -1151,7 +1141,6 @@ int ising_xy_set_spins(ising_xy* x, const double* host_uv) {
     e = cudaGetLastError();
   }
   if (!e) e = cudaStreamSynchronize(x->stream);
-  cudaFree(d);
   if (e) return xfail(ISING_ECUDA, "set spins: %s", cudaGetErrorString(e));
   set_last_error("");
   return ISING_OK;
@@ -1176,6 +1165,7 @@ int ising_xy_destroy(ising_xy* x) {
   cudaFree(x->accepted);
   cudaFree(x->ctl);
   cudaFree(x->strip_x);
+  cudaFree(x->host_layout);
   cudaFreeHost(x->strip_status);
   delete x;
   return ISING_OK;

@@ -473,15 +473,17 @@ int ising_xyfix_set_mode(ising_xyfix* x, int mode) {
 int ising_xyfix_series(ising_xyfix* x, int64_t* E2, int64_t* Mx, int64_t* My, int n) {
   if (!x) return ffail(ISING_EINVAL, "null context");
   if (n < 0 || n > std::min<int64_t>(x->rec_count, kFixRec)) return ffail(ISING_EINVAL, "n exceeds records");
-  std::vector<unsigned long long> h((size_t)3 * kFixRec);
-  FTRY(cudaMemcpyAsync(h.data(), x->rec, h.size() * 8, cudaMemcpyDeviceToHost, x->stream));
+  std::vector<unsigned long long> h((size_t)3 * n);
+  const int64_t s0 = (x->rec_count - n) % kFixRec, n1 = std::min<int64_t>(n, kFixRec - s0);
+  if (n1 > 0) FTRY(cudaMemcpyAsync(h.data(), x->rec + 3 * s0, (size_t)n1 * 24, cudaMemcpyDeviceToHost, x->stream));
+  if (n > n1)
+    FTRY(cudaMemcpyAsync(h.data() + 3 * n1, x->rec, (size_t)(n - n1) * 24, cudaMemcpyDeviceToHost, x->stream));
   FTRY(cudaStreamSynchronize(x->stream));
   if (int st = xyfix_status(x)) return st;
   for (int i = 0; i < n; ++i) {
-    const int64_t slot = (x->rec_count - n + i) % kFixRec;
-    if (E2) E2[i] = (int64_t)h[3 * slot];
-    if (Mx) Mx[i] = (int64_t)h[3 * slot + 1];
-    if (My) My[i] = (int64_t)h[3 * slot + 2];
+    if (E2) E2[i] = (int64_t)h[3 * i];
+    if (Mx) Mx[i] = (int64_t)h[3 * i + 1];
+    if (My) My[i] = (int64_t)h[3 * i + 2];
   }
   set_last_error("");
   return ISING_OK;
