@@ -187,38 +187,23 @@ __device__ __forceinline__ void lazy_planes(uint32_t g, uint32_t t, uint32_t rep
   }
 }
 
-// lazy_planes for two independent words at once (one warp vote for both; two
-// Philox chains in flight per thread).
-template <int B0, int B1>
-__device__ __forceinline__ void lazy_planes2(uint32_t ga, uint32_t gb, uint32_t t, uint32_t rep,
-                                             uint32_t colour, const RngParams& rng, uint32_t& Da,
-                                             uint32_t clsa, uint32_t& acca, uint32_t& Db,
-                                             uint32_t clsb, uint32_t& accb) {
+// Planes of blocks B0 .. 7 of one word by its lane alone, without warp votes: returns
+// the accepted lanes.  For the rare word that is still tied.
+template <int B0>
+__device__ __noinline__ uint32_t finish_word(uint32_t g, uint32_t t, uint32_t rep, uint32_t colour,
+                                             const RngParams& rng, uint32_t D, uint32_t cls) {
+  uint32_t acc = 0;
+  for (int b = B0; b < 8 && D != 0u; ++b) {
+    const uint4 r = philox10_rk(make_uint4(g, t, rep, ctr_w(kTagMet, colour, b)), rng.rk0, rng.rk1);
+    const uint32_t p[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-  for (int b = B0; b < B1; ++b) {
-    if (!__any_sync(0xffffffffu, (Da | Db) != 0u)) break;
-    const uint32_t cw = ctr_w(kTagMet, colour, b);
-    const uint4 ra = philox10_rk(make_uint4(ga, t, rep, cw), rng.rk0, rng.rk1);
-    const uint4 rb = philox10_rk(make_uint4(gb, t, rep, cw), rng.rk0, rng.rk1);
-    const uint32_t pa[4] = {ra.x, ra.y, ra.z, ra.w};
-    const uint32_t pb[4] = {rb.x, rb.y, rb.z, rb.w};
-    uint32_t bora = 0u, borb = 0u, eqa = Da, eqb = Db;
-#pragma unroll
-    for (int q = 3; q >= 0; --q) {
-      const int k = 4 * b + q;
-      const uint32_t m4 = rng.tm4[k], m8 = rng.tm8[k];
-      const uint32_t ta = (clsa & m4) | (~clsa & m8);
-      const uint32_t tb = (clsb & m4) | (~clsb & m8);
-      bora = (~pa[q] & ta) | (~pa[q] & bora) | (ta & bora);
-      borb = (~pb[q] & tb) | (~pb[q] & borb) | (tb & borb);
-      eqa &= ~(ta ^ pa[q]);
-      eqb &= ~(tb ^ pb[q]);
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t tm = (cls & rng.tm4[4 * b + q]) | (~cls & rng.tm8[4 * b + q]);
+      acc |= D & tm & ~p[q];
+      D &= ~(tm ^ p[q]);
     }
-    acca |= Da & bora;
-    accb |= Db & borb;
-    Da = eqa;
-    Db = eqb;
   }
+  return acc;
 }
 
 // Planes 0..7 (Philox blocks 0 and 1) of one or two words, all evaluated, as

@@ -21,7 +21,7 @@
 // with one thread per word.  Above, three blocks per word on the multiply pipe
 // (4 cycles per 32 x 32 -> 64 product and sub-partition).  Time per sweep, before
 // (launches per sweep or half sweep; int8: one CTA) and with strips: L = 64 int8
-// 16.4 -> 0.55 us, L = 256 8.3 -> 1.14, L = 1000 8.2 -> 1.9, L = 2048 21 -> 3.4.
+// 16.4 -> 0.55 us, L = 256 8.3 -> 1.04, L = 1000 8.2 -> 1.9, L = 2048 21 -> 3.4.
 #include "internal.h"
 #include "ising_device.cuh"
 
@@ -174,8 +174,15 @@ __global__ void __launch_bounds__(SPLIT ? kSplitThreads : kStripThreads) k_strip
           uint32_t D = ~k.ge2 & valid1;
           uint32_t acc = D & bor;
           D &= eq;
-          if (__any_sync(0xffffffffu, D != 0u))  // a tie over 16 planes: the other blocks
-            lazy_planes<4, 8>(g1, t, rng.replica, (uint32_t)c, rng, D, k.cls, acc);
+          // a tie over 16 planes (1 word in 2500): the other blocks.  By the lane alone
+          // (no vote: 1.14 -> 1.04 us per sweep at L = 256), in one CTA by vote (0.56 -> 0.53
+          // at L = 64)
+          if (WHOLE) {
+            if (__any_sync(0xffffffffu, D != 0u))
+              lazy_planes<4, 8>(g1, t, rng.replica, (uint32_t)c, rng, D, k.cls, acc);
+          } else if (D != 0u) {
+            acc |= finish_word<4>(g1, t, rng.replica, (uint32_t)c, rng, D, k.cls);
+          }
           const uint32_t ns = s ^ ((k.ge2 & valid1) | acc);
           own[c] = ns;
           if (mine_w && q == 0) So[i1] = ns;

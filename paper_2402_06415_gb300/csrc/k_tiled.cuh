@@ -146,24 +146,6 @@ __global__ void __launch_bounds__(256) k_tiled_bits(const uint32_t* __restrict__
     if (slots.slot[s] >= 0) block_add2(acc_anti[s], acc_ones[s], rec + 2 * (size_t)slots.slot[s]);
 }
 
-// Planes of blocks 2 .. 7 of one word by its lane alone (a full queue; not expected
-// at the automatic tile sizes): returns the accepted lanes.
-__device__ __noinline__ uint32_t finish_word(uint32_t g, uint32_t t, uint32_t rep, uint32_t colour,
-                                             const RngParams& rng, uint32_t D, uint32_t cls) {
-  uint32_t acc = 0;
-  for (int b = 2; b < 8 && D != 0u; ++b) {
-    const uint4 r = philox10_rk(make_uint4(g, t, rep, ctr_w(kTagMet, colour, b)), rng.rk0, rng.rk1);
-    const uint32_t p[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint32_t tm = (cls & rng.tm4[4 * b + q]) | (~cls & rng.tm8[4 * b + q]);
-      acc |= D & tm & ~p[q];
-      D &= ~(tm ^ p[q]);
-    }
-  }
-  return acc;
-}
-
 // Tiled sweep with one warp per 32-word tile row segment.  Same tiling, halo
 // and results as k_tiled_bits; differences are for speed only:
 //  * the inner 32*TWW words of a row are updated by TWW warps (lane = word), the
@@ -298,7 +280,7 @@ __global__ void __launch_bounds__(256, MINB) k_tiled32_bits(const uint32_t* __re
             if (slot < QCAP)
               q_ent[slot] = make_uint4((uint32_t)(r * SP + col), D, cls, g);
             else
-              So[r * SP + col] ^= finish_word(g, t, rng.replica, c, rng, D, cls);
+              So[r * SP + col] ^= finish_word<2>(g, t, rng.replica, c, rng, D, cls);
           }
         }
       };
@@ -344,8 +326,8 @@ __global__ void __launch_bounds__(256, MINB) k_tiled32_bits(const uint32_t* __re
             if (na) q_ent[slot] = make_uint4(pos, Da, ka.cls, ga);
             if (Db != 0u) q_ent[slot + na] = make_uint4(pos + SP, Db, kb.cls, gb);
           } else {
-            So[pos] ^= finish_word(ga, t, rng.replica, c, rng, Da, ka.cls);
-            So[pos + SP] ^= finish_word(gb, t, rng.replica, c, rng, Db, kb.cls);
+            So[pos] ^= finish_word<2>(ga, t, rng.replica, c, rng, Da, ka.cls);
+            So[pos + SP] ^= finish_word<2>(gb, t, rng.replica, c, rng, Db, kb.cls);
             // claimed entries below the capacity must not hold an old word
             for (int e = slot; e < QCAP && e < slot + na + (Db != 0u); ++e) q_ent[e] = make_uint4(0u, 0u, 0u, 0u);
           }
