@@ -20,7 +20,7 @@
 // (cluster_persist.cu) each site did.  Bound by the two grid barriers (~1.3 us each), the
 // dependent walks of the boundary forest and, for long strips, the shared-memory
 // unions.  us per SW step at beta_c, before (cluster_persist.cu up to L = 766, then
-// sw.cu) and now: L = 128 28 -> 13, 256 34 -> 22, 512 71 -> 31, 1024 134 -> 56.
+// sw.cu) and now: L = 128 28 -> 13, 256 34 -> 19, 512 71 -> 27, 1024 134 -> 51.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -57,15 +57,6 @@ struct ClusterStripArgs {
   FastDiv fL;
 };
 
-__device__ __forceinline__ uint32_t groot(uint32_t* parent, uint32_t a) {
-  while (true) {  // path halving stores only ancestors of a
-    const uint32_t p = __ldcg(&parent[a]);
-    if (p == a) return a;
-    const uint32_t gp = __ldcg(&parent[p]);
-    if (gp != p) __stcg(&parent[a], gp);
-    a = gp;
-  }
-}
 __device__ __forceinline__ uint32_t groot_ro(const uint32_t* parent, uint32_t a) {
   while (true) {
     const uint32_t p = __ldcg(&parent[a]);
@@ -73,10 +64,22 @@ __device__ __forceinline__ uint32_t groot_ro(const uint32_t* parent, uint32_t a)
     a = p;
   }
 }
+// Unions walk both trees in step (two loads in flight: 22 -> 19 us per step at L = 256,
+// 56 -> 51 at 1024) with path halving, which stores only ancestors, and link the larger
+// root below the smaller.
 __device__ __forceinline__ void gunite(uint32_t* parent, uint32_t a, uint32_t b) {
   while (true) {
-    a = groot(parent, a);
-    b = groot(parent, b);
+    uint32_t pa = __ldcg(&parent[a]), pb = __ldcg(&parent[b]);
+    while (pa != a || pb != b) {
+      if (pa == pb) return;
+      const uint32_t ga = __ldcg(&parent[pa]), gb = __ldcg(&parent[pb]);
+      if (ga != pa) __stcg(&parent[a], ga);
+      if (gb != pb) __stcg(&parent[b], gb);
+      a = ga;
+      b = gb;
+      pa = __ldcg(&parent[a]);
+      pb = __ldcg(&parent[b]);
+    }
     if (a == b) return;
     if (a < b) {
       const uint32_t t = a;
@@ -88,19 +91,20 @@ __device__ __forceinline__ void gunite(uint32_t* parent, uint32_t a, uint32_t b)
     a = old;
   }
 }
-__device__ __forceinline__ uint32_t lroot(volatile uint32_t* lab, uint32_t a) {
-  while (true) {
-    const uint32_t p = lab[a];
-    if (p == a) return a;
-    const uint32_t gp = lab[p];
-    if (gp != p) lab[a] = gp;
-    a = gp;
-  }
-}
 __device__ __forceinline__ void lunite(uint32_t* lab, uint32_t a, uint32_t b) {
+  volatile uint32_t* v = lab;
   while (true) {
-    a = lroot(lab, a);
-    b = lroot(lab, b);
+    uint32_t pa = v[a], pb = v[b];
+    while (pa != a || pb != b) {
+      if (pa == pb) return;
+      const uint32_t ga = v[pa], gb = v[pb];
+      if (ga != pa) v[a] = ga;
+      if (gb != pb) v[b] = gb;
+      a = ga;
+      b = gb;
+      pa = v[a];
+      pb = v[b];
+    }
     if (a == b) return;
     if (a < b) {
       const uint32_t t = a;
@@ -112,7 +116,6 @@ __device__ __forceinline__ void lunite(uint32_t* lab, uint32_t a, uint32_t b) {
     a = old;
   }
 }
-
 __device__ __forceinline__ uint32_t sroot16(uint16_t* par, uint32_t a) {
   volatile uint16_t* v = par;
   while (true) {
@@ -441,8 +444,8 @@ size_t zeroed_bytes(int L, int G) {  // boundary pairs, barrier flags, edge coun
 
 // Number of strips: more of them shorten the work inside a strip and lengthen the
 // boundary forest.  us per SW step at beta_c for 16 / 32 / 64 / 152 strips: L = 128 (SOLVE)
-// 13.0 / 16.5 / 23 / -, 256 33 / 23 / 22 / 25 (128), 384 60 / 39 / 27 / 28, 512 94 / 56 / 37 / 31,
-// 1024 - / 168 / 98 / 56.
+// 12.9 / 16.0 / 22.7 / -, 256 28.9 / 20.3 / 18.8 / 22.4 (128), 384 52 / 34 / 24.4 / 24.4, 512 82 / 50 /
+// 32 / 27, 1024 - / 151 / 88 / 51.
 int cluster_strip_grid(int L, int sms) {
   const int want = solves(L) ? 16 : L < 448 ? std::min(64, L / 4) : sms;
   const int G = std::min(std::min(want, sms), std::min(L / 2, kThreads));
