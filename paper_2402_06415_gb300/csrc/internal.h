@@ -132,7 +132,8 @@ cudaError_t launch_tiled32_sweep_bits(const BitsLattice& in, uint32_t* out, cons
 size_t tiled32_smem_bytes(int L, int k, int n_tile_rows, int tile_words);
 // Resident strips (k_strip.cu): n sweeps in one launch, in place, on packed
 // planes or int8 spins (the other pointer null).  G row strips, one CTA each
-// (cooperative launch; needs L >= 2 K G), K sweeps between exchanges.
+// (cooperative launch; needs L >= 2 K G), K sweeps between exchanges; K = 0: edge rows
+// exchanged every half sweep (needs L >= 2 G and 2 Wc <= kStripThreads).
 constexpr int kStripThreads = 512, kSplitThreads = 768;
 constexpr int kStripBlocks = 3;  // Philox blocks drawn for every word before the lazy ones
 struct StripArgs {

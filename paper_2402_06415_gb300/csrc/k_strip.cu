@@ -21,23 +21,31 @@
 // with one thread per word.  Above, three blocks per word on the multiply pipe
 // (4 cycles per 32 x 32 -> 64 product and sub-partition).  Time per sweep, before
 // (launches per sweep or half sweep; int8: one CTA) and with strips: L = 64 int8
-// 16.4 -> 0.55 us, L = 256 8.3 -> 1.04, L = 1000 8.2 -> 1.9, L = 2048 21 -> 3.4.
+// 16.4 -> 0.55 us, L = 256 8.3 -> 1.04, L = 1000 8.2 -> 1.85, L = 2048 21 -> 2.5 (k_strip_edge).
+#include <algorithm>
+
 #include "internal.h"
 #include "ising_device.cuh"
 
 namespace ising {
 namespace {
 
-// kBlocks Philox blocks (4 kBlocks planes) of a word as one strict comparison
+// NB Philox blocks (4 NB planes) of a word, and one strict comparison over them
 // (planes8 with a variable number of blocks).
 template <int NB>
-__device__ __forceinline__ void planes_first(uint32_t g, uint32_t t, uint32_t rep, uint32_t colour,
-                                             const RngParams& rng, uint32_t& D, uint32_t cls, uint32_t& acc) {
+__device__ __forceinline__ void draw_planes(uint4 (&pl)[NB], uint32_t g, uint32_t t, uint32_t rep, uint32_t colour,
+                                            const RngParams& rng) {
+#pragma unroll
+  for (int b = 0; b < NB; ++b)
+    pl[b] = philox10_rk(make_uint4(g, t, rep, ctr_w(kTagMet, colour, b)), rng.rk0, rng.rk1);
+}
+template <int NB>
+__device__ __forceinline__ void compare_planes(const uint4 (&pl)[NB], const RngParams& rng, uint32_t& D, uint32_t cls,
+                                               uint32_t& acc) {
   uint32_t bor = 0u, eq = D;
 #pragma unroll
   for (int b = NB - 1; b >= 0; --b) {
-    const uint4 r = philox10_rk(make_uint4(g, t, rep, ctr_w(kTagMet, colour, b)), rng.rk0, rng.rk1);
-    const uint32_t p[4] = {r.x, r.y, r.z, r.w};
+    const uint32_t p[4] = {pl[b].x, pl[b].y, pl[b].z, pl[b].w};
 #pragma unroll
     for (int q = 3; q >= 0; --q) {
       const int k = 4 * b + q;
@@ -48,6 +56,46 @@ __device__ __forceinline__ void planes_first(uint32_t g, uint32_t t, uint32_t re
   }
   acc |= D & bor;
   D = eq;
+}
+
+// Words of a strip's planes (P(c)[i] = word group_of(i) of colour c), and its own rows
+// back to the lattice.  With int8 spins a warp takes a word, lane j site j's byte.
+template <bool I8, typename Plane, typename Group>
+__device__ __forceinline__ void strip_load(const StripArgs& a, int n_words, Plane P, Group group_of) {
+  const int tid = threadIdx.x, nth = blockDim.x, L = a.L, Wc = a.Wc;
+  if (I8) {
+    for (int i = tid >> 5; i < 2 * n_words; i += nth >> 5) {
+      const int c = i >= n_words, g = group_of(i - c * n_words);
+      const int y = (int)fdiv((uint32_t)g, a.fwc), w = g - y * Wc;
+      const int j = 32 * w + (tid & 31);
+      const bool up = j < L / 2 && a.spins[(size_t)y * L + 2 * j + ((y + c) & 1)] > 0;
+      const uint32_t v = __ballot_sync(0xffffffffu, up);
+      if ((tid & 31) == 0) P(c)[i - c * n_words] = v;
+    }
+  } else {
+    for (int i = tid; i < 2 * n_words; i += nth) {
+      const int c = i >= n_words, k = i - c * n_words;
+      P(c)[k] = __ldcg(&a.planes[(size_t)c * L * Wc + group_of(k)]);
+    }
+  }
+}
+template <bool I8, typename Plane>
+__device__ __forceinline__ void strip_store(const StripArgs& a, int y0, int R, int off, Plane P) {
+  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, L = a.L, Wc = a.Wc, n = R * Wc;
+  if (I8) {
+    for (int i = tid >> 5; i < 2 * n; i += nth >> 5) {
+      const int c = i >= n, k = i - c * n;
+      const int r = (int)fdiv((uint32_t)k, a.fwc), w = k - r * Wc, y = y0 + r;
+      const uint32_t v = P(c)[off + k];
+      const int j = 32 * w + lane;
+      if (j < L / 2) a.spins[(size_t)y * L + 2 * j + ((y + c) & 1)] = (v >> lane) & 1u ? 1 : -1;
+    }
+  } else {
+    for (int i = tid; i < 2 * n; i += nth) {
+      const int c = i >= n, k = i - c * n;
+      a.planes[(size_t)c * L * Wc + (size_t)y0 * Wc + k] = P(c)[off + k];
+    }
+  }
 }
 
 template <bool WHOLE, bool I8, bool SPLIT>
@@ -73,22 +121,7 @@ __global__ void __launch_bounds__(SPLIT ? kSplitThreads : kStripThreads) k_strip
     }
     return g;
   };
-  if (I8) {
-    // one warp per word: lane j reads the site's byte
-    for (int i = tid >> 5; i < 2 * n_words; i += nth >> 5) {
-      const int c = i >= n_words, g = group_of(i - c * n_words);
-      const int y = (int)fdiv((uint32_t)g, a.fwc), w = g - y * Wc;
-      const int j = 32 * w + lane;
-      const bool up = j < n_half && a.spins[(size_t)y * L + 2 * j + ((y + c) & 1)] > 0;
-      const uint32_t v = __ballot_sync(0xffffffffu, up);
-      if (lane == 0) P(c)[i - c * n_words] = v;
-    }
-  } else {
-    for (int i = tid; i < 2 * n_words; i += nth) {
-      const int c = i >= n_words, k = i - c * n_words;
-      P(c)[k] = __ldcg(&a.planes[(size_t)c * LW + group_of(k)]);
-    }
-  }
+  strip_load<I8>(a, n_words, P, group_of);
   __syncthreads();
   // slots of this strip: 2 x 4 hw boundary pairs (two buffers used in turn), then
   // one "lattice read" token
@@ -237,7 +270,9 @@ __global__ void __launch_bounds__(SPLIT ? kSplitThreads : kStripThreads) k_strip
           const HalfClasses k = classify_hs(s, up ^ dn, up, dn, mid, side);
           uint32_t D = ~k.ge2 & valid, acc = 0;
           const uint32_t g = (uint32_t)group_of(i);
-          planes_first<kStripBlocks>(g, t, rng.replica, (uint32_t)c, rng, D, k.cls, acc);
+          uint4 p[kStripBlocks];
+          draw_planes(p, g, t, rng.replica, (uint32_t)c, rng);
+          compare_planes(p, rng, D, k.cls, acc);
           lazy_planes<kStripBlocks, 8>(g, t, rng.replica, (uint32_t)c, rng, D, k.cls, acc);
           const uint32_t ns = s ^ ((k.ge2 & valid) | acc);
           if (active) So[i] = ns;
@@ -296,44 +331,165 @@ __global__ void __launch_bounds__(SPLIT ? kSplitThreads : kStripThreads) k_strip
     if (tid < 2) ok = recv_word((tid ? dn_slots : up_slots) + 8 * hw, 1u, a.limit, a.status, word);
     if (!__syncthreads_and(ok)) return;
   }
-  if (I8) {
-    const int n = R * Wc;
-    for (int i = tid >> 5; i < 2 * n; i += nth >> 5) {
-      const int c = i >= n, k = i - c * n;
-      const int r = (int)fdiv((uint32_t)k, a.fwc), w = k - r * Wc, y = y0 + r;
-      const uint32_t v = P(c)[H * Wc + k];
-      const int j = 32 * w + lane;
-      if (j < n_half) a.spins[(size_t)y * L + 2 * j + ((y + c) & 1)] = (v >> lane) & 1u ? 1 : -1;
-    }
-  } else {
-    const int n = R * Wc;
-    for (int i = tid; i < 2 * n; i += nth) {
-      const int c = i >= n, k = i - c * n;
-      a.planes[(size_t)c * LW + (size_t)y0 * Wc + k] = P(c)[H * Wc + k];
+  strip_store<I8>(a, y0, R, H * Wc, P);
+}
+
+// Strips without a halo in shared memory, for rows long enough that a half sweep
+// takes about as long as an exchange: the first and the last row's words belong to
+// threads of their own, which send each new word and wait for the neighbour's one in a
+// register, while the other warps update the inner rows.  A half sweep then costs the
+// longer of the two instead of their sum, and no row is updated twice.  Every thread
+// draws the planes of its (first) word of the next half sweep ahead, edge warps once
+// they have sent; words beyond the CTA's threads are taken in a loop.  us per sweep,
+// k_strip -> here: L = 1300 2.32 -> 2.11, 2048 3.49 -> 2.49, 3072 5.7 -> 4.5, 4096 8.4 -> 7.4; with
+// the planes drawn before the wait 2048 took 2.63, drawn by all after the update 2.60.
+// Bound by the round trip of an edge word (0.85 us per half sweep) up to L ~ 1800, then
+// by the logic and multiply pipes.
+template <bool I8>
+__global__ void __launch_bounds__(kStripThreads) k_strip_edge(StripArgs a, RngParams rng) {
+  extern __shared__ uint32_t strip_smem[];
+  const int L = a.L, Wc = a.Wc, G = a.G, n_half = L / 2;
+  const int nb = n_half - 32 * (Wc - 1);                       // valid bits of a row's last word
+  const uint32_t last_mask = nb >= 32 ? 0xffffffffu : ((1u << nb) - 1u);
+  const int b = blockIdx.x, tid = threadIdx.x, nth = blockDim.x, lane = tid & 31;
+  const int y0 = (int)((long long)b * L / G), y1 = (int)((long long)(b + 1) * L / G);
+  const int R = y1 - y0, n_words = R * Wc;
+  const int plane = ((L + G - 1) / G) * Wc;
+  auto P = [plane](int c) { return strip_smem + c * plane; };
+  strip_load<I8>(a, n_words, P, [&](int i) { return y0 * Wc + i; });
+  // words in the order first row, last row, inner rows: row and index of the k-th
+  auto row_of = [&](int k, int& w) {
+    const int q = (int)fdiv((uint32_t)k, a.fwc);
+    w = k - q * Wc;
+    return q == 0 ? 0 : q == 1 ? R - 1 : q - 1;
+  };
+  const bool active1 = tid < n_words, edge = tid < 2 * Wc, top = tid < Wc;
+  const bool edge_warp = (tid & ~31) < 2 * Wc;
+  int w1;
+  const int r1 = row_of(active1 ? tid : 0, w1), i1 = r1 * Wc + w1;
+  const uint32_t g1 = (uint32_t)(y0 * Wc + i1);
+  // the neighbour's row that an edge word needs: colour 1 as the call found it
+  uint32_t beyond = 0;
+  if (edge) {
+    const int y = top ? (y0 == 0 ? L - 1 : y0 - 1) : (y1 == L ? 0 : y1);
+    if (I8) {
+      for (int j = 0; j < 32 && 32 * w1 + j < n_half; ++j)
+        beyond |= (uint32_t)(a.spins[(size_t)y * L + 2 * (32 * w1 + j) + ((y + 1) & 1)] > 0) << j;
+    } else {
+      beyond = __ldcg(&a.planes[(size_t)L * Wc + (size_t)y * Wc + w1]);
     }
   }
+  __syncthreads();
+  // slots: two buffers used in turn of 2 Wc pairs, first row and last row.  A strip writes
+  // one again only after it received what its neighbour sent having read it
+  unsigned long long* const mine = a.xbuf + (size_t)b * 4 * Wc + tid;
+  const unsigned long long* const theirs =
+      a.xbuf + (size_t)(top ? (b == 0 ? G - 1 : b - 1) : (b == G - 1 ? 0 : b + 1)) * 4 * Wc + (top ? Wc : 0) + w1;
+  uint32_t own[2] = {P(0)[i1], P(1)[i1]};
+  uint4 pl[kStripBlocks];
+  draw_planes(pl, g1, a.t0, rng.replica, 0u, rng);
+  uint32_t sent = 0;
+  int to_rec = a.to_rec;
+  long long slot = a.rec0;
+  for (int s2 = 0; s2 < a.n; ++s2) {
+    const uint32_t t = a.t0 + (uint32_t)s2;
+    const bool meas = to_rec == 1;
+    unsigned int anti = 0, ones = 0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      uint32_t* const So = P(c);
+      const uint32_t* const Sn = P(1 - c);
+      // word w of row r, index i; up / dn: the words above and below
+      auto update = [&](int w, int r, int i, bool active, uint32_t g, uint32_t s, uint32_t mid, uint32_t up,
+                        uint32_t dn, const uint4(&p)[kStripBlocks]) {
+        const bool first = w == 0, last = w == Wc - 1, left = ((y0 + r + c) & 1) == 0;
+        const uint32_t x = Sn[left ? (first ? i + Wc - 1 : i - 1) : (last ? i - Wc + 1 : i + 1)];
+        const uint32_t side = left ? (mid << 1) | ((x >> (first ? nb - 1 : 31)) & 1u)
+                                   : (mid >> 1) | ((x & 1u) << (last ? nb - 1 : 31));
+        const uint32_t valid = active ? (last ? last_mask : 0xffffffffu) : 0u;
+        const HalfClasses k = classify_hs(s, up ^ dn, up, dn, mid, side);
+        uint32_t D = ~k.ge2 & valid, acc = 0;
+        compare_planes(p, rng, D, k.cls, acc);
+        if (D != 0u) acc |= finish_word<kStripBlocks>(g, t, rng.replica, (uint32_t)c, rng, D, k.cls);
+        const uint32_t ns = s ^ ((k.ge2 & valid) | acc);
+        if (active) So[i] = ns;
+        if (c == 1 && meas) {
+          anti += __popc((ns ^ up) & valid) + __popc((ns ^ dn) & valid) + __popc((ns ^ mid) & valid) +
+                  __popc((ns ^ side) & valid);
+          ones += __popc(ns & valid) + __popc(mid & valid);
+        }
+        return ns;
+      };
+      // the next half sweep's planes: edge warps first wait, update and send
+      uint4 nx[kStripBlocks];
+      if (!edge_warp) draw_planes(nx, g1, t + (uint32_t)c, rng.replica, (uint32_t)(1 - c), rng);
+      bool ok = true;
+      if (edge && sent > 0)
+        ok = recv_word(theirs + (sent & 1 ? 2 * Wc : 0), sent, a.limit, a.status, beyond);
+      ++sent;
+      const uint32_t up = edge && top ? beyond : Sn[r1 == 0 ? i1 : i1 - Wc];
+      const uint32_t dn = edge && !top ? beyond : Sn[r1 == R - 1 ? i1 : i1 + Wc];
+      own[c] = update(w1, r1, i1, active1, g1, own[c], own[1 - c], up, dn, pl);
+      if (edge) send_word(mine + (sent & 1 ? 2 * Wc : 0), sent, own[c]);
+      if (edge_warp) draw_planes(nx, g1, t + (uint32_t)c, rng.replica, (uint32_t)(1 - c), rng);
+#pragma unroll
+      for (int j = 0; j < kStripBlocks; ++j) pl[j] = nx[j];
+      // the last warps, which have no edge words, first
+      for (int base = 2 * nth - 32 - (tid & ~31); base < n_words; base += nth) {
+        const bool active = base + lane < n_words;
+        int w;
+        const int r = row_of(active ? base + lane : 2 * Wc, w), i = r * Wc + w;
+        const uint32_t g = (uint32_t)(y0 * Wc + i);
+        uint4 p[kStripBlocks];
+        draw_planes(p, g, t, rng.replica, (uint32_t)c, rng);
+        update(w, r, i, active, g, So[i], Sn[i], Sn[i - Wc], Sn[i + Wc], p);
+      }
+      // (a plain barrier and a failure that is carried to the end: 2 to 7 % slower)
+      if (!__syncthreads_and(ok)) return;
+    }
+    if (meas) {
+      anti = __reduce_add_sync(0xffffffffu, anti);
+      ones = __reduce_add_sync(0xffffffffu, ones);
+      if (lane == 0 && (anti | ones)) {
+        atomicAdd(&a.rec[2 * slot], (unsigned long long)anti);
+        atomicAdd(&a.rec[2 * slot + 1], (unsigned long long)ones);
+      }
+    }
+    if (to_rec > 0 && --to_rec == 0) {
+      to_rec = a.m;
+      slot = slot + 1 == a.rec_cap ? 0 : slot + 1;
+    }
+  }
+  // in place: a neighbour's edge threads read this strip's rows before they sent the
+  // words that its own edge threads have received
+  strip_store<I8>(a, y0, R, 0, P);
 }
 
 }  // namespace
 
 size_t strip_smem_bytes(int L, int G, int K) {
   const int Wc = (L / 2 + 31) / 32;
-  const int H = G == 1 ? 0 : 2 * K;
+  const int H = G == 1 ? 0 : 2 * K;  // K = 0: k_strip_edge, no halo
   return 2ull * (size_t)((L + G - 1) / G + 2 * H) * (size_t)Wc * sizeof(uint32_t);
 }
 
 size_t strip_xbuf_words(int L, int G, int K) {
   const int Wc = (L / 2 + 31) / 32;
-  return G == 1 ? 0 : (size_t)G * (16 * (size_t)K * Wc + 1);
+  return G == 1 ? 0 : K == 0 ? (size_t)G * 4 * Wc : (size_t)G * (16 * (size_t)K * Wc + 1);
 }
 
 // Time model of one sweep in microseconds, fitted to sweeps of (G, K) on GB300
-// for L = 32 ... 8192 (within 15 %): per half sweep 0.10 + 0.085 us per resident
-// warp of an SM sub-partition with four threads per word (SPLIT), 0.45 + 0.25 us
-// with one, and 0.9 us per exchange.
+// for L = 32 ... 6144 (within 15 %): per half sweep 0.10 + 0.085 us per resident
+// warp of an SM sub-partition with four threads per word (SPLIT), 0.33 + 0.23 us
+// with one, and 0.9 us per exchange; without a halo (K = 0) the longer of 0.85 + 0.08 us
+// and 0.25 + 0.25 us per half sweep, and never below the other forms up to L ~ 900.
 static double strip_model_us(int L, int Wc, int G, int K) {
   const int R = (L + G - 1) / G;
   const bool whole = G == 1;
+  if (K == 0) {
+    const int wps = ((R * Wc + 31) / 32 + 3) / 4;
+    return 2 * std::max(0.85 + 0.08 * wps, 0.25 + 0.25 * wps);
+  }
   const int most = (R + (whole ? 0 : 4 * K - 2)) * Wc;
   double t = whole ? 0.0 : 0.9;
   if (4 * most <= kSplitThreads) {
@@ -342,7 +498,7 @@ static double strip_model_us(int L, int Wc, int G, int K) {
   } else {
     for (int h = 0; h < 2 * K; ++h) {
       const int words = (R + (whole ? 0 : 2 * (2 * K - 1 - h))) * Wc;
-      t += 0.45 + 0.25 * (((words + 31) / 32 + 3) / 4);
+      t += 0.33 + 0.23 * (((words + 31) / 32 + 3) / 4);
     }
   }
   return t / K;
@@ -352,7 +508,9 @@ StripShape choose_strip(int L, int sms) {
   const int Wc = (L / 2 + 31) / 32;
   StripShape best{0, 0, 1e30};
   for (int G = 1; G <= sms && G <= L / 2; ++G)
-    for (int K = 1; K <= (G == 1 ? 1 : kStripMaxK); ++K) {
+    for (int K = G == 1 ? 1 : 0; K <= (G == 1 ? 1 : kStripMaxK); ++K) {
+      // k_strip_edge: two rows at least, and a thread for each edge word
+      if (K == 0 && (L / G < 2 || 2 * Wc > kStripThreads)) continue;
       if (G > 1 && L / G < 2 * K) break;  // the halo comes from the next strip only
       if (strip_smem_bytes(L, G, K) > 200 * 1024) break;
       const double t = strip_model_us(L, Wc, G, K);
@@ -362,17 +520,19 @@ StripShape choose_strip(int L, int sms) {
 }
 
 cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, cudaStream_t s) {
-  const bool whole = a.G == 1, i8 = a.spins != nullptr;
+  const bool whole = a.G == 1, edge = a.K == 0, i8 = a.spins != nullptr;
   if (a.K > a.n) a.K = a.n;
   const size_t smem = strip_smem_bytes(a.L, a.G, a.K);
-  const int words = (int)(((a.L + a.G - 1) / a.G + (whole ? 0 : 4 * a.K - 2)) * (long long)a.Wc);
-  const bool split = 4 * words <= kSplitThreads;
-  const void* fns[8] = {(const void*)k_strip<false, false, false>, (const void*)k_strip<true, false, false>,
-                        (const void*)k_strip<false, true, false>,  (const void*)k_strip<true, true, false>,
-                        (const void*)k_strip<false, false, true>,  (const void*)k_strip<true, false, true>,
-                        (const void*)k_strip<false, true, true>,   (const void*)k_strip<true, true, true>};
-  const int which = (whole ? 1 : 0) + (i8 ? 2 : 0) + (split ? 4 : 0);
-  static DeviceCache configured[8];
+  const int words = (int)(((a.L + a.G - 1) / a.G + (whole || edge ? 0 : 4 * a.K - 2)) * (long long)a.Wc);
+  const bool split = !edge && 4 * words <= kSplitThreads;
+  const void* fns[10] = {(const void*)k_strip<false, false, false>, (const void*)k_strip<true, false, false>,
+                         (const void*)k_strip<false, true, false>,  (const void*)k_strip<true, true, false>,
+                         (const void*)k_strip<false, false, true>,  (const void*)k_strip<true, false, true>,
+                         (const void*)k_strip<false, true, true>,   (const void*)k_strip<true, true, true>,
+                         (const void*)k_strip_edge<false>, (const void*)k_strip_edge<true>};
+  a.fwc = make_fastdiv((uint32_t)a.Wc);
+  const int which = edge ? (i8 ? 9 : 8) : (whole ? 1 : 0) + (i8 ? 2 : 0) + (split ? 4 : 0);
+  static DeviceCache configured[10];
   if ((long long)smem > configured[which].get()) {
     cudaError_t e = cudaFuncSetAttribute(fns[which], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -381,7 +541,6 @@ cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, cudaStream_t s
   int threads = (((split ? 4 : 1) * words + 31) / 32) * 32;
   if (threads < 64) threads = 64;
   if (!split && threads > kStripThreads) threads = kStripThreads;
-  a.fwc = make_fastdiv((uint32_t)a.Wc);
   RngParams r = rng;
   void* args[] = {&a, &r};
   if (whole) return cudaLaunchKernel(fns[which], dim3(1), dim3(threads), args, smem, s);

@@ -43,6 +43,18 @@ def test_strips_equal_half_sweeps(L, layout):
         assert np.array_equal(a, b)
 
 
+# strips without a halo: one word a thread and a loop over more, edge words that share a warp with inner ones, ragged last
+# words, uneven strips, and calls of a single sweep (the first exchange only)
+@pytest.mark.parametrize("L", [900, 1300, 2046, 2306, 3074])
+@pytest.mark.parametrize("layout", [BITS, I8])
+def test_edge_strips_equal_half_sweeps(L, layout):
+    calls = [(1, 0), (1, 1), (3, 2), (10, 1)]
+    got = _run(L, 0.4406868, layout, calls)
+    ref = _run(L, 0.4406868, BITS, calls, ising.ISING_KERNEL_HALF)
+    for a, b in zip(got, ref):
+        assert np.array_equal(a, b)
+
+
 @pytest.mark.parametrize("L,beta", [(64, 0.9), (256, 0.05), (258, 0.6), (1026, 0.3)])
 def test_strips_equal_oracle(L, beta):
     ref = oracle.init(L, 40 + L)
