@@ -153,7 +153,7 @@ def tiled32_ctas_per_sm(L: int, k: int, n_ty: int, tile_words: int) -> int:
     of 1536 entries and sums + 1 KiB reserved per CTA), else 2 (the variant with up
     to 128 registers)."""
     ty_max = -(-L // n_ty)
-    per_cta = 2 * (ty_max + 4 * k) * (tile_words + 8) * 4 + (12 * 1536 + 16 + 16 * k) + 1024
+    per_cta = 2 * (ty_max + 4 * k) * (tile_words + 8) * 4 + (16 * 1536 + 16 + 16 * k) + 1024
     return 3 if 3 * per_cta <= 228 * 1024 else 2
 
 
