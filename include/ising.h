@@ -214,8 +214,9 @@ int ising_batch_create(ising_batch** out, int n_ladders, const int* L, int n_bet
  * identity slot assignment, zero counters, sweep counter 0.  Synchronises. */
 int ising_batch_seed(ising_batch* b, uint64_t seed);
 
-/* Work decomposition: replica words per work item (16..16384, default 512),
- * threads per CTA (32, 64, 128 or 256; 0 = 256), grid (0 = all resident CTAs).
+/* Work decomposition: replica words per work item (16..16384; until this call 256 or
+ * 512 by the batch's size), threads per CTA (32, 64, 128 or 256; 0 = 256; until this
+ * call 128), grid (0 = all resident CTAs).
  * Never changes results.  Drops a captured graph. */
 int ising_batch_set_kernel(ising_batch* b, int words_per_item, int threads, int grid);
 
@@ -489,7 +490,7 @@ int ising_xy_create(ising_xy** out, int L, double beta, int precision, void* str
 int ising_xy_seed(ising_xy* x, uint64_t seed);
 /* n_sweeps sweeps (async). */
 int ising_xy_sweep(ising_xy* x, int n_sweeps, int measure_every);
-/* Kernel form: 0 automatic (persistent for L <= 256), 1 one launch per half
+/* Kernel form: 0 automatic (one persistent launch per call for L <= 1024), 1 one launch per half
  * sweep, 2 persistent cooperative kernel (all CTAs co-resident, one launch per
  * ising_xy_sweep call, a bounded grid barrier between half sweeps).  Results
  * are identical in every mode.  If a persistent barrier gives up (after ~2 s)
