@@ -514,7 +514,10 @@ StripShape choose_strip(int L, int sms) {
       if (G > 1 && L / G < 2 * K) break;  // the halo comes from the next strip only
       if (strip_smem_bytes(L, G, K) > 200 * 1024) break;
       const double t = strip_model_us(L, Wc, G, K);
-      if (t < best.us) best = {G, G == 1 ? 1 << 30 : K, t};
+      // without a halo, equal warps a sub-partition: more strips from two warps on (us per sweep
+      // for 128 / 152 strips: L = 1000 1.78 / 1.85, 1600 2.27 / 2.17, 2048 2.58 / 2.49)
+      const bool finer = K == 0 && best.K == 0 && t == best.us && (L + G - 1) / G * Wc > 128;
+      if (t < best.us || finer) best = {G, G == 1 ? 1 << 30 : K, t};
     }
   return best;
 }
