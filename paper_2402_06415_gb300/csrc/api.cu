@@ -180,8 +180,8 @@ int check_ctx(ising_ctx* c) {
 
 // Where the resident strips are the automatic choice: everywhere they fit in
 // shared memory, except lattices from 6144 up that tile into 32-word tiles
-// (flips/ns, strips against the best tiled shape: L = 2048 1540 / 804, 4096
-// 2173 / 1997, 6144 2398 / 2717, 8192 2611 / 3094).  The other automatic paths
+// (flips/ns, strips against the best tiled shape: L = 2048 1635 / 804, 4096
+// 2241 / 2006, 6144 2398 / 2717, 8192 2611 / 3094).  The other automatic paths
 // there, one launch per half sweep or per sweep, gave 115 at L = 1000 and 200 at
 // L = 2048; one CTA with int8 spins 0.25 at L = 64 (strips: 7).
 bool strip_applies(int layout, int L) {
