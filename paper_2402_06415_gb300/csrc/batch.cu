@@ -114,7 +114,10 @@ __device__ __forceinline__ uint32_t valid_mask_bf(int w, int Wc, int n) {
   const uint32_t last = nb >= 32 ? 0xffffffffu : ((1u << (nb & 31)) - 1u);
   return w < Wc - 1 ? 0xffffffffu : last;
 }
-constexpr int kQueueCap = 512;  // undecided words per half sweep finished by whole warps
+// Undecided words finished by whole warps at a time, and the word pairs whose undecided
+// words the queue takes: at most 12 % of the words (a lane stays undecided with
+// probability 2^-8), so 483 of 4096 on average.
+constexpr int kQueueCap = 512, kQueuePairs = 2048;
 
 // Bit-plane compare of Philox blocks B0 .. B1-1 for the undecided lanes D of one
 // word, with the replica's per-plane threshold masks tm[k] = (all ones iff bit
@@ -248,25 +251,30 @@ __device__ void run_item(const BatchDev& d, int item, uint32_t t0, int ns, bool 
   // with every lane of a warp on one of them, instead of each warp waiting for
   // its slowest word.  (Warp-owned replicas with only __syncwarp() between half
   // sweeps measured slower: too few resident warps per SM for this many
-  // replicas.)
+  // replicas.)  Items of more than kQueuePairs pairs alternate between the phases,
+  // so that the queue does not fill: in one go, L = 1024 queued 1150 words and the lanes
+  // that found it full finished theirs alone (20 sweeps of
+  // 64 replicas in 256-thread CTAs 1684 -> 1230 us; L = 768 880 -> 713, L = 512, a single pass, 320 -> 325).
   // the warp's first thread through a shuffle: known to be uniform
   const int lane = threadIdx.x & 31, warp0 = __shfl_sync(0xffffffffu, (int)(threadIdx.x & ~31u), 0);
   const int words = nr * plane;
   const int half = plane / 2, pairs = nr * half;  // word pairs (rows 2 yy, 2 yy + 1)
   const FastDiv fwc = make_fastdiv((uint32_t)Wc);
   const FastDiv fhalf = make_fastdiv((uint32_t)half);
+  int cur = 0;  // queue counter in use (the other is reset meanwhile)
   for (int s = 0; s < ns; ++s) {
     const uint32_t t = t0 + (uint32_t)s;
-    for (int c = 0; c < 2; ++c) {
-      const int cur = c;  // queue counter of this half sweep (the other is reset meanwhile)
+    for (int c = 0; c < 2; ++c)
+    for (int p_lo = 0; p_lo < pairs; p_lo += kQueuePairs, cur ^= 1) {
+      const int p_hi = min(pairs, p_lo + kQueuePairs);
       // two vertically adjacent words of one replica per lane (rows 2 yy and
       // 2 yy + 1; L is even): they share the other colour's rows 2 yy, 2 yy + 1
       // as neighbours (and the half sum of that pair), the replica and the
       // index division, and their two Philox chains interleave; 80 registers
       // keep three CTAs of 256 threads per SM
-      for (int p0 = warp0; p0 < pairs; p0 += blockDim.x) {
+      for (int p0 = p_lo + warp0; p0 < p_hi; p0 += blockDim.x) {
         const int p = p0 + lane;
-        const bool act = p < pairs;
+        const bool act = p < p_hi;
         const int qq = act ? (int)fdiv((uint32_t)p, fhalf) : 0;
         const int rem = act ? p - qq * half : 0;
         const int yy = (int)fdiv((uint32_t)rem, fwc), w = rem - yy * Wc;
