@@ -214,9 +214,9 @@ int ising_batch_create(ising_batch** out, int n_ladders, const int* L, int n_bet
  * identity slot assignment, zero counters, sweep counter 0.  Synchronises. */
 int ising_batch_seed(ising_batch* b, uint64_t seed);
 
-/* Work decomposition: replica words per work item (16..16384; until this call 256 or
- * 512 by the batch's size), threads per CTA (32, 64, 128 or 256; 0 = 256; until this
- * call 128), grid (0 = all resident CTAs).
+/* Work decomposition: replica words per work item (16..16384), threads per CTA (32, 64,
+ * 128 or 256; 0 = 256), grid (0 = all resident CTAs).  Until this call 256 or 512 words
+ * and 128 or 256 threads, by a time model of the batch's replicas.
  * Never changes results.  Drops a captured graph. */
 int ising_batch_set_kernel(ising_batch* b, int words_per_item, int threads, int grid);
 

@@ -569,41 +569,45 @@ void bfree(ising_batch* b) {
 
 int words_per_replica(int L) { return 2 * L * ((L / 2 + 31) / 32); }
 
-// Items and their assignment to CTAs (largest first to the least loaded CTA).
-int plan_items(ising_batch* b) {
-  std::vector<int> il, ii0, inr;
-  std::vector<long long> cost;
+// Items of at most words_per_item words per colour plane (one replica at least), and
+// their assignment to CTAs (largest first to the least loaded CTA).
+struct ItemPlan {
+  std::vector<int> ladder, i0, nr;   // per item
+  std::vector<int> first, items;     // CSR over the CTAs
+  size_t smem = 0;
+  int grid = 0;
+  double cost = 0;  // of a half sweep, for the comparison of plans (choose_items)
+};
+
+int make_plan(const ising_batch* b, int words_per_item, int threads, ItemPlan* p) {
+  std::vector<long long> words;  // per colour plane
   for (int l = 0; l < b->n_ladders; ++l) {
-    const int per = words_per_replica(b->L[l]) / 2;  // words per colour plane
-    int nr = std::max(1, b->words_per_item / std::max(per, 1));
-    nr = std::min(nr, kMaxRepPerItem);
+    const int per = words_per_replica(b->L[l]) / 2;
+    const int nr = std::min(std::max(1, words_per_item / std::max(per, 1)), kMaxRepPerItem);
     for (int i0 = 0; i0 < b->n_beta; i0 += nr) {
       const int k = std::min(nr, b->n_beta - i0);
-      il.push_back(l);
-      ii0.push_back(i0);
-      inr.push_back(k);
-      cost.push_back((long long)k * per);
+      p->ladder.push_back(l);
+      p->i0.push_back(i0);
+      p->nr.push_back(k);
+      words.push_back((long long)k * per);
     }
   }
-  b->n_items = (int)il.size();
-  size_t max_words = 0;
-  for (int j = 0; j < b->n_items; ++j)
-    max_words = std::max(max_words, (size_t)inr[j] * words_per_replica(b->L[il[j]]));
-  b->smem = max_words * sizeof(uint32_t);
-  if (b->smem > 200 * 1024) return bfail(ISING_EINVAL, "an item needs %zu B of shared memory", b->smem);
-  BTRY(cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
+  const int n = (int)words.size();
+  p->smem = 2 * (size_t)*std::max_element(words.begin(), words.end()) * sizeof(uint32_t);
+  if (p->smem > 200 * 1024) return bfail(ISING_EINVAL, "an item needs %zu B of shared memory", p->smem);
+  BTRY(cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->smem));
   int dev = 0, sms = 0, per_sm = 0;
   BTRY(cudaGetDevice(&dev));
   BTRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  BTRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch, b->threads, b->smem));
+  BTRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch, threads, p->smem));
   if (per_sm < 1) return bfail(ISING_EINVAL, "kernel does not fit on an SM with this item size");
   int grid = per_sm * sms;
   if (b->grid > 0) grid = std::min(grid, b->grid);
-  grid = std::max(1, std::min(grid, std::max(b->n_items, b->n_ladders)));
-  b->grid_used = grid;
-  std::vector<int> order(b->n_items);
-  for (int j = 0; j < b->n_items; ++j) order[j] = j;
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[x] > cost[y]; });
+  grid = std::max(1, std::min(grid, std::max(n, b->n_ladders)));
+  p->grid = grid;
+  std::vector<int> order(n);
+  for (int j = 0; j < n; ++j) order[j] = j;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return words[x] > words[y]; });
   using P = std::pair<long long, int>;
   std::priority_queue<P, std::vector<P>, std::greater<P>> pq;
   for (int c = 0; c < grid; ++c) pq.push({0, c});
@@ -612,30 +616,63 @@ int plan_items(ising_batch* b) {
     P top = pq.top();
     pq.pop();
     per_cta[top.second].push_back(j);
-    pq.push({top.first + cost[j], top.second});
+    pq.push({top.first + words[j], top.second});
   }
-  std::vector<int> first(grid + 1, 0), items;
+  p->first.assign(grid + 1, 0);
+  double passes = 0;
   for (int c = 0; c < grid; ++c) {
-    first[c] = (int)items.size();
-    items.insert(items.end(), per_cta[c].begin(), per_cta[c].end());
+    p->first[c] = (int)p->items.size();
+    p->items.insert(p->items.end(), per_cta[c].begin(), per_cta[c].end());
+    double t = 0;
+    for (int j : per_cta[c]) t += std::max(0.5 * (double)words[j] / threads, 1.0);
+    passes = std::max(passes, t);
   }
-  first[grid] = (int)items.size();
-  cudaFree(b->d_item_l);
-  cudaFree(b->d_item_i0);
-  cudaFree(b->d_item_nr);
-  cudaFree(b->d_cta_first);
-  cudaFree(b->d_cta_items);
-  b->d_item_l = b->d_item_i0 = b->d_item_nr = b->d_cta_first = b->d_cta_items = nullptr;
-  if (int st = balloc(&b->d_item_l, il.size())) return st;
-  if (int st = balloc(&b->d_item_i0, il.size())) return st;
-  if (int st = balloc(&b->d_item_nr, il.size())) return st;
-  if (int st = balloc(&b->d_cta_first, first.size())) return st;
-  if (int st = balloc(&b->d_cta_items, items.size())) return st;
-  BTRY(cudaMemcpy(b->d_item_l, il.data(), il.size() * 4, cudaMemcpyHostToDevice));
-  BTRY(cudaMemcpy(b->d_item_i0, ii0.data(), ii0.size() * 4, cudaMemcpyHostToDevice));
-  BTRY(cudaMemcpy(b->d_item_nr, inr.data(), inr.size() * 4, cudaMemcpyHostToDevice));
-  BTRY(cudaMemcpy(b->d_cta_first, first.data(), first.size() * 4, cudaMemcpyHostToDevice));
-  BTRY(cudaMemcpy(b->d_cta_items, items.data(), items.size() * 4, cudaMemcpyHostToDevice));
+  p->first[grid] = (int)p->items.size();
+  p->cost = passes * (2.0 + (double)((grid + sms - 1) / sms) * threads / 128.0);
+  return ISING_OK;
+}
+
+// Default decomposition: of 256 or 512 words an item and 128 or 256 threads a CTA, the
+// pair with the least cost: passes over word pairs that the fullest CTA makes, times
+// the time of a pass, which grows with the warps that share an SM sub-partition (about
+// as 2 + warps).  Measured on 100 batches (L = 16 .. 1024, 4 .. 8192 replicas, one size and
+// mixed): 0.6 % above the best of the four on average, 3 % above it at the 90th
+// percentile.  us for 20 sweeps, (256, 128) / (256, 256) / (512, 128) / (512, 256): 4096 replicas of
+// 16 .. 128 squared 218 / 272 / 208 / 224, 8192 of 64 squared 337 / 349 / 402 / 341, 1024 of 128
+// squared 231 / 215 / 154 / 231, 64 of 256 squared 124 / 99 / 124 / 99, 64 of 1024 squared 1577 / 1124 /
+// 1578 / 1124: a replica is never split, so a large one wants the larger CTA.
+int choose_items(ising_batch* b) {
+  double best = 0;
+  for (int words : {256, 512})
+    for (int threads : {128, 256}) {
+      ItemPlan p;
+      if (int st = make_plan(b, words, threads, &p)) return st;
+      if (best == 0 || p.cost < best) {
+        best = p.cost;
+        b->words_per_item = words;
+        b->threads = threads;
+      }
+    }
+  return ISING_OK;
+}
+
+// Plans the items of the batch's decomposition and hands them to the device.
+int plan_items(ising_batch* b) {
+  ItemPlan p;
+  if (int st = make_plan(b, b->words_per_item, b->threads, &p)) return st;
+  b->n_items = (int)p.nr.size();
+  b->smem = p.smem;
+  b->grid_used = p.grid;
+  int** const dst[5] = {&b->d_item_l, &b->d_item_i0, &b->d_item_nr, &b->d_cta_first, &b->d_cta_items};
+  const std::vector<int>* const src[5] = {&p.ladder, &p.i0, &p.nr, &p.first, &p.items};
+  for (int** d : dst) {
+    cudaFree(*d);
+    *d = nullptr;
+  }
+  for (int k = 0; k < 5; ++k) {
+    if (int st = balloc(dst[k], src[k]->size())) return st;
+    BTRY(cudaMemcpy(*dst[k], src[k]->data(), src[k]->size() * sizeof(int), cudaMemcpyHostToDevice));
+  }
   return ISING_OK;
 }
 
@@ -769,19 +806,7 @@ int ising_batch_create(ising_batch** out, int n_ladders, const int* L, int n_bet
     if (!e) e = cudaMemset(b->d_ctr, 0, sizeof(BatchCounters));
     if (e) st = bfail(ISING_ECUDA, "batch setup copy: %s", cudaGetErrorString(e));
   }
-  if (!st) {
-    // Default decomposition: 128 threads a CTA (six per SM) and the smaller of 256 and
-    // 512 words per item that leaves at most one item per resident CTA.  flips/ns for
-    // (256, 128) / (512, 128) / (512, 256) words and threads: 12.7 k words per colour
-    // plane in all 228 / 161 / 194, 83 k 1033 / 836 / 871, 166 k 1569 / 1349 / 1378, 331 k
-    // 1616 / 1922 / 1587.
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e) st = bfail(ISING_ECUDA, "device query: %s", cudaGetErrorString(e));
-    b->threads = 128;
-    b->words_per_item = o / 2 <= 256LL * 6 * sms ? 256 : 512;
-  }
+  if (!st) st = choose_items(b);
   if (!st) st = plan_items(b);
   if (st) {
     bfree(b);

@@ -72,3 +72,21 @@ def test_cold_replicas_cost_no_more_than_the_words_they_queue():
             b.run(200)  # domains
             ms.append(_ms(b, 120) - _ms(b, 20))
     assert ms[1] < 1.25 * ms[0], ms
+
+
+# one replica an SM, three, a few items more than CTAs of either size, uneven replicas
+@pytest.mark.parametrize("Ls", [[256] * 64, [512] * 64, [1024] * 64, [256] * 456, [64] * 8192, [96] * 1024, [64, 512] * 16,
+                                [16, 32, 64, 128, 256] * 64])
+def test_default_decomposition_loses_to_no_other(Ls):
+    """The automatic decomposition is within 15 % of every one it chooses from (a fixed 128 threads a CTA took 1.2 to
+    1.6 times as long on replicas above 128 x 128)."""
+    import torch
+
+    with ising.Batch(Ls, [0.44], 10, stream=torch.cuda.current_stream(), seed=5) as b:
+        auto = _ms(b, 20)
+        other = {}
+        for words in (256, 512):
+            for threads in (128, 256):
+                ising.ising_batch_set_kernel(b.h, words, threads)
+                other[words, threads] = _ms(b, 20)
+    assert auto < 1.15 * min(other.values()), (auto, other)
