@@ -4,8 +4,11 @@ Searches the kernel choice and its shape (sweeps per launch k, number of row
 strips, words per tile row) for one lattice size on the current GPU, timing
 each candidate with CUDA events on the lattice's stream after a warm-up.  The
 choice never changes results (every configuration is bit-identical), only
-speed.  Results are cached as JSON keyed by (GPU name, SM count, L, layout) in
-``$ISING_TUNE_CACHE`` or ``~/.cache/ising_gb300/tune.json``.
+speed.  Unless the caller names the candidates, the library's own choice (AUTO) is
+timed beside them: the resident strips, which are what AUTO runs on lattices below
+6144, have no shape to search.  Results are cached as JSON keyed by (version of the
+candidates, GPU name, SM count, L, layout) in ``$ISING_TUNE_CACHE`` or
+``~/.cache/ising_gb300/tune.json``.
 """
 from __future__ import annotations
 
@@ -14,6 +17,9 @@ import os
 import time
 
 from . import _binding as B
+
+# raised when kernels or candidates change, so that older answers are timed again
+_VERSION = 2
 
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "ising_gb300", "tune.json")
 
@@ -26,7 +32,7 @@ def _key(L: int, layout: int) -> str:
     import torch
 
     p = torch.cuda.get_device_properties(torch.cuda.current_device())
-    return "%s|%d|L=%d|layout=%d" % (p.name, p.multi_processor_count, L, layout)
+    return "v%d|%s|%d|L=%d|layout=%d" % (_VERSION, p.name, p.multi_processor_count, L, layout)
 
 
 def candidates(L: int, sms: int = 152) -> list[dict]:
@@ -91,7 +97,8 @@ def tune(L: int, beta: float = 0.4406868, sweeps: int = 24, reps: int = 3,
         if key in cache:
             return cache[key]
     sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-    cands = cands if cands is not None else candidates(L, sms)
+    if cands is None:
+        cands = [{"kernel": B.ISING_KERNEL_AUTO, "k": 1, "tile_rows": 1, "tile_words": 4}] + candidates(L, sms)
     table = []
     t0 = time.time()
     with B.Lattice(L, beta, B.ISING_LAYOUT_BITS, stream=torch.cuda.current_stream(),
@@ -126,8 +133,8 @@ def tune_batch(Ls, betas, pt_every: int, sweeps: int = 100, reps: int = 2,
     import numpy as np
     import torch
 
-    key = "batch|%s|%d|nL=%d|Lsum=%d|nb=%d|pt=%d" % (
-        torch.cuda.get_device_properties(torch.cuda.current_device()).name,
+    key = "v%d|batch|%s|%d|nL=%d|Lsum=%d|nb=%d|pt=%d" % (
+        _VERSION, torch.cuda.get_device_properties(torch.cuda.current_device()).name,
         torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count,
         len(Ls), int(np.sum(np.asarray(Ls) ** 2)), len(betas), pt_every)
     path = _cache_path()
