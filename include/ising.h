@@ -59,10 +59,14 @@ typedef enum {
 typedef enum { ISING_LAYOUT_I8 = 0, ISING_LAYOUT_BITS = 1 } ising_layout;
 
 typedef enum {
-  ISING_KERNEL_AUTO = 0,     /* pick per lattice (tiled if it applies, else half) */
+  ISING_KERNEL_AUTO = 0,     /* pick per lattice: strips, except tiled from L = 6144 where 32-word
+                                tiles fit; where strips do not fit tiled, else half (packed),
+                                resident, else half (int8) */
   ISING_KERNEL_HALF = 1,     /* one launch per half sweep, spins in global memory */
   ISING_KERNEL_TILED = 2,    /* packed layout: shared-memory tile + halo, k sweeps per launch */
-  ISING_KERNEL_RESIDENT = 3  /* int8 layout: whole lattice in one CTA's shared memory */
+  ISING_KERNEL_RESIDENT = 3, /* int8 layout: whole lattice in one CTA's shared memory */
+  ISING_KERNEL_STRIP = 4     /* row strips resident in the SMs' shared memory for all sweeps of a
+                                call, either layout, up to what 200 KiB per strip hold */
 } ising_kernel;
 
 /* Create a context for one L x L lattice (Results A; the sweep of Fig. 2b).
@@ -137,12 +141,15 @@ int ising_words_per_row(int L);
  * sweeps_per_launch k (tiled: 1..8), tile_rows = number of row strips the
  * lattice is cut into (tiled), tile_words = words per tile row (tiled; must
  * divide Wc and be a multiple of 4), grid/block: launch shape (0 = default).
+ * The strips' shape is chosen by the library, whatever is passed.
  * The choice never changes results, only speed.  EINVAL if the kernel does
  * not apply to this lattice/layout. */
 int ising_set_kernel(ising_ctx* ctx, int kernel, int sweeps_per_launch, int tile_rows,
                      int tile_words, int grid, int block);
 
-/* The kernel configuration in use (after AUTO resolution). */
+/* The kernel configuration in use (after AUTO resolution); ising_set_kernel takes it back.
+ * Strips: tile_rows = number of strips, sweeps_per_launch = sweeps between exchanges of
+ * boundary rows (0: one strip, or an exchange every half sweep), tile_words = 0. */
 int ising_get_kernel(ising_ctx* ctx, int* kernel, int* sweeps_per_launch, int* tile_rows,
                      int* tile_words, int* grid, int* block);
 

@@ -40,6 +40,7 @@ ISING_KERNEL_AUTO = 0
 ISING_KERNEL_HALF = 1
 ISING_KERNEL_TILED = 2
 ISING_KERNEL_RESIDENT = 3
+ISING_KERNEL_STRIP = 4
 
 _STATUS_NAMES = {0: "OK", -1: "EINVAL", -2: "ENOMEM", -3: "ECUDA", -4: "ETIMEOUT",
                  -5: "EINTERNAL"}

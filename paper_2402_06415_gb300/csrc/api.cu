@@ -231,14 +231,20 @@ int ensure_strip_status(ising_ctx* c) {
   return ISING_OK;
 }
 
+// Strips of this lattice: the automatic choice, or wherever they fit.
+StripShape strip_shape(const ising_ctx* c, bool automatic) {
+  return !automatic || strip_applies(c->layout, c->L) ? choose_strip(c->L, c->sms) : StripShape{0, 0, 0.0};
+}
+
 // Buffers of the strips' boundary exchange, once per context.
-int ensure_strip(ising_ctx* c) {
-  if (c->strip.G <= 1 || c->strip_x) return ISING_OK;
+int ensure_strip(ising_ctx* c, const StripShape& shape) {
+  if (shape.G <= 1) return ISING_OK;
+  if (int st = ensure_strip_status(c)) return st;
+  if (c->strip_x) return ISING_OK;
   void* p = nullptr;
-  int st = dev_alloc(&p, strip_xbuf_words(c->L, c->strip.G, c->strip.K) * sizeof(unsigned long long));
-  if (st) return st;
+  int st = dev_alloc(&p, strip_xbuf_words(c->L, shape.G, shape.K) * sizeof(unsigned long long));
   c->strip_x = (unsigned long long*)p;
-  return ensure_strip_status(c);
+  return st;
 }
 
 // 32-word tiles, four sweeps per launch, and the number of row strips that gives
@@ -269,7 +275,7 @@ void auto_tiles32(ising_ctx* c) {
 }
 
 void resolve_auto(ising_ctx* c) {
-  c->strip = strip_applies(c->layout, c->L) ? choose_strip(c->L, c->sms) : StripShape{0, 0, 0.0};
+  c->strip = strip_shape(c, true);
   if (c->layout == ISING_LAYOUT_BITS) {
     if (c->Wc % 4 == 0 && c->L % 64 == 0 && c->L >= 256) {
       c->kernel = ISING_KERNEL_TILED;
@@ -525,7 +531,7 @@ int ising_create(ising_ctx** out, int L, double beta, int layout, void* stream) 
   }
   if (!st) {
     resolve_auto(c);
-    st = ensure_strip(c);
+    st = ensure_strip(c, c->strip);
     if (!st && c->kernel == ISING_KERNEL_TILED && c->strip.G == 0) st = ensure_second_buffer(c);
   }
   if (!st) {
@@ -829,9 +835,13 @@ int ising_set_kernel(ising_ctx* c, int kernel, int k, int tile_rows, int tile_wo
   if (int st = check_ctx(c)) return st;
   if (grid < 0 || block < 0 || (block && (block % 32 != 0 || block > 1024)))
     return fail(ISING_EINVAL, "grid must be >= 0 and block a multiple of 32 in [32, 1024]");
-  if (kernel == ISING_KERNEL_AUTO) {
+  if (kernel == ISING_KERNEL_AUTO || kernel == ISING_KERNEL_STRIP) {
+    const StripShape shape = strip_shape(c, kernel == ISING_KERNEL_AUTO);
+    if (kernel == ISING_KERNEL_STRIP && shape.G == 0)
+      return fail(ISING_EINVAL, "no strips of an L = %d lattice fit in shared memory", c->L);
+    if (int st = ensure_strip(c, shape)) return st;  // before anything changes
     resolve_auto(c);
-    if (int st = ensure_strip(c)) return st;
+    c->strip = shape;
     if (c->kernel == ISING_KERNEL_TILED && c->strip.G == 0)
       if (int st = ensure_second_buffer(c)) return st;
     return ok();
@@ -854,10 +864,11 @@ int ising_set_kernel(ising_ctx* c, int kernel, int k, int tile_rows, int tile_wo
 int ising_get_kernel(ising_ctx* c, int* kernel, int* k, int* tile_rows, int* tile_words,
                      int* grid, int* block) {
   if (int st = check_ctx(c)) return st;
-  if (kernel) *kernel = c->kernel;
-  if (k) *k = c->k;
-  if (tile_rows) *tile_rows = c->tile_rows;
-  if (tile_words) *tile_words = c->tile_words;
+  const bool strip = c->strip.G > 0;
+  if (kernel) *kernel = strip ? ISING_KERNEL_STRIP : c->kernel;
+  if (k) *k = !strip ? c->k : c->strip.G > 1 ? c->strip.K : 0;
+  if (tile_rows) *tile_rows = strip ? c->strip.G : c->tile_rows;
+  if (tile_words) *tile_words = strip ? 0 : c->tile_words;
   if (grid) *grid = c->grid;
   if (block) *block = c->block;
   return ok();
