@@ -104,7 +104,11 @@ int ising_get_state(ising_ctx* ctx, uint64_t* seed, uint32_t* replica, int64_t* 
  * starting at the current sweep counter t.  After every sweep t with
  * (t + 1) % measure_every == 0 the energy E = -sum s s' (2 L^2 bonds) and
  * magnetisation M = sum s are recorded (measure_every = 0: no records).
- * n_sweeps >= 0, measure_every >= 0, t + n_sweeps < 2^32.  Async. */
+ * n_sweeps >= 0, measure_every >= 0, t + n_sweeps < 2^32.  Async.
+ * Strips (ISING_KERNEL_STRIP) wait for each other's boundary rows; a wait gives up after
+ * about 2 s, and synchronising calls then fail with ISING_ETIMEOUT.  The lattice and the
+ * records of that call and of work queued after it are undefined until ising_seed,
+ * ising_set_spins or ising_set_bits (or their device forms) sets the lattice again. */
 int ising_sweep(ising_ctx* ctx, int n_sweeps, int measure_every);
 
 /* E and M of the current configuration.  Synchronises the stream. */
@@ -501,7 +505,9 @@ int ising_xy_sweep(ising_xy* x, int n_sweeps, int measure_every);
  * sweep, 2 persistent cooperative kernel (all CTAs co-resident, one launch per
  * ising_xy_sweep call, a bounded grid barrier between half sweeps).  Results
  * are identical in every mode.  If a persistent barrier gives up (after ~2 s)
- * the next synchronising call returns ISING_ETIMEOUT until ising_xy_seed. */
+ * or a wait of the automatic form's strips does, synchronising calls return
+ * ISING_ETIMEOUT, and the lattice and its records are undefined, until ising_xy_seed or
+ * ising_xy_set_spins. */
 int ising_xy_set_mode(ising_xy* x, int mode);
 /* Kernels this context has launched. */
 int ising_xy_launch_count(ising_xy* x, int64_t* count);
@@ -586,7 +592,9 @@ int ising_quad_create(ising_quad** out, int lattice, int Lc, double beta, double
 int ising_quad_seed(ising_quad* x, uint64_t seed);
 /* Replica id of the counter map; re-seeds with the current seed. */
 int ising_quad_set_replica(ising_quad* x, uint32_t replica);
-/* n_sweeps sweeps (async). */
+/* n_sweeps sweeps (async).  As in ising_sweep a wait between strips may give up:
+ * synchronising calls then return ISING_ETIMEOUT until ising_quad_seed or
+ * ising_quad_set_spins. */
 int ising_quad_sweep(ising_quad* x, int n_sweeps, int measure_every);
 /* Last n records, oldest first (host arrays; any may be NULL).  Synchronises. */
 int ising_quad_series(ising_quad* x, int64_t* B1, int64_t* B2, int64_t* M, int n);

@@ -39,14 +39,6 @@ int ok() {
   return ISING_OK;
 }
 
-// Host-side fault injection for the failure-path tests: ISING_FAULT=alloc
-// makes device allocations fail, ISING_FAULT=launch makes sweep launches fail,
-// ISING_FAULT=copy makes host<->device copies fail.  Never touches the GPU.
-bool fault(const char* what) {
-  const char* f = std::getenv("ISING_FAULT");
-  return f && std::strstr(f, what) != nullptr;
-}
-
 #define CUDA_TRY(expr)                                                                   \
   do {                                                                                   \
     cudaError_t e__ = (expr);                                                            \
@@ -87,7 +79,7 @@ struct ising_ctx {
   // resident strips (the automatic choice where they are the fastest; G = 0: not used)
   StripShape strip{0, 0, 0.0};
   unsigned long long* strip_x = nullptr;  // boundary exchange buffer (G > 1)
-  int* strip_status = nullptr;            // pinned host word a strip sets when a wait gave up
+  StripStatus strip_status;
   int kernel = ISING_KERNEL_HALF, k = 1, tile_rows = 1, tile_words = 4, grid = 0, block = 0;
   __nv_bfloat16* nn_w = nullptr;    // BF16 weights of the block proposal
   __nv_bfloat16* nn_w2t = nullptr;
@@ -143,9 +135,8 @@ void free_all(ising_ctx* c) {
   cudaFree(c->rec);
   cudaFree(c->meas);
   cudaFree(c->strip_x);
-  cudaFreeHost(c->strip_status);
   c->strip_x = nullptr;
-  c->strip_status = nullptr;
+  c->strip_status.release();
   cudaFree(c->nn_w);
   cudaFree(c->nn_w2t);
   cudaFree(c->blk_stats);
@@ -221,13 +212,11 @@ int validate_kernel(const ising_ctx* c, int kernel, int k, int tile_rows, int ti
 }
 
 int ensure_strip_status(ising_ctx* c) {
-  if (c->strip_status) return ISING_OK;
-  cudaError_t e = cudaHostAlloc((void**)&c->strip_status, sizeof(int), cudaHostAllocDefault);
+  cudaError_t e = c->strip_status.ensure();
   if (e != cudaSuccess) {
-    c->strip_status = nullptr;
+    cudaGetLastError();
     return fail(ISING_ENOMEM, "pinned status word: %s", cudaGetErrorString(e));
   }
-  *c->strip_status = 0;
   return ISING_OK;
 }
 
@@ -392,8 +381,8 @@ int sweep_chunk(ising_ctx* c, int64_t t0, int n, int m) {
     a.rec_cap = kRecCap;
     a.rec = c->rec;
     a.xbuf = c->strip_x;
-    a.status = c->strip_status;
-    a.limit = kClusterSpinLimit;
+    a.status = c->strip_status.wait();
+    a.limit = fault("wait") ? -1 : kClusterSpinLimit;
     if (int st = launch_result(c, launch_strip_sweep(a, rng, c->stream), "strip sweep")) return st;
   } else if (c->layout == ISING_LAYOUT_BITS && c->kernel == ISING_KERNEL_HALF) {
     for (int64_t t = t0; t < t0 + n; ++t) {
@@ -450,14 +439,21 @@ int to_host_sync(ising_ctx* c, void* dst, const void* src, size_t bytes) {
   if (fault("copy")) return fail(ISING_ECUDA, "device-to-host copy failed (injected)");
   CUDA_TRY(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(cudaStreamSynchronize(c->stream));
-  if (c->strip_status && *(volatile int*)c->strip_status)
+  if (c->strip_status.failed())
     return fail(ISING_ETIMEOUT, "a strip's wait for its neighbour timed out");
   if (c->cluster_gctl) {
-    // a grid barrier of the persistent cluster kernel that gave up stays recorded until the next seed
+    // a grid barrier of the persistent cluster kernel that gave up stays recorded until the lattice is set again
     int status = 0;
     CUDA_TRY(cudaMemcpy(&status, &c->cluster_gctl->status, sizeof(int), cudaMemcpyDeviceToHost));
     if (status) return fail(ISING_ETIMEOUT, "grid barrier timed out in the persistent cluster kernel");
   }
+  return ISING_OK;
+}
+
+// The whole lattice is about to be written: a wait that gave up before no longer matters.
+int lattice_defined(ising_ctx* c) {
+  ++c->strip_status.epoch;
+  if (c->cluster_gctl) CUDA_TRY(cudaMemsetAsync(c->cluster_gctl, 0, sizeof(GridCtl), c->stream));
   return ISING_OK;
 }
 
@@ -472,6 +468,15 @@ int to_device_sync(ising_ctx* c, void* dst, const void* src, size_t bytes) {
 
 namespace ising {
 void set_last_error(const char* msg) { g_err = msg ? msg : ""; }
+
+// Fault injection for the failure-path tests: ISING_FAULT=alloc makes device allocations
+// fail, ISING_FAULT=launch sweep launches, ISING_FAULT=copy host<->device copies, all
+// without touching the GPU; ISING_FAULT=wait gives strips no time for a wait that is
+// not over at once (they set the status and return).
+bool fault(const char* what) {
+  const char* f = std::getenv("ISING_FAULT");
+  return f && std::strstr(f, what) != nullptr;
+}
 }  // namespace ising
 
 extern "C" {
@@ -568,14 +573,10 @@ int ising_seed(ising_ctx* c, uint64_t seed) {
   c->rec_count = 0;
   c->sw_steps = 0;
   c->wolff_steps = 0;
-  if (c->strip_status) *c->strip_status = 0;
+  if (int st = lattice_defined(c)) return st;
   cudaError_t e;
   if (c->wolff) {
     e = cudaMemsetAsync(c->wolff, 0, sizeof(WolffCtl), c->stream);
-    if (e) return fail(ISING_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
-  }
-  if (c->cluster_gctl) {
-    e = cudaMemsetAsync(c->cluster_gctl, 0, sizeof(GridCtl), c->stream);
     if (e) return fail(ISING_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
   }
   if (c->layout == ISING_LAYOUT_BITS) {
@@ -694,6 +695,7 @@ static int get_spins_dev(ising_ctx* c, int8_t* dst) {
 }
 
 static int set_spins_dev(ising_ctx* c, const int8_t* src) {
+  if (int st = lattice_defined(c)) return st;
   if (c->layout == ISING_LAYOUT_I8) {
     CUDA_TRY(cudaMemcpyAsync(c->spins, src, (size_t)c->N(), cudaMemcpyDeviceToDevice, c->stream));
     return ISING_OK;
@@ -712,6 +714,7 @@ static int get_bits_dev(ising_ctx* c, uint32_t* dst) {
 }
 
 static int set_bits_dev(ising_ctx* c, const uint32_t* src) {
+  if (int st = lattice_defined(c)) return st;
   if (c->layout == ISING_LAYOUT_BITS) {
     CUDA_TRY(cudaMemcpyAsync(c->bits[c->cur], src, c->plane_words() * 4, cudaMemcpyDeviceToDevice,
                              c->stream));
@@ -771,6 +774,7 @@ int ising_set_spins(ising_ctx* c, const int8_t* host_in) {
     if (host_in[i] != 1 && host_in[i] != -1)
       return fail(ISING_EINVAL, "spin %lld is %d, not +-1", (long long)i, (int)host_in[i]);
   if (c->layout == ISING_LAYOUT_I8) {
+    if (int st = lattice_defined(c)) return st;
     if (int st = to_device_sync(c, c->spins, host_in, (size_t)c->N())) return st;
     return ok();
   }
@@ -815,6 +819,7 @@ int ising_set_bits(ising_ctx* c, const uint32_t* host_in) {
     src = masked.data();
   }
   if (c->layout == ISING_LAYOUT_BITS) {
+    if (int st = lattice_defined(c)) return st;
     if (int st = to_device_sync(c, c->bits[c->cur], src, c->plane_words() * 4)) return st;
     return ok();
   }
@@ -1037,7 +1042,7 @@ int cluster_persist_run(ising_ctx* c, bool wolff, int64_t step0, int n, int meas
       cudaError_t e = launch_cluster_strip(c->lat(c->cur), wolff, (uint32_t)t, k, measure_every,
                                            n_rec ? (int)((before + 1) * m - t) : 0, bond_threshold(c->beta), c->rng(),
                                            G, c->cluster_strip, c->rec, c->rec_count % kRecCap, kRecCap, c->wolff,
-                                           c->strip_status, c->stream);
+                                           c->strip_status.wait(), c->stream);
       if (int st = launch_result(c, e, "cluster strips")) return st;
       c->rec_count += n_rec;
       done += k;

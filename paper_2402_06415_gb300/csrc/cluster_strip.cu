@@ -52,7 +52,7 @@ struct ClusterStripArgs {
   unsigned int* flags;
   unsigned int* n_edges;
   WolffCtl* wctl;
-  int* status;
+  WaitStatus status;
   long long limit;
   FastDiv fL;
 };
@@ -145,9 +145,9 @@ __device__ __forceinline__ void sunite16(uint16_t* par, uint32_t a, uint32_t b) 
 // Grid barrier of up to kThreads CTAs, all resident: every CTA raises its flag and
 // polls everybody's, one thread per CTA, so it takes one store and one load through
 // L2 instead of an atomic, its answer and a load.  False after `limit` cycles
-// (and *status = 1).
+// (and the status set).
 __device__ __forceinline__ bool flag_barrier(unsigned int* flags, int G, unsigned int epoch, long long limit,
-                                             int* status) {
+                                             const WaitStatus& status) {
   __syncthreads();
   const int tid = threadIdx.x;
   if (tid == 0) {
@@ -159,7 +159,7 @@ __device__ __forceinline__ bool flag_barrier(unsigned int* flags, int G, unsigne
     const long long start = clock64();
     while (ld_acquire_gpu(flags + tid) < epoch) {
       if (clock64() - start > limit) {
-        *reinterpret_cast<volatile int*>(status) = 1;
+        gave_up(status);
         ok = false;
         break;
       }
@@ -460,7 +460,7 @@ size_t cluster_strip_bytes(int L, int G) {
 cudaError_t launch_cluster_strip(const BitsLattice& lat, bool wolff, uint32_t step0, int n_steps, int measure_every,
                                  int to_rec, uint32_t thr, const RngParams& rng, int G, void* scratch,
                                  unsigned long long* rec, long long rec0, long long rec_cap, WolffCtl* wctl,
-                                 int* status, cudaStream_t s) {
+                                 const WaitStatus& status, cudaStream_t s) {
   ClusterStripArgs a{};
   a.planes = lat.planes;
   a.L = lat.L;
@@ -484,7 +484,7 @@ cudaError_t launch_cluster_strip(const BitsLattice& lat, bool wolff, uint32_t st
   a.n_edges = a.flags + G;
   a.wctl = wctl;
   a.status = status;
-  a.limit = kClusterSpinLimit;
+  a.limit = fault("wait") ? -1 : kClusterSpinLimit;
   a.fL = make_fastdiv((uint32_t)a.L);
   const size_t smem = strip_smem(a.L, G);
   const void* fns[4] = {(const void*)k_cluster_strip<false, false>, (const void*)k_cluster_strip<true, false>,

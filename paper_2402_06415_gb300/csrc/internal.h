@@ -134,6 +134,33 @@ size_t tiled32_smem_bytes(int L, int k, int n_tile_rows, int tile_words);
 // planes or int8 spins (the other pointer null).  G row strips, one CTA each
 // (cooperative launch; needs L >= 2 K G), K sweeps between exchanges; K = 0: edge rows
 // exchanged every half sweep (needs L >= 2 G and 2 Wc <= kStripThreads).
+// What a strip writes to a host-visible word when a wait for a neighbour gave up.
+struct WaitStatus {
+  int* word;
+  int code;
+};
+// The host's side of it.  The code is the context's epoch, which every call that defines
+// the whole lattice raises: a launch that is still queued then reports an epoch that
+// is over, so the order on the stream decides and not the moment of the host's call.
+struct StripStatus {
+  int* word = nullptr;  // pinned
+  int epoch = 1;
+  cudaError_t ensure() {
+    if (word) return cudaSuccess;
+    const cudaError_t e = cudaHostAlloc((void**)&word, sizeof(int), cudaHostAllocDefault);
+    if (e != cudaSuccess) word = nullptr;
+    else *word = 0;
+    return e;
+  }
+  void release() {
+    cudaFreeHost(word);
+    word = nullptr;
+  }
+  bool failed() const { return word && *(volatile int*)word == epoch; }
+  WaitStatus wait() const { return WaitStatus{word, epoch}; }
+};
+// Whether ISING_FAULT names this kind of failure (api.cu).
+bool fault(const char* what);
 constexpr int kStripThreads = 512, kSplitThreads = 768;
 constexpr int kStripBlocks = 3;  // Philox blocks drawn for every word before the lazy ones
 struct StripArgs {
@@ -146,7 +173,7 @@ struct StripArgs {
   long long rec0, rec_cap;  // ring slot of the first record
   unsigned long long* rec;
   unsigned long long* xbuf;  // strip_xbuf_words(L, G, K) words (G > 1), zeroed by the launcher
-  int* status;         // host-visible word, set to 1 when a wait gave up
+  WaitStatus status;
   long long limit;     // clock64 cycles a wait may take
   FastDiv fwc;         // set by the launcher
 };
@@ -280,14 +307,13 @@ cudaError_t launch_cluster_persist(const BitsLattice& lat, bool wolff, uint32_t 
 // The same on resident row strips (cluster_strip.cu).  cluster_strip_grid: strips of
 // an L x L lattice (0: they do not fit in shared memory); scratch: device memory
 // of cluster_strip_bytes(L, G) bytes; the record slots are zero on entry; to_rec:
-// steps until the first record (0: none); *status: host-visible word set to 1
-// when a wait gave up.
+// steps until the first record (0: none).
 int cluster_strip_grid(int L, int sms);
 size_t cluster_strip_bytes(int L, int G);
 cudaError_t launch_cluster_strip(const BitsLattice& lat, bool wolff, uint32_t step0, int n_steps, int measure_every,
                                  int to_rec, uint32_t thr, const RngParams& rng, int G, void* scratch,
                                  unsigned long long* rec, long long rec0, long long rec_cap, WolffCtl* wctl,
-                                 int* status, cudaStream_t s);
+                                 const WaitStatus& status, cudaStream_t s);
 
 // Sets the message returned by ising_last_error() on the calling thread.
 void set_last_error(const char* msg);

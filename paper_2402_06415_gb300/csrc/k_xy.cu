@@ -458,7 +458,7 @@ struct XYStripArgs {
   long long rec0, rec_cap;
   unsigned long long* accepted;
   unsigned long long* xbuf;  // xy_strip_words(...) pairs, zeroed by the launcher (G > 1)
-  int* status;
+  WaitStatus status;
   long long limit;
   FastDiv fh;
 };
@@ -740,7 +740,7 @@ struct ising_xy {
   // resident strips of the automatic mode (G = 0: one launch per half sweep)
   int strip_G = 0, strip_gh = 0;
   unsigned long long* strip_x = nullptr;
-  int* strip_status = nullptr;  // pinned host word a strip sets when a wait gave up
+  StripStatus strip_status;
 };
 
 namespace {
@@ -800,8 +800,8 @@ cudaError_t xy_strip_t(ising_xy* x, int n, int m) {
   a.rec_cap = kXYRec;
   a.accepted = x->accepted;
   a.xbuf = x->strip_x;
-  a.status = x->strip_status;
-  a.limit = kXYSpinLimit;
+  a.status = x->strip_status.wait();
+  a.limit = fault("wait") ? -1 : kXYSpinLimit;
   a.fh = make_fastdiv((uint32_t)(x->L / 2));
   const bool whole = a.G == 1;
   const long long sites = (long long)((a.L + a.G - 1) / a.G + (whole ? 0 : 2 * a.gh)) * (a.L / 2);
@@ -992,14 +992,13 @@ int ising_xy_create(ising_xy** out, int L, double beta, int precision, void* str
     if (st.G > 1) {
       const size_t words = precision == 64 ? xy_strip_words<double>(L, st.G, st.gh) : xy_strip_words<float>(L, st.G, st.gh);
       e = cudaMalloc((void**)&x->strip_x, words * sizeof(unsigned long long));
-      if (!e) e = cudaHostAlloc((void**)&x->strip_status, sizeof(int), cudaHostAllocDefault);
-      if (!e) *x->strip_status = 0;
+      if (!e) e = x->strip_status.ensure();
     }
   }
   if (e) {
     cudaGetLastError();
     cudaFree(x->strip_x);
-    cudaFreeHost(x->strip_status);
+    x->strip_status.release();
     cudaFree(x->u);
     cudaFree(x->rec);
     cudaFree(x->accepted);
@@ -1017,7 +1016,7 @@ int ising_xy_seed(ising_xy* x, uint64_t seed) {
   x->sweep = 0;
   x->rec_count = 0;
   x->grid_used = false;
-  if (x->strip_status) *x->strip_status = 0;
+  ++x->strip_status.epoch;
   const RngParams rng = make_rng(seed, 0, 0, 0);
   const long long N = (long long)x->L * x->L;
   if (x->precision == 64)
@@ -1044,9 +1043,9 @@ int ising_xy_sweep(ising_xy* x, int n_sweeps, int measure_every) {
 }
 
 // After a synchronising call: ETIMEOUT if a persistent kernel's grid barrier
-// gave up (the flag stays set until the next seed).
+// or a strip's wait gave up (until the lattice is seeded or set again).
 static int xy_status(ising_xy* x) {
-  if (x->strip_status && *(volatile int*)x->strip_status)
+  if (x->strip_status.failed())
     return xfail(ISING_ETIMEOUT, "a strip's wait for its neighbour timed out in the XY kernel");
   if (!x->grid_used) return ISING_OK;
   int st = 0;
@@ -1132,6 +1131,8 @@ int ising_xy_set_spins(ising_xy* x, const double* host_uv) {
   const long long N = (long long)x->L * x->L;
   if (!x->host_layout) XTRY(cudaMalloc((void**)&x->host_layout, N * 2 * sizeof(double)));
   double* d = x->host_layout;
+  ++x->strip_status.epoch;
+  XTRY(cudaMemsetAsync(x->ctl, 0, sizeof(GridCtl), x->stream));
   cudaError_t e = cudaMemcpyAsync(d, host_uv, N * 2 * sizeof(double), cudaMemcpyHostToDevice, x->stream);
   if (!e) {
     if (x->precision == 64)
@@ -1166,7 +1167,7 @@ int ising_xy_destroy(ising_xy* x) {
   cudaFree(x->ctl);
   cudaFree(x->strip_x);
   cudaFree(x->host_layout);
-  cudaFreeHost(x->strip_status);
+  x->strip_status.release();
   delete x;
   return ISING_OK;
 }

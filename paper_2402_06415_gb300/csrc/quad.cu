@@ -359,7 +359,7 @@ struct QuadStripArgs {
   unsigned long long* rec;
   long long rec0, rec_cap;
   unsigned long long* xbuf;  // quad_strip_words(...) pairs, zeroed by the launcher
-  int* status;
+  WaitStatus status;
   long long limit;
 };
 constexpr int kQuadStripThreads = 512, kQuadStripMaxK = 4;
@@ -553,7 +553,7 @@ struct ising_quad {
   int64_t launches = 0;
   int strip_G = 0, strip_K = 0;  // resident strips (G = 0: not used)
   unsigned long long* strip_x = nullptr;
-  int* strip_status = nullptr;   // pinned host word a strip sets when a wait gave up
+  StripStatus strip_status;
   int8_t* spins = nullptr;       // unpacked spins for get_spins, allocated by its first call
 };
 
@@ -597,8 +597,8 @@ cudaError_t launch_quad_strip(ising_quad* x, int n, int m, const RngParams& rng)
   a.rec0 = x->rec_count % kQuadRec;
   a.rec_cap = kQuadRec;
   a.xbuf = x->strip_x;
-  a.status = x->strip_status;
-  a.limit = kQuadSpinLimit;
+  a.status = x->strip_status.wait();
+  a.limit = fault("wait") ? -1 : kQuadSpinLimit;
   cudaError_t e;
   int64_t n_rec = 0;
   if (m > 0) {
@@ -764,13 +764,12 @@ int ising_quad_create(ising_quad** out, int lattice, int Lc, double beta, double
   if (!e) choose_quad_strip(x->geom, sms, &x->strip_G, &x->strip_K);
   if (!e && x->strip_G > 0) {
     e = cudaMalloc((void**)&x->strip_x, quad_strip_words(x->geom, x->strip_G, x->strip_K) * sizeof(unsigned long long));
-    if (!e) e = cudaHostAlloc((void**)&x->strip_status, sizeof(int), cudaHostAllocDefault);
-    if (!e) *x->strip_status = 0;
+    if (!e) e = x->strip_status.ensure();
   }
   if (e) {
     cudaGetLastError();
     cudaFree(x->strip_x);
-    cudaFreeHost(x->strip_status);
+    x->strip_status.release();
     cudaFree(x->planes);
     cudaFree(x->rec);
     delete x;
@@ -785,7 +784,7 @@ int ising_quad_seed(ising_quad* x, uint64_t seed) {
   x->seed = seed;
   x->sweep = 0;
   x->rec_count = 0;
-  if (x->strip_status) *x->strip_status = 0;
+  ++x->strip_status.epoch;
   const RngParams rng = make_rng(seed, x->replica, 0, 0);
   k_quad_init<<<qgrid(4LL * x->Lc * x->geom.Wq), 256, 0, x->stream>>>(x->planes, x->geom, rng);
   QTRY(cudaGetLastError());
@@ -810,9 +809,9 @@ int ising_quad_sweep(ising_quad* x, int n_sweeps, int measure_every) {
   return ISING_OK;
 }
 
-// After a synchronising call: ETIMEOUT if a strip's wait gave up (until the next seed).
+// After a synchronising call: ETIMEOUT if a strip's wait gave up (until the lattice is set again).
 static int quad_status(ising_quad* x) {
-  if (x->strip_status && *(volatile int*)x->strip_status)
+  if (x->strip_status.failed())
     return qfail(ISING_ETIMEOUT, "a strip's wait for its neighbour timed out");
   return ISING_OK;
 }
@@ -860,6 +859,7 @@ int ising_quad_set_spins(ising_quad* x, const int8_t* host_in) {
         if (v != 1 && v != -1) return qfail(ISING_EINVAL, "spins must be +1 or -1");
         if (v == 1) h[((size_t)q * Lc + Y) * Wq + (X >> 5)] |= 1u << (X & 31);
       }
+  ++x->strip_status.epoch;
   QTRY(cudaMemcpyAsync(x->planes, h.data(), h.size() * 4, cudaMemcpyHostToDevice, x->stream));
   QTRY(cudaStreamSynchronize(x->stream));
   set_last_error("");
@@ -878,7 +878,7 @@ int ising_quad_destroy(ising_quad* x) {
   cudaFree(x->planes);
   cudaFree(x->rec);
   cudaFree(x->strip_x);
-  cudaFreeHost(x->strip_status);
+  x->strip_status.release();
   cudaFree(x->spins);
   delete x;
   return ISING_OK;
