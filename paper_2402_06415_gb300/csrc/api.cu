@@ -100,6 +100,7 @@ struct ising_ctx {
   int cluster_mode = ISING_CLUSTER_AUTO;
   GridCtl* cluster_gctl = nullptr;  // barrier of the persistent cluster kernels
   void* cluster_strip = nullptr;    // scratch of the strip form (cluster_strip_bytes)
+  bool cluster_strips_refused = false;  // the stream has too few SMs for them
   bool timing = false;
   std::vector<cudaEvent_t> ev;
   size_t ev_used = 0;
@@ -383,7 +384,17 @@ int sweep_chunk(ising_ctx* c, int64_t t0, int n, int m) {
     a.xbuf = c->strip_x;
     a.status = c->strip_status.wait();
     a.limit = fault("wait") ? -1 : kClusterSpinLimit;
-    if (int st = launch_result(c, launch_strip_sweep(a, rng, c->stream), "strip sweep")) return st;
+    const cudaError_t e = launch_strip_sweep(a, rng, c->stream);
+    if (strips_refused(e)) {
+      if (c->kernel == ISING_KERNEL_TILED)
+        if (int st = ensure_second_buffer(c)) return st;
+      c->strip = StripShape{0, 0, 0.0};
+    } else if (int st = launch_result(c, e, "strip sweep")) {
+      return st;
+    }
+  }
+  if (c->strip.G > 0) {
+    // done
   } else if (c->layout == ISING_LAYOUT_BITS && c->kernel == ISING_KERNEL_HALF) {
     for (int64_t t = t0; t < t0 + n; ++t) {
       const int64_t sl = slot_of(t);
@@ -471,7 +482,8 @@ void set_last_error(const char* msg) { g_err = msg ? msg : ""; }
 
 // Fault injection for the failure-path tests: ISING_FAULT=alloc makes device allocations
 // fail, ISING_FAULT=launch sweep launches, ISING_FAULT=copy host<->device copies, all
-// without touching the GPU; ISING_FAULT=wait gives strips no time for a wait that is
+// without touching the GPU; ISING_FAULT=coop refuses the strips' cooperative launches, as a
+// stream with few SMs does; ISING_FAULT=wait gives strips no time for a wait that is
 // not over at once (they set the status and return).
 bool fault(const char* what) {
   const char* f = std::getenv("ISING_FAULT");
@@ -1009,6 +1021,10 @@ int cluster_checks(ising_ctx* c, int64_t counter, int n_steps, int measure_every
 constexpr int kClusterPersistMaxL = 768;
 constexpr int kClusterSmemMaxL = 64;  // up to here one CTA holds the lattice (cluster_persist.cu)
 
+int cluster_strips(const ising_ctx* c) {
+  return c->L > kClusterSmemMaxL && !c->cluster_strips_refused ? cluster_strip_grid(c->L, c->sms) : 0;
+}
+
 // Whether cluster steps on this context run as one persistent kernel per call.
 bool cluster_persistent(const ising_ctx* c, bool wolff) {
   if (c->cluster_mode == ISING_CLUSTER_PERSISTENT) return true;
@@ -1018,14 +1034,16 @@ bool cluster_persistent(const ising_ctx* c, bool wolff) {
   // 112 / 221; tiled: 2048 170 / 111).  Wolff: below 768, where a step that grows from
   // the seed is not yet worth a launch.
   if (c->L <= kClusterSmemMaxL) return true;
-  if (wolff) return c->L < kClusterPersistMaxL;
-  return !sw_tiled(c->L) && cluster_strip_grid(c->L, c->sms) > 0;
+  if (wolff && c->L >= kClusterPersistMaxL) return false;
+  return (wolff || !sw_tiled(c->L)) && cluster_strips(c) > 0;
 }
 
-// n persistent-kernel cluster steps from step0, records included.
-int cluster_persist_run(ising_ctx* c, bool wolff, int64_t step0, int n, int measure_every) {
+// n persistent-kernel cluster steps from step0, records included.  *refused: the strips
+// were not accepted and nothing ran.
+int cluster_persist_run(ising_ctx* c, bool wolff, int64_t step0, int n, int measure_every, bool* refused) {
+  *refused = false;
   if (n <= 0) return ISING_OK;
-  const int G = c->L > kClusterSmemMaxL ? cluster_strip_grid(c->L, c->sms) : 0;
+  const int G = cluster_strips(c);
   if (G > 0) {
     if (!c->cluster_strip) {
       if (int st = dev_alloc(&c->cluster_strip, cluster_strip_bytes(c->L, G))) return st;
@@ -1043,6 +1061,10 @@ int cluster_persist_run(ising_ctx* c, bool wolff, int64_t step0, int n, int meas
                                            n_rec ? (int)((before + 1) * m - t) : 0, bond_threshold(c->beta), c->rng(),
                                            G, c->cluster_strip, c->rec, c->rec_count % kRecCap, kRecCap, c->wolff,
                                            c->strip_status.wait(), c->stream);
+      if (done == 0 && strips_refused(e)) {
+        c->cluster_strips_refused = *refused = true;
+        return ISING_OK;
+      }
       if (int st = launch_result(c, e, "cluster strips")) return st;
       c->rec_count += n_rec;
       done += k;
@@ -1109,8 +1131,10 @@ int ising_wolff_step(ising_ctx* c, int n_steps, int measure_every) {
     cudaError_t e = cudaMemsetAsync(c->wolff, 0, sizeof(WolffCtl), c->stream);
     if (e) return fail(ISING_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
   }
-  if (cluster_persistent(c, true)) {
-    if (int st = cluster_persist_run(c, true, c->wolff_steps, n_steps, measure_every)) return st;
+  while (cluster_persistent(c, true)) {
+    bool refused;
+    if (int st = cluster_persist_run(c, true, c->wolff_steps, n_steps, measure_every, &refused)) return st;
+    if (refused) continue;
     c->wolff_steps += n_steps;
     return ok();
   }
@@ -1185,8 +1209,10 @@ int ising_sw_step(ising_ctx* c, int n_steps, int measure_every) {
   if (int st = check_ctx(c)) return st;
   if (int st = cluster_checks(c, c->sw_steps, n_steps, measure_every)) return st;
   NvtxRange nvtx("ising_sw_step");
-  if (cluster_persistent(c, false)) {
-    if (int st = cluster_persist_run(c, false, c->sw_steps, n_steps, measure_every)) return st;
+  while (cluster_persistent(c, false)) {
+    bool refused;
+    if (int st = cluster_persist_run(c, false, c->sw_steps, n_steps, measure_every, &refused)) return st;
+    if (refused) continue;
     c->sw_steps += n_steps;
     return ok();
   }

@@ -500,7 +500,7 @@ cudaError_t launch_cluster_strip(const BitsLattice& lat, bool wolff, uint32_t st
   if ((e = cudaMemsetAsync(a.xbuf, 0, zeroed, s))) return e;
   RngParams r = rng;
   void* args[] = {&a, &r};
-  return cudaLaunchCooperativeKernel(fn, dim3((unsigned)G), dim3(kThreads), args, smem, s);
+  return launch_strips(fn, G, kThreads, args, smem, s);
 }
 
 }  // namespace ising

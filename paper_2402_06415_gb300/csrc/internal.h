@@ -161,6 +161,18 @@ struct StripStatus {
 };
 // Whether ISING_FAULT names this kind of failure (api.cu).
 bool fault(const char* what);
+// cudaLaunchCooperativeKernel of strips.  A stream may have fewer SMs than the device
+// (a green context's); the launch is refused there (strips_refused) and the callers go on
+// with the kernels that run where strips do not fit.
+inline cudaError_t launch_strips(const void* fn, int grid, int threads, void** args, size_t smem, cudaStream_t s) {
+  if (fault("coop")) return cudaErrorCooperativeLaunchTooLarge;
+  return cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args, smem, s);
+}
+inline bool strips_refused(cudaError_t e) {
+  if (e != cudaErrorCooperativeLaunchTooLarge) return false;
+  cudaGetLastError();
+  return true;
+}
 constexpr int kStripThreads = 512, kSplitThreads = 768;
 constexpr int kStripBlocks = 3;  // Philox blocks drawn for every word before the lazy ones
 struct StripArgs {

@@ -549,7 +549,7 @@ cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, cudaStream_t s
   if (whole) return cudaLaunchKernel(fns[which], dim3(1), dim3(threads), args, smem, s);
   cudaError_t e = cudaMemsetAsync(a.xbuf, 0, strip_xbuf_words(a.L, a.G, a.K) * 8, s);
   if (e != cudaSuccess) return e;
-  return cudaLaunchCooperativeKernel(fns[which], dim3(a.G), dim3(threads), args, smem, s);
+  return launch_strips(fns[which], a.G, threads, args, smem, s);
 }
 
 }  // namespace ising

@@ -836,7 +836,7 @@ cudaError_t xy_strip_t(ising_xy* x, int n, int m) {
     e = cudaLaunchKernel(fns[which], dim3(1), dim3(threads), args, smem, x->stream);
   } else {
     e = cudaMemsetAsync(a.xbuf, 0, xy_strip_words<T>(a.L, a.G, a.gh) * 8, x->stream);
-    if (!e) e = cudaLaunchCooperativeKernel(fns[which], dim3(a.G), dim3(threads), args, smem, x->stream);
+    if (!e) e = launch_strips(fns[which], a.G, threads, args, smem, x->stream);
   }
   if (e) return e;
   ++x->launches;
@@ -921,15 +921,21 @@ cudaError_t xy_sweep_t(ising_xy* x, int n, int m) {
   if (x->mode == 0 && x->strip_G > 0) {
     // chunks whose records fit the ring
     const int most = m > 0 ? (int)std::min<int64_t>(kXYRec * (int64_t)m, 1 << 29) : 1 << 29;
-    for (int done = 0; done < n;) {
+    cudaError_t e = cudaSuccess;
+    int done = 0;
+    for (; done < n && !e;) {
       const int k = std::min(most, n - done);
-      cudaError_t e = xy_strip_t<T>(x, k, m);
-      if (e) return e;
+      e = xy_strip_t<T>(x, k, m);
+      if (strips_refused(e)) {
+        x->strip_G = 0;
+        e = xy_sweep_t<T>(x, n - done, m);
+        break;
+      }
       x->sweep += k;
       done += k;
     }
-    x->sweep -= n;  // the caller advances the counter
-    return cudaSuccess;
+    x->sweep -= done;  // the caller advances the counter
+    return e;
   }
   const bool persist = x->mode == 2;
   if (persist) return n > 0 ? xy_persist_t<T>(x, n, m) : cudaSuccess;

@@ -622,7 +622,7 @@ cudaError_t launch_quad_strip(ising_quad* x, int n, int m, const RngParams& rng)
   RngParams r = rng;
   QuadTable tab = x->tab;
   void* args[] = {&a, &r, &tab};
-  if ((e = cudaLaunchCooperativeKernel(fn, dim3(a.G), dim3(threads), args, smem, x->stream))) return e;
+  if ((e = launch_strips(fn, a.G, threads, args, smem, x->stream))) return e;
   ++x->launches;
   x->rec_count += n_rec;
   return cudaSuccess;
@@ -685,6 +685,11 @@ cudaError_t quad_sweeps(ising_quad* x, int n, int m) {
       const int k = std::min(most, n - done);
       e = x->lattice == ISING_QUAD_SQUARE ? strip_dispatch<ISING_QUAD_SQUARE>(x, k, m, rng)
                                           : strip_dispatch<ISING_QUAD_SQOCT>(x, k, m, rng);
+      if (strips_refused(e)) {
+        x->strip_G = 0;
+        e = quad_sweeps(x, n - done, m);
+        break;
+      }
       x->sweep += k;
       done += k;
     }
