@@ -1,0 +1,47 @@
+"""Calls of a single sweep, as the interleaved schedule makes them, cost no more than one launch per half sweep did."""
+import pytest
+
+import paper_2402_06415_gb300 as ising
+
+pytestmark = pytest.mark.gpu
+
+BITS, I8 = ising.ISING_LAYOUT_BITS, ising.ISING_LAYOUT_I8
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    ising.lib()
+
+
+def _us(run, n=200, reps=5):
+    """us per call of run(), n calls in a row, best of reps."""
+    import torch
+
+    run()
+    best = 1e30
+    for _ in range(reps):
+        torch.cuda.synchronize()
+        e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        e0.record()
+        for _ in range(n):
+            run()
+        e1.record()
+        e1.synchronize()
+        best = min(best, e0.elapsed_time(e1) * 1e3 / n)
+    return best
+
+
+def test_int8_edge_strips_start_as_fast_as_the_others():
+    """1000 x 1000 int8 spins are 1.7 times the bytes of 768 x 768, where the strips still keep a halo: a call of one
+    sweep takes no longer than that (reading the neighbour's row byte after byte made it 2.0 times)."""
+    import torch
+
+    us = []
+    for L in (768, 1000):
+        with ising.Lattice(L, 0.44, I8, seed=1, stream=torch.cuda.current_stream()) as lat:
+            lat.set_kernel(ising.ISING_KERNEL_STRIP)
+            us.append(_us(lambda: lat.sweep(2)))
+    assert us[1] < 1.7 * us[0], us
