@@ -59,7 +59,8 @@ typedef enum {
 typedef enum { ISING_LAYOUT_I8 = 0, ISING_LAYOUT_BITS = 1 } ising_layout;
 
 typedef enum {
-  ISING_KERNEL_AUTO = 0,     /* pick per lattice: strips, except tiled from L = 6144 where 32-word
+  ISING_KERNEL_AUTO = 0,     /* pick per lattice: strips (calls of one sweep: half sweeps where
+                                those are faster), except tiled from L = 6144 where 32-word
                                 tiles fit; where strips do not fit tiled, else half (packed),
                                 resident, else half (int8) */
   ISING_KERNEL_HALF = 1,     /* one launch per half sweep, spins in global memory */
@@ -501,9 +502,10 @@ int ising_xy_create(ising_xy** out, int L, double beta, int precision, void* str
 int ising_xy_seed(ising_xy* x, uint64_t seed);
 /* n_sweeps sweeps (async). */
 int ising_xy_sweep(ising_xy* x, int n_sweeps, int measure_every);
-/* Kernel form: 0 automatic (one persistent launch per call for L <= 1024), 1 one launch per half
- * sweep, 2 persistent cooperative kernel (all CTAs co-resident, one launch per
- * ising_xy_sweep call, a bounded grid barrier between half sweeps).  Results
+/* Kernel form: 0 automatic (one persistent launch per call for L <= 1024, but half sweeps for
+ * single-precision calls of one sweep), 1 one launch per half sweep, 2 persistent
+ * cooperative kernel (all CTAs co-resident, one launch per ising_xy_sweep call, a bounded
+ * grid barrier between half sweeps).  Results
  * are identical in every mode.  If a persistent barrier gives up (after ~2 s)
  * or a wait of the automatic form's strips does, synchronising calls return
  * ISING_ETIMEOUT, and the lattice and its records are undefined, until ising_xy_seed or

@@ -80,6 +80,7 @@ struct ising_ctx {
   StripShape strip{0, 0, 0.0};
   unsigned long long* strip_x = nullptr;  // boundary exchange buffer (G > 1)
   StripStatus strip_status;
+  bool strip_asked = false;               // the caller chose strips: for calls of one sweep too
   int kernel = ISING_KERNEL_HALF, k = 1, tile_rows = 1, tile_words = 4, grid = 0, block = 0;
   __nv_bfloat16* nn_w = nullptr;    // BF16 weights of the block proposal
   __nv_bfloat16* nn_w2t = nullptr;
@@ -178,6 +179,17 @@ int check_ctx(ising_ctx* c) {
 // L = 2048; one CTA with int8 spins 0.25 at L = 64 (strips: 7).
 bool strip_applies(int layout, int L) {
   return layout == ISING_LAYOUT_I8 || L < 6144 || words_per_row(L) % 32 != 0 || L % 64 != 0;
+}
+
+// Whether a call of one sweep is faster as two half-sweep launches than on strips, which
+// load and store the whole lattice and clear the exchange buffer first.  us per call,
+// strips / half sweeps: packed L = 128 6.5 / 8.2, 256 to 1280 10.3 / 8.2, 2048 12.3 / 8.2, 4096 18.4 / 16.4,
+// 6000 26.7 / 27.0, with a record 256 10.7 / 9.9, 3000 16.8 / 16.2, 4096 18.9 / 20.1; int8 512 14.4 / 12.3,
+// 576 14.4 / 16.4, with a record strips everywhere (14.8 / 20.6 at 512).
+bool one_sweep_as_halves(const ising_ctx* c, bool recorded) {
+  if (c->strip.G <= 1 || c->strip_asked) return false;
+  if (c->layout == ISING_LAYOUT_I8) return !recorded && c->L < 544;
+  return c->L > 128 && c->L < (recorded ? 3584 : 5632);
 }
 
 // Kernel configuration validity for this lattice.
@@ -365,7 +377,9 @@ int sweep_chunk(ising_ctx* c, int64_t t0, int n, int m) {
   const RngParams rng = c->rng();
   if (fault("launch")) return fail(ISING_ECUDA, "sweep launch failed (injected)");
 
-  if (c->strip.G > 0) {
+  const bool halves = n == 1 && one_sweep_as_halves(c, n_rec > 0);
+  const int kernel = halves ? ISING_KERNEL_HALF : c->kernel;
+  if (c->strip.G > 0 && !halves) {
     Timed tm(c);
     StripArgs a{};
     a.planes = c->layout == ISING_LAYOUT_BITS ? c->bits[c->cur] : nullptr;
@@ -393,9 +407,9 @@ int sweep_chunk(ising_ctx* c, int64_t t0, int n, int m) {
       return st;
     }
   }
-  if (c->strip.G > 0) {
+  if (c->strip.G > 0 && !halves) {
     // done
-  } else if (c->layout == ISING_LAYOUT_BITS && c->kernel == ISING_KERNEL_HALF) {
+  } else if (c->layout == ISING_LAYOUT_BITS && kernel == ISING_KERNEL_HALF) {
     for (int64_t t = t0; t < t0 + n; ++t) {
       const int64_t sl = slot_of(t);
       for (int col = 0; col < 2; ++col) {
@@ -406,7 +420,7 @@ int sweep_chunk(ising_ctx* c, int64_t t0, int n, int m) {
         if (int st = launch_result(c, e, "half sweep")) return st;
       }
     }
-  } else if (c->layout == ISING_LAYOUT_BITS && c->kernel == ISING_KERNEL_TILED) {
+  } else if (c->layout == ISING_LAYOUT_BITS && kernel == ISING_KERNEL_TILED) {
     for (int64_t t = t0; t < t0 + n; t += c->k) {
       const int kk = (int)std::min<int64_t>(c->k, t0 + n - t);
       RecordSlots slots;
@@ -424,7 +438,7 @@ int sweep_chunk(ising_ctx* c, int64_t t0, int n, int m) {
       if (int st = launch_result(c, e, "tiled sweep")) return st;
       c->cur = 1 - c->cur;
     }
-  } else if (c->layout == ISING_LAYOUT_I8 && c->kernel == ISING_KERNEL_RESIDENT) {
+  } else if (c->layout == ISING_LAYOUT_I8 && kernel == ISING_KERNEL_RESIDENT) {
     Timed tm(c);
     cudaError_t e = launch_resident_sweep_i8(
         c->spins, c->L, rng, (uint32_t)t0, n, m, (uint32_t)(first_t < 0 ? 0 : first_t),
@@ -859,6 +873,7 @@ int ising_set_kernel(ising_ctx* c, int kernel, int k, int tile_rows, int tile_wo
     if (int st = ensure_strip(c, shape)) return st;  // before anything changes
     resolve_auto(c);
     c->strip = shape;
+    c->strip_asked = kernel == ISING_KERNEL_STRIP;
     if (c->kernel == ISING_KERNEL_TILED && c->strip.G == 0)
       if (int st = ensure_second_buffer(c)) return st;
     return ok();

@@ -916,9 +916,20 @@ cudaError_t xy_persist_t(ising_xy* x, int n, int m) {
   return cudaSuccess;
 }
 
+// Single-precision calls of one sweep that the strips make slower than the forms before
+// them.  us per call: half sweeps / strips (which clear their exchange buffer first) L = 64 8.2 /
+// 10.3, 512 12.3 / 14.4, 1024 20.5 / 22.6; with a record, one CTA: separate measurement / in the
+// sweep L = 32 10.3 / 11.4 (FP64: at most even).
+int xy_one_sweep_mode(const ising_xy* x, bool recorded) {
+  if (x->mode != 0 || x->precision != 32) return x->mode;
+  if (x->strip_G > 1 && !recorded) return 1;
+  return x->strip_G == 1 && recorded && x->L > 24 ? 2 : 0;
+}
+
 template <typename T>
 cudaError_t xy_sweep_t(ising_xy* x, int n, int m) {
-  if (x->mode == 0 && x->strip_G > 0) {
+  const int mode = n == 1 ? xy_one_sweep_mode(x, m > 0 && (x->sweep + 1) % m == 0) : x->mode;
+  if (mode == 0 && x->strip_G > 0) {
     // chunks whose records fit the ring
     const int most = m > 0 ? (int)std::min<int64_t>(kXYRec * (int64_t)m, 1 << 29) : 1 << 29;
     cudaError_t e = cudaSuccess;
@@ -937,8 +948,7 @@ cudaError_t xy_sweep_t(ising_xy* x, int n, int m) {
     x->sweep -= done;  // the caller advances the counter
     return e;
   }
-  const bool persist = x->mode == 2;
-  if (persist) return n > 0 ? xy_persist_t<T>(x, n, m) : cudaSuccess;
+  if (mode == 2) return n > 0 ? xy_persist_t<T>(x, n, m) : cudaSuccess;
   const RngParams rng = make_rng(x->seed, 0, 0, 0);
   const long long blocks = ((long long)x->L * (x->L / 2) + 1) / 2;
   using V = typename Vec<T>::type;
