@@ -67,7 +67,8 @@ typedef enum {
   ISING_KERNEL_TILED = 2,    /* packed layout: shared-memory tile + halo, k sweeps per launch */
   ISING_KERNEL_RESIDENT = 3, /* int8 layout: whole lattice in one CTA's shared memory */
   ISING_KERNEL_STRIP = 4     /* row strips resident in the SMs' shared memory for all sweeps of a
-                                call, either layout, up to what 200 KiB per strip hold */
+                                call (launches of about 20 ms), either layout, up to what 200 KiB
+                                per strip hold */
 } ising_kernel;
 
 /* Create a context for one L x L lattice (Results A; the sweep of Fig. 2b).
@@ -381,7 +382,7 @@ int ising_sweep_blocks(ising_ctx* ctx, int n_sweeps, int measure_every, int bloc
 int ising_sw_step(ising_ctx* ctx, int n_steps, int measure_every);
 
 /* How cluster steps (ising_sw_step, ising_wolff_step) run: AUTO = one
- * persistent launch per call for L < 768 (up to 64 x 64 sites one CTA with the
+ * persistent launch per call, or per 20 ms of a longer one, for L < 768 (up to 64 x 64 sites one CTA with the
  * lattice in shared memory, else row strips resident in shared memory with
  * bounded grid barriers around the unions across strips; a barrier wait gives up
  * after about 2 s and later synchronising calls then fail with ISING_ETIMEOUT;
@@ -502,8 +503,8 @@ int ising_xy_create(ising_xy** out, int L, double beta, int precision, void* str
 int ising_xy_seed(ising_xy* x, uint64_t seed);
 /* n_sweeps sweeps (async). */
 int ising_xy_sweep(ising_xy* x, int n_sweeps, int measure_every);
-/* Kernel form: 0 automatic (one persistent launch per call for L <= 1024, but half sweeps for
- * single-precision calls of one sweep), 1 one launch per half sweep, 2 persistent
+/* Kernel form: 0 automatic (for L <= 1024 one persistent launch per call, or per 20 ms of a
+ * longer one, but half sweeps for single-precision calls of one sweep), 1 one launch per half sweep, 2 persistent
  * cooperative kernel (all CTAs co-resident, one launch per ising_xy_sweep call, a bounded
  * grid barrier between half sweeps).  Results
  * are identical in every mode.  If a persistent barrier gives up (after ~2 s)

@@ -663,7 +663,8 @@ int ising_sweep(ising_ctx* c, int n_sweeps, int measure_every) {
   const int64_t max_chunk = measure_every > 0 ? kRecCap * (int64_t)measure_every : end - t;
   while (t < end) {
     const int64_t n = std::min<int64_t>(end - t, std::max<int64_t>(max_chunk, 1));
-    int chunk = (int)std::min<int64_t>(n, 1 << 30);
+    const int most = c->strip.G > 0 ? strip_launch_sweeps(c->strip.us) : 1 << 30;
+    const int chunk = (int)std::min<int64_t>(n, most);
     if (int st = sweep_chunk(c, t, chunk, measure_every)) return st;
     t += chunk;
     c->sweep = t;
@@ -1065,8 +1066,10 @@ int cluster_persist_run(ising_ctx* c, bool wolff, int64_t step0, int n, int meas
     }
     if (int st = ensure_strip_status(c)) return st;
     const int64_t m = measure_every;
-    // chunks whose records fit the ring
-    const int64_t most = m > 0 ? std::min<int64_t>(kRecCap * m, 1 << 29) : 1 << 29;
+    // chunks whose records fit the ring, of about 20 ms (a step takes 12 us at L = 128, 27 at
+    // 512, 51 at 1024, 230 at 2400)
+    const int64_t launch = strip_launch_sweeps(12.0 + 4e-5 * (double)c->N());
+    const int64_t most = m > 0 ? std::min<int64_t>(kRecCap * m, launch) : launch;
     for (int64_t done = 0; done < n;) {
       const int k = (int)std::min<int64_t>(most, n - done);
       const int64_t t = step0 + done, before = m > 0 ? t / m : 0, n_rec = m > 0 ? (t + k) / m - before : 0;

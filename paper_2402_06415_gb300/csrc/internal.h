@@ -161,6 +161,13 @@ struct StripStatus {
 };
 // Whether ISING_FAULT names this kind of failure (api.cu).
 bool fault(const char* what);
+// Sweeps or steps per launch of strips, by their modelled time: about 20 ms.  A cooperative
+// launch starts once all its SMs are free, so without a bound another context's strips
+// waited for the whole of a long call (0.9 s behind 2,000,000 sweeps on one SM; so
+// 2 to 24 ms).  A launch costs 10 us.
+inline int strip_launch_sweeps(double us_per_sweep) {
+  return us_per_sweep < 20000.0 ? (int)(20000.0 / us_per_sweep) : 1;
+}
 // cudaLaunchCooperativeKernel of strips.  A stream may have fewer SMs than the device
 // (a green context's); the launch is refused there (strips_refused) and the callers go on
 // with the kernels that run where strips do not fit.

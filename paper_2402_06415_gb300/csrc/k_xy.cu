@@ -739,6 +739,7 @@ struct ising_xy {
   double* host_layout = nullptr;     // spins in the host's layout, allocated by the first call that needs it
   // resident strips of the automatic mode (G = 0: one launch per half sweep)
   int strip_G = 0, strip_gh = 0;
+  double strip_us = 0;  // modelled time of a sweep
   unsigned long long* strip_x = nullptr;
   StripStatus strip_status;
 };
@@ -930,8 +931,9 @@ template <typename T>
 cudaError_t xy_sweep_t(ising_xy* x, int n, int m) {
   const int mode = n == 1 ? xy_one_sweep_mode(x, m > 0 && (x->sweep + 1) % m == 0) : x->mode;
   if (mode == 0 && x->strip_G > 0) {
-    // chunks whose records fit the ring
-    const int most = m > 0 ? (int)std::min<int64_t>(kXYRec * (int64_t)m, 1 << 29) : 1 << 29;
+    // chunks whose records fit the ring, of about 20 ms
+    const int launch = strip_launch_sweeps(x->strip_us);
+    const int most = m > 0 ? (int)std::min<int64_t>(kXYRec * (int64_t)m, launch) : launch;
     cudaError_t e = cudaSuccess;
     int done = 0;
     for (; done < n && !e;) {
@@ -1005,6 +1007,7 @@ int ising_xy_create(ising_xy** out, int L, double beta, int precision, void* str
     const XYStrip st = precision == 64 ? choose_xy_strip<double>(L, sms) : choose_xy_strip<float>(L, sms);
     x->strip_G = st.G;
     x->strip_gh = st.gh;
+    x->strip_us = st.us;
     if (st.G > 1) {
       const size_t words = precision == 64 ? xy_strip_words<double>(L, st.G, st.gh) : xy_strip_words<float>(L, st.G, st.gh);
       e = cudaMalloc((void**)&x->strip_x, words * sizeof(unsigned long long));

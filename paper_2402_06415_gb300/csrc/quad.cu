@@ -552,6 +552,7 @@ struct ising_quad {
   int64_t rec_count = 0;
   int64_t launches = 0;
   int strip_G = 0, strip_K = 0;  // resident strips (G = 0: not used)
+  double strip_us = 0;           // modelled time of a sweep
   unsigned long long* strip_x = nullptr;
   StripStatus strip_status;
   int8_t* spins = nullptr;       // unpacked spins for get_spins, allocated by its first call
@@ -565,7 +566,7 @@ constexpr long long kQuadSpinLimit = 4000000000LL;  // ~2 s of SM clock per wait
 // sweep takes 0.45 + 0.25 per resident warp of an SM sub-partition, an exchange
 // 1.0; G = 0 where one CTA (the same time per quarter, no exchange) is as fast
 // or the strips do not fit.
-void choose_quad_strip(const QuadGeom& g, int sms, int* G_out, int* K_out) {
+void choose_quad_strip(const QuadGeom& g, int sms, int* G_out, int* K_out, double* us_out) {
   auto quarter = [](double words) { return 0.45 + 0.25 * std::ceil(std::ceil(words / 32) / 4); };
   double best = g.Lc <= 256 ? 4 * quarter((double)g.Lc * g.Wq) : 1e30;
   *G_out = *K_out = 0;
@@ -579,6 +580,7 @@ void choose_quad_strip(const QuadGeom& g, int sms, int* G_out, int* K_out) {
         best = t / K;
         *G_out = G;
         *K_out = K;
+        *us_out = best;
       }
     }
 }
@@ -677,8 +679,9 @@ cudaError_t persist_dispatch(ising_quad* x, int n, int m, const RngParams& rng) 
 cudaError_t quad_sweeps(ising_quad* x, int n, int m) {
   const RngParams rng = make_rng(x->seed, x->replica, 0, 0);
   if (x->strip_G > 0 && n > 0) {
-    // chunks whose records fit the ring
-    const int most = m > 0 ? (int)std::min<int64_t>(kQuadRec * (int64_t)m, 1 << 29) : 1 << 29;
+    // chunks whose records fit the ring, of about 20 ms
+    const int launch = strip_launch_sweeps(x->strip_us);
+    const int most = m > 0 ? (int)std::min<int64_t>(kQuadRec * (int64_t)m, launch) : launch;
     cudaError_t e = cudaSuccess;
     int done = 0;
     for (; done < n && !e;) {
@@ -766,7 +769,7 @@ int ising_quad_create(ising_quad** out, int lattice, int Lc, double beta, double
   int dev = 0, sms = 0;
   if (!e) e = cudaGetDevice(&dev);
   if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (!e) choose_quad_strip(x->geom, sms, &x->strip_G, &x->strip_K);
+  if (!e) choose_quad_strip(x->geom, sms, &x->strip_G, &x->strip_K, &x->strip_us);
   if (!e && x->strip_G > 0) {
     e = cudaMalloc((void**)&x->strip_x, quad_strip_words(x->geom, x->strip_G, x->strip_K) * sizeof(unsigned long long));
     if (!e) e = x->strip_status.ensure();
