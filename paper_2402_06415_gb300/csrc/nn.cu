@@ -889,8 +889,7 @@ namespace {
 // loss and gradients of count windows with the trainer's kernel
 cudaError_t launch_train(ising_nn* n, const int8_t* dev_windows, int count) {
   if (n->train_prec == kTrainBf16Tc)
-    return nn_train_tc(dev_windows, count, n->plan, n->n_net, n->p, n->g, n->loss, sms_of_current(),
-                       n->stream);
+    return nn_train_tc(dev_windows, count, n->plan, n->p, n->g, n->loss, sms_of_current(), n->stream);
   const int grid = std::max(1, std::min(count * n->n_net, sms_of_current()));
   k_nn_train<<<grid, kThreads, train_smem(), n->stream>>>(dev_windows, count, n->B, n->plan, n->p, n->g,
                                                           n->loss);

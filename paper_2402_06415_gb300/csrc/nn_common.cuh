@@ -145,9 +145,9 @@ cudaError_t nn_log_q(const int8_t* windows, int count, const StagedPlan* d_plan,
                      cudaStream_t s);
 // Loss and gradient sums (added to grads, loss) of count windows on the tensor
 // cores (nn_train_tc.cu): the objective of the FP32 training kernel with BF16
-// operands and FP32 accumulation in the 32 -> 32 convolution; at most `grid`
+// operands and FP32 accumulation in the 32 -> 32 convolution; `grid`
 // CTAs (one per SM fits).
-cudaError_t nn_train_tc(const int8_t* windows, int count, const StagedPlan* d_plan, int n_net,
+cudaError_t nn_train_tc(const int8_t* windows, int count, const StagedPlan* d_plan,
                         const float* params, float* grads, float* loss, int grid, cudaStream_t s);
 // training precisions
 constexpr int kTrainFp32 = 0;
