@@ -520,7 +520,8 @@ int ising_xy_launch_count(ising_xy* x, int64_t* count);
 int ising_selftest_grid_barrier(double timeout_s, int* timed_out);
 /* Last n records (oldest first): E, Mx, My (host arrays; any may be NULL). */
 int ising_xy_series(ising_xy* x, double* E, double* Mx, double* My, int n);
-/* Spins as host [L][L][2] doubles (cos, sin), row-major y*L + x. */
+/* Spins as host [L][L][2] doubles (cos, sin), row-major y*L + x.  The context keeps a
+ * device buffer of at most 32 MB for them. */
 int ising_xy_get_spins(ising_xy* x, double* host_uv);
 int ising_xy_set_spins(ising_xy* x, const double* host_uv);
 /* Accepted updates since the last seed (synchronises). */
@@ -601,7 +602,8 @@ int ising_quad_set_replica(ising_quad* x, uint32_t replica);
 int ising_quad_sweep(ising_quad* x, int n_sweeps, int measure_every);
 /* Last n records, oldest first (host arrays; any may be NULL).  Synchronises. */
 int ising_quad_series(ising_quad* x, int64_t* B1, int64_t* B2, int64_t* M, int n);
-/* Spins as host int8 [4][Lc][Lc] (+1 / -1).  Synchronise. */
+/* Spins as host int8 [4][Lc][Lc] (+1 / -1).  Synchronise.  The context keeps a device
+ * buffer of at most 32 MB for get. */
 int ising_quad_get_spins(ising_quad* x, int8_t* host_out);
 int ising_quad_set_spins(ising_quad* x, const int8_t* host_in);
 /* Kernels this context has launched. */

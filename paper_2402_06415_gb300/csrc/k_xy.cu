@@ -673,25 +673,25 @@ __global__ void k_grid_barrier_selftest(GridCtl* ctl, long long limit) {
 }
 
 template <typename T>
-__global__ void k_xy_to_host_layout(const typename Vec<T>::type* __restrict__ u, int L,
+__global__ void k_xy_to_host_layout(const typename Vec<T>::type* __restrict__ u, int L, long long n0, long long count,
                                     double* __restrict__ out, int to_dev) {
-  // to_dev = 0: planes -> [L][L][2] double; 1: the reverse (out is the source)
+  // sites [n0, n0 + count); to_dev = 0: planes -> [count][2] double; 1: the reverse (out is the source)
   using V = typename Vec<T>::type;
-  const long long N = (long long)L * L;
   const int half = L / 2;
   V* uu = const_cast<V*>(u);
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-       n += (long long)gridDim.x * blockDim.x) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long n = n0 + i;
     const int y = (int)(n / L), x = (int)(n - (n / L) * L);
     const size_t idx = (size_t)((x + y) & 1) * L * half + (size_t)y * half + (x >> 1);
     if (to_dev) {
       V v;
-      v.x = (T)out[2 * n];
-      v.y = (T)out[2 * n + 1];
+      v.x = (T)out[2 * i];
+      v.y = (T)out[2 * i + 1];
       uu[idx] = v;
     } else {
-      out[2 * n] = (double)u[idx].x;
-      out[2 * n + 1] = (double)u[idx].y;
+      out[2 * i] = (double)u[idx].x;
+      out[2 * i + 1] = (double)u[idx].y;
     }
   }
 }
@@ -736,7 +736,7 @@ struct ising_xy {
   int64_t rec_count = 0;
   unsigned long long* accepted = nullptr;
   bool grid_used = false;            // a grid barrier ran since the last seed: its status is worth reading
-  double* host_layout = nullptr;     // spins in the host's layout, allocated by the first call that needs it
+  double* host_layout = nullptr;     // spins in the host's layout, at most kXYLayoutSites at a time (xy_layout)
   // resident strips of the automatic mode (G = 0: one launch per half sweep)
   int strip_G = 0, strip_gh = 0;
   double strip_us = 0;  // modelled time of a sweep
@@ -746,6 +746,7 @@ struct ising_xy {
 
 namespace {
 constexpr int64_t kXYRec = 65536;
+constexpr long long kXYLayoutSites = 2 << 20;  // 16 bytes a site in the host's layout
 
 // Largest L for which the automatic mode runs the resident strips.
 // (us per sweep, strips / one launch per half sweep: FP64 L = 256 8.9 / 17.6, 1024 76 / 78; FP32 L = 256 3.1 / 8.2,
@@ -1127,18 +1128,35 @@ int ising_xy_series(ising_xy* x, double* E, double* Mx, double* My, int n) {
   return ISING_OK;
 }
 
+// Spins between the planes and the host's layout, through a device buffer of at most 32 MB
+// that the context keeps (an allocation per call took 100 us; one for the whole lattice
+// would hold 17 GB at L = 32768).
+static cudaError_t xy_layout(ising_xy* x, double* host, bool to_dev) {
+  const long long N = (long long)x->L * x->L, most = std::min(N, kXYLayoutSites);
+  cudaError_t e = cudaSuccess;
+  if (!x->host_layout) {
+    e = cudaMalloc((void**)&x->host_layout, most * 2 * sizeof(double));
+    if (e) return e;
+  }
+  double* const d = x->host_layout;
+  for (long long n0 = 0; n0 < N && !e; n0 += most) {
+    const long long count = std::min(most, N - n0);
+    const size_t bytes = (size_t)count * 2 * sizeof(double);
+    if (to_dev) e = cudaMemcpyAsync(d, host + 2 * n0, bytes, cudaMemcpyHostToDevice, x->stream);
+    if (e) return e;
+    if (x->precision == 64)
+      k_xy_to_host_layout<double><<<grid_of(count), 256, 0, x->stream>>>((const double2*)x->u, x->L, n0, count, d, to_dev);
+    else
+      k_xy_to_host_layout<float><<<grid_of(count), 256, 0, x->stream>>>((const float2*)x->u, x->L, n0, count, d, to_dev);
+    e = cudaGetLastError();
+    if (!e && !to_dev) e = cudaMemcpyAsync(host + 2 * n0, d, bytes, cudaMemcpyDeviceToHost, x->stream);
+  }
+  return e ? e : cudaStreamSynchronize(x->stream);
+}
+
 int ising_xy_get_spins(ising_xy* x, double* host_uv) {
   if (!x || !host_uv) return xfail(ISING_EINVAL, "null argument");
-  const long long N = (long long)x->L * x->L;
-  if (!x->host_layout) XTRY(cudaMalloc((void**)&x->host_layout, N * 2 * sizeof(double)));
-  double* d = x->host_layout;
-  if (x->precision == 64)
-    k_xy_to_host_layout<double><<<grid_of(N), 256, 0, x->stream>>>((const double2*)x->u, x->L, d, 0);
-  else
-    k_xy_to_host_layout<float><<<grid_of(N), 256, 0, x->stream>>>((const float2*)x->u, x->L, d, 0);
-  cudaError_t e = cudaGetLastError();
-  if (!e) e = cudaMemcpyAsync(host_uv, d, N * 2 * sizeof(double), cudaMemcpyDeviceToHost, x->stream);
-  if (!e) e = cudaStreamSynchronize(x->stream);
+  cudaError_t e = xy_layout(x, host_uv, false);
   if (e) return xfail(ISING_ECUDA, "get spins: %s", cudaGetErrorString(e));
   if (int st = xy_status(x)) return st;
   set_last_error("");
@@ -1147,20 +1165,9 @@ int ising_xy_get_spins(ising_xy* x, double* host_uv) {
 
 int ising_xy_set_spins(ising_xy* x, const double* host_uv) {
   if (!x || !host_uv) return xfail(ISING_EINVAL, "null argument");
-  const long long N = (long long)x->L * x->L;
-  if (!x->host_layout) XTRY(cudaMalloc((void**)&x->host_layout, N * 2 * sizeof(double)));
-  double* d = x->host_layout;
   ++x->strip_status.epoch;
   XTRY(cudaMemsetAsync(x->ctl, 0, sizeof(GridCtl), x->stream));
-  cudaError_t e = cudaMemcpyAsync(d, host_uv, N * 2 * sizeof(double), cudaMemcpyHostToDevice, x->stream);
-  if (!e) {
-    if (x->precision == 64)
-      k_xy_to_host_layout<double><<<grid_of(N), 256, 0, x->stream>>>((const double2*)x->u, x->L, d, 1);
-    else
-      k_xy_to_host_layout<float><<<grid_of(N), 256, 0, x->stream>>>((const float2*)x->u, x->L, d, 1);
-    e = cudaGetLastError();
-  }
-  if (!e) e = cudaStreamSynchronize(x->stream);
+  cudaError_t e = xy_layout(x, const_cast<double*>(host_uv), true);
   if (e) return xfail(ISING_ECUDA, "set spins: %s", cudaGetErrorString(e));
   set_last_error("");
   return ISING_OK;

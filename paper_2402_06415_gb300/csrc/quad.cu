@@ -464,15 +464,16 @@ __global__ void __launch_bounds__(kQuadStripThreads) k_quad_strip(QuadStripArgs 
     for (int i = tid; i < R * Wq; i += nth) a.planes[(size_t)q * LW + (size_t)y0 * Wq + i] = sp[q * plane + hw + i];
 }
 
-// Bit planes -> one int8 (+-1) per site, [4][Lc][Lc].
-__global__ void __launch_bounds__(256) k_quad_unpack(const uint32_t* __restrict__ planes, QuadGeom g,
-                                                     int8_t* __restrict__ out) {
-  const long long words = 4LL * g.Lc * g.Wq;
+// Rows [row0, row0 + rows) of the bit planes (row q Lc + Y) -> one int8 (+-1) per site.
+__global__ void __launch_bounds__(256) k_quad_unpack(const uint32_t* __restrict__ planes, QuadGeom g, long long row0,
+                                                     int rows, int8_t* __restrict__ out) {
+  const long long words = (long long)rows * g.Wq;
+  planes += row0 * g.Wq;
   const int lane = threadIdx.x & 31;
   // one warp per word, one lane per site
   for (long long i = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; i < words;
        i += ((long long)gridDim.x * blockDim.x) >> 5) {
-    const long long row = i / g.Wq;  // q Lc + Y
+    const long long row = i / g.Wq;
     const int X = 32 * (int)(i - row * g.Wq) + lane;
     const uint32_t v = __ldg(&planes[i]);
     if (X < g.Lc) out[row * g.Lc + X] = (v >> lane) & 1u ? 1 : -1;
@@ -555,11 +556,12 @@ struct ising_quad {
   double strip_us = 0;           // modelled time of a sweep
   unsigned long long* strip_x = nullptr;
   StripStatus strip_status;
-  int8_t* spins = nullptr;       // unpacked spins for get_spins, allocated by its first call
+  int8_t* spins = nullptr;       // unpacked rows for get_spins, at most kQuadUnpackBytes
 };
 
 namespace {
 constexpr int64_t kQuadRec = 65536;
+constexpr long long kQuadUnpackBytes = 32 << 20;
 constexpr long long kQuadSpinLimit = 4000000000LL;  // ~2 s of SM clock per wait
 
 // Strips of an Lc x Lc lattice by a time model (us per sweep, GB300): a quarter
@@ -845,11 +847,16 @@ int ising_quad_series(ising_quad* x, int64_t* B1, int64_t* B2, int64_t* M, int n
 
 int ising_quad_get_spins(ising_quad* x, int8_t* host_out) {
   if (!x || !host_out) return qfail(ISING_EINVAL, "null argument");
-  const size_t N = (size_t)4 * x->Lc * x->Lc;
-  if (!x->spins) QTRY(cudaMalloc((void**)&x->spins, N));
-  k_quad_unpack<<<qgrid(4LL * x->Lc * x->geom.Wq * 32), 256, 0, x->stream>>>(x->planes, x->geom, x->spins);
-  QTRY(cudaGetLastError());
-  QTRY(cudaMemcpyAsync(host_out, x->spins, N, cudaMemcpyDeviceToHost, x->stream));
+  const int Lc = x->Lc, Wq = x->geom.Wq;
+  const long long rows = 4LL * Lc, most = std::min(rows, std::max(1LL, kQuadUnpackBytes / Lc));
+  // through a buffer that the context keeps, so many rows at a time
+  if (!x->spins) QTRY(cudaMalloc((void**)&x->spins, most * Lc));
+  for (long long r0 = 0; r0 < rows; r0 += most) {
+    const int n = (int)std::min(most, rows - r0);
+    k_quad_unpack<<<qgrid((long long)n * Wq * 32), 256, 0, x->stream>>>(x->planes, x->geom, r0, n, x->spins);
+    QTRY(cudaGetLastError());
+    QTRY(cudaMemcpyAsync(host_out + r0 * Lc, x->spins, (size_t)n * Lc, cudaMemcpyDeviceToHost, x->stream));
+  }
   QTRY(cudaStreamSynchronize(x->stream));
   if (int st = quad_status(x)) return st;
   set_last_error("");

@@ -1,0 +1,47 @@
+"""Spins to and from the host: through a bounded device buffer, piece by piece, and on the host where that is faster."""
+import numpy as np
+import pytest
+
+import paper_2402_06415_gb300 as ising
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    ising.lib()
+
+
+def _free():
+    import torch
+
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+# one piece, a last piece of a few rows, and a size that is no multiple of a piece
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("L", [1448, 1450, 3002])
+def test_xy_round_trip_in_bounded_memory(precision, L):
+    rng = np.random.default_rng(L)
+    u = rng.standard_normal((L, L, 2)).astype(np.float32).astype(np.float64)  # exact in both precisions
+    with ising.XY(L, 1.0, precision, seed=1) as x:
+        before = _free()
+        x.set_spins(u)
+        assert np.array_equal(x.spins(), u)
+        assert before - _free() <= 40 << 20
+
+
+@pytest.mark.parametrize("Lc", [2, 31, 48, 49, 97, 2896, 3001])
+def test_quad_round_trip_in_bounded_memory(Lc):
+    rng = np.random.default_rng(Lc)
+    s = np.where(rng.integers(0, 2, (4, Lc, Lc)), 1, -1).astype(np.int8)
+    with ising.Quad(ising.ISING_QUAD_SQUARE, Lc, 0.44, 1.0, 0.5, seed=1) as x:
+        before = _free()
+        x.set_spins(s)
+        assert np.array_equal(x.spins(), s)
+        assert before - _free() <= 40 << 20
+
