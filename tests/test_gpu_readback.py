@@ -45,3 +45,19 @@ def test_quad_round_trip_in_bounded_memory(Lc):
         assert np.array_equal(x.spins(), s)
         assert before - _free() <= 40 << 20
 
+
+def test_small_quad_lattices_are_read_faster_than_larger_ones():
+    """32 x 32 cells are a quarter of 64 x 64, and the host unpacks them while a launch would be under way (unpacked on
+    the device, both took the same time)."""
+    import time
+
+    us = []
+    for Lc in (32, 64):
+        with ising.Quad(ising.ISING_QUAD_SQUARE, Lc, 0.44, 1.0, 0.5, seed=1) as x:
+            best = 1e30
+            for _ in range(300):
+                t0 = time.perf_counter()
+                x.spins()
+                best = min(best, time.perf_counter() - t0)
+            us.append(best * 1e6)
+    assert us[0] < 0.9 * us[1], us
