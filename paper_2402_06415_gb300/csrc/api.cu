@@ -396,9 +396,9 @@ int sweep_chunk(ising_ctx* c, int64_t t0, int n, int m) {
     a.rec_cap = kRecCap;
     a.rec = c->rec;
     a.xbuf = c->strip_x;
-    a.status = c->strip_status.wait();
-    a.limit = fault("wait") ? -1 : kClusterSpinLimit;
-    const cudaError_t e = launch_strip_sweep(a, rng, c->stream);
+    a.status = c->strip_status.word();
+    a.limit = c->strip_status.limit(kClusterSpinLimit);
+    const cudaError_t e = launch_strip_sweep(a, rng, c->strip_status.refuse, c->stream);
     if (strips_refused(e)) {
       if (c->kernel == ISING_KERNEL_TILED)
         if (int st = ensure_second_buffer(c)) return st;
@@ -477,7 +477,7 @@ int to_host_sync(ising_ctx* c, void* dst, const void* src, size_t bytes) {
 
 // The whole lattice is about to be written: a wait that gave up before no longer matters.
 int lattice_defined(ising_ctx* c) {
-  ++c->strip_status.epoch;
+  CUDA_TRY(c->strip_status.begin(c->stream));
   if (c->cluster_gctl) CUDA_TRY(cudaMemsetAsync(c->cluster_gctl, 0, sizeof(GridCtl), c->stream));
   return ISING_OK;
 }
@@ -498,7 +498,8 @@ void set_last_error(const char* msg) { g_err = msg ? msg : ""; }
 // fail, ISING_FAULT=launch sweep launches, ISING_FAULT=copy host<->device copies, all
 // without touching the GPU; ISING_FAULT=coop refuses the strips' cooperative launches, as a
 // stream with few SMs does; ISING_FAULT=wait gives strips no time for a wait that is
-// not over at once (they set the status and return).
+// not over at once (they set the status and return).  The last two are looked up when
+// the context is made and when its lattice is set.
 bool fault(const char* what) {
   const char* f = std::getenv("ISING_FAULT");
   return f && std::strstr(f, what) != nullptr;
@@ -1078,7 +1079,7 @@ int cluster_persist_run(ising_ctx* c, bool wolff, int64_t step0, int n, int meas
       cudaError_t e = launch_cluster_strip(c->lat(c->cur), wolff, (uint32_t)t, k, measure_every,
                                            n_rec ? (int)((before + 1) * m - t) : 0, bond_threshold(c->beta), c->rng(),
                                            G, c->cluster_strip, c->rec, c->rec_count % kRecCap, kRecCap, c->wolff,
-                                           c->strip_status.wait(), c->stream);
+                                           c->strip_status, c->stream);
       if (done == 0 && strips_refused(e)) {
         c->cluster_strips_refused = *refused = true;
         return ISING_OK;

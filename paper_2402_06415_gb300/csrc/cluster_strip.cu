@@ -52,7 +52,7 @@ struct ClusterStripArgs {
   unsigned int* flags;
   unsigned int* n_edges;
   WolffCtl* wctl;
-  WaitStatus status;
+  int* status;
   long long limit;
   FastDiv fL;
 };
@@ -145,9 +145,9 @@ __device__ __forceinline__ void sunite16(uint16_t* par, uint32_t a, uint32_t b) 
 // Grid barrier of up to kThreads CTAs, all resident: every CTA raises its flag and
 // polls everybody's, one thread per CTA, so it takes one store and one load through
 // L2 instead of an atomic, its answer and a load.  False after `limit` cycles
-// (and the status set).
+// (and *status = 1).
 __device__ __forceinline__ bool flag_barrier(unsigned int* flags, int G, unsigned int epoch, long long limit,
-                                             const WaitStatus& status) {
+                                             int* status) {
   __syncthreads();
   const int tid = threadIdx.x;
   if (tid == 0) {
@@ -159,7 +159,7 @@ __device__ __forceinline__ bool flag_barrier(unsigned int* flags, int G, unsigne
     const long long start = clock64();
     while (ld_acquire_gpu(flags + tid) < epoch) {
       if (clock64() - start > limit) {
-        gave_up(status);
+        *reinterpret_cast<volatile int*>(status) = 1;
         ok = false;
         break;
       }
@@ -460,7 +460,7 @@ size_t cluster_strip_bytes(int L, int G) {
 cudaError_t launch_cluster_strip(const BitsLattice& lat, bool wolff, uint32_t step0, int n_steps, int measure_every,
                                  int to_rec, uint32_t thr, const RngParams& rng, int G, void* scratch,
                                  unsigned long long* rec, long long rec0, long long rec_cap, WolffCtl* wctl,
-                                 const WaitStatus& status, cudaStream_t s) {
+                                 const StripStatus& status, cudaStream_t s) {
   ClusterStripArgs a{};
   a.planes = lat.planes;
   a.L = lat.L;
@@ -483,8 +483,8 @@ cudaError_t launch_cluster_strip(const BitsLattice& lat, bool wolff, uint32_t st
   a.flags = (unsigned int*)(a.xbuf + xwords);
   a.n_edges = a.flags + G;
   a.wctl = wctl;
-  a.status = status;
-  a.limit = fault("wait") ? -1 : kClusterSpinLimit;
+  a.status = status.word();
+  a.limit = status.limit(kClusterSpinLimit);
   a.fL = make_fastdiv((uint32_t)a.L);
   const size_t smem = strip_smem(a.L, G);
   const void* fns[4] = {(const void*)k_cluster_strip<false, false>, (const void*)k_cluster_strip<true, false>,
@@ -500,7 +500,7 @@ cudaError_t launch_cluster_strip(const BitsLattice& lat, bool wolff, uint32_t st
   if ((e = cudaMemsetAsync(a.xbuf, 0, zeroed, s))) return e;
   RngParams r = rng;
   void* args[] = {&a, &r};
-  return launch_strips(fn, G, kThreads, args, smem, s);
+  return launch_strips(fn, G, kThreads, args, smem, status.refuse, s);
 }
 
 }  // namespace ising

@@ -6,6 +6,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <cstdint>
+#include <cstring>
 
 namespace ising {
 
@@ -134,33 +135,51 @@ size_t tiled32_smem_bytes(int L, int k, int n_tile_rows, int tile_words);
 // planes or int8 spins (the other pointer null).  G row strips, one CTA each
 // (cooperative launch; needs L >= 2 K G), K sweeps between exchanges; K = 0: edge rows
 // exchanged every half sweep (needs L >= 2 G and 2 Wc <= kStripThreads).
-// What a strip writes to a host-visible word when a wait for a neighbour gave up.
-struct WaitStatus {
-  int* word;
-  int code;
-};
-// The host's side of it.  The code is the context's epoch, which every call that defines
-// the whole lattice raises: a launch that is still queued then reports an epoch that
-// is over, so the order on the stream decides and not the moment of the host's call.
+// Pinned words that a strip sets to 1 when a wait for a neighbour gave up: one for each
+// epoch of the context, and every call that defines the whole lattice begins a new one.  A
+// launch that is still queued then sets the word of an epoch that is over, so the order
+// on the stream decides and not the moment of the host's call.  (Kernels that write a
+// number of the epoch instead of 1 came out up to 9 % slower: other register
+// allocations, k_quad_strip with spills.)
+// Whether ISING_FAULT names this kind of failure (api.cu).
+bool fault(const char* what);
+
 struct StripStatus {
-  int* word = nullptr;  // pinned
-  int epoch = 1;
+  static constexpr int kEpochs = 1024;
+  int* words = nullptr;
+  int epoch = 0;
+  // injected failures, looked up when the context is made and when its lattice is set (a
+  // look at the environment per launch took 0.2 us): waits get no time, launches are refused
+  bool hurry = false, refuse = false;
+  long long limit(long long cycles) const { return hurry ? -1 : cycles; }
   cudaError_t ensure() {
-    if (word) return cudaSuccess;
-    const cudaError_t e = cudaHostAlloc((void**)&word, sizeof(int), cudaHostAllocDefault);
-    if (e != cudaSuccess) word = nullptr;
-    else *word = 0;
+    if (words) return cudaSuccess;
+    look_up();
+    const cudaError_t e = cudaHostAlloc((void**)&words, kEpochs * sizeof(int), cudaHostAllocDefault);
+    if (e != cudaSuccess) words = nullptr;
+    else std::memset(words, 0, kEpochs * sizeof(int));
     return e;
   }
   void release() {
-    cudaFreeHost(word);
-    word = nullptr;
+    cudaFreeHost(words);
+    words = nullptr;
   }
-  bool failed() const { return word && *(volatile int*)word == epoch; }
-  WaitStatus wait() const { return WaitStatus{word, epoch}; }
+  // The words are used again only after every launch that may set them is over.
+  cudaError_t begin(cudaStream_t s) {
+    look_up();
+    epoch = (epoch + 1) % kEpochs;
+    if (epoch != 0 || !words) return cudaSuccess;
+    const cudaError_t e = cudaStreamSynchronize(s);
+    std::memset(words, 0, kEpochs * sizeof(int));
+    return e;
+  }
+  int* word() const { return words ? words + epoch : nullptr; }
+  bool failed() const { return words && *(volatile int*)word(); }
+  void look_up() {
+    hurry = fault("wait");
+    refuse = fault("coop");
+  }
 };
-// Whether ISING_FAULT names this kind of failure (api.cu).
-bool fault(const char* what);
 // Sweeps or steps per launch of strips, by their modelled time: about 20 ms.  A cooperative
 // launch starts once all its SMs are free, so without a bound another context's strips
 // waited for the whole of a long call (0.9 s behind 2,000,000 sweeps on one SM; so
@@ -171,8 +190,9 @@ inline int strip_launch_sweeps(double us_per_sweep) {
 // cudaLaunchCooperativeKernel of strips.  A stream may have fewer SMs than the device
 // (a green context's); the launch is refused there (strips_refused) and the callers go on
 // with the kernels that run where strips do not fit.
-inline cudaError_t launch_strips(const void* fn, int grid, int threads, void** args, size_t smem, cudaStream_t s) {
-  if (fault("coop")) return cudaErrorCooperativeLaunchTooLarge;
+inline cudaError_t launch_strips(const void* fn, int grid, int threads, void** args, size_t smem, bool refuse,
+                                 cudaStream_t s) {
+  if (refuse) return cudaErrorCooperativeLaunchTooLarge;
   return cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args, smem, s);
 }
 inline bool strips_refused(cudaError_t e) {
@@ -192,7 +212,7 @@ struct StripArgs {
   long long rec0, rec_cap;  // ring slot of the first record
   unsigned long long* rec;
   unsigned long long* xbuf;  // strip_xbuf_words(L, G, K) words (G > 1), zeroed by the launcher
-  WaitStatus status;
+  int* status;         // host-visible word, set to 1 when a wait gave up
   long long limit;     // clock64 cycles a wait may take
   FastDiv fwc;         // set by the launcher
 };
@@ -206,7 +226,7 @@ constexpr int kStripMaxK = 8;
 StripShape choose_strip(int L, int sms);
 size_t strip_smem_bytes(int L, int G, int K);
 size_t strip_xbuf_words(int L, int G, int K);
-cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, cudaStream_t s);
+cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, bool refuse, cudaStream_t s);
 cudaError_t launch_measure_bits(const BitsLattice& lat, unsigned long long* out2,
                                 cudaStream_t s);
 cudaError_t launch_unpack_bits(const BitsLattice& lat, int8_t* spins, cudaStream_t s);
@@ -326,13 +346,13 @@ cudaError_t launch_cluster_persist(const BitsLattice& lat, bool wolff, uint32_t 
 // The same on resident row strips (cluster_strip.cu).  cluster_strip_grid: strips of
 // an L x L lattice (0: they do not fit in shared memory); scratch: device memory
 // of cluster_strip_bytes(L, G) bytes; the record slots are zero on entry; to_rec:
-// steps until the first record (0: none).
+// steps until the first record (0: none); status: of the context.
 int cluster_strip_grid(int L, int sms);
 size_t cluster_strip_bytes(int L, int G);
 cudaError_t launch_cluster_strip(const BitsLattice& lat, bool wolff, uint32_t step0, int n_steps, int measure_every,
                                  int to_rec, uint32_t thr, const RngParams& rng, int G, void* scratch,
                                  unsigned long long* rec, long long rec0, long long rec_cap, WolffCtl* wctl,
-                                 const WaitStatus& status, cudaStream_t s);
+                                 const StripStatus& status, cudaStream_t s);
 
 // Sets the message returned by ising_last_error() on the calling thread.
 void set_last_error(const char* msg);

@@ -343,16 +343,15 @@ __device__ __forceinline__ unsigned long long poll_word(const unsigned long long
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(slot) : "memory");
   return v;
 }
-__device__ __forceinline__ void gave_up(const WaitStatus& s) { *reinterpret_cast<volatile int*>(s.word) = s.code; }
-// Waits for the pair with this tag; false (and the status set) after `limit` cycles.
-__device__ __forceinline__ bool recv_word(const unsigned long long* slot, uint32_t tag, long long limit,
-                                          const WaitStatus& status, uint32_t& word) {
+// Waits for the pair with this tag; false (and *status = 1) after `limit` cycles.
+__device__ __forceinline__ bool recv_word(const unsigned long long* slot, uint32_t tag, long long limit, int* status,
+                                          uint32_t& word) {
   unsigned long long v = poll_word(slot);
   if ((uint32_t)(v >> 32) != tag) {
     const long long start = clock64();
     do {
       if (clock64() - start > limit) {
-        gave_up(status);
+        *reinterpret_cast<volatile int*>(status) = 1;
         return false;
       }
       v = poll_word(slot);
@@ -366,7 +365,7 @@ __device__ __forceinline__ bool recv_word(const unsigned long long* slot, uint32
 // trip is 0.4 us): src(i) is the slot, put(i, word) takes the word.
 template <int N, typename Src, typename Put>
 __device__ __forceinline__ void recv_words(int tid, int nth, int n, Src src, uint32_t tag, long long limit,
-                                           const WaitStatus& status, bool& ok, Put put) {
+                                           int* status, bool& ok, Put put) {
   for (int base = tid; base < n; base += N * nth) {
     unsigned long long v[N];
 #pragma unroll

@@ -539,7 +539,7 @@ StripShape choose_strip(int L, int sms) {
   return best;
 }
 
-cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, cudaStream_t s) {
+cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, bool refuse, cudaStream_t s) {
   const bool whole = a.G == 1, edge = a.K == 0, i8 = a.spins != nullptr;
   if (a.K > a.n) a.K = a.n;
   const size_t smem = strip_smem_bytes(a.L, a.G, a.K);
@@ -566,7 +566,7 @@ cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, cudaStream_t s
   if (whole) return cudaLaunchKernel(fns[which], dim3(1), dim3(threads), args, smem, s);
   cudaError_t e = cudaMemsetAsync(a.xbuf, 0, strip_xbuf_words(a.L, a.G, a.K) * 8, s);
   if (e != cudaSuccess) return e;
-  return launch_strips(fns[which], a.G, threads, args, smem, s);
+  return launch_strips(fns[which], a.G, threads, args, smem, refuse, s);
 }
 
 }  // namespace ising

@@ -458,7 +458,7 @@ struct XYStripArgs {
   long long rec0, rec_cap;
   unsigned long long* accepted;
   unsigned long long* xbuf;  // xy_strip_words(...) pairs, zeroed by the launcher (G > 1)
-  WaitStatus status;
+  int* status;
   long long limit;
   FastDiv fh;
 };
@@ -802,8 +802,8 @@ cudaError_t xy_strip_t(ising_xy* x, int n, int m) {
   a.rec_cap = kXYRec;
   a.accepted = x->accepted;
   a.xbuf = x->strip_x;
-  a.status = x->strip_status.wait();
-  a.limit = fault("wait") ? -1 : kXYSpinLimit;
+  a.status = x->strip_status.word();
+  a.limit = x->strip_status.limit(kXYSpinLimit);
   a.fh = make_fastdiv((uint32_t)(x->L / 2));
   const bool whole = a.G == 1;
   const long long sites = (long long)((a.L + a.G - 1) / a.G + (whole ? 0 : 2 * a.gh)) * (a.L / 2);
@@ -838,7 +838,7 @@ cudaError_t xy_strip_t(ising_xy* x, int n, int m) {
     e = cudaLaunchKernel(fns[which], dim3(1), dim3(threads), args, smem, x->stream);
   } else {
     e = cudaMemsetAsync(a.xbuf, 0, xy_strip_words<T>(a.L, a.G, a.gh) * 8, x->stream);
-    if (!e) e = launch_strips(fns[which], a.G, threads, args, smem, x->stream);
+    if (!e) e = launch_strips(fns[which], a.G, threads, args, smem, x->strip_status.refuse, x->stream);
   }
   if (e) return e;
   ++x->launches;
@@ -1036,7 +1036,7 @@ int ising_xy_seed(ising_xy* x, uint64_t seed) {
   x->sweep = 0;
   x->rec_count = 0;
   x->grid_used = false;
-  ++x->strip_status.epoch;
+  XTRY(x->strip_status.begin(x->stream));
   const RngParams rng = make_rng(seed, 0, 0, 0);
   const long long N = (long long)x->L * x->L;
   if (x->precision == 64)
@@ -1165,7 +1165,7 @@ int ising_xy_get_spins(ising_xy* x, double* host_uv) {
 
 int ising_xy_set_spins(ising_xy* x, const double* host_uv) {
   if (!x || !host_uv) return xfail(ISING_EINVAL, "null argument");
-  ++x->strip_status.epoch;
+  XTRY(x->strip_status.begin(x->stream));
   XTRY(cudaMemsetAsync(x->ctl, 0, sizeof(GridCtl), x->stream));
   cudaError_t e = xy_layout(x, const_cast<double*>(host_uv), true);
   if (e) return xfail(ISING_ECUDA, "set spins: %s", cudaGetErrorString(e));

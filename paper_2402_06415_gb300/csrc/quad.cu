@@ -359,7 +359,7 @@ struct QuadStripArgs {
   unsigned long long* rec;
   long long rec0, rec_cap;
   unsigned long long* xbuf;  // quad_strip_words(...) pairs, zeroed by the launcher
-  WaitStatus status;
+  int* status;
   long long limit;
 };
 constexpr int kQuadStripThreads = 512, kQuadStripMaxK = 4;
@@ -601,8 +601,8 @@ cudaError_t launch_quad_strip(ising_quad* x, int n, int m, const RngParams& rng)
   a.rec0 = x->rec_count % kQuadRec;
   a.rec_cap = kQuadRec;
   a.xbuf = x->strip_x;
-  a.status = x->strip_status.wait();
-  a.limit = fault("wait") ? -1 : kQuadSpinLimit;
+  a.status = x->strip_status.word();
+  a.limit = x->strip_status.limit(kQuadSpinLimit);
   cudaError_t e;
   int64_t n_rec = 0;
   if (m > 0) {
@@ -626,7 +626,7 @@ cudaError_t launch_quad_strip(ising_quad* x, int n, int m, const RngParams& rng)
   RngParams r = rng;
   QuadTable tab = x->tab;
   void* args[] = {&a, &r, &tab};
-  if ((e = launch_strips(fn, a.G, threads, args, smem, x->stream))) return e;
+  if ((e = launch_strips(fn, a.G, threads, args, smem, x->strip_status.refuse, x->stream))) return e;
   ++x->launches;
   x->rec_count += n_rec;
   return cudaSuccess;
@@ -794,7 +794,7 @@ int ising_quad_seed(ising_quad* x, uint64_t seed) {
   x->seed = seed;
   x->sweep = 0;
   x->rec_count = 0;
-  ++x->strip_status.epoch;
+  QTRY(x->strip_status.begin(x->stream));
   const RngParams rng = make_rng(seed, x->replica, 0, 0);
   k_quad_init<<<qgrid(4LL * x->Lc * x->geom.Wq), 256, 0, x->stream>>>(x->planes, x->geom, rng);
   QTRY(cudaGetLastError());
@@ -884,7 +884,7 @@ int ising_quad_set_spins(ising_quad* x, const int8_t* host_in) {
         if (v != 1 && v != -1) return qfail(ISING_EINVAL, "spins must be +1 or -1");
         if (v == 1) h[((size_t)q * Lc + Y) * Wq + (X >> 5)] |= 1u << (X & 31);
       }
-  ++x->strip_status.epoch;
+  QTRY(x->strip_status.begin(x->stream));
   QTRY(cudaMemcpyAsync(x->planes, h.data(), h.size() * 4, cudaMemcpyHostToDevice, x->stream));
   QTRY(cudaStreamSynchronize(x->stream));
   set_last_error("");

@@ -1,6 +1,6 @@
 """A wait between strips that runs out: the status reaches the caller, the context stays usable, and setting the
-lattice again (in stream order) clears it.  ISING_FAULT=wait gives the waits no time, so some give up at once; nothing
-hangs and nothing is read out of range: the strips set the status and return."""
+lattice again (in stream order) clears it.  A lattice set under ISING_FAULT=wait gives the waits no time, so some give up
+at once; nothing hangs and nothing is read out of range: the strips set the status and return."""
 import numpy as np
 import pytest
 
@@ -46,10 +46,15 @@ def _read(x):
     return x.series(0), x.spins().sum()
 
 
-def _give_up(x, step, monkeypatch):
+def _hurry(x, monkeypatch):
     monkeypatch.setenv("ISING_FAULT", "wait")
-    getattr(x, step)(60)
+    x.seed(4)
     monkeypatch.delenv("ISING_FAULT")
+
+
+def _give_up(x, step, monkeypatch):
+    _hurry(x, monkeypatch)
+    getattr(x, step)(60)
 
 
 def _times_out(x):
@@ -83,13 +88,14 @@ def test_cleared_by_setting_the_spins(case, monkeypatch):
 
 @pytest.mark.parametrize("case", ["split", "edge", "xy32", "quad"])
 def test_a_seed_clears_what_is_still_queued(case, monkeypatch):
-    """The call that gives up is still behind a long one when the host seeds the context again."""
+    """The call that gives up is still behind a long one on the stream when the host seeds its context again."""
     make, step = CASES[case]
-    with make() as x:
-        x.sweep(2)
+    with make() as x, _lattice(256, BITS)() as other:  # both on the default stream
+        _read(x), other.measure()
+        _hurry(x, monkeypatch)
         _read(x)
-        x.sweep(20000)
-        _give_up(x, step, monkeypatch)
+        other.sweep(20000)
+        getattr(x, step)(60)
         x.seed(5)
         _read(x)
 
@@ -107,3 +113,15 @@ def test_bits_and_device_forms_clear_it_too(monkeypatch):
             assert _times_out(x)
             put()
             assert np.array_equal(x.bits(), words)
+
+
+def test_a_status_word_that_is_used_again_is_clear(monkeypatch):
+    """The context has 1024 status words, one after the other for each lattice that is set."""
+    with ising.Lattice(256, 0.44, BITS, seed=3) as x:
+        _give_up(x, "sweep", monkeypatch)
+        assert _times_out(x)
+        for k in range(1024):
+            x.seed(k)
+        _read(x)
+        x.sweep(20)
+        _read(x)
