@@ -90,3 +90,12 @@ def test_default_decomposition_loses_to_no_other(Ls):
                 ising.ising_batch_set_kernel(b.h, words, threads)
                 other[words, threads] = _ms(b, 20)
     assert auto < 1.15 * min(other.values()), (auto, other)
+
+
+def test_a_small_batch_does_not_take_a_large_one_its_shared_memory():
+    with _batch(1024, 2) as large:
+        large.run(1)
+        with _batch(16, 2) as small:
+            small.run(1)
+            large.run(1)
+            assert ising.ising_batch_status(large.h) == (0, 2) and ising.ising_batch_status(small.h) == (0, 1)
