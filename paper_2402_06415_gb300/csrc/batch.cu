@@ -595,12 +595,8 @@ int make_plan(const ising_batch* b, int words_per_item, int threads, ItemPlan* p
   const int n = (int)words.size();
   p->smem = 2 * (size_t)*std::max_element(words.begin(), words.end()) * sizeof(uint32_t);
   if (p->smem > 200 * 1024) return bfail(ISING_EINVAL, "an item needs %zu B of shared memory", p->smem);
-  // the limit belongs to the kernel and not to a batch: only ever raised
   static DeviceCache configured;
-  if ((long long)p->smem > configured.get()) {
-    BTRY(cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->smem));
-    configured.set((long long)p->smem);
-  }
+  BTRY(allow_dynamic_smem((const void*)k_batch, configured));
   int dev = 0, sms = 0, per_sm = 0;
   BTRY(cudaGetDevice(&dev));
   BTRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

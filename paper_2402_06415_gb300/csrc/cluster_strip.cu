@@ -493,10 +493,7 @@ cudaError_t launch_cluster_strip(const BitsLattice& lat, bool wolff, uint32_t st
   const void* fn = fns[which];
   static DeviceCache configured[4];
   cudaError_t e;
-  if ((long long)smem > configured[which].get()) {
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-    configured[which].set((long long)smem);
-  }
+  if ((e = allow_dynamic_smem(fn, configured[which]))) return e;
   if ((e = cudaMemsetAsync(a.xbuf, 0, zeroed, s))) return e;
   RngParams r = rng;
   void* args[] = {&a, &r};

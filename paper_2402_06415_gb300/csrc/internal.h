@@ -71,6 +71,21 @@ struct DeviceCache {
   void set(long long x) { v[device()].store(x, std::memory_order_relaxed); }
 };
 
+// Lets a kernel launch with as much dynamic shared memory as a block may have; `done` is
+// the kernel's own.  The limit belongs to the kernel and not to a launch, so it is set once
+// and to the same value by every thread: set to each launch's need, a thread with a
+// small lattice could lower it between another thread's call and its launch.
+inline cudaError_t allow_dynamic_smem(const void* fn, DeviceCache& done) {
+  if (done.get()) return cudaSuccess;
+  cudaFuncAttributes a;
+  int most = 0;
+  cudaError_t e = cudaFuncGetAttributes(&a, fn);
+  if (!e) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, DeviceCache::device());
+  if (!e) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
+  if (!e) done.set(1);
+  return e;
+}
+
 // Unsigned 32-bit division by a divisor fixed per launch, as a multiply-high, an
 // add and a shift (Granlund & Montgomery, PLDI 1994, the round-up method):
 // l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1, n / d = (mulhi(m, n) + n) >> l,

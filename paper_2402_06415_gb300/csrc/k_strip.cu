@@ -553,18 +553,15 @@ cudaError_t launch_strip_sweep(StripArgs a, const RngParams& rng, bool refuse, c
   a.fwc = make_fastdiv((uint32_t)a.Wc);
   const int which = edge ? (i8 ? 9 : 8) : (whole ? 1 : 0) + (i8 ? 2 : 0) + (split ? 4 : 0);
   static DeviceCache configured[10];
-  if ((long long)smem > configured[which].get()) {
-    cudaError_t e = cudaFuncSetAttribute(fns[which], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured[which].set((long long)smem);
-  }
+  cudaError_t e = allow_dynamic_smem(fns[which], configured[which]);
+  if (e != cudaSuccess) return e;
   int threads = (((split ? 4 : 1) * words + 31) / 32) * 32;
   if (threads < 64) threads = 64;
   if (!split && threads > kStripThreads) threads = kStripThreads;
   RngParams r = rng;
   void* args[] = {&a, &r};
   if (whole) return cudaLaunchKernel(fns[which], dim3(1), dim3(threads), args, smem, s);
-  cudaError_t e = cudaMemsetAsync(a.xbuf, 0, strip_xbuf_words(a.L, a.G, a.K) * 8, s);
+  e = cudaMemsetAsync(a.xbuf, 0, strip_xbuf_words(a.L, a.G, a.K) * 8, s);
   if (e != cudaSuccess) return e;
   return launch_strips(fns[which], a.G, threads, args, smem, refuse, s);
 }

@@ -816,12 +816,8 @@ cudaError_t xy_strip_t(ising_xy* x, int n, int m) {
                         (const void*)k_xy_strip<T, false, true>, (const void*)k_xy_strip<T, true, true>};
   const int which = (whole ? 1 : 0) + (ahead ? 2 : 0);
   static DeviceCache configured[4];
-  cudaError_t e;
-  if ((long long)smem > configured[which].get()) {
-    e = cudaFuncSetAttribute(fns[which], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e) return e;
-    configured[which].set((long long)smem);
-  }
+  cudaError_t e = allow_dynamic_smem(fns[which], configured[which]);
+  if (e) return e;
   // records of this launch: zeroed, then summed into by every CTA
   int64_t n_rec = 0;
   if (m > 0) {

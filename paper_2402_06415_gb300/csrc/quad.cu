@@ -616,10 +616,7 @@ cudaError_t launch_quad_strip(ising_quad* x, int n, int m, const RngParams& rng)
   const size_t smem = quad_strip_smem(a.g, a.G, a.K);
   const void* fn = (const void*)k_quad_strip<LAT, NV>;
   static DeviceCache configured;
-  if ((long long)smem > configured.get()) {
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-    configured.set((long long)smem);
-  }
+  if ((e = allow_dynamic_smem(fn, configured))) return e;
   const long long words = (long long)((a.g.Lc + a.G - 1) / a.G + 2 * a.K - 1) * a.g.Wq;
   const int threads = (int)std::min<long long>(kQuadStripThreads, std::max(64LL, (words + 31) / 32 * 32));
   if ((e = cudaMemsetAsync(a.xbuf, 0, quad_strip_words(a.g, a.G, a.K) * 8, x->stream))) return e;
