@@ -24,9 +24,10 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <new>
-#include <queue>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "internal.h"
@@ -580,20 +581,29 @@ struct ItemPlan {
 };
 
 int make_plan(const ising_batch* b, int words_per_item, int threads, ItemPlan* p) {
-  std::vector<long long> words;  // per colour plane
+  // items of one size that follow each other
+  struct Run {
+    long long words;  // of an item's colour plane
+    int first, n;
+  };
+  std::vector<Run> runs;
+  int n = 0;
+  long long most = 0;
   for (int l = 0; l < b->n_ladders; ++l) {
     const int per = words_per_replica(b->L[l]) / 2;
     const int nr = std::min(std::max(1, words_per_item / std::max(per, 1)), kMaxRepPerItem);
-    for (int i0 = 0; i0 < b->n_beta; i0 += nr) {
+    for (int i0 = 0; i0 < b->n_beta; i0 += nr, ++n) {
       const int k = std::min(nr, b->n_beta - i0);
       p->ladder.push_back(l);
       p->i0.push_back(i0);
       p->nr.push_back(k);
-      words.push_back((long long)k * per);
+      const long long words = (long long)k * per;
+      most = std::max(most, words);
+      if (!runs.empty() && runs.back().words == words) ++runs.back().n;
+      else runs.push_back({words, n, 1});
     }
   }
-  const int n = (int)words.size();
-  p->smem = 2 * (size_t)*std::max_element(words.begin(), words.end()) * sizeof(uint32_t);
+  p->smem = 2 * (size_t)most * sizeof(uint32_t);
   if (p->smem > 200 * 1024) return bfail(ISING_EINVAL, "an item needs %zu B of shared memory", p->smem);
   static DeviceCache configured;
   BTRY(allow_dynamic_smem((const void*)k_batch, configured));
@@ -606,30 +616,42 @@ int make_plan(const ising_batch* b, int words_per_item, int threads, ItemPlan* p
   if (b->grid > 0) grid = std::min(grid, b->grid);
   grid = std::max(1, std::min(grid, std::max(n, b->n_ladders)));
   p->grid = grid;
-  std::vector<int> order(n);
-  for (int j = 0; j < n; ++j) order[j] = j;
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return words[x] > words[y]; });
+  // largest first to the least loaded CTA, the first of them among equals: the first `grid`
+  // items have a CTA each, in order; from then on a heap, whose top takes the item in place
+  std::stable_sort(runs.begin(), runs.end(), [](const Run& x, const Run& y) { return x.words > y.words; });
   using P = std::pair<long long, int>;
-  std::priority_queue<P, std::vector<P>, std::greater<P>> pq;
-  for (int c = 0; c < grid; ++c) pq.push({0, c});
-  std::vector<std::vector<int>> per_cta(grid);
-  for (int j : order) {
-    P top = pq.top();
-    pq.pop();
-    per_cta[top.second].push_back(j);
-    pq.push({top.first + words[j], top.second});
-  }
-  p->first.assign(grid + 1, 0);
-  double passes = 0;
-  for (int c = 0; c < grid; ++c) {
-    p->first[c] = (int)p->items.size();
-    p->items.insert(p->items.end(), per_cta[c].begin(), per_cta[c].end());
-    double t = 0;
-    for (int j : per_cta[c]) t += std::max(0.5 * (double)words[j] / threads, 1.0);
-    passes = std::max(passes, t);
-  }
-  p->first[grid] = (int)p->items.size();
-  p->cost = passes * (2.0 + (double)((grid + sms - 1) / sms) * threads / 128.0);
+  std::vector<P> heap(grid);
+  for (int c = 0; c < grid; ++c) heap[c] = {0, c};
+  std::vector<int> order(n), cta(n), count(grid, 0);
+  std::vector<double> passes(grid, 0.0);
+  int at = 0;
+  for (const Run& r : runs)
+    for (int j = 0; j < r.n; ++j, ++at) {
+      if (at == grid) std::make_heap(heap.begin(), heap.end(), std::greater<P>());
+      const int slot = at < grid ? at : 0, c = heap[slot].second;
+      order[at] = r.first + j;
+      cta[at] = c;
+      ++count[c];
+      passes[c] += std::max(0.5 * (double)r.words / threads, 1.0);
+      heap[slot].first += r.words;
+      if (at < grid) continue;
+      const P x = heap[0];
+      int k = 0;
+      for (int l = 1; l < grid; l = 2 * k + 1) {
+        if (l + 1 < grid && heap[l + 1] < heap[l]) ++l;
+        if (!(heap[l] < x)) break;
+        heap[k] = heap[l];
+        k = l;
+      }
+      heap[k] = x;
+    }
+  p->first.resize(grid + 1);
+  p->first[0] = 0;
+  for (int c = 0; c < grid; ++c) p->first[c + 1] = p->first[c] + count[c];
+  p->items.resize(n);
+  std::vector<int> next(p->first.begin(), p->first.end() - 1);
+  for (int k = 0; k < n; ++k) p->items[next[cta[k]]++] = order[k];
+  p->cost = *std::max_element(passes.begin(), passes.end()) * (2.0 + (double)((grid + sms - 1) / sms) * threads / 128.0);
   return ISING_OK;
 }
 
@@ -642,14 +664,13 @@ int make_plan(const ising_batch* b, int words_per_item, int threads, ItemPlan* p
 // 16 .. 128 squared 218 / 272 / 208 / 224, 8192 of 64 squared 337 / 349 / 402 / 341, 1024 of 128
 // squared 231 / 215 / 154 / 231, 64 of 256 squared 124 / 99 / 124 / 99, 64 of 1024 squared 1577 / 1124 /
 // 1578 / 1124: a replica is never split, so a large one wants the larger CTA.
-int choose_items(ising_batch* b) {
-  double best = 0;
+int choose_items(ising_batch* b, ItemPlan* best) {
   for (int words : {256, 512})
     for (int threads : {128, 256}) {
       ItemPlan p;
       if (int st = make_plan(b, words, threads, &p)) return st;
-      if (best == 0 || p.cost < best) {
-        best = p.cost;
+      if (best->grid == 0 || p.cost < best->cost) {
+        *best = std::move(p);
         b->words_per_item = words;
         b->threads = threads;
       }
@@ -657,10 +678,8 @@ int choose_items(ising_batch* b) {
   return ISING_OK;
 }
 
-// Plans the items of the batch's decomposition and hands them to the device.
-int plan_items(ising_batch* b) {
-  ItemPlan p;
-  if (int st = make_plan(b, b->words_per_item, b->threads, &p)) return st;
+// Hands a plan's items to the device.
+int use_plan(ising_batch* b, const ItemPlan& p) {
   b->n_items = (int)p.nr.size();
   b->smem = p.smem;
   b->grid_used = p.grid;
@@ -807,8 +826,11 @@ int ising_batch_create(ising_batch** out, int n_ladders, const int* L, int n_bet
     if (!e) e = cudaMemset(b->d_ctr, 0, sizeof(BatchCounters));
     if (e) st = bfail(ISING_ECUDA, "batch setup copy: %s", cudaGetErrorString(e));
   }
-  if (!st) st = choose_items(b);
-  if (!st) st = plan_items(b);
+  if (!st) {
+    ItemPlan plan;
+    st = choose_items(b, &plan);
+    if (!st) st = use_plan(b, plan);
+  }
   if (st) {
     bfree(b);
     delete b;
@@ -858,7 +880,9 @@ int ising_batch_set_kernel(ising_batch* b, int words_per_item, int threads, int 
     b->graph = nullptr;
     b->graph_sweeps = -1;
   }
-  if (int st = plan_items(b)) return st;
+  ItemPlan plan;
+  if (int st = make_plan(b, b->words_per_item, b->threads, &plan)) return st;
+  if (int st = use_plan(b, plan)) return st;
   set_last_error("");
   return ISING_OK;
 }
