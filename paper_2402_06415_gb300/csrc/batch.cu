@@ -632,7 +632,7 @@ int make_plan(const ising_batch* b, int words_per_item, int threads, ItemPlan* p
       order[at] = r.first + j;
       cta[at] = c;
       ++count[c];
-      passes[c] += std::max(0.5 * (double)r.words / threads, 1.0);
+      passes[c] += std::max(0.5 * (double)r.words / threads, 1.0) + 0.01;  // of equals, the fewer items
       heap[slot].first += r.words;
       if (at < grid) continue;
       const P x = heap[0];
@@ -658,9 +658,11 @@ int make_plan(const ising_batch* b, int words_per_item, int threads, ItemPlan* p
 // Default decomposition: of 256 or 512 words an item and 128 or 256 threads a CTA, the
 // pair with the least cost: passes over word pairs that the fullest CTA makes, times
 // the time of a pass, which grows with the warps that share an SM sub-partition (about
-// as 2 + warps).  Measured on 100 batches (L = 16 .. 1024, 4 .. 8192 replicas, one size and
-// mixed): 0.6 % above the best of the four on average, 3 % above it at the 90th
-// percentile.  us for 20 sweeps, (256, 128) / (256, 256) / (512, 128) / (512, 256): 4096 replicas of
+// as 2 + warps).  Two items of one pass take longer than one of two (4096 replicas 220 and
+// 210 us), so equal plans are told apart by their items.  Measured on 120 batches (L = 8 .. 512,
+// 4 .. 8192 replicas, one size and mixed): 0.3 % above the best of the four on average, 1.7 % at
+// the 95th percentile, 3 % at most (10 % where the first of equals was taken).
+// us for 20 sweeps, (256, 128) / (256, 256) / (512, 128) / (512, 256): 4096 replicas of
 // 16 .. 128 squared 218 / 272 / 208 / 224, 8192 of 64 squared 337 / 349 / 402 / 341, 1024 of 128
 // squared 231 / 215 / 154 / 231, 64 of 256 squared 124 / 99 / 124 / 99, 64 of 1024 squared 1577 / 1124 /
 // 1578 / 1124: a replica is never split, so a large one wants the larger CTA.

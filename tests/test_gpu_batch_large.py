@@ -99,3 +99,12 @@ def test_a_small_batch_does_not_take_a_large_one_its_shared_memory():
             small.run(1)
             large.run(1)
             assert ising.ising_batch_status(large.h) == (0, 2) and ising.ising_batch_status(small.h) == (0, 1)
+
+
+def test_of_equal_plans_the_one_with_fewer_items():
+    """64 ladders of 64 replicas of 16 .. 128 squared: items of 512 words are one for a CTA, those of 256 up to two (5 % slower)."""
+    from paper_2402_06415_gb300 import workloads
+
+    with ising.Batch(workloads.batch_ladder_sizes(64, 6), workloads.batch_betas(64), workloads.BATCH_PT_EVERY) as b:
+        info = ising.ising_batch_info(b.h)
+        assert info["items"] == info["grid"]
