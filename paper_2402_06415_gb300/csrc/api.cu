@@ -12,6 +12,8 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -70,7 +72,8 @@ struct ising_ctx {
   int64_t sweep = 0;
   cudaStream_t stream = nullptr;
   int Wc = 0;
-  uint32_t* bits[2] = {nullptr, nullptr};
+  void* mem = nullptr;  // lattice, records and exchange buffer of the automatic strips, in one allocation
+  uint32_t* bits[2] = {nullptr, nullptr};  // bits[0] lies in mem
   int cur = 0;
   int8_t* spins = nullptr;
   unsigned long long* rec = nullptr;  // [kRecCap][2]: anti-bond count, up-spin count
@@ -79,6 +82,7 @@ struct ising_ctx {
   // resident strips (the automatic choice where they are the fastest; G = 0: not used)
   StripShape strip{0, 0, 0.0};
   unsigned long long* strip_x = nullptr;  // boundary exchange buffer (G > 1)
+  bool strip_x_own = false;               // strip_x does not lie in mem
   StripStatus strip_status;
   bool strip_asked = false;               // the caller chose strips: for calls of one sweep too
   int kernel = ISING_KERNEL_HALF, k = 1, tile_rows = 1, tile_words = 4, grid = 0, block = 0;
@@ -131,12 +135,10 @@ void free_all(ising_ctx* c) {
   if (!c) return;
   for (auto e : c->ev) cudaEventDestroy(e);
   c->ev.clear();
-  cudaFree(c->bits[0]);
+  cudaFree(c->mem);
   cudaFree(c->bits[1]);
-  cudaFree(c->spins);
-  cudaFree(c->rec);
-  cudaFree(c->meas);
-  cudaFree(c->strip_x);
+  if (c->strip_x_own) cudaFree(c->strip_x);
+  c->mem = nullptr;
   c->strip_x = nullptr;
   c->strip_status.release();
   cudaFree(c->nn_w);
@@ -246,6 +248,7 @@ int ensure_strip(ising_ctx* c, const StripShape& shape) {
   void* p = nullptr;
   int st = dev_alloc(&p, strip_xbuf_words(c->L, shape.G, shape.K) * sizeof(unsigned long long));
   c->strip_x = (unsigned long long*)p;
+  c->strip_x_own = true;
   return st;
 }
 
@@ -494,6 +497,61 @@ int to_device_sync(ising_ctx* c, void* dst, const void* src, size_t bytes) {
 namespace ising {
 void set_last_error(const char* msg) { g_err = msg ? msg : ""; }
 
+// Pinned pages are dear: allocating and freeing them for each context took 300 us, twice
+// as long as everything else that creating a lattice does.  Contexts take blocks of slabs of 128 KB.
+// A slab is freed with its last block, unless it is the only one.
+namespace {
+struct StatusSlab {
+  static constexpr int kBlocks = 32, kWords = StripStatus::kEpochs;
+  int* base;
+  uint32_t used;
+  StatusSlab* next;
+};
+std::mutex g_slab_mutex;
+StatusSlab* g_slabs = nullptr;
+}  // namespace
+
+cudaError_t take_status_words(int** words, int n) {
+  *words = nullptr;
+  if (n > StatusSlab::kWords) return cudaErrorInvalidValue;
+  std::lock_guard<std::mutex> lock(g_slab_mutex);
+  StatusSlab* s = g_slabs;
+  while (s && s->used == 0xffffffffu) s = s->next;
+  if (!s) {
+    s = new (std::nothrow) StatusSlab{nullptr, 0u, g_slabs};
+    if (!s) return cudaErrorMemoryAllocation;
+    const cudaError_t e =
+        cudaHostAlloc((void**)&s->base, StatusSlab::kBlocks * StatusSlab::kWords * sizeof(int), cudaHostAllocPortable);
+    if (e != cudaSuccess) {
+      delete s;
+      return e;
+    }
+    g_slabs = s;
+  }
+  int k = 0;
+  while (s->used >> k & 1u) ++k;
+  s->used |= 1u << k;
+  *words = s->base + k * StatusSlab::kWords;
+  std::memset(*words, 0, StatusSlab::kWords * sizeof(int));
+  return cudaSuccess;
+}
+
+void give_status_words(int* words) {
+  if (!words) return;
+  std::lock_guard<std::mutex> lock(g_slab_mutex);
+  for (StatusSlab** p = &g_slabs; *p; p = &(*p)->next) {
+    StatusSlab* const s = *p;
+    if (words < s->base || words >= s->base + StatusSlab::kBlocks * StatusSlab::kWords) continue;
+    s->used &= ~(1u << ((words - s->base) / StatusSlab::kWords));
+    if (s->used == 0u && g_slabs->next) {
+      *p = s->next;
+      cudaFreeHost(s->base);
+      delete s;
+    }
+    return;
+  }
+}
+
 // Fault injection for the failure-path tests: ISING_FAULT=alloc makes device allocations
 // fail, ISING_FAULT=launch sweep launches, ISING_FAULT=copy host<->device copies, all
 // without touching the GPU; ISING_FAULT=coop refuses the strips' cooperative launches, as a
@@ -545,26 +603,24 @@ int ising_create(ising_ctx** out, int L, double beta, int layout, void* stream) 
     delete c;
     return fail(ISING_ECUDA, "no usable CUDA device: %s", cudaGetErrorString(e));
   }
-  void* p = nullptr;
-  if (layout == ISING_LAYOUT_BITS) {
-    st = dev_alloc(&p, c->plane_words() * sizeof(uint32_t));
-    c->bits[0] = (uint32_t*)p;
-  } else {
-    st = dev_alloc(&p, (size_t)c->N());
-    c->spins = (int8_t*)p;
-  }
+  resolve_auto(c);
+  // one allocation: each that starts a 2 MB page of its own takes 80 us
+  const StripShape& sh = c->strip;
+  const size_t sizes[4] = {layout == ISING_LAYOUT_BITS ? c->plane_words() * sizeof(uint32_t) : (size_t)c->N(),
+                           (size_t)kRecCap * 2 * sizeof(unsigned long long), 2 * sizeof(unsigned long long),
+                           sh.G > 1 ? strip_xbuf_words(L, sh.G, sh.K) * sizeof(unsigned long long) : 0};
+  size_t at[5] = {0};
+  for (int k = 0; k < 4; ++k) at[k + 1] = at[k] + (sizes[k] + 255) / 256 * 256;
+  st = dev_alloc(&c->mem, at[4]);
   if (!st) {
-    st = dev_alloc(&p, (size_t)kRecCap * 2 * sizeof(unsigned long long));
-    c->rec = (unsigned long long*)p;
-  }
-  if (!st) {
-    st = dev_alloc(&p, 2 * sizeof(unsigned long long));
-    c->meas = (unsigned long long*)p;
-  }
-  if (!st) {
-    resolve_auto(c);
-    st = ensure_strip(c, c->strip);
-    if (!st && c->kernel == ISING_KERNEL_TILED && c->strip.G == 0) st = ensure_second_buffer(c);
+    char* const m = (char*)c->mem;
+    if (layout == ISING_LAYOUT_BITS) c->bits[0] = (uint32_t*)m;
+    else c->spins = (int8_t*)m;
+    c->rec = (unsigned long long*)(m + at[1]);
+    c->meas = (unsigned long long*)(m + at[2]);
+    if (sh.G > 1) c->strip_x = (unsigned long long*)(m + at[3]);
+    st = ensure_strip(c, sh);
+    if (!st && c->kernel == ISING_KERNEL_TILED && sh.G == 0) st = ensure_second_buffer(c);
   }
   if (!st) {
     // all -1 start: zero bits / int8 0xff

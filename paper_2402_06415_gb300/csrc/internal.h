@@ -156,6 +156,9 @@ size_t tiled32_smem_bytes(int L, int k, int n_tile_rows, int tile_words);
 // on the stream decides and not the moment of the host's call.  (Kernels that write a
 // number of the epoch instead of 1 came out up to 9 % slower: other register
 // allocations, k_quad_strip with spills.)
+// Pinned, cleared words for one context, and back (api.cu).
+cudaError_t take_status_words(int** words, int n);
+void give_status_words(int* words);
 // Whether ISING_FAULT names this kind of failure (api.cu).
 bool fault(const char* what);
 
@@ -170,13 +173,11 @@ struct StripStatus {
   cudaError_t ensure() {
     if (words) return cudaSuccess;
     look_up();
-    const cudaError_t e = cudaHostAlloc((void**)&words, kEpochs * sizeof(int), cudaHostAllocDefault);
-    if (e != cudaSuccess) words = nullptr;
-    else std::memset(words, 0, kEpochs * sizeof(int));
-    return e;
+    return take_status_words(&words, kEpochs);
   }
+  // After the context's last launch is over.
   void release() {
-    cudaFreeHost(words);
+    give_status_words(words);
     words = nullptr;
   }
   // The words are used again only after every launch that may set them is over.

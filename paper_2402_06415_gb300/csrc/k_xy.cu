@@ -991,14 +991,9 @@ int ising_xy_create(ising_xy** out, int L, double beta, int precision, void* str
   x->precision = precision;
   x->stream = (cudaStream_t)stream;
   const size_t bytes = (size_t)L * L * (precision == 64 ? 16 : 8);
-  cudaError_t e = cudaMalloc(&x->u, bytes);
-  if (!e) e = cudaMalloc((void**)&x->rec, kXYRec * 3 * sizeof(double));
-  if (!e) e = cudaMalloc((void**)&x->accepted, sizeof(unsigned long long));
-  if (!e) e = cudaMemset(x->accepted, 0, sizeof(unsigned long long));
-  if (!e) e = cudaMalloc((void**)&x->ctl, sizeof(GridCtl));
-  if (!e) e = cudaMemset(x->ctl, 0, sizeof(GridCtl));
   int dev = 0, sms = 0;
-  if (!e) e = cudaGetDevice(&dev);
+  size_t strip_words = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (!e && L <= kXYStripMaxL) {
     const XYStrip st = precision == 64 ? choose_xy_strip<double>(L, sms) : choose_xy_strip<float>(L, sms);
@@ -1006,19 +1001,28 @@ int ising_xy_create(ising_xy** out, int L, double beta, int precision, void* str
     x->strip_gh = st.gh;
     x->strip_us = st.us;
     if (st.G > 1) {
-      const size_t words = precision == 64 ? xy_strip_words<double>(L, st.G, st.gh) : xy_strip_words<float>(L, st.G, st.gh);
-      e = cudaMalloc((void**)&x->strip_x, words * sizeof(unsigned long long));
-      if (!e) e = x->strip_status.ensure();
+      strip_words = precision == 64 ? xy_strip_words<double>(L, st.G, st.gh) : xy_strip_words<float>(L, st.G, st.gh);
+      e = x->strip_status.ensure();
     }
+  }
+  // one allocation: each that starts a 2 MB page of its own takes 80 us
+  const size_t sizes[5] = {bytes, kXYRec * 3 * sizeof(double), strip_words * sizeof(unsigned long long),
+                           sizeof(unsigned long long), sizeof(GridCtl)};
+  size_t at[6] = {0};
+  for (int k = 0; k < 5; ++k) at[k + 1] = at[k] + (sizes[k] + 255) / 256 * 256;
+  if (!e) e = cudaMalloc(&x->u, at[5]);
+  if (!e) {
+    char* const m = (char*)x->u;
+    x->rec = (double*)(m + at[1]);
+    if (strip_words) x->strip_x = (unsigned long long*)(m + at[2]);
+    x->accepted = (unsigned long long*)(m + at[3]);
+    x->ctl = (GridCtl*)(m + at[4]);
+    e = cudaMemset(x->accepted, 0, at[5] - at[3]);
   }
   if (e) {
     cudaGetLastError();
-    cudaFree(x->strip_x);
     x->strip_status.release();
     cudaFree(x->u);
-    cudaFree(x->rec);
-    cudaFree(x->accepted);
-    cudaFree(x->ctl);
     delete x;
     return xfail(ISING_ENOMEM, "XY allocation: %s", cudaGetErrorString(e));
   }
@@ -1184,10 +1188,6 @@ int ising_xy_destroy(ising_xy* x) {
   if (!x) return ISING_OK;
   cudaStreamSynchronize(x->stream);
   cudaFree(x->u);
-  cudaFree(x->rec);
-  cudaFree(x->accepted);
-  cudaFree(x->ctl);
-  cudaFree(x->strip_x);
   cudaFree(x->host_layout);
   x->strip_status.release();
   delete x;

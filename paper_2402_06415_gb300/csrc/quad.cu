@@ -763,22 +763,26 @@ int ising_quad_create(ising_quad** out, int lattice, int Lc, double beta, double
     return qfail(ISING_EINTERNAL, "threshold table overflow");
   }
   const size_t bytes = (size_t)4 * Lc * x->geom.Wq * sizeof(uint32_t);
-  cudaError_t e = cudaMalloc((void**)&x->planes, bytes);
-  if (!e) e = cudaMalloc((void**)&x->rec, kQuadRec * 3 * sizeof(unsigned long long));
   int dev = 0, sms = 0;
-  if (!e) e = cudaGetDevice(&dev);
+  size_t strip_words = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (!e) choose_quad_strip(x->geom, sms, &x->strip_G, &x->strip_K, &x->strip_us);
   if (!e && x->strip_G > 0) {
-    e = cudaMalloc((void**)&x->strip_x, quad_strip_words(x->geom, x->strip_G, x->strip_K) * sizeof(unsigned long long));
-    if (!e) e = x->strip_status.ensure();
+    strip_words = quad_strip_words(x->geom, x->strip_G, x->strip_K);
+    e = x->strip_status.ensure();
+  }
+  // one allocation: each that starts a 2 MB page of its own takes 80 us
+  const size_t at_rec = (bytes + 255) / 256 * 256, at_x = at_rec + kQuadRec * 3 * sizeof(unsigned long long);
+  if (!e) e = cudaMalloc((void**)&x->planes, at_x + strip_words * sizeof(unsigned long long));
+  if (!e) {
+    x->rec = (unsigned long long*)((char*)x->planes + at_rec);
+    if (strip_words) x->strip_x = (unsigned long long*)((char*)x->planes + at_x);
   }
   if (e) {
     cudaGetLastError();
-    cudaFree(x->strip_x);
     x->strip_status.release();
     cudaFree(x->planes);
-    cudaFree(x->rec);
     delete x;
     return qfail(ISING_ENOMEM, "quad allocation: %s", cudaGetErrorString(e));
   }
@@ -898,8 +902,6 @@ int ising_quad_destroy(ising_quad* x) {
   if (!x) return ISING_OK;
   cudaStreamSynchronize(x->stream);
   cudaFree(x->planes);
-  cudaFree(x->rec);
-  cudaFree(x->strip_x);
   x->strip_status.release();
   cudaFree(x->spins);
   delete x;
