@@ -187,11 +187,13 @@ bool strip_applies(int layout, int L) {
 // load and store the whole lattice and clear the exchange buffer first.  us per call,
 // strips / half sweeps: packed L = 128 6.5 / 8.2, 256 to 1280 10.3 / 8.2, 2048 12.3 / 8.2, 4096 18.4 / 16.4,
 // 6000 26.7 / 27.0, with a record 256 10.7 / 9.9, 3000 16.8 / 16.2, 4096 18.9 / 20.1; int8 512 14.4 / 12.3,
-// 576 14.4 / 16.4, with a record strips everywhere (14.8 / 20.6 at 512).
+// 576 14.4 / 16.4, with a record strips everywhere (14.8 / 20.6 at 512).  Below 128 packed strips
+// with a record win where they are few (7 to 15 of 86 to 128 rows: 7.3 to 8.6 / 9.0) and lose where the
+// time model takes more and thinner ones (96, 102, 114, 126: 10.3 / 9.0).
 bool one_sweep_as_halves(const ising_ctx* c, bool recorded) {
   if (c->strip.G <= 1 || c->strip_asked) return false;
   if (c->layout == ISING_LAYOUT_I8) return !recorded && c->L < 544;
-  return c->L > 128 && c->L < (recorded ? 3584 : 5632);
+  return (c->L > 128 || (recorded && c->strip.G > 15)) && c->L < (recorded ? 3584 : 5632);
 }
 
 // Kernel configuration validity for this lattice.

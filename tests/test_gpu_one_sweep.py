@@ -60,6 +60,17 @@ def test_one_sweep_a_call(L, layout):
     assert auto < 1.07 * half, (auto, half)
 
 
+@pytest.mark.parametrize("L", [90, 96, 114, 126, 128, 256])
+def test_one_recorded_sweep_a_call(L):
+    import torch
+
+    with ising.Lattice(L, 0.44, BITS, seed=1, stream=torch.cuda.current_stream()) as lat:
+        auto = _us(lambda: lat.sweep(1, 1))
+        lat.set_kernel(ising.ISING_KERNEL_HALF)
+        half = _us(lambda: lat.sweep(1, 1))
+    assert auto < 1.07 * half, (auto, half)
+
+
 @pytest.mark.parametrize("L,every,mode", [(64, 0, 1), (512, 0, 1), (1024, 0, 1), (32, 1, 2)])
 def test_one_xy_sweep_a_call(L, every, mode):
     import torch
