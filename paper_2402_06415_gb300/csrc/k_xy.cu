@@ -916,12 +916,14 @@ cudaError_t xy_persist_t(ising_xy* x, int n, int m) {
 
 // Single-precision calls of one sweep that the strips make slower than the forms before
 // them.  us per call: half sweeps / strips (which clear their exchange buffer first) L = 64 8.2 /
-// 10.3, 512 12.3 / 14.4, 1024 20.5 / 22.6; with a record, one CTA: separate measurement / in the
-// sweep L = 32 10.3 / 11.4 (FP64: at most even).
+// 10.3, 512 12.3 / 14.4, 1024 20.5 / 22.6; with a record, one CTA or one cluster: separate measurement /
+// in the sweep L = 8 6.2 / 6.9, 10 to 20 8.2 / 6.9, 32 10.3 / 11.4, on strips 48 12.3 / 11.4, 50 11.3 / 12.5, 64 11.4 / 12.5, 72 12.3 /
+// 12.6, 80 13.3 / 12.4 (FP64: at most even).
 int xy_one_sweep_mode(const ising_xy* x, bool recorded) {
   if (x->mode != 0 || x->precision != 32) return x->mode;
   if (x->strip_G > 1 && !recorded) return 1;
-  return x->strip_G == 1 && recorded && x->L > 24 ? 2 : 0;
+  if (!recorded) return 0;
+  return x->L < 10 || (x->strip_G == 1 && x->L > 24) || (x->L >= 50 && x->L <= 72) ? 2 : 0;
 }
 
 template <typename T>

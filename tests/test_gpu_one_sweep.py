@@ -71,7 +71,7 @@ def test_one_recorded_sweep_a_call(L):
     assert auto < 1.07 * half, (auto, half)
 
 
-@pytest.mark.parametrize("L,every,mode", [(64, 0, 1), (512, 0, 1), (1024, 0, 1), (32, 1, 2)])
+@pytest.mark.parametrize("L,every,mode", [(64, 0, 1), (512, 0, 1), (1024, 0, 1), (8, 1, 2), (32, 1, 2), (50, 1, 2), (64, 1, 2)])
 def test_one_xy_sweep_a_call(L, every, mode):
     import torch
 
