@@ -675,9 +675,20 @@ cudaError_t persist_dispatch(ising_quad* x, int n, int m, const RngParams& rng) 
   return cudaErrorInvalidValue;
 }
 
+// Calls of few sweeps that one CTA finishes before strips, which are launched cooperatively and
+// clear their exchange buffer first.  us per call, strips / one CTA: one sweep, 4.8.8 Lc = 65 10.3 / 8.3, 128 12.3 /
+// 10.1, 129 11.3 / 12.3; square J2 = 0 66 11.7 / 8.3, 128 14.3 / 12.3, 129 11.4 / 16.2; J2 = 0.5 66 16.0 / 12.3, 96 14.4 / 14.4, 97 14.4 /
+// 18.4; two sweeps, in the same order, 84 12.4 / 10.3, 14.6 / 14.4, 22.7 / 20.5, 89 12.3 / 12.4, 14.5 / 16.5, 22.6 /
+// 26.6; three at 76 15.9 / 14.4, 19.9 / 18.5, 32.3 / 28.7; five 20.5 / 20.5, 28.3 / 28.0, 47.1 / 44.8, 20 strips from 65 on.
+bool quad_one_cta(const ising_quad* x, int n) {
+  if (n > 3) return false;
+  const bool many_classes = x->lattice == ISING_QUAD_SQUARE && x->tab.n_vals > 2;
+  return x->Lc < (n > 1 ? 88 : many_classes ? 97 : 129);
+}
+
 cudaError_t quad_sweeps(ising_quad* x, int n, int m) {
   const RngParams rng = make_rng(x->seed, x->replica, 0, 0);
-  if (x->strip_G > 0 && n > 0) {
+  if (x->strip_G > 0 && n > 0 && !quad_one_cta(x, n)) {
     // chunks whose records fit the ring, of about 20 ms
     const int launch = strip_launch_sweeps(x->strip_us);
     const int most = m > 0 ? (int)std::min<int64_t>(kQuadRec * (int64_t)m, launch) : launch;

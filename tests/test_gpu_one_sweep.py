@@ -88,3 +88,34 @@ def test_strips_that_are_asked_for_run_single_sweeps_too():
         before = ising.ising_launch_count(lat.ctx)
         lat.sweep(1)
         assert ising.ising_launch_count(lat.ctx) == before + 1
+
+
+# a context whose strips are refused when they are first used runs one CTA from then on
+@pytest.mark.parametrize("lattice,J2", [(ising.ISING_QUAD_SQOCT, 1.0), (ising.ISING_QUAD_SQUARE, 0.0), (ising.ISING_QUAD_SQUARE, 0.5)])
+@pytest.mark.parametrize("Lc,n", [(66, 1), (96, 1), (128, 1), (76, 2), (84, 2), (76, 3)])
+def test_few_quad_sweeps_a_call(lattice, J2, Lc, n, monkeypatch):
+    import torch
+
+    us = []
+    for refuse in (False, True):
+        if refuse:
+            monkeypatch.setenv("ISING_FAULT", "coop")
+        with ising.Quad(lattice, Lc, 0.44, 1.0, J2, seed=1, stream=torch.cuda.current_stream()) as x:
+            monkeypatch.delenv("ISING_FAULT", raising=False)
+            x.sweep(5, 0)
+            us.append(_us(lambda: x.sweep(n, 0)))
+    assert us[0] < 1.07 * us[1], us
+
+
+def test_few_and_many_quad_sweeps_are_one_chain():
+    import numpy as np
+
+    for Lc in (66, 87, 96, 127, 128):
+        with ising.Quad(ising.ISING_QUAD_SQUARE, Lc, 0.44, 1.0, 0.0, seed=4) as x, \
+                ising.Quad(ising.ISING_QUAD_SQUARE, Lc, 0.44, 1.0, 0.0, seed=4) as y:
+            for n in (1, 2, 3, 4, 1, 9):
+                x.sweep(n, 2)
+            y.sweep(20, 2)
+            assert np.array_equal(x.spins(), y.spins())
+            for a, b in zip(x.series(10), y.series(10)):
+                assert np.array_equal(a, b)
