@@ -681,9 +681,9 @@ cudaError_t persist_dispatch(ising_quad* x, int n, int m, const RngParams& rng) 
 // 18.4; two sweeps, in the same order, 84 12.4 / 10.3, 14.6 / 14.4, 22.7 / 20.5, 89 12.3 / 12.4, 14.5 / 16.5, 22.6 /
 // 26.6; three at 76 15.9 / 14.4, 19.9 / 18.5, 32.3 / 28.7; five 20.5 / 20.5, 28.3 / 28.0, 47.1 / 44.8, 20 strips from 65 on.
 bool quad_one_cta(const ising_quad* x, int n) {
-  if (n > 3) return false;
-  const bool many_classes = x->lattice == ISING_QUAD_SQUARE && x->tab.n_vals > 2;
-  return x->Lc < (n > 1 ? 88 : many_classes ? 97 : 129);
+  const bool more_classes = x->tab.n_vals > 2;
+  if (n > (more_classes ? 5 : 3)) return false;
+  return x->Lc < (n > 1 ? 88 : more_classes && x->lattice == ISING_QUAD_SQUARE ? 97 : 129);
 }
 
 cudaError_t quad_sweeps(ising_quad* x, int n, int m) {

@@ -92,7 +92,7 @@ def test_strips_that_are_asked_for_run_single_sweeps_too():
 
 # a context whose strips are refused when they are first used runs one CTA from then on
 @pytest.mark.parametrize("lattice,J2", [(ising.ISING_QUAD_SQOCT, 1.0), (ising.ISING_QUAD_SQUARE, 0.0), (ising.ISING_QUAD_SQUARE, 0.5)])
-@pytest.mark.parametrize("Lc,n", [(66, 1), (96, 1), (128, 1), (76, 2), (84, 2), (76, 3)])
+@pytest.mark.parametrize("Lc,n", [(66, 1), (96, 1), (128, 1), (76, 2), (84, 2), (76, 3), (76, 5)])
 def test_few_quad_sweeps_a_call(lattice, J2, Lc, n, monkeypatch):
     import torch
 
