@@ -27,9 +27,10 @@
 // The windows of all stages are dealt to the CTAs in contiguous ranges of equal
 // estimated work, so a CTA builds the tables of one or two stages.
 //
-// What bounds it: the two gathered contractions, whose ldmatrix traffic (the
-// weights are read again by every warp) and mma.sync rate (8 cycles per
-// m16n8k16 and sub-partition) are about equal, and the barriers between phases.
+// What bounds it: the barriers between phases and the latency of ldmatrix, with 4
+// warps a sub-partition (stalls per instruction: barrier 2.6, fixed latency 2.2, shared
+// memory 2.0); the tensor pipe is 29 % busy, the load / store unit, through which every warp
+// reads the weights again, 18 %.  128 registers, 100 bytes of them spilled.
 // 512 windows x 8 stages: kernel 1520 -> 192 us, loss and gradients through the
 // API 1560 -> 236 us (before: full frames, one sample at a time, and one thread
 // listing the loss sites).

@@ -345,8 +345,9 @@ __global__ void __launch_bounds__(1024) k_quad_persist(uint32_t* __restrict__ pl
 // further than the second on the side it does not read from.  The halo has
 // H = K + 1 rows, because the bond sums of a recorded sweep read one row beyond
 // the strip.
-// Bound by the dependent chain of a quarter sweep (~0.6 us) up to 512^2 cells, then by
-// issue slots.  us per sweep, before (one CTA up to 256^2 cells, else a launch per
+// Bound by the dependent chain of a quarter sweep (~0.6 us) up to 1024^2 cells (there two
+// warps a sub-partition, ALU pipe 40 % busy), then by the ALU pipe.  The 4.8.8 form for up to
+// 8 classes spills 56 bytes at its 64 registers.  us per sweep, before (one CTA up to 256^2 cells, else a launch per
 // quarter sweep) and with strips: 4.8.8 at 256^2 19.5 -> 2.7, 1024^2 16.5 -> 4.5, 4096^2
 // 49.8 -> 34.5; square J2 = 0.5 at 1024^2 24.7 -> 8.8.  8192^2 does not fit and keeps
 // the launches (152 us, ALU pipe bound).
